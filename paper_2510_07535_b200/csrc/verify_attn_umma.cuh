@@ -91,6 +91,14 @@ struct Segment {
     }
     __device__ __forceinline__ int tile(int s, int i) const { return tile0 + (shared ? i : 2 * i + s); }
     __device__ __forceinline__ bool whole() const { return tile0 == 0 && tile1 == tiles; }
+    // Warps of a stream's warpgroup that hold a row of a unit of up to 128 rows (both streams hold the same ones).  The
+    // others take no part in the key loop.  A chain of 8 nodes x 4 heads fills one warp of four: its three idle warps used
+    // to weigh 96 zero rows a tile, and their weights of 1 kept the multipliers of P V busy; left alone, those rows of P
+    // stay the zeros that the zero rows of Q gave S (16 mixed sequences 756 -> 738 us, 48 short ones 180 -> 176 us per
+    // step).  The instances for units above 128 rows keep every warp: there a hand-off barrier whose count is not an
+    // immediate costs the issuing warp more than the rare idle warp (4 x 64 nodes 631 -> 642 us).
+    template <bool kWide>
+    __device__ __forceinline__ int live_warps() const { return kWide ? 4 : (M + 31) >> 5; }
 };
 
 // Walks the CTA's piece [t, t_end) of the flat tile range unit by unit.  Every role runs its own
@@ -344,6 +352,8 @@ __device__ __forceinline__ void mma_loop(const AttnParams& p, Aux* aux, uint32_t
         if (!__any_sync(kAll, more)) break;
         const int tile0 = __reduce_max_sync(kAll, g.tile0), tile1 = __reduce_max_sync(kAll, g.tile1);
         const bool shared = kWide && __reduce_max_sync(kAll, g.shared ? 1 : 0) != 0;
+        // threads on the hand-off barrier of P: a stream's live softmax warps and this one
+        const int p_threads = kWide ? 160 : 32 + 32 * __reduce_max_sync(kAll, g.template live_warps<kWide>());
         bool ok = __all_sync(kAll, mbar_wait(smem_u32(&aux->q_full), seg_no & 1u, abort_flag));
         const int T = tile1 - tile0;
         const int n_it[2] = {shared ? T : (T + 1) >> 1, shared ? T : T >> 1};
@@ -420,7 +430,7 @@ __device__ __forceinline__ void mma_loop(const AttnParams& p, Aux* aux, uint32_t
             for (int s = 0; s < 2; ++s) {
                 const bool last_reader = !shared || s == 1;
                 const bool do_pv = i >= 0 && i < n_it[s], do_qk = i + 1 < n_it[s];
-                if (do_pv) asm volatile("bar.sync %0, 160;" ::"r"(4 + s) : "memory");
+                if (do_pv) asm volatile("bar.sync %0, %1;" ::"r"(4 + s), "r"(p_threads) : "memory");
                 if (i < 0 && do_qk && !(shared && s == 1)) {
                     const uint32_t seq = (item_base >> 1) + (uint32_t)s;
                     ok = __all_sync(kAll, mbar_wait(smem_u32(&aux->full[seq % kTilesInFlight]),
@@ -450,7 +460,7 @@ __device__ __forceinline__ void mma_loop(const AttnParams& p, Aux* aux, uint32_t
                 const uint32_t issue = ok ? elected : 0u;
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
-                    asm volatile("bar.sync %0, 160;" ::"r"(4 + s) : "memory");
+                    asm volatile("bar.sync %0, %1;" ::"r"(4 + s), "r"(p_threads) : "memory");
                     tc_fence_after();
                     issue_pv(s, issue, i > 0 ? 1u : 0u);
                     if (!shared || s == 1) umma_commit_if(issue, smem_u32(&aux->empty[v_slot[s]]));
@@ -597,11 +607,13 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         const unsigned long long anc_row = rr < g.M ? aux->anc[rr / G] : 0ull;
         const bool bad_tree = aux->seg_bad_tree != 0;
         const int n_it = g.iters(s);
+        const int live = g.template live_warps<kWide>();
+        const bool idle = (wtid >> 5) >= live;       // no row of the unit in this warp: straight to the segment's end
         float m = -INFINITY, l = 0.f, lx = 0.f;   // l: sum of the bf16 weights (normaliser); lx: exact sum (LSE)
 
-        for (int i = 0; i < n_it; ++i) {
+        for (int i = 0; i < (idle ? 0 : n_it); ++i) {
             const int t = g.tile(s, i);
-            mbar_wait(smem_u32(&aux->s_full[s]), it & 1u, abort_flag);
+            mbar_wait(smem_u32(&aux->s_full[s]), (it + i) & 1u, abort_flag);
             tc_fence_after();
             if ((t + 1) * kTileKeys > g.L) {
                 // The tile reaches drafted positions (or the end of the sequence): at most two tiles per unit.
@@ -641,7 +653,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
                     const uint32_t seq = tile_base + (uint32_t)(g.shared ? i : 2 * i + s);
                     unsigned char* vslot = smem + kRingOff + ((2u * seq + 1u) % kSlots) * kSlotBytes;
 #pragma unroll 1
-                    for (int k = kv_valid + (wtid >> 4); k < kv_end; k += 8)   // 16 threads x 16 bytes per 256-byte row
+                    for (int k = kv_valid + (wtid >> 4); k < kv_end; k += 2 * live)   // 16 threads x 16 bytes per 256-byte row
                         *reinterpret_cast<uint4*>(vslot + (k >> 3) * 2048 + ((wtid >> 3) & 1) * 1024 + (k & 7) * 128 +
                                                   (wtid & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
                     fence_proxy_async_smem();
@@ -788,10 +800,10 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             }
             tmem_wait_st();
             tc_fence_before();
-            // Hand-off of P: hardware barrier 4 + s, 160 threads (this warpgroup + the MMA warp).  Executed once per
+            // Hand-off of P: hardware barrier 4 + s, the live warps of this warpgroup + the MMA warp.  Executed once per
             // key tile of this stream - n_it times per segment, the count of the MMA warp's bar.sync on it - on every
             // path: nothing above leaves the loop body early, and a wait that gave up only changed what was computed.
-            asm volatile("bar.arrive %0, 160;" ::"r"(4 + s) : "memory");
+            asm volatile("bar.arrive %0, %1;" ::"r"(4 + s), "r"(32 * live + 32) : "memory");
             // In a unit of more than 128 rows the MMA warp polls no mbarrier between O += P V of this tile and
             // S = Q K^T of the next one: the first warp of the warpgroup looks at that tile's arrival barrier for it
             // (after P is announced, so that nothing this tile holds is released any later) and passes the news on
@@ -804,11 +816,15 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
                 // T - 1 times, matching the MMA warp's bar.sync 6 before S of tiles 1 .. T - 1; unconditional
                 asm volatile("bar.arrive 6, 64;" ::: "memory");
             }
-            ++it;
         }
+        it += (uint32_t)n_it;
 
         // ---- segment end: every product of this stream has completed
-        if (n_it > 0) { mbar_wait(smem_u32(&aux->o_done[s]), od_phase & 1u, abort_flag); ++od_phase; }
+        // (an idle warp sleeps on the hardware barrier below instead; it reads nothing)
+        if (n_it > 0) {
+            if (!idle) mbar_wait(smem_u32(&aux->o_done[s]), od_phase & 1u, abort_flag);
+            ++od_phase;
+        }
         tc_fence_after();
         // split mode: the streams exchange (m, l, lx) through the second Q block, which only the shared mode uses
         float (*ml)[128][3] = reinterpret_cast<float (*)[128][3]>(smem + kQBytes);
@@ -850,6 +866,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             write_lse = s == 0;
             c_first = 2 * s; c_count = 2;
         }
+        if (idle) c_count = 0;
 #pragma unroll 1
         for (int c4 = c_first; c4 < c_first + c_count; ++c4) {
             uint32_t oa[32], ob[32];

@@ -1,30 +1,38 @@
-// Weight-streaming product C[M, N] = A[M, K] B[N, K]^T on the 5th-generation tensor cores (bf16 operands,
-// fp32 accumulators in tensor memory), for the two producers either side of the verify step:
-//   LM head     A = hidden states of the drafted nodes [nodes, 4096], B = head weight [vocab, 4096]; the epilogue
-//               keeps of every row only its arg-max over the vocabulary - the logits are never written;
+// Weight-streaming product C[M, N] = A[M, K] B[N, K]^T on the 5th-generation tensor cores (bf16 operands, fp32
+// accumulators in tensor memory), for the two producers either side of the verify step:
+//   LM head     A = hidden states of the drafted nodes [nodes, K], B = head weight [vocab, K]; the epilogue keeps of every
+//               row of A only its arg-max over the vocabulary - the logits are never written;
 //   drafter     A = h [rows, d_in], B = [W^f; W^i; W^o; W^c] ([4d, d_in]), Eq. 2; the epilogue stores fp32.
-// M is small (up to 384 rows: 1 to 3 blocks of 128), N is huge: B is read from HBM exactly once, A comes again and
-// again out of L2.  One persistent CTA per SM takes column tiles of C round-robin:
-//   warp 0     TMA producer: per 64-wide k-block one box per row block of A and one or two boxes of B into a ring
-//   warp 1     issues the tcgen05.mma (one thread): per k-block 4 k-steps x row blocks, 128 x width x 16 each
-//   warps 4-7  epilogue, thread = row: reads its accumulators of every row block and reduces or stores them
-// Tile width.  A 128 x 128 x 16 instruction reads 4 KB of A and 4 KB of B from shared memory in its 64 clocks, which
-// together with the TMA writes is more than the 128 B / clock shared memory delivers: two row blocks ran at 875
-// clocks per k-block for 512 of tensor-pipe time.  A 128 x 256 x 16 instruction reads 12 KB in 128 clocks, so up to
-// two row blocks take tiles of up to 256 columns (all 512 columns of tensor memory as one accumulator buffer for two
-// row blocks, two buffers for one); three row blocks take up to 160 (3 x 160 = 480 columns: 7-9 % faster than 128).
-// Balance.  B is read once and every CTA streams at the same rate, so the columns are dealt out evenly: each CTA
-// gets ceil(N / 16 / CTAs) units of 16 columns, cut into as few tiles as the width limit allows, the tiles of one
-// round equally wide on every CTA (widths differ by at most 16 between rounds).  The instruction's N is the tile
-// width (any multiple of 16), one TMA box brings the tile's rows of B.  N = 49152 on 148 CTAs: rounds of 176 and
-// 160 columns, 98.8 % of the last round filled, against 65 % with 256-wide tiles only.
-// Ring.  At 6.5 TB/s over 148 SMs and 2.5-3 us of loaded memory latency a CTA needs 110-130 KB of B in flight, so a
-// stage holds what is loaded and nothing else: the tile's rows of B and the valid rows of A rounded up to 8 (one
-// swizzle atom).  The instruction still reads 128 rows of A: past the loaded ones it finds whatever follows in
-// shared memory (the stage's B, the next stage, the pad behind the ring), which only feeds accumulator rows >= M that
-// nobody reads - an output row depends on its own row of A alone.  10 rows against 176 of B: 24 KB per stage, 8
-// stages, 176 KB in flight (with 48 KB stages there were 88 KB in flight and the product ran at 4.2 TB/s).
-// Every wait is bounded as in the attention kernel.
+// M is small (up to 384 rows), N is huge: B is read from HBM exactly once, A comes again and again out of L2.
+//
+// The WEIGHTS are the instruction's M operand: the accumulator is C^T, one row of B per lane of tensor memory, one row of
+// A (rounded up to 16) per column.  What bounds the product is B's bytes and, run in a loop, the board's power.  With A as
+// the M operand every instruction multiplied 128 rows however few exist: at 30 rows and 6 TB/s the tensor cores did the
+// work of an 800 TFLOP/s product, three quarters of it on rows that nobody reads, and the power cap took the SM clock from
+// 1965 to 1140 MHz, which slows the memory system as well.
+//
+// CTA pairs (cta_group::2) at every M: two CTAs on neighbouring SMs run one tcgen05.mma of M = 256 together.  CTA r stages
+// half of the tile's rows of B (its own 128 accumulator lanes) and half of A's rows, so A is staged once per 256 rows of
+// B and per SM half as often; each SM's tensor memory holds two accumulator buffers, so the epilogue of a tile hides under
+// the next tile's products.  One thread issues for two SMs, and its time is the other limit: a wait, a commit and the loop
+// around them cost it some 800 clocks a stage when written plainly (divisions by the ring's length, 64-bit descriptor
+// arithmetic, one k-block a stage).  A stage holds two k-blocks (eight products per wait and commit), slot and phase run
+// along as counters, and each thread looks at its next barrier before it needs it.
+// Above 256 rows of A the accumulator is two groups of up to 192 columns in one buffer, a stage one k-block (the same
+// eight products).
+//
+// Measured (128256 x 4096 weights, us in a loop at the power cap; before = A as the M operand): 16 rows 192 -> 161, 32 rows
+// 195 -> 158, 64 rows 205 -> 163, 96 rows 195 -> 172, 128 rows 203 -> 183, 144 rows 281 -> 216, 192 rows 279 -> 233,
+// 256 rows 286 -> 273.  One CTA per SM instead of pairs: 162 / 163 / 175 / 185 / 193 us at 16 / 32 / 64 / 96 / 128 rows.
+//
+// Balance.  Every pair gets ceil(N / 16 / pairs) units of 16 rows of B, cut into as few tiles of at most 256 as
+// possible, the tiles of one round equally high on every pair (heights differ by at most 16 between rounds).
+// Ring.  At 6.5 TB/s over 148 SMs and 2.5-3 us of loaded memory latency a CTA needs 110-130 KB of B in flight, so a stage
+// holds the tile's rows of B and A's rows and nothing else; a 128-row window on fewer rows runs on into whatever follows
+// in shared memory, which feeds accumulator lanes that nobody reads.
+// Roles (256 threads): warp 0 TMA producer (copies complete on the EVEN CTA's arrival barrier; no multicast), warp 1 of the
+// even CTA issues, warps 4-7 epilogue (thread = lane of tensor memory = row of B).  Every wait is bounded; a wait that
+// gives up raises both CTAs' abort flags.
 #pragma once
 
 #include <cuda.h>
@@ -41,25 +49,26 @@ namespace gemm_path {
 
 using namespace sm100;
 
-constexpr int kBM = 128, kBN = 128, kBK = 64;
-constexpr int kThreads = 256;
-constexpr int kTileBytes = kBM * kBK * 2;        // 16 KB: 128 rows of one 128-byte swizzle row each
-constexpr int kMaxRowBlocks = 3;
-constexpr int kMaxStages = 12;
-constexpr int kAuxBytes = 1024;
-constexpr int kSmemLimit = 232448;               // 227 KB
-
 enum Epilogue { kEpiArgmax = 0, kEpiStore = 1 };
+
+constexpr int kBK = 64;                          // a k-block: one 128-byte swizzle row per operand row
+constexpr int kThreads = 256;
+constexpr int kWindowBytes = 128 * kBK * 2;      // what an instruction reads of one CTA's rows of B: 16 KB
+constexpr int kMaxStages = 8;
+constexpr int kAuxBytes = 4096;
+constexpr int kSmemLimit = 232448;               // 227 KB
+constexpr int kMaxTile = 256;                    // rows of B per tile, both CTAs
+constexpr int kMaxRows = 384;                    // rows of A
+constexpr int kGroupRows = 256;                  // rows of A in one column group; above, two groups
 
 struct GemmParams {
     int M, N, K;
-    int row_blocks;                 // ceil(M / 128)
-    int stages;                     // ring depth: what fits beside the aux area and the pad
-    int a_bytes;                    // per stage: full row blocks of 16 KB, then the last block's rows rounded up to 8
-    int stage_bytes;                // a_bytes + the widest tile's rows of B, 128 bytes each
-    int rounds;                     // tiles per CTA; round t holds one tile per CTA, all of the same width
-    int wide_rounds;                // rounds [0, wide_rounds) are w_lo + 16 columns wide, the others w_lo
-    int w_lo;                       // multiple of 16, <= 256 (160 with three row blocks)
+    int group_rows;                 // rows of A per column group, a multiple of 16: the instruction's N
+    int stages;
+    int block_bytes;                // a k-block of a stage: this CTA's rows of B, then its rows of A, 128 bytes each
+    int rounds;                     // tiles per pair; all tiles of a round are equally high
+    int tall_rounds;                // rounds [0, tall_rounds) are h_lo + 16 rows of B high, the others h_lo
+    int h_lo;                       // multiple of 16, <= 256
     int32_t* status;
     unsigned long long* row_key;    // kEpiArgmax: [M] keys (value, ~column), raised by atomicMax; cleared by the caller
     float* c;                       // kEpiStore: fp32 [M, ldc]
@@ -67,201 +76,255 @@ struct GemmParams {
 };
 
 struct Aux {
-    uint64_t full[kMaxStages], empty[kMaxStages];
-    uint64_t acc_full[2], acc_empty[2];
+    uint64_t full[kMaxStages], empty[kMaxStages];   // `full` is used in the even CTA only
+    uint64_t acc_full[2], acc_empty[2];             // `acc_empty` is used in the even CTA only (256 arrivals)
+    unsigned long long best[kMaxRows];              // kEpiArgmax: the CTA's best key per row of A
     uint32_t tmem_base;
     int abort_flag;
 };
 static_assert(sizeof(Aux) <= kAuxBytes, "aux area too small");
 
-// up to two row blocks take tiles of 256 columns, three of 128 (tensor memory: row blocks x width <= 512 columns)
-// widest tile: row blocks x width columns of fp32 accumulators must fit the 512 columns of tensor memory
-__host__ __device__ inline int max_tile_width(int row_blocks) { return row_blocks <= 2 ? 256 : 160; }
-// shared memory: [aux][stages x stage_bytes][pad: the A operand window of the last stage may reach one tile past it]
-__host__ inline int ring_stages(int stage_bytes) {
-    const int s = (kSmemLimit - kAuxBytes - kTileBytes) / stage_bytes;
+// k-blocks per stage for one or two column groups: eight products either way
+__host__ __device__ constexpr int stage_kblocks(int groups) { return groups == 1 ? 2 : 1; }
+__host__ inline int ring_stages(int groups, int block_bytes) {
+    const int s = (kSmemLimit - kAuxBytes - kWindowBytes) / (stage_kblocks(groups) * block_bytes);
     return s < kMaxStages ? s : kMaxStages;
 }
-__host__ inline int smem_bytes(int stages, int stage_bytes) { return kAuxBytes + stages * stage_bytes + kTileBytes; }
-
-// 2-D tile load global -> shared with an L2 cache policy, completion counted in bytes on an mbarrier of this CTA.
-__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
-        : : "r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "l"(policy) : "memory");
+// (the pad behind the ring: the window of the last stage may reach one window past it)
+__host__ inline int smem_bytes(int groups, int stages, int block_bytes) {
+    return kAuxBytes + stages * stage_kblocks(groups) * block_bytes + kWindowBytes;
 }
+
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
+// .cta_group::2 form of the tile copy: destination in this CTA, completion counted on `bar_cluster`, a
+// shared::cluster address that may lie in the peer CTA.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* tmap, uint32_t bar_cluster, int c0, int c1, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+        : : "r"(dst), "l"(tmap), "r"(bar_cluster), "r"(c0), "r"(c1), "l"(policy) : "memory");
+}
 
-template <int kEpi>
-__global__ void __launch_bounds__(kThreads, 1)
-gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap amap_last,
-                 const __grid_constant__ CUtensorMap bmap_hi, const __grid_constant__ CUtensorMap bmap_lo) {
+// The arg-max of 32 columns (rows of A) over a warp's 32 lanes (rows of B): lane j gets column j's key.  `hi` of a lane
+// without a row of B is 0, below every real value's image.
+__device__ __forceinline__ unsigned long long warp_column_argmax(const uint32_t (&v)[32], bool lane_valid, uint32_t row0) {
+    const int lane = threadIdx.x & 31;
+    uint32_t best = 0u, who = 0u;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const uint32_t hi = lane_valid ? (uint32_t)(argmax_key(__uint_as_float(v[j]), 0u) >> 32) : 0u;
+        const uint32_t m = __reduce_max_sync(0xffffffffu, hi);
+        const uint32_t first = (uint32_t)__ffs((int)__ballot_sync(0xffffffffu, hi == m)) - 1u;   // lowest row of B among equals
+        if (lane == j) { best = m; who = first; }
+    }
+    return best ? ((unsigned long long)best << 32) | (uint32_t)(~(row0 + who)) : 0ull;
+}
+
+// gridDim.x is even: CTAs 2j and 2j + 1 are pair j.
+template <int kEpi, int kGroups>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap_hi,
+                 const __grid_constant__ CUtensorMap bmap_lo) {
     extern __shared__ __align__(1024) unsigned char smem[];
+    constexpr int kQ = stage_kblocks(kGroups);
+    constexpr uint32_t kBufs = kGroups == 1 ? 2 : 1;    // accumulator buffers
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t smem_base = smem_u32(smem) + kAuxBytes;       // the ring
-    const int rb = p.row_blocks, stages = p.stages;
-    const int sbytes = p.stage_bytes;
+    const uint32_t ring = smem_u32(smem) + kAuxBytes;
+    const int stages = p.stages, bbytes = p.block_bytes;
     Aux* aux = reinterpret_cast<Aux*>(smem);
     volatile int* abort_flag = &aux->abort_flag;
-    if (smem_base & 1023u) {                       // operand tiles must sit on swizzle-atom boundaries
-        if (tid == 0) report(p.status, kErrTimeout);
-        return;
-    }
+    const uint32_t rank = cluster_cta_rank();           // 0: issues the products; 1: its peer
+    const int pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
+    // the peer's abort flag: a wait that gives up here ends the peer's waits too
+    const uint32_t peer_abort = cluster_map(smem_u32(&aux->abort_flag), rank ^ 1u);
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        const bool ok = mbar_wait_cluster_ns(bar, parity, abort_flag, kWaitLimitNs);
+        if (!ok) st_cluster_u32(peer_abort, 1u);
+        return ok;
+    };
+    const bool misaligned = (ring & 1023u) != 0;       // operand tiles must sit on swizzle-atom boundaries (same in both CTAs)
     if (tid == 0) {
         for (int i = 0; i < stages; ++i) { mbar_init(smem_u32(&aux->full[i]), 1); mbar_init(smem_u32(&aux->empty[i]), 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&aux->acc_full[i]), 1); mbar_init(smem_u32(&aux->acc_empty[i]), 128); }
+        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&aux->acc_full[i]), 1); mbar_init(smem_u32(&aux->acc_empty[i]), 256); }
         aux->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&amap);
-        tma_prefetch_desc(&amap_last);
         tma_prefetch_desc(&bmap_hi);
         tma_prefetch_desc(&bmap_lo);
     }
-    if (warp == 0) { tmem_alloc(smem_u32(&aux->tmem_base), 512); tmem_relinquish(); }
+    if (kEpi == kEpiArgmax)
+        for (int i = tid; i < kMaxRows; i += kThreads) aux->best[i] = 0ull;
+    if (warp == 0 && !misaligned) { tmem_alloc_pair(smem_u32(&aux->tmem_base), 512); tmem_relinquish_pair(); }
     // may be launched as a programmatic dependent of the kernel before it in the stream: the set-up above touched no
     // input and ran beside that kernel's tail; from here on it has completed (a no-op in an ordinary launch).  The
     // kernel after this one may queue up in turn; it waits likewise before it reads anything.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();            // both CTAs' barriers are initialised and both halves of tensor memory allocated
     tc_fence_after();
+    if (misaligned) {
+        if (tid == 0) report(p.status, kErrTimeout);
+        return;
+    }
     const uint32_t tmem = aux->tmem_base;
     const int kblocks = p.K / kBK;
-    const int wmax = max_tile_width(rb);         // widest tile: 256 columns, 160 with three row blocks
-    const int nbuf = rb * wmax * 2 <= 512 ? 2 : 1; // accumulator buffers of rb x wmax columns each
-    // round t: one tile per CTA, the rounds' column bands one after the other; a tile that starts past N is empty
-    auto tile_width = [&](int t) { return t < p.wide_rounds ? p.w_lo + 16 : p.w_lo; };
-    auto tile_col0 = [&](int t) {
-        const int hi = t < p.wide_rounds ? t : p.wide_rounds;
-        return (int)gridDim.x * (hi * (p.w_lo + 16) + (t - hi) * p.w_lo) + (int)blockIdx.x * tile_width(t);
+    const int a_half = p.group_rows >> 1;                            // rows of a group of A that this CTA stages
+    // round t: one tile per pair, the rounds' bands of B one after the other; a tile that starts past N is empty
+    auto tile_rows = [&](int t) { return t < p.tall_rounds ? p.h_lo + 16 : p.h_lo; };
+    auto tile_row0 = [&](int t) {
+        const int hi = t < p.tall_rounds ? t : p.tall_rounds;
+        return pairs * (hi * (p.h_lo + 16) + (t - hi) * p.h_lo) + pair * tile_rows(t);
     };
+    const uint32_t full_bar = smem_u32(&aux->full[0]), empty_bar = smem_u32(&aux->empty[0]);
     uint32_t issued = 0;
 
     if (warp == 0) {
         if (lane == 0) {
             const uint64_t stream_policy = l2_policy_evict_first();   // B is read once
-            const uint64_t keep_policy = l2_policy_evict_last();      // A is read by every CTA for every tile
-            uint32_t it = 0;
+            const uint64_t keep_policy = l2_policy_evict_last();      // A is read by every pair for every tile
+            uint32_t stage = 0, ph = 1;
+            bool peek = true;                                         // the first pass over the ring finds it empty
             for (int t = 0; t < p.rounds; ++t) {
-                const int col0 = tile_col0(t), w = tile_width(t);
-                if (col0 >= p.N) break;
-                const CUtensorMap* bmap = t < p.wide_rounds ? &bmap_hi : &bmap_lo;   // box = the tile's w rows of B
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const uint32_t stage = it % stages, ph = (it / stages) & 1u;
-                    if (!mbar_wait(smem_u32(&aux->empty[stage]), ph ^ 1u, abort_flag)) continue;
-                    const uint32_t full = smem_u32(&aux->full[stage]);
-                    const uint32_t dst = smem_base + stage * sbytes;
-                    mbar_arrive_expect_tx(full, (uint32_t)(p.a_bytes + w * kBK * 2));
-                    for (int r = 0; r < rb; ++r)       // the last row block's box is as high as its valid rows (rounded up to 8)
-                        tma_load_2d_hint(dst + r * kTileBytes, r + 1 < rb ? &amap : &amap_last, full, kb * kBK, r * kBM, keep_policy);
-                    tma_load_2d_hint(dst + p.a_bytes, bmap, full, kb * kBK, col0, stream_policy);
-                    issued = it + 1;
+                const int row0 = tile_row0(t), share = tile_rows(t) >> 1;
+                if (row0 >= p.N) break;
+                const CUtensorMap* bmap = t < p.tall_rounds ? &bmap_hi : &bmap_lo;   // box = this CTA's half of the tile's rows
+                const int brow = row0 + (int)rank * share, arow = (int)rank * a_half;
+                // both CTAs' copies of a stage complete on the even CTA's barrier, which expects all their bytes
+                const uint32_t bytes = (uint32_t)(2 * kQ * (share + kGroups * a_half) * kBK * 2);
+                for (int kb = 0; kb < kblocks; kb += kQ) {
+                    if (peek || wait(empty_bar + stage * 8u, ph)) {
+                        const uint32_t full = full_bar + stage * 8u, full0 = cluster_map(full, 0);
+                        const uint32_t dst = ring + stage * (uint32_t)(kQ * bbytes);
+                        if (rank == 0) mbar_arrive_expect_tx(full, bytes);
+#pragma unroll
+                        for (int q = 0; q < kQ; ++q) {
+                            // (with an odd number of k-blocks the last stage's second one lies past K: the boxes read zeros)
+                            const int k0 = (kb + q) * kBK;
+                            uint32_t d = dst + q * bbytes;
+                            tma_load_2d_pair(d, bmap, full0, k0, brow, stream_policy);
+                            d += (uint32_t)share * (kBK * 2);
+#pragma unroll
+                            for (int g = 0; g < kGroups; ++g)
+                                tma_load_2d_pair(d + g * a_half * (kBK * 2), &amap, full0, k0, arow + g * p.group_rows, keep_policy);
+                        }
+                        ++issued;
+                    }
+                    if (++stage == (uint32_t)stages) { stage = 0; ph ^= 1u; }
+                    peek = mbar_try_wait_cluster(empty_bar + stage * 8u, ph);
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            uint32_t it = 0, tcount = 0;
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc = umma_idesc_16bit(256, p.group_rows, 0, 0, false);
+            const uint64_t desc0 = umma_smem_desc_sw128(ring, 16, 1024);     // operands differ in the start address only
+            const uint32_t desc_hi = (uint32_t)(desc0 >> 32), desc_lo = (uint32_t)desc0;
+            uint32_t stage = 0, ph = 0, tcount = 0;
+            bool peek = false;
             for (int t = 0; t < p.rounds; ++t, ++tcount) {
-                if (tile_col0(t) >= p.N) break;
-                const uint32_t buf = tcount % nbuf, acc_ph = (tcount / nbuf) & 1u;
-                const uint32_t idesc = umma_idesc_16bit(kBM, tile_width(t), 0, 0, false);
-                bool ok = mbar_wait(smem_u32(&aux->acc_empty[buf]), acc_ph ^ 1u, abort_flag);   // the epilogue has read this buffer
-                tc_fence_after();
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const uint32_t stage = it % stages, ph = (it / stages) & 1u;
-                    ok = mbar_wait(smem_u32(&aux->full[stage]), ph, abort_flag) && ok;
+                if (tile_row0(t) >= p.N) break;
+                const uint32_t buf = tcount % kBufs, acc_ph = (tcount / kBufs) & 1u;
+                const uint32_t a_off = (uint32_t)(tile_rows(t) >> 1) * (kBK * 2) >> 4, a_step = (uint32_t)a_half * (kBK * 2) >> 4;
+                const uint32_t d = tmem + buf * 256u;
+                bool ok = wait(smem_u32(&aux->acc_empty[buf]), acc_ph ^ 1u);      // both epilogues have read this buffer
+                for (int kb = 0; kb < kblocks; kb += kQ) {
+                    ok = (peek || wait(full_bar + stage * 8u, ph)) && ok;
                     tc_fence_after();
+                    const uint32_t used = empty_bar + stage * 8u;
+                    const uint32_t stage_lo = desc_lo + (stage * (uint32_t)(kQ * bbytes) >> 4);
+                    if (++stage == (uint32_t)stages) { stage = 0; ph ^= 1u; }
                     if (ok) {
-                        const uint32_t a0 = smem_base + stage * sbytes;
-                        const uint64_t bdesc = umma_smem_desc_sw128(a0 + p.a_bytes, 16, 1024);
-                        for (int r = 0; r < rb; ++r) {
-                            const uint64_t adesc = umma_smem_desc_sw128(a0 + r * kTileBytes, 16, 1024);
-                            const uint32_t d = tmem + buf * (uint32_t)(rb * wmax) + r * wmax;
 #pragma unroll
-                            for (int ks = 0; ks < kBK / 16; ++ks)    // 32 bytes along K inside the 128-byte swizzle row
-                                umma_ss(d, adesc + (uint64_t)(ks * 2), bdesc + (uint64_t)(ks * 2), idesc, (kb | ks) ? 1u : 0u);
+                        for (int q = 0; q < kQ; ++q) {
+                            const uint32_t b_lo = stage_lo + (uint32_t)(q * bbytes >> 4);
+#pragma unroll
+                            for (int g = 0; g < kGroups; ++g) {
+                                const uint32_t a_lo = b_lo + a_off + g * a_step;
+#pragma unroll
+                                for (int ks = 0; ks < kBK / 16; ++ks)    // 32 bytes along K inside the 128-byte swizzle row
+                                    umma_ss_pair_lh(d + g * 256u, b_lo + ks * 2, desc_hi, a_lo + ks * 2, desc_hi, idesc,
+                                                    (q | ks) ? 1u : (kb ? 1u : 0u));
+                            }
                         }
-                        umma_commit(smem_u32(&aux->empty[stage]));
+                        umma_commit_pair(used, 3);                       // the slot is free in both CTAs
                     }
+                    peek = mbar_try_wait_cluster(full_bar + stage * 8u, ph);
                 }
-                if (ok) umma_commit(smem_u32(&aux->acc_full[buf]));
+                if (ok) umma_commit_pair(smem_u32(&aux->acc_full[buf]), 3);
             }
         }
     } else if (warp >= 4) {
-        const int lane_row = (warp & 3) * 32 + lane;                    // TMEM lane = row inside a row block
         const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
+        const int chunks = (p.group_rows + 31) / 32;
         uint32_t tcount = 0;
         for (int t = 0; t < p.rounds; ++t, ++tcount) {
-            const int n0 = tile_col0(t);
-            if (n0 >= p.N) break;
-            const uint32_t buf = tcount % nbuf, acc_ph = (tcount / nbuf) & 1u;
-            const bool ok = mbar_wait(smem_u32(&aux->acc_full[buf]), acc_ph, abort_flag);
+            const int row0 = tile_row0(t);
+            if (row0 >= p.N) break;
+            const uint32_t buf = tcount % kBufs, acc_ph = (tcount / kBufs) & 1u;
+            const int share = tile_rows(t) >> 1;
+            const bool ok = wait(smem_u32(&aux->acc_full[buf]), acc_ph);
             tc_fence_after();
-            // columns [n0, n_end) are this tile's; a width that is an odd multiple of 16 leaves half of the last chunk
-            // of 32 unused (those columns of tensor memory hold another tile's or no data)
-            const int n_end = n0 + tile_width(t) < p.N ? n0 + tile_width(t) : p.N;
-            const int chunks = (tile_width(t) + 31) / 32;
-            for (int r = 0; r < rb; ++r) {
-                const int row = r * kBM + lane_row;
-                const uint32_t taddr = tmem + lane_sel + buf * (uint32_t)(rb * wmax) + r * wmax;
-                float bv = -INFINITY;
-                uint32_t bi = 0xffffffffu;
+            const int first = row0 + (int)rank * share;                 // this CTA's rows of B: [first, end)
+            const int end = first + share < p.N ? first + share : p.N;
+            const int warp_row = first + (warp & 3) * 32;               // row of B in the warp's lane 0
+            const bool lane_valid = warp_row + lane < end;
+            if (ok && warp_row < end) {
 #pragma unroll 1
-                for (int c4 = 0; c4 < chunks; ++c4) {
-                    uint32_t v[32];
-                    tmem_ld32(taddr + c4 * 32, v);
-                    tmem_wait_ld();
-                    if (!ok || row >= p.M) continue;
-                    const int col0 = n0 + c4 * 32;
-                    if (kEpi == kEpiArgmax) {
+                for (int g = 0; g < kGroups; ++g) {
+#pragma unroll 1
+                    for (int c4 = 0; c4 < chunks; ++c4) {
+                        // (a chunk's columns past the group's rows hold no data of this tile)
+                        const int a0 = g * p.group_rows + c4 * 32, left = min(p.M - a0, p.group_rows - c4 * 32);
+                        uint32_t v[32];
+                        tmem_ld32(tmem + lane_sel + buf * 256u + g * 256u + c4 * 32, v);
+                        tmem_wait_ld();
+                        if (kEpi == kEpiArgmax) {
+                            const unsigned long long key = warp_column_argmax(v, lane_valid, (uint32_t)warp_row);
+                            if (lane < left) atomicMax(&aux->best[a0 + lane], key);
+                        } else if (lane_valid) {
+                            float* dst = p.c + (long long)a0 * p.ldc + warp_row + lane;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            // NaN reads as -inf; strict '>' keeps the lowest column among equal values
-                            const float x = __uint_as_float(v[j]);
-                            const float e = x != x ? -INFINITY : x;
-                            if (col0 + j < n_end && (bi == 0xffffffffu || e > bv)) { bv = e; bi = (uint32_t)(col0 + j); }
-                        }
-                    } else {
-                        float* dst = p.c + (long long)row * p.ldc + col0;
-                        if (col0 + 32 <= n_end && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                reinterpret_cast<uint4*>(dst)[j] = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                        } else {
-                            for (int j = 0; j < 32 && col0 + j < n_end; ++j) dst[j] = __uint_as_float(v[j]);
+                            for (int j = 0; j < 32; ++j)
+                                if (j < left) dst[j * p.ldc] = __uint_as_float(v[j]);
                         }
                     }
                 }
-                if (kEpi == kEpiArgmax && ok && row < p.M && bi != 0xffffffffu) atomicMax(p.row_key + row, argmax_key(bv, bi));
             }
             tc_fence_before();
-            mbar_arrive(smem_u32(&aux->acc_empty[buf]));    // unconditional: the issuing thread's wait must end
+            // unconditional: the issuing thread's wait on the even CTA's barrier must end
+            mbar_arrive_cluster(cluster_map(smem_u32(&aux->acc_empty[buf]), 0));
+        }
+        if (kEpi == kEpiArgmax) {
+            asm volatile("bar.sync 1, 128;" ::: "memory");              // the four epilogue warps
+            for (int i = tid - 128; i < p.M; i += 128)
+                if (aux->best[i]) atomicMax(p.row_key + i, aux->best[i]);
         }
     }
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
-        if (aux->abort_flag) {
-            // give the copies still in flight a bounded time to land before the CTA's shared memory is released
-            if (lane == 0) {
-                const uint32_t first = issued > (uint32_t)stages ? issued - stages : 0u;
-                for (uint32_t it = first; it < issued; ++it) {
-                    const uint32_t bar = smem_u32(&aux->full[it % stages]), ph = (it / stages) & 1u;
-                    for (int polls = 0; polls < (1 << 20) && !mbar_try_wait(bar, ph); ++polls) {}
-                }
-                report(p.status, kErrTimeout);
+    if (aux->abort_flag && warp == 0 && lane == 0) {
+        if (rank == 0) {
+            // both CTAs' copies complete on this CTA's barriers: give those in flight a bounded time to land before
+            // either CTA's shared memory is released (the peer leaves only after the cluster barrier below)
+            const uint32_t first = issued > (uint32_t)stages ? issued - stages : 0u;
+            for (uint32_t it = first; it < issued; ++it) {
+                const uint32_t bar = smem_u32(&aux->full[it % stages]), ph = (it / stages) & 1u;
+                for (int polls = 0; polls < (1 << 20) && !mbar_try_wait_cluster(bar, ph); ++polls) {}
             }
-            __syncwarp();
         }
+        report(p.status, kErrTimeout);
+    }
+    // no CTA leaves while its peer may still send it an arrival or read or write its half of a product
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem, 512);
+        tmem_dealloc_pair(tmem, 512);
     }
 }
 

@@ -12,7 +12,7 @@
 
 #include "accept.cuh"
 #include "combine.cuh"
-#include "gemm_umma_pair.cuh"
+#include "gemm_umma.cuh"
 #include "owl_common.cuh"
 #include "spec_loop.cuh"
 #include "verify_attn_umma.cuh"
@@ -180,63 +180,35 @@ __global__ void selftest_wait_kernel(int32_t* status, unsigned long long limit_n
 
 // C[M, N] = A[M, K] B[N, K]^T on the tensor cores with one of the two epilogues (gemm_umma.cuh).
 template <int kEpi>
-static int launch_gemm(owl_ctx* ctx, const void* a, const void* b, int M, int N, int K, unsigned long long* row_key, float* c,
-                       long long ldc, cudaStream_t stream) {
-    gemm_path::GemmParams g{};
+int launch_gemm(owl_ctx* ctx, const void* a, const void* b, int M, int N, int K, unsigned long long* row_key, float* c,
+                long long ldc, cudaStream_t stream) {
+    using namespace gemm_path;
+    const int groups = M <= kGroupRows ? 1 : 2;
+    GemmParams g{};
     g.M = M; g.N = N; g.K = K;
-    g.row_blocks = (M + gemm_path::kBM - 1) / gemm_path::kBM;
+    g.group_rows = (M + 16 * groups - 1) / (16 * groups) * 16;
     g.status = ctx->status;
     g.row_key = row_key; g.c = c; g.ldc = ldc;
-    if (g.row_blocks == 2 && ctx->sm_count >= 2 && K % (2 * gemm_path::kBK) == 0) {
-        // 129 to 256 rows: CTA pairs (gemm_umma_pair.cuh).  The columns are dealt out to the pairs as to single CTAs
-        // below; a CTA stages half of a tile's rows of B.
-        const int units = (N + 15) / 16, max_pairs = ctx->sm_count / 2;
-        const int pairs = units < max_pairs ? units : max_pairs;
-        const int per_pair = (units + pairs - 1) / pairs;
-        g.rounds = (per_pair + 15) / 16;
-        g.w_lo = per_pair / g.rounds * 16;
-        g.wide_rounds = per_pair % g.rounds;
-        g.a_bytes = gemm_path::kTileBytes;
-        g.stage_bytes = 2 * (g.a_bytes + (g.w_lo + (g.wide_rounds ? 16 : 0)) / 2 * gemm_path::kBK * 2);   // two k-blocks
-        const int fit = (gemm_path::kSmemLimit - gemm_path::kAuxBytes) / g.stage_bytes;
-        g.stages = fit < gemm_path::kMaxStages ? fit : gemm_path::kMaxStages;
-        CUtensorMap amap, bmap_hi, bmap_lo;
-        const int ra = gemm_path::make_operand_map(ctx->encode, &amap, a, M, K, gemm_path::kBM);
-        int rb = gemm_path::make_operand_map(ctx->encode, &bmap_lo, b, N, K, g.w_lo / 2);
-        if (rb == 0) rb = g.wide_rounds ? gemm_path::make_operand_map(ctx->encode, &bmap_hi, b, N, K, (g.w_lo + 16) / 2) : (bmap_hi = bmap_lo, 0);
-        if (ra != 0 || rb != 0) {
-            snprintf(ctx->err, sizeof ctx->err, "cuTensorMapEncodeTiled failed (%d, %d): operands must be 16-byte aligned", ra, rb);
-            return OWL_ERR_CUDA;
-        }
-        launch_dependent_smem(gemm_path::gemm_umma_pair_kernel<kEpi>, dim3(2u * (unsigned)pairs), dim3(gemm_path::kThreads),
-                              (size_t)(gemm_path::kAuxBytes + g.stages * g.stage_bytes), stream, g, amap, bmap_hi, bmap_lo);
-        ++ctx->launches;
-        return OWL_OK;
-    }
-    // every CTA gets the same number of 16-column units, cut into as few tiles as the width limit allows
-    const int units = (N + 15) / 16;
-    const int grid = units < ctx->sm_count ? units : ctx->sm_count;
-    const int per_cta = (units + grid - 1) / grid;
-    const int wmax_units = gemm_path::max_tile_width(g.row_blocks) / 16;
-    g.rounds = (per_cta + wmax_units - 1) / wmax_units;
-    g.w_lo = per_cta / g.rounds * 16;
-    g.wide_rounds = per_cta % g.rounds;
-    // a stage: the rows of A that exist (the last row block rounded up to 8 rows) and the widest tile's rows of B
-    const int last_rows = (M - (g.row_blocks - 1) * gemm_path::kBM + 7) / 8 * 8;
-    g.a_bytes = (g.row_blocks - 1) * gemm_path::kTileBytes + last_rows * gemm_path::kBK * 2;
-    g.stage_bytes = g.a_bytes + (g.w_lo + (g.wide_rounds ? 16 : 0)) * gemm_path::kBK * 2;
-    g.stages = gemm_path::ring_stages(g.stage_bytes);
-    CUtensorMap amap, amap_last, bmap_hi, bmap_lo;
-    int ra = gemm_path::make_operand_map(ctx->encode, &amap, a, M, K, gemm_path::kBM);
-    if (ra == 0) ra = gemm_path::make_operand_map(ctx->encode, &amap_last, a, M, K, last_rows);
-    int rb = gemm_path::make_operand_map(ctx->encode, &bmap_lo, b, N, K, g.w_lo);
-    if (rb == 0) rb = g.wide_rounds ? gemm_path::make_operand_map(ctx->encode, &bmap_hi, b, N, K, g.w_lo + 16) : (bmap_hi = bmap_lo, 0);
+    // every pair gets the same number of 16-row units of B, cut into as few tiles as the height limit allows
+    const int units = (N + 15) / 16, max_pairs = ctx->sm_count / 2;
+    const int pairs = units < max_pairs ? units : max_pairs;
+    const int per_pair = (units + pairs - 1) / pairs;
+    g.rounds = (per_pair + kMaxTile / 16 - 1) / (kMaxTile / 16);
+    g.h_lo = per_pair / g.rounds * 16;
+    g.tall_rounds = per_pair % g.rounds;
+    const int h_hi = g.h_lo + (g.tall_rounds ? 16 : 0);
+    g.block_bytes = (h_hi + groups * g.group_rows) / 2 * kBK * 2;
+    g.stages = ring_stages(groups, g.block_bytes);
+    CUtensorMap amap, bmap_hi, bmap_lo;
+    const int ra = make_operand_map(ctx->encode, &amap, a, M, K, g.group_rows / 2);
+    int rb = make_operand_map(ctx->encode, &bmap_lo, b, N, K, g.h_lo / 2);
+    if (rb == 0) rb = g.tall_rounds ? make_operand_map(ctx->encode, &bmap_hi, b, N, K, h_hi / 2) : (bmap_hi = bmap_lo, 0);
     if (ra != 0 || rb != 0) {
         snprintf(ctx->err, sizeof ctx->err, "cuTensorMapEncodeTiled failed (%d, %d): operands must be 16-byte aligned", ra, rb);
         return OWL_ERR_CUDA;
     }
-    launch_dependent_smem(gemm_path::gemm_umma_kernel<kEpi>, dim3(grid), dim3(gemm_path::kThreads),
-                          (size_t)gemm_path::smem_bytes(g.stages, g.stage_bytes), stream, g, amap, amap_last, bmap_hi, bmap_lo);
+    launch_dependent_smem(groups == 1 ? gemm_umma_kernel<kEpi, 1> : gemm_umma_kernel<kEpi, 2>, dim3(2u * (unsigned)pairs),
+                          dim3(kThreads), (size_t)smem_bytes(groups, g.stages, g.block_bytes), stream, g, amap, bmap_hi, bmap_lo);
     ++ctx->launches;
     return OWL_OK;
 }
@@ -326,14 +298,12 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
              cudaFuncSetAttribute(combine_sched_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_) == cudaSuccess;
     }
     if (ok) {
-        ok = cudaFuncSetAttribute(gemm_path::gemm_umma_kernel<gemm_path::kEpiArgmax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  gemm_path::kSmemLimit) == cudaSuccess &&
-             cudaFuncSetAttribute(gemm_path::gemm_umma_kernel<gemm_path::kEpiStore>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  gemm_path::kSmemLimit) == cudaSuccess &&
-             cudaFuncSetAttribute(gemm_path::gemm_umma_pair_kernel<gemm_path::kEpiArgmax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  gemm_path::kSmemLimit) == cudaSuccess &&
-             cudaFuncSetAttribute(gemm_path::gemm_umma_pair_kernel<gemm_path::kEpiStore>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  gemm_path::kSmemLimit) == cudaSuccess;
+        using namespace gemm_path;
+        auto full_smem = [](auto* kernel) {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess;
+        };
+        ok = full_smem(gemm_umma_kernel<kEpiArgmax, 1>) && full_smem(gemm_umma_kernel<kEpiArgmax, 2>) &&
+             full_smem(gemm_umma_kernel<kEpiStore, 1>) && full_smem(gemm_umma_kernel<kEpiStore, 2>);
     }
     if (!ok || cudaDeviceSynchronize() != cudaSuccess) {
         cudaGetLastError();
@@ -665,7 +635,7 @@ int owl_lm_head_accept(owl_ctx* ctx, const owl_dims* d, int32_t hidden_dim, cons
     if (!hidden || !weight || !draft_tokens || !tree_parent || !accept_len || !accept_path || !bonus_token) return OWL_ERR_INVALID_ARG;
     if (!node_offsets && d->total_nodes % d->batch != 0) return OWL_ERR_INVALID_ARG;
     if (hidden_dim < gemm_path::kBK) return OWL_ERR_INVALID_ARG;
-    if (hidden_dim % gemm_path::kBK != 0 || d->total_nodes > gemm_path::kMaxRowBlocks * gemm_path::kBM) return OWL_ERR_UNSUPPORTED;
+    if (hidden_dim % gemm_path::kBK != 0 || d->total_nodes > gemm_path::kMaxRows) return OWL_ERR_UNSUPPORTED;
     if (!ctx->lm_keys || d->batch > ctx->max_dims.batch || d->total_nodes > ctx->max_dims.total_nodes) return OWL_ERR_TOO_LARGE;
     DeviceGuard guard(ctx->device);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
@@ -705,7 +675,7 @@ int owl_lstm_cell(owl_ctx* ctx, int32_t rows, int32_t d_in, int32_t d, const voi
                   float* z, float* h_out_f32, void* h_out_bf16, float* workspace, void* stream_) {
     if (!ctx || !h || !emb || !w || !z || !workspace || (!h_out_f32 && !h_out_bf16)) return OWL_ERR_INVALID_ARG;
     if (rows < 1 || d < 1 || d_in < gemm_path::kBK || !(eps >= 0.f) || alpha != alpha) return OWL_ERR_INVALID_ARG;
-    if (d_in % gemm_path::kBK != 0 || rows > gemm_path::kMaxRowBlocks * gemm_path::kBM || d > kCellMaxD ||
+    if (d_in % gemm_path::kBK != 0 || rows > gemm_path::kMaxRows || d > kCellMaxD ||
         d % 4 != 0)
         return OWL_ERR_UNSUPPORTED;
     DeviceGuard guard(ctx->device);

@@ -1,7 +1,8 @@
 """Kernel branches at the sizes where they can go wrong, against the CPU oracle (tolerances as in test_gpu_parity)."""
 import pytest
+import torch
 
-from paper_2510_07535_b200 import workloads as W
+from paper_2510_07535_b200 import OwlContext, make_dims, workloads as W
 from test_gpu_parity import check_attention
 
 pytestmark = pytest.mark.gpu
@@ -26,3 +27,24 @@ def test_units_that_fill_one_to_four_softmax_warps(nodes):
     wl = W.generate(W.Spec("live", 8, 2, [700 + nodes, 129, 40], [("chain", nodes)] * 3, page_size=64, shuffle_pages=True,
                            seed=700 + nodes, with_logits=False))
     check_attention(fill_dead_slots(wl))
+
+
+@pytest.mark.parametrize("rows,d_in", [(1, 64), (16, 192), (17, 64), (32, 320), (33, 192), (128, 192), (129, 64), (256, 192), (257, 64), (383, 192)])
+def test_product_row_padding_and_odd_k_blocks(rows, d_in):
+    """The weight-streaming product behind the drafter cell, element by element: rows around the padding to 16 and the
+    switch to two column groups (257), one, three and five k-blocks (a stage holds two), several tiles per CTA pair.
+    Bound: fp32 accumulation of K exact products, K 2^-24 sum_k |h_k| |w_k| per element."""
+    d = 4096 + 20
+    g = torch.Generator().manual_seed(rows)
+    h = torch.randn(rows, d_in, generator=g).bfloat16()
+    w = torch.randn(4 * d, d_in, generator=g).bfloat16()
+    emb = torch.zeros(rows, d, dtype=torch.bfloat16, device="cuda")
+    z, hf = torch.zeros(rows, d, device="cuda"), torch.empty(rows, d, device="cuda")
+    ws = torch.full((rows, 4 * d), float("nan"), device="cuda")
+    ctx = OwlContext(make_dims(batch=1, total_nodes=1, max_nodes=1))
+    ctx.owl_lstm_cell(h.cuda(), emb, w.cuda(), 0.0, z, hf, None, ws)
+    assert ctx.owl_get_status() == 0
+    ref = h.double() @ w.double().t()
+    bound = d_in * 2.0 ** -24 * (h.double().abs() @ w.double().abs().t())
+    assert bool(((ws.cpu().double() - ref).abs() <= bound).all())
+    ctx.close()

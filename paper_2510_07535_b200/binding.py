@@ -1,6 +1,8 @@
-"""Thin ctypes binding of libowlverify (argument marshalling only; every step runs in the CUDA
-kernels).  PyTorch supplies device memory and streams.  There is no fallback: if the shared
-library has not been built, loading raises."""
+"""Thin binding of libowlverify (argument marshalling only; every step runs in the CUDA kernels).
+PyTorch supplies device memory and streams.  The calls a decoding loop makes go through the native
+half of the binding (csrc/torch_binding.cpp), which checks the tensors and takes torch's current
+stream; the rest uses ctypes.  There is no fallback: if a shared library has not been built,
+loading raises."""
 from __future__ import annotations
 
 import ctypes
@@ -12,6 +14,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libowlverify.so")
 _lib = None
+_native = None
 
 OWL_OK = 0
 STATUS = {0: "OWL_OK", -1: "OWL_ERR_INVALID_ARG", -2: "OWL_ERR_UNSUPPORTED", -3: "OWL_ERR_CUDA",
@@ -33,46 +36,24 @@ class OwlError(RuntimeError):
 
 def load_library() -> ctypes.CDLL:
     """dlopen the in-tree libowlverify.so; raises if it was not built (no CPU fallback exists)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
         raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2510_07535_b200.build` "
                           "(nvcc, sm_100a). There is no fallback path.")
     lib = ctypes.CDLL(LIB_PATH)
+    from . import _owl_native as native      # built beside the library; finds it there
     vp, i32, i64 = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64
     dp = ctypes.POINTER(OwlDims)
     lib.owl_create.restype = i32
     lib.owl_create.argtypes = [ctypes.POINTER(vp), i32, dp]
     lib.owl_destroy.restype = i32
     lib.owl_destroy.argtypes = [vp]
-    lib.owl_verify_attn.restype = i32
-    lib.owl_verify_attn.argtypes = [vp, dp] + [vp] * 10
-    lib.owl_verify_attn_f16.restype = i32
-    lib.owl_verify_attn_f16.argtypes = [vp, dp] + [vp] * 10
-    lib.owl_tree_accept.restype = i32
-    lib.owl_tree_accept.argtypes = [vp, dp] + [vp] * 9
-    lib.owl_tree_accept_spec.restype = i32
-    lib.owl_tree_accept_spec.argtypes = [vp, dp] + [vp] * 10
-    lib.owl_prepare_spec_tree.restype = i32
-    lib.owl_prepare_spec_tree.argtypes = [vp, dp] + [vp] * 4 + [ctypes.c_int32] + [vp] * 6
-    lib.owl_prepare_hybrid.restype = i32
-    lib.owl_prepare_hybrid.argtypes = [vp, dp] + [vp] * 5 + [ctypes.c_int32] + [vp] * 6
     lib.owl_howl_route.restype = i32
     lib.owl_howl_route.argtypes = [ctypes.c_int32, vp, ctypes.c_float, vp, vp]
-    lib.owl_kv_commit.restype = i32
-    lib.owl_kv_commit.argtypes = [vp, dp] + [vp] * 8
-    lib.owl_lm_head_accept.restype = i32
-    lib.owl_lm_head_accept.argtypes = [vp, dp, ctypes.c_int32] + [vp] * 10
-    lib.owl_lstm_cell.restype = i32
-    lib.owl_lstm_cell.argtypes = [vp, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, vp, vp, vp, ctypes.c_float, vp, vp, vp, vp,
-                                  ctypes.c_float, vp, vp, vp, vp, vp]
     lib.owl_lstm_alpha.restype = ctypes.c_double
     lib.owl_lstm_alpha.argtypes = [ctypes.c_int32, ctypes.c_int32]
-    lib.owl_tree_accept_static.restype = i32
-    lib.owl_tree_accept_static.argtypes = [dp] + [vp] * 10
-    lib.owl_verify_step.restype = i32
-    lib.owl_verify_step.argtypes = [vp, dp] + [vp] * 16
     lib.owl_verify_step_host.restype = i32
     lib.owl_verify_step_host.argtypes = [vp, dp] + [vp] * 15
     lib.owl_get_status.restype = i32
@@ -89,7 +70,7 @@ def load_library() -> ctypes.CDLL:
     lib.owl_set_profiling.argtypes = [vp, i32]
     lib.owl_last_kernel_times.restype = i32
     lib.owl_last_kernel_times.argtypes = [vp, vp, ctypes.POINTER(ctypes.c_double)]
-    _lib = lib
+    _lib, _native = lib, native
     return lib
 
 
@@ -124,12 +105,14 @@ class OwlContext:
         rc = self.lib.owl_create(ctypes.byref(self._h), self.device.index, ctypes.byref(max_dims))
         if rc != OWL_OK:
             raise OwlError(rc, "owl_create")
+        self._handle, self._dev = self._h.value, self.device.index      # as the native half takes them
 
     def close(self):
         if getattr(self, "_h", None) and self._h.value:
             torch.cuda.synchronize(self.device)
             self.lib.owl_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._handle = 0
 
     def __del__(self):
         try:
@@ -137,146 +120,71 @@ class OwlContext:
         except Exception:
             pass
 
+    def _done(self, rc: int, check: bool, where: str) -> int:
+        if rc != OWL_OK and check:
+            raise OwlError(rc, where, self.last_error())
+        return rc
+
     def owl_verify_attn(self, dims: OwlDims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent,
                         out, lse, check: bool = True) -> int:
-        dev = self.device
-        rc = self.lib.owl_verify_attn(
-            self._h, ctypes.byref(dims), _ptr(q, torch.bfloat16, dev, "q"), _ptr(k_cache, torch.bfloat16, dev, "k_cache"),
-            _ptr(v_cache, torch.bfloat16, dev, "v_cache"), _ptr(block_table, torch.int32, dev, "block_table"),
-            _ptr(ctx_lens, torch.int32, dev, "ctx_lens"), _ptr(node_offsets, torch.int32, dev, "node_offsets"),
-            _ptr(tree_parent, torch.int32, dev, "tree_parent"), _ptr(out, torch.bfloat16, dev, "out"),
-            _ptr(lse, torch.float32, dev, "lse"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_verify_attn", self.last_error())
-        return rc
+        rc = _native.verify_attn(self._handle, self._dev, dims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse)
+        return self._done(rc, check, "owl_verify_attn")
 
     def owl_verify_attn_f16(self, dims: OwlDims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent,
                             out, lse, check: bool = True) -> int:
-        dev = self.device
-        h = torch.float16
-        rc = self.lib.owl_verify_attn_f16(
-            self._h, ctypes.byref(dims), _ptr(q, h, dev, "q"), _ptr(k_cache, h, dev, "k_cache"), _ptr(v_cache, h, dev, "v_cache"),
-            _ptr(block_table, torch.int32, dev, "block_table"), _ptr(ctx_lens, torch.int32, dev, "ctx_lens"),
-            _ptr(node_offsets, torch.int32, dev, "node_offsets"), _ptr(tree_parent, torch.int32, dev, "tree_parent"),
-            _ptr(out, h, dev, "out"), _ptr(lse, torch.float32, dev, "lse"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_verify_attn_f16", self.last_error())
-        return rc
+        rc = _native.verify_attn_f16(self._handle, self._dev, dims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent,
+                                     out, lse)
+        return self._done(rc, check, "owl_verify_attn_f16")
 
     def owl_tree_accept(self, dims: OwlDims, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path,
                         bonus_token, node_argmax=None, check: bool = True) -> int:
-        dev = self.device
-        rc = self.lib.owl_tree_accept(
-            self._h, ctypes.byref(dims), _ptr(logits, torch.float32, dev, "logits"),
-            _ptr(draft_tokens, torch.int32, dev, "draft_tokens"), _ptr(node_offsets, torch.int32, dev, "node_offsets"),
-            _ptr(tree_parent, torch.int32, dev, "tree_parent"), _ptr(accept_len, torch.int32, dev, "accept_len"),
-            _ptr(accept_path, torch.int32, dev, "accept_path"), _ptr(bonus_token, torch.int32, dev, "bonus_token"),
-            _ptr(node_argmax, torch.int32, dev, "node_argmax"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_tree_accept", self.last_error())
-        return rc
+        rc = _native.tree_accept(self._handle, self._dev, dims, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path,
+                                 bonus_token, node_argmax)
+        return self._done(rc, check, "owl_tree_accept")
 
     def owl_tree_accept_spec(self, dims: OwlDims, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path,
                              bonus_token, spec_node, node_argmax=None, check: bool = True) -> int:
-        dev = self.device
-        i32 = torch.int32
-        rc = self.lib.owl_tree_accept_spec(
-            self._h, ctypes.byref(dims), _ptr(logits, torch.float32, dev, "logits"), _ptr(draft_tokens, i32, dev, "draft_tokens"),
-            _ptr(node_offsets, i32, dev, "node_offsets"), _ptr(tree_parent, i32, dev, "tree_parent"),
-            _ptr(accept_len, i32, dev, "accept_len"), _ptr(accept_path, i32, dev, "accept_path"),
-            _ptr(bonus_token, i32, dev, "bonus_token"), _ptr(spec_node, i32, dev, "spec_node"),
-            _ptr(node_argmax, i32, dev, "node_argmax"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_tree_accept_spec", self.last_error())
-        return rc
+        rc = _native.tree_accept_spec(self._handle, self._dev, dims, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path,
+                                      bonus_token, spec_node, node_argmax)
+        return self._done(rc, check, "owl_tree_accept_spec")
 
     def owl_prepare_spec_tree(self, dims: OwlDims, node_offsets, tree_parent, draft_tokens, ctx_lens, spec_token: int,
                               out_node_offsets, out_tree_parent, out_draft_tokens, out_input_ids, out_position_ids,
                               check: bool = True) -> int:
-        dev = self.device
-        i32 = torch.int32
-        rc = self.lib.owl_prepare_spec_tree(
-            self._h, ctypes.byref(dims), _ptr(node_offsets, i32, dev, "node_offsets"), _ptr(tree_parent, i32, dev, "tree_parent"),
-            _ptr(draft_tokens, i32, dev, "draft_tokens"), _ptr(ctx_lens, i32, dev, "ctx_lens"), int(spec_token),
-            _ptr(out_node_offsets, i32, dev, "out_node_offsets"), _ptr(out_tree_parent, i32, dev, "out_tree_parent"),
-            _ptr(out_draft_tokens, i32, dev, "out_draft_tokens"), _ptr(out_input_ids, i32, dev, "out_input_ids"),
-            _ptr(out_position_ids, i32, dev, "out_position_ids"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_prepare_spec_tree", self.last_error())
-        return rc
+        rc = _native.prepare_spec_tree(self._handle, self._dev, dims, int(spec_token), node_offsets, tree_parent, draft_tokens, ctx_lens,
+                                       out_node_offsets, out_tree_parent, out_draft_tokens, out_input_ids, out_position_ids)
+        return self._done(rc, check, "owl_prepare_spec_tree")
 
     def owl_prepare_hybrid(self, dims: OwlDims, node_offsets, tree_parent, draft_tokens, ctx_lens, route, spec_token: int,
                            out_node_offsets, out_tree_parent, out_draft_tokens, out_input_ids, out_position_ids,
                            check: bool = True) -> int:
-        dev = self.device
-        i32 = torch.int32
-        rc = self.lib.owl_prepare_hybrid(
-            self._h, ctypes.byref(dims), _ptr(node_offsets, i32, dev, "node_offsets"), _ptr(tree_parent, i32, dev, "tree_parent"),
-            _ptr(draft_tokens, i32, dev, "draft_tokens"), _ptr(ctx_lens, i32, dev, "ctx_lens"), _ptr(route, i32, dev, "route"),
-            int(spec_token), _ptr(out_node_offsets, i32, dev, "out_node_offsets"), _ptr(out_tree_parent, i32, dev, "out_tree_parent"),
-            _ptr(out_draft_tokens, i32, dev, "out_draft_tokens"), _ptr(out_input_ids, i32, dev, "out_input_ids"),
-            _ptr(out_position_ids, i32, dev, "out_position_ids"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_prepare_hybrid", self.last_error())
-        return rc
+        rc = _native.prepare_hybrid(self._handle, self._dev, dims, int(spec_token), node_offsets, tree_parent, draft_tokens, ctx_lens, route,
+                                    out_node_offsets, out_tree_parent, out_draft_tokens, out_input_ids, out_position_ids)
+        return self._done(rc, check, "owl_prepare_hybrid")
 
     def owl_kv_commit(self, dims: OwlDims, k_cache, v_cache, block_table, ctx_lens, node_offsets, accept_len, accept_path,
                       check: bool = True) -> int:
-        dev = self.device
-        i32, bf = torch.int32, torch.bfloat16
-        rc = self.lib.owl_kv_commit(
-            self._h, ctypes.byref(dims), _ptr(k_cache, bf, dev, "k_cache"), _ptr(v_cache, bf, dev, "v_cache"),
-            _ptr(block_table, i32, dev, "block_table"), _ptr(ctx_lens, i32, dev, "ctx_lens"),
-            _ptr(node_offsets, i32, dev, "node_offsets"), _ptr(accept_len, i32, dev, "accept_len"),
-            _ptr(accept_path, i32, dev, "accept_path"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_kv_commit", self.last_error())
-        return rc
+        rc = _native.kv_commit(self._handle, self._dev, dims, k_cache, v_cache, block_table, ctx_lens, node_offsets, accept_len, accept_path)
+        return self._done(rc, check, "owl_kv_commit")
 
     def owl_lm_head_accept(self, dims: OwlDims, hidden, weight, draft_tokens, node_offsets, tree_parent, accept_len, accept_path,
                            bonus_token, node_argmax=None, check: bool = True) -> int:
-        dev = self.device
-        i32, bf = torch.int32, torch.bfloat16
-        rc = self.lib.owl_lm_head_accept(
-            self._h, ctypes.byref(dims), int((weight if hidden is None else hidden).shape[-1]), _ptr(hidden, bf, dev, "hidden"),
-            _ptr(weight, bf, dev, "weight"),
-            _ptr(draft_tokens, i32, dev, "draft_tokens"), _ptr(node_offsets, i32, dev, "node_offsets"),
-            _ptr(tree_parent, i32, dev, "tree_parent"), _ptr(accept_len, i32, dev, "accept_len"),
-            _ptr(accept_path, i32, dev, "accept_path"), _ptr(bonus_token, i32, dev, "bonus_token"),
-            _ptr(node_argmax, i32, dev, "node_argmax"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_lm_head_accept", self.last_error())
-        return rc
+        rc = _native.lm_head_accept(self._handle, self._dev, dims, int((weight if hidden is None else hidden).shape[-1]), hidden, weight,
+                                    draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token, node_argmax)
+        return self._done(rc, check, "owl_lm_head_accept")
 
     def owl_lstm_cell(self, h, emb, w, alpha: float, z, h_out_f32, h_out_bf16, workspace, ln_c=(None, None), ln_z=(None, None),
                       eps: float = 1e-5, check: bool = True) -> int:
-        dev = self.device
-        bf, f32 = torch.bfloat16, torch.float32
         rows, d_in = h.shape
-        d = emb.shape[-1]
-        rc = self.lib.owl_lstm_cell(
-            self._h, rows, d_in, d, _ptr(h, bf, dev, "h"), _ptr(emb, bf, dev, "emb"), _ptr(w, bf, dev, "w"), float(alpha),
-            _ptr(ln_c[0], f32, dev, "ln_c_gamma"), _ptr(ln_c[1], f32, dev, "ln_c_beta"), _ptr(ln_z[0], f32, dev, "ln_z_gamma"),
-            _ptr(ln_z[1], f32, dev, "ln_z_beta"), float(eps), _ptr(z, f32, dev, "z"), _ptr(h_out_f32, f32, dev, "h_out_f32"),
-            _ptr(h_out_bf16, bf, dev, "h_out_bf16"), _ptr(workspace, f32, dev, "workspace"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_lstm_cell", self.last_error())
-        return rc
+        rc = _native.lstm_cell(self._handle, self._dev, rows, d_in, emb.shape[-1], float(alpha), float(eps), h, emb, w, ln_c[0], ln_c[1],
+                               ln_z[0], ln_z[1], z, h_out_f32, h_out_bf16, workspace)
+        return self._done(rc, check, "owl_lstm_cell")
 
     def owl_verify_step(self, dims: OwlDims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse,
                         logits, draft_tokens, accept_len, accept_path, bonus_token, node_argmax=None, check: bool = True) -> int:
-        dev = self.device
-        i32, bf, f32 = torch.int32, torch.bfloat16, torch.float32
-        rc = self.lib.owl_verify_step(
-            self._h, ctypes.byref(dims), _ptr(q, bf, dev, "q"), _ptr(k_cache, bf, dev, "k_cache"), _ptr(v_cache, bf, dev, "v_cache"),
-            _ptr(block_table, i32, dev, "block_table"), _ptr(ctx_lens, i32, dev, "ctx_lens"),
-            _ptr(node_offsets, i32, dev, "node_offsets"), _ptr(tree_parent, i32, dev, "tree_parent"), _ptr(out, bf, dev, "out"),
-            _ptr(lse, f32, dev, "lse"), _ptr(logits, f32, dev, "logits"), _ptr(draft_tokens, i32, dev, "draft_tokens"),
-            _ptr(accept_len, i32, dev, "accept_len"), _ptr(accept_path, i32, dev, "accept_path"),
-            _ptr(bonus_token, i32, dev, "bonus_token"), _ptr(node_argmax, i32, dev, "node_argmax"), _stream(dev))
-        if check and rc != OWL_OK:
-            raise OwlError(rc, "owl_verify_step", self.last_error())
-        return rc
+        rc = _native.verify_step(self._handle, self._dev, dims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent,
+                                 out, lse, logits, draft_tokens, accept_len, accept_path, bonus_token, node_argmax)
+        return self._done(rc, check, "owl_verify_step")
 
     def owl_verify_step_host(self, dims: OwlDims, q, k_cache, v_cache, block_table, ctx_lens, node_offsets,
                              tree_parent, logits, draft_tokens, out, lse, accept_len, accept_path, bonus_token) -> int:
@@ -329,15 +237,9 @@ def owl_tree_accept_static(dims: OwlDims, logits, draft_tokens, node_offsets, tr
     (allocated by the caller, as always) must live on the current CUDA device; scratch is the library's
     fixed array, shared by every call on that device, so overlapping calls must be serialised by the
     caller.  ``device_status`` (optional int32[1] on the device) receives 0 or OWL_ERR_BAD_TREE."""
-    lib = load_library()
-    dev = torch.device("cuda", torch.cuda.current_device())
-    rc = lib.owl_tree_accept_static(
-        ctypes.byref(dims), _ptr(logits, torch.float32, dev, "logits"),
-        _ptr(draft_tokens, torch.int32, dev, "draft_tokens"), _ptr(node_offsets, torch.int32, dev, "node_offsets"),
-        _ptr(tree_parent, torch.int32, dev, "tree_parent"), _ptr(accept_len, torch.int32, dev, "accept_len"),
-        _ptr(accept_path, torch.int32, dev, "accept_path"), _ptr(bonus_token, torch.int32, dev, "bonus_token"),
-        _ptr(node_argmax, torch.int32, dev, "node_argmax"), _ptr(device_status, torch.int32, dev, "device_status"),
-        _stream(dev))
+    load_library()
+    rc = _native.tree_accept_static(0, torch.cuda.current_device(), dims, logits, draft_tokens, node_offsets, tree_parent, accept_len,
+                                    accept_path, bonus_token, node_argmax, device_status)
     if check and rc != OWL_OK:
         raise OwlError(rc, "owl_tree_accept_static")
     return rc

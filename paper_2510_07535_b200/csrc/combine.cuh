@@ -11,6 +11,29 @@
 namespace owl {
 
 constexpr int kCombineWarps = 8;
+constexpr int kCombineCtasPerSm = 4;
+
+// Partials per round of the merge, for `units` units (sequence, KV head) cut by `ctas` CTAs: as many as a unit of
+// average length is cut into, plus one at either end, so that its rows take one memory round trip; longer units take
+// several rounds.  A stage of 32 rows for everybody made a CTA 128 KB large: one per SM, and the 1920 rows of a 60-node
+// tree (240 CTAs) ran in two waves.
+inline int combine_group(long long units, int ctas) {
+    const long long g = (ctas + units - 1) / units + 2;
+    return (int)(g < 4 ? 4 : g < 32 ? g : 32);
+}
+inline size_t combine_stage_bytes(int group) { return (size_t)kCombineWarps * group * 32 * sizeof(float4); }
+inline int combine_ctas_per_sm(int group) {
+    const int fit = (int)((227u << 10) / (combine_stage_bytes(group) + 1024));
+    return fit < kCombineCtasPerSm ? fit : kCombineCtasPerSm;
+}
+// What a launch of `ctas` CTAs asks for: its stage, and enough that no SM takes more than its share of them.  The
+// SMs whose attention CTA ends first would otherwise collect several merge CTAs each (2K context, 33 CTAs: 15.5 -> 16.1 us
+// per step).
+inline size_t combine_smem_bytes(int group, unsigned ctas, int sms) {
+    const unsigned share = (ctas + (unsigned)sms - 1) / (unsigned)sms;
+    const size_t spread = (227u << 10) / (share + 1) + 16, stage = combine_stage_bytes(group);
+    return stage > spread ? stage : spread;
+}
 
 // One warp per output row finds the CTAs whose pieces cut the row's unit
 // and merges their partials in CTA order.  A CTA stores at most two partials: slot 2c if its piece starts inside
@@ -25,18 +48,16 @@ constexpr int kCombineWarps = 8;
 // kFused (verify step): the grid has one more CTA per sequence after the row CTAs; each of those runs one
 // sequence's acceptance walk over the arg-max keys that the pass's spare warps left (`ap`).
 //
-// kGroup: partials fetched per round, 16 or 32.  A unit cut into 17 to 32 pieces (8 units of a 32K context over 148
-// CTAs: 18 or 19) costs a second round of loads with 16, which is a whole memory round trip of a kernel that is
-// all latency.  A round's rows go through a warp-private stage in shared memory (16 or 8 KB per warp: 128 or 64 KB
-// per CTA, which is what limits 32 to launches with few rows; the host takes it up to 4096 output rows).
+// p.combine_group: partials fetched per round, at most 32 (combine_group below).  A round's rows go through a
+// warp-private stage in shared memory of that many rows, which is what limits the CTAs per SM.
 //
 // The stage is there for the sake of the code's length, not of the data: with the rows in registers the fetch and
 // the fold were two loops unrolled 32 times, some 450 instructions that a warp with one row executes exactly once,
 // at the pace of instruction fetches from L2.  Copied with cp.async in a short rolled loop and folded in another,
 // the same work is two dozen instructions executed from the instruction cache after their first trip (attention +
 // merge call at 32K context 37.5 -> 36.8 us, with 8192 output rows 586 -> 578 us).
-template <bool kFused, int kGroup>
-__global__ void __launch_bounds__(kCombineWarps * 32) combine_sched_kernel(const AttnParams p, const AcceptParams ap) {
+template <bool kFused>
+__global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine_sched_kernel(const AttnParams p, const AcceptParams ap) {
     const long long rows = (long long)p.total_nodes * p.num_q_heads;
     const unsigned row_ctas = (unsigned)p.combine_row_ctas;
     if (kFused) {
@@ -51,8 +72,9 @@ __global__ void __launch_bounds__(kCombineWarps * 32) combine_sched_kernel(const
     // The row CTAs are persistent: a warp derives the schedule once and then takes rows first, first + stride, ...
     // (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived 8192 times).
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    extern __shared__ float4 combine_stage[];          // [warps][kGroup][32]: a round's partial rows, warp-private
-    float4* stage = combine_stage + warp * kGroup * 32;
+    extern __shared__ float4 combine_stage[];          // [warps][group][32]: a round's partial rows, warp-private
+    const int group = p.combine_group;
+    float4* stage = combine_stage + warp * group * 32;
     const long long first = (long long)blockIdx.x * kCombineWarps + warp, stride = (long long)row_ctas * kCombineWarps;
     const bool small = p.batch <= 32;
     WarpSchedule ws{};
@@ -73,7 +95,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) combine_sched_kernel(const
         t0 = seq_begin + (long long)(hq / G) * tiles;
         c0 = part.owner(t0);
         c1 = part.owner(t0 + tiles - 1);
-        prow_first = row_of(c0 + min(lane & (kGroup - 1), c1 - c0));
+        prow_first = row_of(c0 + min(lane, c1 - c0));
     };
     auto locate = [&](long long row_id) {       // every lane of the warp, same row
         n = (int)(row_id / p.num_q_heads);
@@ -116,17 +138,17 @@ __global__ void __launch_bounds__(kCombineWarps * 32) combine_sched_kernel(const
         const int bad_epoch = __ldcg(p.seq_bad + b);   // (its round trip overlaps the partial loads below)
         const int count = c1 - c0 + 1;
 
-        // Partials are taken kGroup at a time: lane j (< kGroup) of a group owns partial base + j.  The row loads do
+        // Partials are taken `group` at a time: lane j (< group) owns partial base + j.  The row loads do
         // not depend on the LSE values, so both go out together: one memory round trip per group.  Groups are folded
         // online (running maximum).
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         float sum = 0.f, mx = -INFINITY;
-        for (int base = 0; base < count; base += kGroup) {
-            const int mine = base + (lane & (kGroup - 1));
-            const bool have = mine < count;
+        for (int base = 0; base < count; base += group) {
+            const int mine = base + lane;
+            const bool have = lane < group && mine < count;
             const long long prow = base == 0 ? prow_first : row_of(c0 + (have ? mine : 0));
             const float my_lse = have ? __ldcg(p.part_lse + prow) : -INFINITY;
-            const int cnt = count - base < kGroup ? count - base : kGroup;
+            const int cnt = count - base < group ? count - base : group;
             if (base > 0) __syncwarp();                  // the stage's rows of the round before have been folded
 #pragma unroll 1
             for (int j = 0; j < cnt; ++j) {
@@ -137,7 +159,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) combine_sched_kernel(const
             asm volatile("cp.async.commit_group;" ::: "memory");
             float gmx = my_lse;
 #pragma unroll
-            for (int o = kGroup / 2; o > 0; o >>= 1) gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, o));
+            for (int o = 16; o > 0; o >>= 1) gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, o));
             const float mx_new = fmaxf(mx, gmx);
             if (mx_new > -INFINITY) {
                 const float rescale = mx > -INFINITY ? __expf(mx - mx_new) : 0.f;

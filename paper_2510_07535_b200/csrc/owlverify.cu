@@ -291,11 +291,9 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         ok = set_umma_smem_attr();
     }
     if (ok) {
-        const int big = kCombineWarps * 32 * 32 * (int)sizeof(float4), small_ = big / 2;
-        ok = cudaFuncSetAttribute(combine_sched_kernel<true, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) == cudaSuccess &&
-             cudaFuncSetAttribute(combine_sched_kernel<false, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) == cudaSuccess &&
-             cudaFuncSetAttribute(combine_sched_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_) == cudaSuccess &&
-             cudaFuncSetAttribute(combine_sched_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_) == cudaSuccess;
+        const int most = (int)combine_stage_bytes(32);
+        ok = cudaFuncSetAttribute(combine_sched_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
+             cudaFuncSetAttribute(combine_sched_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
     }
     if (ok) {
         using namespace gemm_path;
@@ -411,9 +409,11 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
 
     if (ctx->profiling) cudaEventRecord(ctx->ev[0], stream);
     const long long rows = (long long)d->total_nodes * d->num_q_heads;
-    // one warp per row up to two CTAs per SM; beyond that the merge kernel's warps stride over the rows
+    // one warp per row while all CTAs are resident at once; beyond that the merge kernel's warps stride over the rows
+    p.combine_group = combine_group((long long)d->batch * d->num_kv_heads, ctx->num_ctas);
     const long long want_ctas = (rows + kCombineWarps - 1) / kCombineWarps;
-    const unsigned grid = (unsigned)(want_ctas < 2ll * ctx->sm_count ? want_ctas : 2ll * ctx->sm_count);
+    const long long most_ctas = (long long)ctx->sm_count * combine_ctas_per_sm(p.combine_group);
+    const unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas : most_ctas);
     p.combine_row_ctas = (int32_t)grid;
     {
         cudaLaunchConfig_t cfg = {};
@@ -433,14 +433,12 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     }
     ++ctx->launches;
     if (ctx->profiling) cudaEventRecord(ctx->ev[1], stream);
-    const bool few_rows = rows <= 4096;      // latency-bound merge: 32 partials per round (see combine.cuh)
-    const size_t stage_bytes = (size_t)kCombineWarps * (few_rows ? 32 : 16) * 32 * sizeof(float4);
+    const size_t stage_bytes = combine_smem_bytes(p.combine_group, grid + (ap ? (unsigned)d->batch : 0u), ctx->sm_count);
     if (ap)
-        launch_dependent_smem(few_rows ? combine_sched_kernel<true, 32> : combine_sched_kernel<true, 16>,
-                              dim3(grid + (unsigned)d->batch), dim3(kCombineWarps * 32), stage_bytes, stream, p, *ap);
+        launch_dependent_smem(combine_sched_kernel<true>, dim3(grid + (unsigned)d->batch), dim3(kCombineWarps * 32), stage_bytes, stream,
+                              p, *ap);
     else
-        launch_dependent_smem(few_rows ? combine_sched_kernel<false, 32> : combine_sched_kernel<false, 16>, dim3(grid),
-                              dim3(kCombineWarps * 32), stage_bytes, stream, p, AcceptParams{});
+        launch_dependent_smem(combine_sched_kernel<false>, dim3(grid), dim3(kCombineWarps * 32), stage_bytes, stream, p, AcceptParams{});
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[2], stream); ctx->ev_attn_valid = true; }
     cudaError_t e = cudaGetLastError();

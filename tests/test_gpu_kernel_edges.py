@@ -29,6 +29,17 @@ def test_units_that_fill_one_to_four_softmax_warps(nodes):
     check_attention(fill_dead_slots(wl))
 
 
+@pytest.mark.parametrize("hkv,ctx", [
+    (1, [9000]),                       # one unit cut into 71 pieces: 32 partials per round, three rounds
+    (2, [6000] + [20] * 7),            # 12 partials per round, the long units cut into dozens of pieces
+    (2, [3000] + [150] * 39),          # 80 units: 4 partials per round, schedule read from global memory
+])
+def test_merge_rounds_of_partials(hkv, ctx):
+    wl = W.generate(W.Spec("merge", 4 * hkv, hkv, ctx, [("tree", 9, 3)] * len(ctx), shuffle_pages=True, seed=800 + len(ctx),
+                           with_logits=False))
+    check_attention(wl)
+
+
 @pytest.mark.parametrize("rows,d_in", [(1, 64), (16, 192), (17, 64), (32, 320), (33, 192), (128, 192), (129, 64), (256, 192), (257, 64), (383, 192)])
 def test_product_row_padding_and_odd_k_blocks(rows, d_in):
     """The weight-streaming product behind the drafter cell, element by element: rows around the padding to 16 and the

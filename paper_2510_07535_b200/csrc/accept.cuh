@@ -1,6 +1,6 @@
 // Greedy tree acceptance: row arg-max over the vocabulary, then the acceptance walk.
 //
-// The scan reads fp32 logits with 16-byte loads, one warp per (row, 8192-float vocabulary chunk) item.  Every
+// The scan reads fp32 logits with 16-byte loads, one warp per (row, vocabulary chunk of 2048 to 8192 floats) item.  Every
 // (value, index) candidate is folded into one 64-bit key, high word = the float mapped to an unsigned
 // integer that sorts like the float (NaN mapped to -inf, -0 to +0), low word = ~index, so that an unsigned
 // max picks the larger value and, among equal values, the lower index.  Per-lane and warp (shuffle) maxima
@@ -24,7 +24,16 @@ namespace owl {
 
 constexpr int kArgmaxThreads = 256;
 static_assert(kArgmaxThreads >= kMaxNodes, "the walk needs one thread per node");
-constexpr int kArgmaxChunk = 8192;  // floats per CTA: 8 x float4 per thread
+constexpr int kArgmaxChunk = 8192;     // floats per item when there are items enough for every warp
+constexpr int kArgmaxMinChunk = 2048;  // two rounds of eight 16-byte loads per lane
+// Floats per (row, chunk) item of a scan by `warps` warps: halved as long as every warp still gets one item at most.  A
+// small scan is bound by the loads a warp can keep in flight, so it needs all the warps (60 rows x 128256: 960 items of
+// 8192 kept 960 of 2368 warps busy).
+__host__ inline int argmax_chunk(long long rows, int vocab, long long warps) {
+    int chunk = kArgmaxChunk;
+    while (chunk > kArgmaxMinChunk && rows * ((vocab + chunk / 2 - 1) / (chunk / 2)) <= warps) chunk /= 2;
+    return chunk;
+}
 
 // 16-byte load of data that is read once: no L1 allocation, first in line for eviction from L2
 // (`policy` from createpolicy.fractional.L2::evict_first).
@@ -55,7 +64,8 @@ struct AcceptParams {
     uint32_t epoch;                  // call number: the other set is cleared for the next call
     int32_t counter_stride;          // distance between the two sets
     int32_t* status;
-    int32_t batch, total_nodes, nodes_uniform, max_nodes, vocab, path_stride, chunks;
+    int32_t batch, total_nodes, nodes_uniform, max_nodes, vocab, path_stride;
+    int32_t chunk, chunks;           // floats per item, items per row
 };
 
 __device__ __forceinline__ unsigned long long argmax_key(float x, uint32_t idx) {
@@ -66,7 +76,8 @@ __device__ __forceinline__ unsigned long long argmax_key(float x, uint32_t idx) 
     return ((unsigned long long)u << 32) | (uint32_t)(~idx);
 }
 
-// Called by every thread of the CTA (threads >= kMaxNodes only keep the barriers company).
+// Called by every thread of a CTA of kArgmaxThreads: a node's chunk keys are read by several neighbouring threads, all
+// in one memory round trip; after that thread i is node i and the others only keep the barriers company.
 __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int b) {
     const int i = threadIdx.x;
     const int base = p.node_offsets ? p.node_offsets[b] : b * p.nodes_uniform;
@@ -80,23 +91,35 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
     }
     __syncthreads();
     if (s_bad) { if (i == 0) report(p.status, kErrBadTree); return; }
+    {
+        static_assert(kArgmaxThreads >= 4 * kMaxNodes, "at least four threads per node");
+        const int lg = n > 32 ? 2 : n > 16 ? 3 : n > 8 ? 4 : 5;       // 4 to 32 threads per node
+        const int node = i >> lg, sub = i & ((1 << lg) - 1);
+        unsigned long long k = 0;
+        if (node < n) {
+            const unsigned long long* pk = p.part_keys + (long long)(base + node) * p.chunks;
+            for (int c0 = sub; c0 < p.chunks; c0 += 8 << lg) {
+                unsigned long long v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = c0 + (j << lg) < p.chunks ? __ldcg(pk + c0 + (j << lg)) : 0ull;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) k = v[j] > k ? v[j] : k;
+            }
+        }
+        for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
+            k = other > k ? other : k;
+        }
+        if (node < n && sub == 0) {
+            const int am = (int)(~(uint32_t)(k & 0xffffffffull));
+            s_am[node] = am;
+            if (p.node_argmax) p.node_argmax[base + node] = am;
+        }
+    }
     if (i < n) {
         const int pi = p.tree_parent[base + i];
         s_parent[i] = pi;
         s_tok[i] = p.draft_tokens[base + i];
-        unsigned long long k = 0;
-        const unsigned long long* pk = p.part_keys + (long long)(base + i) * p.chunks;
-        // independent loads, eight in flight (a dependent one-by-one walk would cost a memory round trip per chunk)
-        for (int c0 = 0; c0 < p.chunks; c0 += 8) {
-            unsigned long long v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = c0 + j < p.chunks ? __ldcg(pk + c0 + j) : 0ull;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) k = v[j] > k ? v[j] : k;
-        }
-        const int am = (int)(~(uint32_t)(k & 0xffffffffull));
-        s_am[i] = am;
-        if (p.node_argmax) p.node_argmax[base + i] = am;
         if ((i == 0 && pi != -1) || (i > 0 && (pi < 0 || pi >= i))) atomicExch(&s_bad, 1);
     }
     __syncthreads();
@@ -147,8 +170,8 @@ template <bool kPipelined>
 __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, const int row, const int chunk) {
     const int lane = threadIdx.x & 31;
     const long long V = p.vocab;
-    const long long c0 = (long long)chunk * kArgmaxChunk;
-    const long long c1 = c0 + kArgmaxChunk < V ? c0 + kArgmaxChunk : V;
+    const long long c0 = (long long)chunk * p.chunk;
+    const long long c1 = c0 + p.chunk < V ? c0 + p.chunk : V;
     const float* base = p.logits + row * V;
     // [c0, a0) scalar head up to 16-byte alignment, [a0, a1) float4 body, [a1, c1) scalar tail
     const uintptr_t addr = reinterpret_cast<uintptr_t>(base + c0);
@@ -228,6 +251,7 @@ __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, co
 // out of items it walks the trees of the sequences it noted.  (A CTA can note at most as many as it scanned items.)
 constexpr int kArgmaxWarps = kArgmaxThreads / 32;
 constexpr int kArgmaxCtasPerSm = 2;     // what fits at the kernel's register count
+__host__ inline long long argmax_warps(int sms) { return (long long)sms * kArgmaxCtasPerSm * kArgmaxWarps; }
 constexpr int kArgmaxNoteMax = 64;
 constexpr int kArgmaxOffsMax = 1024;            // sequences whose packed offsets a CTA keeps in shared memory
 
@@ -308,7 +332,7 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const Ac
 // every warp the same number of items (4096 items on 2368 resident warps would leave a quarter of the warps idle
 // during the second half of the kernel; 2048 warps with two items each do not).
 __host__ inline unsigned argmax_grid(long long items, int sms) {
-    const long long max_warps = (long long)sms * kArgmaxCtasPerSm * kArgmaxWarps;
+    const long long max_warps = argmax_warps(sms);
     const long long rounds = (items + max_warps - 1) / max_warps;
     const long long warps = rounds > 0 ? (items + rounds - 1) / rounds : 1;
     const long long ctas = (warps + kArgmaxWarps - 1) / kArgmaxWarps;

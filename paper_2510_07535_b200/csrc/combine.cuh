@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
     const unsigned row_ctas = (unsigned)p.combine_row_ctas;
     if (kFused) {
         if (blockIdx.x >= row_ctas) {
-            static_assert(kCombineWarps * 32 >= kMaxNodes, "the walk needs one thread per node");
+            static_assert(kCombineWarps * 32 == kArgmaxThreads, "the walk's block");
             asm volatile("griddepcontrol.wait;" ::: "memory");
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             accept_walk_seq(ap, (int)(blockIdx.x - row_ctas));

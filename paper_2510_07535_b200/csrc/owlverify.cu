@@ -275,7 +275,9 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     alloc((void**)&ctx->sched_seq_begin, ((size_t)max_dims->batch + 1) * sizeof(long long));
     alloc((void**)&ctx->sched_header, sizeof(SchedHeader));
     if (acc) {
-        ctx->part_keys_len = (long long)max_dims->total_nodes * ((max_dims->vocab + kArgmaxChunk - 1) / kArgmaxChunk);
+        // room for the smallest chunks of any call whose rows x 8192-float chunks do not exceed the context's
+        ctx->part_keys_len = (long long)max_dims->total_nodes * ((max_dims->vocab + kArgmaxChunk - 1) / kArgmaxChunk) *
+                             (kArgmaxChunk / kArgmaxMinChunk);
         alloc((void**)&ctx->part_keys, (size_t)ctx->part_keys_len * sizeof(unsigned long long));
         alloc((void**)&ctx->lm_keys, 2 * (size_t)max_dims->total_nodes * sizeof(unsigned long long));
         if (ok) ok = cudaMemset(ctx->lm_keys, 0, 2 * (size_t)max_dims->total_nodes * sizeof(unsigned long long)) == cudaSuccess;
@@ -464,7 +466,7 @@ int owl_verify_attn_f16(owl_ctx* ctx, const owl_dims* d, const void* q, const vo
 static int accept_params(owl_ctx* ctx, const owl_dims* d, const float* logits, const int32_t* draft_tokens,
                          const int32_t* node_offsets, const int32_t* tree_parent, int32_t* accept_len,
                          int32_t* accept_path, int32_t* bonus_token, int32_t* node_argmax, AcceptParams& p,
-                         int32_t* spec_node = nullptr) {
+                         int32_t* spec_node = nullptr, int chunk = 0 /* floats per item; 0: by the scan's size */) {
     if (!ctx) return OWL_ERR_INVALID_ARG;
     int rc = check_dims(d, false, true);
     if (rc != OWL_OK) return rc;
@@ -472,8 +474,8 @@ static int accept_params(owl_ctx* ctx, const owl_dims* d, const float* logits, c
     if (!node_offsets && d->total_nodes % d->batch != 0) return OWL_ERR_INVALID_ARG;
     if (d->batch > ctx->max_dims.batch || d->total_nodes > ctx->max_dims.total_nodes) return OWL_ERR_TOO_LARGE;
     if (d->total_nodes > 65535) return OWL_ERR_UNSUPPORTED;
-    const int chunks = (d->vocab + kArgmaxChunk - 1) / kArgmaxChunk;
-    if (!ctx->part_keys || (long long)d->total_nodes * chunks > ctx->part_keys_len) return OWL_ERR_TOO_LARGE;
+    const long long wide_items = (long long)d->total_nodes * ((d->vocab + kArgmaxChunk - 1) / kArgmaxChunk);
+    if (!ctx->part_keys || wide_items * (kArgmaxChunk / kArgmaxMinChunk) > ctx->part_keys_len) return OWL_ERR_TOO_LARGE;
     p = AcceptParams{};
     p.logits = logits;
     p.draft_tokens = draft_tokens;
@@ -485,7 +487,8 @@ static int accept_params(owl_ctx* ctx, const owl_dims* d, const float* logits, c
     p.node_argmax = node_argmax;
     p.spec_node = spec_node;
     p.part_keys = ctx->part_keys;
-    p.chunks = chunks;
+    p.chunk = chunk ? chunk : argmax_chunk(d->total_nodes, d->vocab, argmax_warps(ctx->sm_count));
+    p.chunks = (d->vocab + p.chunk - 1) / p.chunk;
     p.status = ctx->status;
     p.batch = d->batch;
     p.total_nodes = d->total_nodes;
@@ -506,12 +509,11 @@ static int tree_accept_impl(owl_ctx* ctx, const owl_dims* d, const float* logits
     if (rc != OWL_OK) return rc;
     DeviceGuard guard(ctx->device);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    const int chunks = p.chunks;
     p.seq_counter = ctx->seq_counter;
     p.counter_stride = ctx->max_dims.batch;
     p.epoch = ++ctx->accept_epoch;
     if (ctx->profiling) cudaEventRecord(ctx->ev[3], stream);
-    dim3 grid(argmax_grid((long long)chunks * d->total_nodes, ctx->sm_count));
+    dim3 grid(argmax_grid((long long)p.chunks * d->total_nodes, ctx->sm_count));
     launch_dependent(argmax_partial_kernel, grid, dim3(kArgmaxThreads), stream, p);   // the walk runs in the CTA that finishes a sequence
     ++ctx->launches;
     if (ctx->profiling) cudaEventRecord(ctx->ev[4], stream);
@@ -712,7 +714,8 @@ int owl_verify_step(owl_ctx* ctx, const owl_dims* d, const void* q, const void* 
     // Two launches: the attention kernel, whose two spare warps per CTA scan the logits while K/V stream in, and the
     // merge kernel, which also walks the trees.
     AcceptParams ap;
-    rc = accept_params(ctx, d, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token, node_argmax, ap);
+    rc = accept_params(ctx, d, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token, node_argmax, ap,
+                       nullptr, kArgmaxMinChunk);   // a handful of small items per spare warp: the last ones end together
     if (rc != OWL_OK) return rc;
     ctx->ev_accept_valid = false;
     return verify_attn_impl(ctx, d, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse, stream_, &ap);
@@ -901,6 +904,7 @@ extern "C" int owl_tree_accept_static(const owl_dims* d, const float* logits, co
     p.bonus_token = bonus_token;
     p.node_argmax = node_argmax;
     p.part_keys = scratch;
+    p.chunk = kArgmaxChunk;
     p.chunks = chunks;
     p.status = status;
     p.batch = d->batch;

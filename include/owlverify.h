@@ -228,7 +228,7 @@ int owl_prepare_hybrid(owl_ctx* ctx, const owl_dims* dims, const int32_t* node_o
  * for every KV head, in k_cache and v_cache, IN PLACE, and ctx_lens[b] becomes L_b + a.  Whatever else was
  * drafted stays behind as dead slots past the new length.  Uses dims->batch, total_nodes, max_nodes,
  * num_kv_heads, head_dim, page_size, max_pages_per_seq, num_pages, path_stride.  All pointers device; k_cache,
- * v_cache and ctx_lens are read and written.  Asynchronous on `stream` (two small kernels in stream order).  A
+ * v_cache and ctx_lens are read and written.  Asynchronous on `stream`.  A
  * path that is not a root path in node order sets OWL_ERR_BAD_TREE, a page id out of range OWL_ERR_BAD_PAGE;
  * that sequence is then left untouched, length included.
  */

@@ -33,6 +33,7 @@ struct owl_ctx {
     int32_t* status = nullptr;
     unsigned long long* selftest_ns = nullptr;
     int32_t* seq_bad = nullptr;
+    unsigned int* commit_done = nullptr;        // CommitParams::seq_done
     long long* sched_seq_begin = nullptr;
     SchedHeader* sched_header = nullptr;
     unsigned long long* part_keys = nullptr;
@@ -250,10 +251,11 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     ctx->max_dims = *max_dims;
     DeviceGuard guard(device);
     cudaError_t e;
-    cudaDeviceProp prop;
-    if ((e = cudaGetDeviceProperties(&prop, device)) != cudaSuccess) { delete ctx; return OWL_ERR_CUDA; }
-    if (prop.major != 10) { delete ctx; return OWL_ERR_UNSUPPORTED; }  // sm_100a code only
-    ctx->sm_count = prop.multiProcessorCount;
+    // (two attributes: cudaGetDeviceProperties gathers dozens and was 2.7 of this call's 3.1 ms)
+    int major = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { delete ctx; return OWL_ERR_CUDA; }
+    if (major != 10) { delete ctx; return OWL_ERR_UNSUPPORTED; }  // sm_100a code only
     ctx->num_ctas = ctx->sm_count;
 
     ctx->encode = load_encode_tiled();
@@ -272,6 +274,7 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     alloc((void**)&ctx->status, sizeof(int32_t));
     alloc((void**)&ctx->selftest_ns, 2 * sizeof(unsigned long long));
     alloc((void**)&ctx->seq_bad, (size_t)max_dims->batch * sizeof(int32_t));
+    alloc((void**)&ctx->commit_done, kMaxBatch * sizeof(unsigned int));      // owl_kv_commit takes any batch
     alloc((void**)&ctx->sched_seq_begin, ((size_t)max_dims->batch + 1) * sizeof(long long));
     alloc((void**)&ctx->sched_header, sizeof(SchedHeader));
     if (acc) {
@@ -286,7 +289,8 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     }
     if (ok) {
         ok = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess &&
-             cudaMemset(ctx->seq_bad, 0, (size_t)max_dims->batch * sizeof(int32_t)) == cudaSuccess;
+             cudaMemset(ctx->seq_bad, 0, (size_t)max_dims->batch * sizeof(int32_t)) == cudaSuccess &&
+             cudaMemset(ctx->commit_done, 0, kMaxBatch * sizeof(unsigned int)) == cudaSuccess;
     }
     for (int i = 0; ok && i < 6; ++i) ok = cudaEventCreate(&ctx->ev[i]) == cudaSuccess;
     if (ok && attn) {
@@ -322,6 +326,7 @@ int owl_destroy(owl_ctx* ctx) {
     cudaFree(ctx->status);
     cudaFree(ctx->selftest_ns);
     cudaFree(ctx->seq_bad);
+    cudaFree(ctx->commit_done);
     cudaFree(ctx->sched_seq_begin);
     cudaFree(ctx->sched_header);
     cudaFree(ctx->part_keys);
@@ -617,10 +622,9 @@ int owl_kv_commit(owl_ctx* ctx, const owl_dims* d, void* k_cache, void* v_cache,
     p.max_nodes = d->max_nodes; p.num_kv_heads = d->num_kv_heads;
     p.page_size = d->page_size; p.page_shift = log2_exact(d->page_size);
     p.max_pages_per_seq = d->max_pages_per_seq; p.num_pages = d->num_pages; p.path_stride = d->path_stride;
-    // the second kernel's wait is what keeps a length from being bumped while a CTA of the first still reads it
-    launch_dependent(kv_commit_move_kernel, dim3(2u * (unsigned)d->num_kv_heads, (unsigned)d->batch), dim3(kCommitThreads), stream, p);
-    launch_dependent(kv_commit_lens_kernel, dim3((unsigned)d->batch), dim3(kCommitThreads), stream, p);
-    ctx->launches += 2;
+    p.seq_done = ctx->commit_done;
+    launch_dependent(kv_commit_kernel, dim3(2u * (unsigned)d->num_kv_heads, (unsigned)d->batch), dim3(kCommitThreads), stream, p);
+    ++ctx->launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_kv_commit launch");
     return OWL_OK;

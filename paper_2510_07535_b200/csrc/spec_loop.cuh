@@ -1,7 +1,7 @@
 // The steps of the decoding loop on either side of the verify pass (Algorithm 1):
 //   prepare_spec_kernel   Prepare(d): one [SPEC] leaf after every tree path, parents (= attention mask),
 //                         depth-based position ids (Section 3.2.2 "Decode Stage")
-//   kv_commit_*_kernel    "l <- l; d", "N <- N + |d|": the accepted nodes' K/V move from logical position
+//   kv_commit_kernel      "l <- l; d", "N <- N + |d|": the accepted nodes' K/V move from logical position
 //                         L + path[k] to L + k in the paged cache, the committed length grows by accept_len
 // Both are tiny and latency-bound: one CTA per sequence (and per KV head and cache for the move).
 #pragma once
@@ -101,13 +101,14 @@ struct CommitParams {
     const int32_t* accept_len;
     const int32_t* accept_path;
     int32_t* status;
+    unsigned int* seq_done;        // [kMaxBatch], 0 between calls: CTAs of the sequence that have read its length
     int32_t batch, total_nodes, nodes_uniform, max_nodes, num_kv_heads;
     int32_t page_size, page_shift, max_pages_per_seq, num_pages, path_stride;
 };
 
 constexpr int kCommitThreads = 256;
 
-// What both commit kernels decide alike for sequence b, from the inputs alone: 0 = commit, else the error code.
+// What every CTA of sequence b decides alike, from the inputs alone: 0 = commit, else the error code.
 // The accepted path must be a root path in node order (path[0] = 0, strictly increasing, below n) and every page
 // the drafted positions L .. L + n - 1 touch must exist.  Called by all threads of a CTA (uses two barriers).
 __device__ __forceinline__ int commit_verdict(const CommitParams& p, int b, int& L, int& n, int& a, int* s_path /*[kMaxNodes]*/,
@@ -139,7 +140,9 @@ __device__ __forceinline__ int commit_verdict(const CommitParams& p, int b, int&
 
 // grid (2 * Hkv, B): blockIdx.x = 2 * head + (0: K, 1: V).  Every source row is read into shared memory before any
 // destination is written, because a position can be the source of one move and the destination of a later one.
-__global__ void __launch_bounds__(kCommitThreads) kv_commit_move_kernel(const CommitParams p) {
+// The committed length grows by accept_len once all CTAs of the sequence have read the old one: each counts itself in
+// after that and the last one writes (and the counter wraps to zero for the next call).
+__global__ void __launch_bounds__(kCommitThreads) kv_commit_kernel(const CommitParams p) {
     // may be launched as a programmatic dependent: nothing is read before the kernel before it in the stream has
     // completed (a no-op in an ordinary launch); the kernel after this one may queue up and waits likewise
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -154,6 +157,11 @@ __global__ void __launch_bounds__(kCommitThreads) kv_commit_move_kernel(const Co
         if (threadIdx.x == 0 && blockIdx.x == 0) report(p.status, verdict);
         return;
     }
+    if (threadIdx.x == 0) {
+        // every thread's read of the length came before the barriers of commit_verdict
+        __threadfence();
+        if (atomicInc(p.seq_done + b, gridDim.x - 1u) == gridDim.x - 1u) p.ctx_lens[b] = L + a;
+    }
     __nv_bfloat16* cache = (blockIdx.x & 1) ? p.v_cache : p.k_cache;
     const int32_t* table = p.block_table + (long long)b * p.max_pages_per_seq;
     auto row_ptr = [&](int pos) {
@@ -166,19 +174,6 @@ __global__ void __launch_bounds__(kCommitThreads) kv_commit_move_kernel(const Co
     __syncthreads();
     for (int k = threadIdx.x >> 4; k < a; k += kCommitThreads / 16)
         if (s_path[k] != k) row_ptr(L + k)[piece] = s_rows[k * 16 + piece];
-}
-
-// One CTA per sequence, after the move kernel in stream order: the committed length grows by accept_len.
-__global__ void __launch_bounds__(kCommitThreads) kv_commit_lens_kernel(const CommitParams p) {
-    // may be launched as a programmatic dependent: nothing is read before the kernel before it in the stream has
-    // completed (a no-op in an ordinary launch); the kernel after this one may queue up and waits likewise
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ int s_path[kMaxNodes];
-    __shared__ int s_flag;
-    int L, n, a;
-    const int verdict = commit_verdict(p, blockIdx.x, L, n, a, s_path, &s_flag);
-    if (verdict == 0 && threadIdx.x == 0) p.ctx_lens[blockIdx.x] = L + a;
 }
 
 }  // namespace owl

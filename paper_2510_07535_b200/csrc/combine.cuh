@@ -92,9 +92,9 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
         if (tiles == 0) return;
         const int G = p.group;
         lrow = (n - node_base) * G + hq % G;
-        t0 = seq_begin + (long long)(hq / G) * tiles;
-        c0 = part.owner(t0);
-        c1 = part.owner(t0 + tiles - 1);
+        t0 = seq_begin + (long long)(hq / G) * (tiles + part.pen);
+        c0 = part.owner(t0 + part.pen);
+        c1 = part.owner(t0 + part.pen + tiles - 1);
         prow_first = row_of(c0 + min(lane, c1 - c0));
     };
     auto locate = [&](long long row_id) {       // every lane of the warp, same row
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             b = hit ? __ffs(hit) - 1 : 0;
             node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
             tiles = hit ? __shfl_sync(0xffffffffu, ws.tiles, b) : 0;
-            seq_begin = __shfl_sync(0xffffffffu, ws.excl_t, b);
+            seq_begin = __shfl_sync(0xffffffffu, ws.excl_t + (long long)part.pen * ws.excl_u, b);
         } else {
             int lo = 0, hi = p.batch;  // largest b with node_offsets[b] <= n
             if (p.node_offsets) {
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
             node_base = seq_node_base(p, b);
             seq_begin = sb;
-            tiles = (int)((se - sb) / p.num_kv_heads);
+            tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
         }
         plan();
     };

@@ -59,44 +59,47 @@ __device__ __forceinline__ float fast_exp2(float x) {
 __device__ __forceinline__ void report(int32_t* status, int code) { atomicCAS(status, 0, code); }
 
 // ---------------------------------------------------------------------------------------------
-// Flat partition of the split-KV pass.
+// Partition of the split-KV pass.
 //
 // A unit is (sequence b, KV head h) with all its G * n_b packed rows; it owns
-// tiles_b = ceil((L_b + n_b) / TileKeys) key tiles.  Units are laid out sequence-major, then head;
-// all their tiles form one flat range [0, total) which is cut into num_ctas contiguous pieces.  A
-// CTA's piece may start and end inside a unit; only its first and its last unit can be cut, so a
-// CTA stores at most two partials (o, lse): slot 2c for the unit its piece starts in, 2c + 1 for a later one.
-// ---------------------------------------------------------------------------------------------
-// Cut of the flat tile range [0, total) into `ctas` pieces, one per CTA.
-//   flat:    contiguous, nearly equal pieces; a piece may start and end inside a unit.
+// tiles_b = ceil((L_b + n_b) / TileKeys) key tiles.  Units are laid out sequence-major, then head, on one line, which
+// is cut into num_ctas contiguous pieces, one per CTA.  A piece may start and end inside a unit; only its first and its
+// last unit can be cut, so a CTA stores at most two partials (o, lse): slot 2c for the unit its piece starts in, 2c + 1
+// for a later one.
+//   flat:    pieces of (nearly) equal length.  On the line a unit is `pen` = kBoundaryPenaltyTiles longer than its tiles,
+//            the gap lying in front of them: what it costs a CTA to go from one unit to the next (pipeline drain,
+//            epilogue, new Q: 6.8 us at 1.23 us per tile for units of up to 128 rows, 12.3 at 2.0 for 256).  With pieces
+//            of equally many tiles the CTAs that held many short units ended last by far: 48 sequences of 200 to 6000
+//            tokens 83 to 130 us, 4 x 128K 441 to 493 us.
 //   aligned: only when every unit has the same number of tiles (`unit_tiles`) and there are at least as
 //            many CTAs as units: unit u is cut into base + (u < urem) nearly equal pieces, so no piece
-//            crosses a unit boundary.  Chosen when its largest piece is smaller than the flat piece plus
-//            what a unit boundary costs a CTA (pipeline drain, epilogue, new Q), counted in tiles.
+//            crosses a unit boundary (and there are no gaps).  Chosen when its largest piece is smaller than the flat one.
+// ---------------------------------------------------------------------------------------------
 constexpr int kBoundaryPenaltyTiles = 5;
 struct Partition {
-    long long total, q;
+    long long total, q;           // length of the line, of a piece
     int rem, ctas;
     int unit_tiles, base, urem;   // aligned mode iff unit_tiles > 0
+    int pen;                      // gap in front of a unit's tiles
     // (Every CTA runs this once, on its critical path and with cold instruction caches, where each instruction costs
     // tens of nanoseconds: one 32-bit division where the numbers allow it instead of 64-bit ones.)
-    __device__ __host__ void init(long long total_, int ctas_) {
-        total = total_; ctas = ctas_;
-        if (total_ >= 0 && total_ <= 0x7fffffffll) {
-            const unsigned qq = (unsigned)total_ / (unsigned)ctas_;
-            q = qq; rem = (int)((unsigned)total_ - qq * (unsigned)ctas_);
+    __device__ __host__ void init(long long tiles, int ctas_, int units, int uniform_tiles) {
+        ctas = ctas_;
+        pen = kBoundaryPenaltyTiles;
+        total = tiles + (long long)pen * units;
+        if (total >= 0 && total <= 0x7fffffffll) {
+            const unsigned qq = (unsigned)total / (unsigned)ctas_;
+            q = qq; rem = (int)((unsigned)total - qq * (unsigned)ctas_);
         } else {
-            q = total_ / ctas_; rem = (int)(total_ % ctas_);
+            q = total / ctas_; rem = (int)(total % ctas_);
         }
         unit_tiles = 0; base = 0; urem = 0;
-    }
-    __device__ __host__ void init(long long total_, int ctas_, int units, int uniform_tiles) {
-        init(total_, ctas_);
         if (uniform_tiles > 0 && units > 1 && units <= ctas_) {
             const int b = ctas_ / units;
-            const long long cost_aligned = (uniform_tiles + b - 1) / b;
-            const long long cost_flat = q + (rem ? 1 : 0) + kBoundaryPenaltyTiles;   // ceil(total / ctas) + penalty
-            if (cost_aligned < cost_flat) { unit_tiles = uniform_tiles; base = b; urem = ctas_ - b * units; }
+            if ((uniform_tiles + b - 1) / b < q + (rem ? 1 : 0)) {
+                unit_tiles = uniform_tiles; base = b; urem = ctas_ - b * units;
+                total = tiles; pen = 0;
+            }
         }
     }
     // [begin(c), begin(c + 1)) with one set of divisions (the pieces of a unit tile it exactly, so a piece's end is
@@ -124,7 +127,7 @@ struct Partition {
         const int qq = unit_tiles / cu, rr = unit_tiles % cu;
         return (long long)u * unit_tiles + (long long)k * qq + (k < rr ? k : rr);
     }
-    __device__ __host__ int owner(long long t) const {
+    __device__ __host__ int owner(long long t) const {        // of a place on the line
         if (unit_tiles == 0) {
             long long big = (long long)rem * (q + 1);
             if (total <= 0x7fffffffll) {      // the usual case: 32-bit divisions
@@ -143,7 +146,7 @@ struct Partition {
 
 // What the split-KV pass leaves for the combine kernel: totals and the choice of partition.
 struct SchedHeader {
-    long long total_tiles;
+    long long total_tiles;   // of all units, without gaps
     int uniform_tiles;   // tiles per unit if every schedulable sequence has the same count, else 0
     int units;
 };
@@ -173,7 +176,7 @@ constexpr int kSchedTileKeys = 128;      // key tile of the split-KV pass
 struct WarpSchedule {
     int n, L, node_base, tiles;          // this lane's sequence (tiles = 0 if it is not schedulable)
     bool ok;
-    long long my_tiles, excl_t, total;   // flat tiles of this sequence (all KV heads), of the ones before it, of all
+    long long my_tiles, excl_t, total;   // tiles of this sequence (all KV heads), of the ones before it, of all
     int my_units, excl_u, units;
     int uniform_tiles;                   // tiles per unit if every schedulable sequence has the same count, else 0
 };

@@ -23,8 +23,8 @@
 // than 2^8), writes P, then O += P V (8 MMAs over the keys, A operand from tensor memory, V as an
 // MN-major B operand).
 //
-// Work is cut as in owl_common.cuh (flat range of 128-key tiles over all units, equal pieces per
-// CTA); a CTA whose piece covers a whole unit writes the final bf16 output, otherwise a normalised
+// Work is cut as in owl_common.cuh (Partition: all units' 128-key tiles on one line, an equal piece
+// per CTA); a CTA whose piece covers a whole unit writes the final bf16 output, otherwise a normalised
 // fp32 partial and its LSE for the combine kernel.
 //
 // Every mbarrier wait is bounded (sm100_ptx.cuh).  When a wait gives up, the CTA's abort flag makes
@@ -75,14 +75,13 @@ struct Aux {
     long long total_tiles;
     int scan_units[12];
     int scan_tmin[12], scan_tmax[12];
-    int sched_unit_begin;
     short parent[kMaxNodes];
     unsigned long long anc[kMaxNodes];
 };
 static_assert(sizeof(Aux) <= kAuxBytes, "aux area too small");
 
 struct Segment {
-    int b, h, unit, n, L, node_base, M;
+    int b, h, n, L, node_base, M;
     int tiles, tile0, tile1;
     bool shared;
     __device__ __forceinline__ int iters(int s) const {
@@ -101,11 +100,11 @@ struct Segment {
     __device__ __forceinline__ int live_warps() const { return kWide ? 4 : (M + 31) >> 5; }
 };
 
-// Walks the CTA's piece [t, t_end) of the flat tile range unit by unit.  Every role runs its own
+// Walks the CTA's piece [t, t_end) of the line unit by unit.  Every role runs its own
 // copy; all copies see the same sequence of segments.
 struct Walker {
-    int b, unit_begin;
-    long long seq_begin, t, t_end;
+    int b, pen;
+    long long seq_begin, t, t_end;      // places on the line of Partition
     // the sequence `b` as last loaded (most segments of a piece lie in the same sequence)
     int cur_b = -1, cur_n = 0, cur_L = 0, cur_tiles = 0, cur_node_base = 0;
     bool cur_ok = false;
@@ -124,30 +123,31 @@ struct Walker {
         if (t >= t_end) return false;
         while (b < p.batch) {
             if (cur_b != b) load_seq(p);
-            const long long flat = (long long)cur_tiles * p.num_kv_heads;
+            const long long flat = cur_ok ? (long long)(cur_tiles + pen) * p.num_kv_heads : 0;
             if (t < seq_begin + flat) break;
             seq_begin += flat;
-            unit_begin += cur_ok ? p.num_kv_heads : 0;
             ++b;
         }
         if (b >= p.batch) { t = t_end; return false; }
-        const int tiles = cur_tiles;
-        const unsigned local = (unsigned)(t - seq_begin);   // < tiles * Hkv <= 2^24 * 2^7
-        g.b = b; g.n = cur_n; g.L = cur_L; g.tiles = tiles;
-        g.h = (int)(local / (unsigned)tiles);
-        g.tile0 = (int)(local - (unsigned)g.h * (unsigned)tiles);
+        const int len = cur_tiles + pen;
+        const unsigned local = (unsigned)(t - seq_begin);   // < len * Hkv <= 2^24 * 2^7
+        g.b = b; g.n = cur_n; g.L = cur_L; g.tiles = cur_tiles;
+        g.h = (int)(local / (unsigned)len);
+        const int at = (int)(local - (unsigned)g.h * (unsigned)len);
         const long long left = t_end - t;
-        g.tile1 = (int)(g.tile0 + left < tiles ? g.tile0 + left : tiles);
-        g.unit = unit_begin + g.h;
+        const int end = (int)(at + left < len ? at + left : len);
+        t += end - at;
+        g.tile0 = max(at - pen, 0);
+        g.tile1 = end - pen;
+        if (g.tile1 <= 0) return false;                     // the piece ends in the gap before the unit
         g.node_base = cur_node_base;
         g.M = cur_n * p.group;
         g.shared = kWide && g.M > 128;
-        t += g.tile1 - g.tile0;
         return true;
     }
 };
 
-// Block-wide: totals of the flat tile range, the choice of partition and the first sequence of this
+// Block-wide: totals of tiles and units, the choice of partition and the first sequence of this
 // CTA's piece.  CTA 0 also leaves the per-sequence prefix and the header for the combine kernel.
 __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker& w) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -191,37 +191,37 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
         tmin = min(tmin, aux->scan_tmin[w2]); tmax = max(tmax, aux->scan_tmax[w2]);
     }
     const int uniform_tiles = (units > 0 && tmin == tmax) ? tmin : 0;
-    const long long excl_t = off_t + inc_t - my_tiles;
-    const int excl_u = off_u + inc_u - my_units;
     Partition part;
     part.init(total, gridDim.x, units, uniform_tiles);
+    // this thread's sequences on the line
+    const long long excl = off_t + inc_t - my_tiles + (long long)part.pen * (off_u + inc_u - my_units);
+    const long long my_len = my_tiles + (long long)part.pen * my_units;
     long long t_begin, t_end;
     part.range(blockIdx.x, t_begin, t_end);
-    if (t_begin < t_end && my_tiles > 0 && t_begin >= excl_t && t_begin < excl_t + my_tiles) {
+    if (t_begin < t_end && my_len > 0 && t_begin >= excl && t_begin < excl + my_len) {
         aux->sched_b0 = b_lo;                 // the walker skips ahead from the first sequence of this thread
-        aux->sched_tile_begin = excl_t;
-        aux->sched_unit_begin = excl_u;
+        aux->sched_tile_begin = excl;
     }
     if (blockIdx.x == 0) {
-        long long run = excl_t;
+        long long run = excl;
         for (int b = b_lo; b < b_hi; ++b) {
             p.sched_seq_begin[b] = run;
             const int n = seq_nodes(p, b), L = p.ctx_lens[b];
-            if (seq_shape_ok(p, b, n, L)) run += (long long)((L + n + kTileKeys - 1) / kTileKeys) * p.num_kv_heads;
+            if (seq_shape_ok(p, b, n, L)) run += (long long)((L + n + kTileKeys - 1) / kTileKeys + part.pen) * p.num_kv_heads;
         }
         if (tid == 0) {
-            p.sched_seq_begin[p.batch] = total;
+            p.sched_seq_begin[p.batch] = part.total;
             p.sched_header->total_tiles = total;
             p.sched_header->uniform_tiles = uniform_tiles;
             p.sched_header->units = units;
         }
     }
     __syncthreads();
+    w.pen = part.pen;
     w.t = t_begin;
     w.t_end = t_end;
     w.b = aux->sched_b0;
     w.seq_begin = aux->sched_tile_begin;
-    w.unit_begin = aux->sched_unit_begin;
 }
 
 // Batches of at most 32 sequences: every warp derives the same schedule on its own (lane b holds sequence
@@ -236,28 +236,27 @@ __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w)
         report(p.status, seq_tree_shape_ok(p, lane, n) ? kErrBadPage : kErrBadTree);
         p.seq_bad[lane] = p.epoch;
     }
-    const long long my_tiles = ws.my_tiles, total = ws.total, excl_t = ws.excl_t;
-    const int units = ws.units, uniform_tiles = ws.uniform_tiles, excl_u = ws.excl_u;
     Partition part;
-    part.init(total, gridDim.x, units, uniform_tiles);
+    part.init(ws.total, gridDim.x, ws.units, ws.uniform_tiles);
+    const long long excl = ws.excl_t + (long long)part.pen * ws.excl_u, my_len = ws.my_tiles + (long long)part.pen * ws.my_units;
     long long t_begin, t_end;
     part.range(blockIdx.x, t_begin, t_end);
-    const unsigned owner = __ballot_sync(0xffffffffu, my_tiles > 0 && t_begin >= excl_t && t_begin < excl_t + my_tiles);
+    const unsigned owner = __ballot_sync(0xffffffffu, my_len > 0 && t_begin >= excl && t_begin < excl + my_len);
     if (blockIdx.x == 0 && threadIdx.x < 32) {
-        if (lane < p.batch) p.sched_seq_begin[lane] = excl_t;
+        if (lane < p.batch) p.sched_seq_begin[lane] = excl;
         if (lane == 0) {
-            p.sched_seq_begin[p.batch] = total;
-            p.sched_header->total_tiles = total;
-            p.sched_header->uniform_tiles = uniform_tiles;
-            p.sched_header->units = units;
+            p.sched_seq_begin[p.batch] = part.total;
+            p.sched_header->total_tiles = ws.total;
+            p.sched_header->uniform_tiles = ws.uniform_tiles;
+            p.sched_header->units = ws.units;
         }
     }
+    w.pen = part.pen;
     w.t = t_begin;
     w.t_end = (t_begin < t_end && owner) ? t_end : t_begin;
     const int b0 = owner ? __ffs(owner) - 1 : 0;
     w.b = b0;
-    w.seq_begin = __shfl_sync(0xffffffffu, excl_t, b0);
-    w.unit_begin = __shfl_sync(0xffffffffu, excl_u, b0);
+    w.seq_begin = __shfl_sync(0xffffffffu, excl, b0);
     w.cur_b = b0;
     w.cur_n = __shfl_sync(0xffffffffu, n, b0);
     w.cur_L = __shfl_sync(0xffffffffu, L, b0);
@@ -922,7 +921,7 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         mbar_init(smem_u32(&aux->q_full), 256);
         aux->abort_flag = 0;
         aux->seg_bad_tree = 0;
-        aux->sched_b0 = 0; aux->sched_tile_begin = 0; aux->sched_unit_begin = 0;
+        aux->sched_b0 = 0; aux->sched_tile_begin = 0;
         fence_barrier_init();
         tma_prefetch_desc(&kmap);
         tma_prefetch_desc(&vmap);

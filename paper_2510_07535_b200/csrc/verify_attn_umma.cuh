@@ -61,29 +61,15 @@ constexpr int kSmemBytes = kAuxOff + kAuxBytes;          // 232448 = 227 KB
 constexpr uint32_t kTmemCols = 512;
 constexpr float kLazyRescale = 8.0f;       // log2 units
 
-struct Aux {
-    uint64_t full[kTilesInFlight];   // one per tile: its K and its V slot complete the same barrier
-    uint64_t empty[kSlots];
-    uint64_t s_full[2], o_done[2];
-    uint64_t q_full;
-    uint32_t tmem_base;
-    int abort_flag;
-    int seg_bad_tree;
-    int sched_b0;
-    long long sched_tile_begin;
-    long long scan_tiles[12];
-    long long total_tiles;
-    int scan_units[12];
-    int scan_tmin[12], scan_tmax[12];
-    short parent[kMaxNodes];
-    unsigned long long anc[kMaxNodes];
-};
-static_assert(sizeof(Aux) <= kAuxBytes, "aux area too small");
-
+// A unit's tiles [tile0, tile1) that this CTA works through, as the producer announces it to the other roles.  Eight
+// places are enough: the producer is never more than four segments ahead of the slowest reader (three tiles fit the
+// ring, and a segment's products wait for its Q, which is loaded after the stores of the segment before).
+constexpr int kSegs = 8;
 struct Segment {
     int b, h, n, L, node_base, M;
-    int tiles, tile0, tile1;
+    int tiles, tile0, tile1;        // tile1 == 0: no more segments
     bool shared;
+    int bad_page;                   // the producer met a page out of range (set before the arrival of the tile)
     __device__ __forceinline__ int iters(int s) const {
         const int T = tile1 - tile0;
         return shared ? T : (s == 0 ? (T + 1) >> 1 : T >> 1);
@@ -100,8 +86,30 @@ struct Segment {
     __device__ __forceinline__ int live_warps() const { return kWide ? 4 : (M + 31) >> 5; }
 };
 
-// Walks the CTA's piece [t, t_end) of the line unit by unit.  Every role runs its own
-// copy; all copies see the same sequence of segments.
+struct Aux {
+    uint64_t seg_full[kSegs];
+    uint64_t full[kTilesInFlight];   // one per tile: its K and its V slot complete the same barrier
+    uint64_t empty[kSlots];
+    uint64_t s_full[2], o_done[2];
+    uint64_t q_full;
+    uint32_t tmem_base;
+    int abort_flag;
+    int seg_bad_tree;
+    Segment seg[kSegs];
+    int sched_b0;
+    long long sched_tile_begin;
+    long long scan_tiles[12];
+    long long total_tiles;
+    int scan_units[12];
+    int scan_tmin[12], scan_tmax[12];
+    short parent[kMaxNodes];
+    unsigned long long anc[kMaxNodes];
+};
+static_assert(sizeof(Aux) <= kAuxBytes, "aux area too small");
+
+// Walks the CTA's piece [t, t_end) of the line unit by unit.  The producer warp does, one segment after the other, and
+// announces each to the other roles in shared memory: with a walker and the schedule's arithmetic in every role the
+// text was a third longer and a CTA barrier stood between the schedule and the first copy.
 struct Walker {
     int b, pen;
     long long seq_begin, t, t_end;      // places on the line of Partition
@@ -224,15 +232,14 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
     w.seq_begin = aux->sched_tile_begin;
 }
 
-// Batches of at most 32 sequences: every warp derives the same schedule on its own (lane b holds sequence
-// b, prefix sums by shuffle), with no shared memory and no CTA-wide barrier, so that each role can start
-// as soon as its own loads have returned.
+// Batches of at most 32 sequences: the producer warp derives the schedule on its own (lane b holds sequence
+// b, prefix sums by shuffle), with no shared memory and no CTA-wide barrier.
 __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w) {
     static_assert(kTileKeys == kSchedTileKeys, "the merge kernel derives the same schedule");
     const int lane = threadIdx.x & 31;
     const WarpSchedule ws = warp_schedule(p);
     const int n = ws.n, L = ws.L, node_base = ws.node_base, tiles = ws.tiles;
-    if (lane < p.batch && !ws.ok && threadIdx.x < 32) {
+    if (lane < p.batch && !ws.ok) {
         report(p.status, seq_tree_shape_ok(p, lane, n) ? kErrBadPage : kErrBadTree);
         p.seq_bad[lane] = p.epoch;
     }
@@ -242,7 +249,7 @@ __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w)
     long long t_begin, t_end;
     part.range(blockIdx.x, t_begin, t_end);
     const unsigned owner = __ballot_sync(0xffffffffu, my_len > 0 && t_begin >= excl && t_begin < excl + my_len);
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
+    if (blockIdx.x == 0) {
         if (lane < p.batch) p.sched_seq_begin[lane] = excl;
         if (lane == 0) {
             p.sched_seq_begin[p.batch] = part.total;
@@ -265,6 +272,22 @@ __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w)
     w.cur_ok = true;
 }
 
+// The CTA's segment seg_no, once the producer has announced it (tile1 == 0: there is none).  The wait does not look at
+// the abort flag: every role must take the same segments, whatever gave up.  The producer announces all of them in any
+// case, its own waits being bounded; the limit here, ten times theirs, is never reached.
+__device__ __forceinline__ Segment next_segment(Aux* aux, uint32_t seg_no) {
+    const uint32_t bar = smem_u32(&aux->seg_full[seg_no % kSegs]), parity = (seg_no / kSegs) & 1u;
+    uint64_t t0 = 0;
+    for (uint32_t polls = 0; !mbar_try_wait(bar, parity); ++polls) {
+        if ((polls & 255u) == 255u) {
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > 10 * kWaitLimitNs) { Segment none{}; return none; }
+        }
+    }
+    return aux->seg[seg_no % kSegs];
+}
+
 // ------------------------------------------------------------------------------------------ producer
 template <bool kWide>
 __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtensorMap* kmap, const CUtensorMap* vmap,
@@ -277,8 +300,18 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
     uint32_t item = 0;
     // K/V are read once: let them leave L2 first, so that Q, the partials, the tables and the code stay
     const uint64_t stream_policy = l2_policy_evict_first();
-    Segment g;
-    while (w.template next<kWide>(p, g)) {
+    for (uint32_t seg_no = 0;; ++seg_no) {
+        Segment g;
+        const bool more = w.template next<kWide>(p, g);
+        Segment& announced = aux->seg[seg_no % kSegs];
+        if (lane == 0) {
+            if (!more) g.tile0 = g.tile1 = 0;
+            g.bad_page = 0;
+            announced = g;
+            mbar_arrive(smem_u32(&aux->seg_full[seg_no % kSegs]));
+        }
+        __syncwarp();
+        if (!more) break;
         const int keys = g.L + g.n;
         const int pages_valid = (keys + p.page_size - 1) >> p.page_shift;
         const int32_t* table = p.block_table + (long long)g.b * p.max_pages_per_seq;
@@ -288,7 +321,11 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
             if (lane < ppt && lp < pages_valid) {
                 const int pg = table[lp];
                 if ((unsigned)pg < (unsigned)p.num_pages) c = pg * p.num_kv_heads + g.h;
-                else { report(p.status, kErrBadPage); p.seq_bad[g.b] = p.epoch; }
+                else {
+                    report(p.status, kErrBadPage);
+                    p.seq_bad[g.b] = p.epoch;                 // for the merge
+                    const_cast<volatile int&>(announced.bad_page) = 1;
+                }
             }
             return c;
         };
@@ -332,7 +369,7 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
 //  * the iterations in which both streams have both products to issue run in a loop of their own without
 //    per-product conditions; the first and the last ones of a segment take the general form.
 template <bool kWide, bool kF16>
-__device__ __forceinline__ void mma_loop(const AttnParams& p, Aux* aux, uint32_t smem_base, uint32_t tmem, Walker w) {
+__device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t tmem) {
     constexpr unsigned kAll = 0xffffffffu;
     volatile int* abort_flag = &aux->abort_flag;
     constexpr uint32_t idesc_qk = umma_idesc_16bit(128, kTileKeys, 0, 0, kF16);
@@ -344,12 +381,11 @@ __device__ __forceinline__ void mma_loop(const AttnParams& p, Aux* aux, uint32_t
     const uint64_t q_desc0 = umma_smem_desc_sw128(smem_base, 16, 1024);
     const uint64_t k_desc0 = umma_smem_desc_sw128(ring, 16, 2048), v_desc0 = umma_smem_desc_sw128(ring, 1024, 2048);
     uint32_t seg_no = 0, item_base = 0;
-    Segment g;
 
     for (;;) {
-        const bool more = w.template next<kWide>(p, g);
-        if (!__any_sync(kAll, more)) break;
+        const Segment g = next_segment(aux, seg_no);
         const int tile0 = __reduce_max_sync(kAll, g.tile0), tile1 = __reduce_max_sync(kAll, g.tile1);
+        if (tile1 == 0) break;
         const bool shared = kWide && __reduce_max_sync(kAll, g.shared ? 1 : 0) != 0;
         // threads on the hand-off barrier of P: a stream's live softmax warps and this one
         const int p_threads = kWide ? 160 : 32 + 32 * __reduce_max_sync(kAll, g.template live_warps<kWide>());
@@ -538,7 +574,7 @@ __device__ __forceinline__ void store_rows32(const AttnParams& p, float* stage, 
 }
 
 template <bool kWide, bool kF16>
-__device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsigned char* smem, uint32_t tmem, Walker w,
+__device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsigned char* smem, uint32_t tmem,
                                              const int s /*stream*/) {
     const int wtid = threadIdx.x - 128 - s * 128;          // 0..127 inside the warpgroup
     const int row_local = wtid;                             // TMEM lane = (warp % 4) * 32 + lane
@@ -549,9 +585,10 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
     const int G = p.group;
     uint32_t it = 0, seg_no = 0, od_phase = 0;   // od_phase: segments of this stream that issued a product
     uint32_t tile_base = 0;                      // key tiles of the CTA's earlier segments (the ring counts them through)
-    Segment g;
 
-    while (w.template next<kWide>(p, g)) {
+    for (;;) {
+        const Segment g = next_segment(aux, seg_no);
+        if (g.tile1 == 0) break;
         // ---- Q rows (16-byte asynchronous copies, rows beyond M zero-filled) and, in stream 0's warpgroup, the
         // ancestor masks; every global read of the segment start is in flight at the same time
         int parent_i = -1;
@@ -829,7 +866,8 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         float (*ml)[128][3] = reinterpret_cast<float (*)[128][3]>(smem + kQBytes);
         if (!g.shared) { ml[s][row_local][0] = m; ml[s][row_local][1] = l; ml[s][row_local][2] = lx; }
         named_barrier(1, 256);                 // both streams done: all MMAs of the segment have completed
-        const bool write_ok = !bad_tree && !*abort_flag && *reinterpret_cast<volatile int32_t*>(p.seq_bad + g.b) != p.epoch;
+        // (looking up seq_bad in global memory here stood between a unit's last product and its stores)
+        const bool write_ok = !bad_tree && !*abort_flag && !const_cast<volatile int&>(aux->seg[seg_no % kSegs].bad_page);
         // only the first and the last unit of a CTA's piece can be cut: two partial slots per CTA
         const long long part_row = (2ll * blockIdx.x + (seg_no > 0 ? 1 : 0)) * p.rows_per_slot + rr;
         const long long out_row = rr < g.M ? (long long)(g.node_base + rr / G) * p.num_q_heads + g.h * G + rr % G : 0;
@@ -919,6 +957,7 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
             mbar_init(smem_u32(&aux->o_done[s]), 1);
         }
         mbar_init(smem_u32(&aux->q_full), 256);
+        for (int i = 0; i < kSegs; ++i) mbar_init(smem_u32(&aux->seg_full[i]), 1);
         aux->abort_flag = 0;
         aux->seg_bad_tree = 0;
         aux->sched_b0 = 0; aux->sched_tile_begin = 0;
@@ -927,36 +966,45 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         tma_prefetch_desc(&vmap);
     }
     if (warp == 0) { tmem_alloc(smem_u32(&aux->tmem_base), kTmemCols); tmem_relinquish(); }
-    // launched as a programmatic dependent itself: everything above touched no input; from here on the kernel
-    // before this one in the stream has completed (a no-op in an ordinary launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // The combine kernel is launched as a programmatic dependent and may queue up behind this grid's CTAs from here
-    // on.  It reads the call's inputs (lengths, offsets) before its own wait: triggering only after this grid's wait
-    // keeps those reads ordered after whatever kernel wrote them earlier in the stream.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    Walker w;
-    if (!kManySeqs) build_walk_small(p, w);        // its global loads overlap the set-up above
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = aux->tmem_base;
-    if (kManySeqs) build_walk(p, aux, w);
+    // Launched as a programmatic dependent itself: everything so far touched no input.  Each role waits for the kernel
+    // before this one in the stream itself, after the jump into its code (a no-op in an ordinary launch).
+    // The combine kernel is launched as a programmatic dependent and may queue up behind this grid's CTAs from then
+    // on.  It reads the call's inputs (lengths, offsets) before its own wait: triggering only after this grid's wait
+    // keeps those reads ordered after whatever kernel wrote them earlier in the stream.
+    auto wait_for_inputs = [] {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    };
+    Walker w;
+    if (kManySeqs) {                    // the block-wide schedule
+        wait_for_inputs();
+        build_walk(p, aux, w);
+    }
 
     // registers move from the warpgroup of the producer / MMA warps to the two softmax warpgroups,
     // whose threads each hold a 128-column row of S: 128 x 72 + 256 x 216 = 384 x 168, the registers the CTA was launched with
     uint32_t items = 0;
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-        if (warp == 0) producer_loop<kWide>(p, &kmap, &vmap, aux, smem_base + kRingOff, w, items);
-        else if (warp == 1) mma_loop<kWide, kF16>(p, aux, smem_base, tmem, w);
-        else if (kFused) {
+        if (!kManySeqs) wait_for_inputs();
+        if (warp == 0) {
+            if (!kManySeqs) build_walk_small(p, w);
+            producer_loop<kWide>(p, &kmap, &vmap, aux, smem_base + kRingOff, w, items);
+        } else if (warp == 1) {
+            mma_loop<kWide, kF16>(aux, smem_base, tmem);
+        } else if (kFused) {
             const long long items = (long long)ap.total_nodes * ap.chunks;
             for (long long it = 2ll * blockIdx.x + (warp - 2); it < items; it += 2ll * gridDim.x)
                 argmax_scan_chunk_warp<false>(ap, (int)(it / ap.chunks), (int)(it % ap.chunks));
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-        softmax_loop<kWide, kF16>(p, aux, smem, tmem, w, warp >= 8 ? 1 : 0);
+        if (!kManySeqs) wait_for_inputs();
+        softmax_loop<kWide, kF16>(p, aux, smem, tmem, warp >= 8 ? 1 : 0);
     }
 
     tc_fence_before();

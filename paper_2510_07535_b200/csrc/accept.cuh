@@ -63,6 +63,7 @@ struct AcceptParams {
     unsigned int* seq_counter;       // [2, batch]: chunk keys of the sequence stored so far; set epoch & 1 is in use
     uint32_t epoch;                  // call number: the other set is cleared for the next call
     int32_t counter_stride;          // distance between the two sets
+    int32_t early;                   // the kernel before this one in the stream is the attention pass of the same step
     int32_t* status;
     int32_t batch, total_nodes, nodes_uniform, max_nodes, vocab, path_stride;
     int32_t chunk, chunks;           // floats per item, items per row
@@ -257,8 +258,11 @@ constexpr int kArgmaxOffsMax = 1024;            // sequences whose packed offset
 
 __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const AcceptParams p) {
     // may be launched as a programmatic dependent of the kernel before it in the stream: nothing is read
-    // before that kernel has completed (a no-op in an ordinary launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // before that kernel has completed (a no-op in an ordinary launch).  After the attention pass of the same step the
+    // scan need not wait: the pass lets its dependents start only once everything before it has completed, and the
+    // scan reads nothing of the pass.  The CTAs then fill the SMs as their attention CTAs end (which is tens of
+    // microseconds apart), and wait before they exit, so that the merge that follows finds the pass completed.
+    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may queue up; it waits likewise
     __shared__ int s_note[kArgmaxNoteMax];
     __shared__ int s_notes;
@@ -326,6 +330,7 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const Ac
         accept_walk_seq(p, s_note[k]);
         __syncthreads();
     }
+    if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Grid of the scan for `items` (row, chunk) items on a device with `sms` multiprocessors: as many warps as give

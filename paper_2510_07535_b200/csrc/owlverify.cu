@@ -339,12 +339,15 @@ int owl_destroy(owl_ctx* ctx) {
     return OWL_OK;
 }
 
-// Attention of a verify step.  `ap` non-null: the logits scan rides in the attention kernel's
-// spare warps and the acceptance walk in the merge kernel, two launches for the whole step.
+static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool early);
+
+// Attention of a verify step.  `ap` non-null: the acceptance of the same step.  A small scan rides in the attention
+// kernel's spare warps and the walk in the merge kernel, two launches for the whole step; a larger one (`own_scan`) is a
+// kernel of its own between the attention pass and its merge, where it fills the SMs that the pass leaves one by one.
 static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, const void* k_cache, const void* v_cache,
                             const int32_t* block_table, const int32_t* ctx_lens, const int32_t* node_offsets,
-                            const int32_t* tree_parent, void* out, float* lse, void* stream_, const AcceptParams* ap,
-                            bool fp16 = false) {
+                            const int32_t* tree_parent, void* out, float* lse, void* stream_, AcceptParams* ap,
+                            bool fp16 = false, bool own_scan = false) {
     if (!ctx) return OWL_ERR_INVALID_ARG;
     int rc = check_dims(d, true, false);
     if (rc != OWL_OK) return rc;
@@ -436,18 +439,24 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
         // the instance that holds only this call's case: block-wide schedule above 32 sequences, the two-row-block
         // mode only if a unit (G * max_nodes rows at most) can exceed 128 rows, the logits scan only in a step
         const bool many = d->batch > 32, wide = G * d->max_nodes > 128;
-        cudaLaunchKernelEx(&cfg, umma_kernel(many, wide, ap != nullptr, fp16), p, maps->kmap, maps->vmap, ap ? *ap : AcceptParams{});
+        cudaLaunchKernelEx(&cfg, umma_kernel(many, wide, ap && !own_scan, fp16), p, maps->kmap, maps->vmap, ap ? *ap : AcceptParams{});
     }
     ++ctx->launches;
     if (ctx->profiling) cudaEventRecord(ctx->ev[1], stream);
-    const size_t stage_bytes = combine_smem_bytes(p.combine_group, grid + (ap ? (unsigned)d->batch : 0u), ctx->sm_count);
-    if (ap)
+    if (own_scan) {
+        if (!ctx->profiling) launch_accept(ctx, *ap, stream, true);
+        ap = ctx->profiling ? ap : nullptr;
+    }
+    const bool walk_here = ap && !own_scan;
+    const size_t stage_bytes = combine_smem_bytes(p.combine_group, grid + (walk_here ? (unsigned)d->batch : 0u), ctx->sm_count);
+    if (walk_here)
         launch_dependent_smem(combine_sched_kernel<true>, dim3(grid + (unsigned)d->batch), dim3(kCombineWarps * 32), stage_bytes, stream,
                               p, *ap);
     else
         launch_dependent_smem(combine_sched_kernel<false>, dim3(grid), dim3(kCombineWarps * 32), stage_bytes, stream, p, AcceptParams{});
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[2], stream); ctx->ev_attn_valid = true; }
+    if (own_scan && ap) launch_accept(ctx, *ap, stream, false);      // profiling: each kernel timed by itself
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_verify_attn launch");
     return OWL_OK;
@@ -504,6 +513,19 @@ static int accept_params(owl_ctx* ctx, const owl_dims* d, const float* logits, c
     return OWL_OK;
 }
 
+// The scan with its walk as a kernel of its own; the walk runs in the CTA that finishes a sequence.
+static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool early) {
+    p.seq_counter = ctx->seq_counter;
+    p.counter_stride = ctx->max_dims.batch;
+    p.epoch = ++ctx->accept_epoch;
+    p.early = early ? 1 : 0;
+    if (ctx->profiling) cudaEventRecord(ctx->ev[3], stream);
+    launch_dependent(argmax_partial_kernel, dim3(argmax_grid((long long)p.chunks * p.total_nodes, ctx->sm_count)), dim3(kArgmaxThreads),
+                     stream, p);
+    ++ctx->launches;
+    if (ctx->profiling) { cudaEventRecord(ctx->ev[4], stream); ctx->ev_accept_valid = true; }
+}
+
 static int tree_accept_impl(owl_ctx* ctx, const owl_dims* d, const float* logits, const int32_t* draft_tokens,
                             const int32_t* node_offsets, const int32_t* tree_parent, int32_t* accept_len,
                             int32_t* accept_path, int32_t* bonus_token, int32_t* spec_node, int32_t* node_argmax,
@@ -513,16 +535,7 @@ static int tree_accept_impl(owl_ctx* ctx, const owl_dims* d, const float* logits
                                  node_argmax, p, spec_node);
     if (rc != OWL_OK) return rc;
     DeviceGuard guard(ctx->device);
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    p.seq_counter = ctx->seq_counter;
-    p.counter_stride = ctx->max_dims.batch;
-    p.epoch = ++ctx->accept_epoch;
-    if (ctx->profiling) cudaEventRecord(ctx->ev[3], stream);
-    dim3 grid(argmax_grid((long long)p.chunks * d->total_nodes, ctx->sm_count));
-    launch_dependent(argmax_partial_kernel, grid, dim3(kArgmaxThreads), stream, p);   // the walk runs in the CTA that finishes a sequence
-    ++ctx->launches;
-    if (ctx->profiling) cudaEventRecord(ctx->ev[4], stream);
-    if (ctx->profiling) ctx->ev_accept_valid = true;
+    launch_accept(ctx, p, static_cast<cudaStream_t>(stream_), false);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_tree_accept launch");
     return OWL_OK;
@@ -709,20 +722,16 @@ int owl_verify_step(owl_ctx* ctx, const owl_dims* d, const void* q, const void* 
     // a larger one slows the attention down by more than its own kernel costs (measured: 4 x 64 nodes of a 128K
     // vocabulary, 570 -> 605 us), so it follows as a kernel of its own in stream order.
     const long long scan_items = (long long)d->total_nodes * ((d->vocab + kArgmaxChunk - 1) / kArgmaxChunk);
-    if (scan_items > 1024) {
-        rc = owl_verify_attn(ctx, d, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse, stream_);
-        if (rc != OWL_OK) return rc;
-        return owl_tree_accept(ctx, d, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token,
-                               node_argmax, stream_);
-    }
+    const bool own_scan = scan_items > 1024;
     // Two launches: the attention kernel, whose two spare warps per CTA scan the logits while K/V stream in, and the
     // merge kernel, which also walks the trees.
     AcceptParams ap;
     rc = accept_params(ctx, d, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token, node_argmax, ap,
-                       nullptr, kArgmaxMinChunk);   // a handful of small items per spare warp: the last ones end together
+                       nullptr, own_scan ? 0 : kArgmaxMinChunk);   // guests: small items, so that the last ones end together
     if (rc != OWL_OK) return rc;
     ctx->ev_accept_valid = false;
-    return verify_attn_impl(ctx, d, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse, stream_, &ap);
+    return verify_attn_impl(ctx, d, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse, stream_, &ap, false,
+                            own_scan);
 }
 
 int owl_verify_step_host(owl_ctx* ctx, const owl_dims* d, const void* q_h, const void* k_h, const void* v_h,

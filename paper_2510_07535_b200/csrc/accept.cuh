@@ -6,12 +6,12 @@
 // max picks the larger value and, among equal values, the lower index.  Per-lane and warp (shuffle) maxima
 // give one key per item, stored to part_keys[row][chunk] (no atomics, nothing to initialise).
 //
-// The warp that stores the last chunk key of a sequence (a per-sequence counter, bumped after a
-// __threadfence; nobody waits for anybody) notes the sequence, and its CTA does that sequence's walk in the
-// same launch: it reduces the chunk keys to arg-max tokens, evaluates for every node whether all edges on its
+// The walk reduces the chunk keys to arg-max tokens, evaluates for every node whether all edges on its
 // root path match (draft token == parent's arg-max), picks the deepest matching node (lowest index among
-// equals) and writes accept_len / accept_path / bonus_token.  Calls alternate between two sets of counters and
-// clear the idle one as a whole, so no separate clearing pass is needed.
+// equals) and writes accept_len / accept_path / bonus_token.  It follows the scan as a kernel of its own (one CTA per
+// sequence), in a verify step as extra CTAs of the merge kernel.  (The scan used to count its items per sequence, and
+// the CTA that completed one walked its tree: the fence and the atomic after every item cost 1.35 us each with the
+// warp's loads drained, 7 of the 68 us of a 756-row scan.)
 //
 // Inside a verify step with a small scan both halves run as guests of the attention kernels: the scan in warps
 // the attention pass does not use (argmax_scan_chunk_warp), the walk in extra CTAs of the merge kernel, after
@@ -60,9 +60,6 @@ struct AcceptParams {
     int32_t* node_argmax;
     int32_t* spec_node;              // optional [B]: the [SPEC] leaf (negative draft token) under the last accepted node
     unsigned long long* part_keys;   // [total_nodes, chunks]
-    unsigned int* seq_counter;       // [2, batch]: chunk keys of the sequence stored so far; set epoch & 1 is in use
-    uint32_t epoch;                  // call number: the other set is cleared for the next call
-    int32_t counter_stride;          // distance between the two sets
     int32_t early;                   // the kernel before this one in the stream is the attention pass of the same step
     int32_t* status;
     int32_t batch, total_nodes, nodes_uniform, max_nodes, vocab, path_stride;
@@ -247,14 +244,10 @@ __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, co
 
 // Persistent scan: the grid's warps take the (row, vocabulary chunk) items in turn (consecutive warps read
 // consecutive chunks), each with eight 16-byte loads per lane in flight, so that a warp streams without the
-// per-item cost of a CTA's launch, barriers and fences.  After storing an item's key, the warp counts it for
-// the row's sequence; the warp that counts a sequence's last item notes the sequence, and when the CTA has run
-// out of items it walks the trees of the sequences it noted.  (A CTA can note at most as many as it scanned items.)
+// per-item cost of a CTA's launch and barriers.
 constexpr int kArgmaxWarps = kArgmaxThreads / 32;
 constexpr int kArgmaxCtasPerSm = 2;     // what fits at the kernel's register count
 __host__ inline long long argmax_warps(int sms) { return (long long)sms * kArgmaxCtasPerSm * kArgmaxWarps; }
-constexpr int kArgmaxNoteMax = 64;
-constexpr int kArgmaxOffsMax = 1024;            // sequences whose packed offsets a CTA keeps in shared memory
 
 __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const AcceptParams p) {
     // may be launched as a programmatic dependent of the kernel before it in the stream: nothing is read
@@ -264,23 +257,10 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const Ac
     // microseconds apart), and wait before they exit, so that the merge that follows finds the pass completed.
     if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may queue up; it waits likewise
-    __shared__ int s_note[kArgmaxNoteMax];
-    __shared__ int s_notes;
-    // packed offsets of up to kArgmaxOffsMax sequences: every item looks its sequence up by binary search, and from
-    // global memory that is log2(B) dependent round trips per item with the warp's loads drained
-    __shared__ int s_offs[kArgmaxOffsMax + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool offs_staged = p.node_offsets && p.batch <= kArgmaxOffsMax;
-    if (offs_staged)
-        for (int b = threadIdx.x; b <= p.batch; b += kArgmaxThreads) s_offs[b] = p.node_offsets[b];
-    if (threadIdx.x == 0) s_notes = 0;
+    const int warp = threadIdx.x >> 5;
     if (blockIdx.x == 0) {
-        // Once per call: clear every counter of the idle set (the next call counts there, whatever its batch), and
-        // check that the packed offsets describe this call's rows: start at 0, end at total_nodes, 1..max_nodes
-        // nodes per sequence.  With inconsistent offsets a row would count for the wrong sequence and a walk could
-        // run on keys not yet stored; the status word says so (that call's outputs are then meaningless).
-        unsigned int* idle = p.seq_counter + (size_t)((p.epoch + 1u) & 1u) * p.counter_stride;
-        for (int b = threadIdx.x; b < p.counter_stride; b += kArgmaxThreads) idle[b] = 0u;
+        // Do the packed offsets describe this call's rows: start at 0, end at total_nodes, 1..max_nodes nodes per sequence?
+        // (If not, the status word says so; the walks check what they touch.)
         if (p.node_offsets) {
             bool bad = false;
             for (int b = threadIdx.x; b < p.batch; b += kArgmaxThreads) {
@@ -290,47 +270,23 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const Ac
             if (bad) report(p.status, kErrBadTree);
         }
     }
-    __syncthreads();
     const long long items = (long long)p.total_nodes * p.chunks;
     const long long stride = (long long)gridDim.x * kArgmaxWarps;
     for (long long it = (long long)blockIdx.x * kArgmaxWarps + warp; it < items; it += stride) {
         const int row = (int)(it / p.chunks), chunk = (int)(it - (long long)row * p.chunks);
         argmax_scan_chunk_warp<true>(p, row, chunk);
-        if (lane == 0) {
-            // which sequence owns this row, and is this the last of its chunk keys?
-            int b, n_b;
-            if (p.node_offsets) {
-                const int* offs = offs_staged ? s_offs : p.node_offsets;
-                int lo = 0, hi = p.batch;   // largest b with node_offsets[b] <= row
-                while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (offs[mid] <= row) lo = mid; else hi = mid; }
-                b = lo;
-                n_b = offs[b + 1] - offs[b];
-            } else {
-                b = row / p.nodes_uniform;
-                n_b = p.nodes_uniform;
-            }
-            __threadfence();
-            // two sets of counters: this call counts in set (epoch & 1); the other one is cleared as a whole (above)
-            // for the next call, so a counter left dirty by malformed input is gone two calls later at the latest and
-            // is never counted in
-            unsigned int* ctr = p.seq_counter + (size_t)(p.epoch & 1u) * p.counter_stride + b;
-            const unsigned int want = atomicAdd(ctr, 1u) + 1u;
-            if ((long long)want == (long long)p.chunks * n_b) {
-                *ctr = 0u;                                   // a completed counter is left clean as well
-                const int slot = atomicAdd(&s_notes, 1);
-                if (slot < kArgmaxNoteMax) s_note[slot] = b;
-                else report(p.status, kErrBadTree);          // only inconsistent offsets can complete that many here
-            }
-        }
-    }
-    __threadfence();
-    __syncthreads();
-    const int notes = min(s_notes, kArgmaxNoteMax);
-    for (int k = 0; k < notes; ++k) {
-        accept_walk_seq(p, s_note[k]);
-        __syncthreads();
     }
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// One sequence's acceptance walk per CTA over the keys the scan or the LM-head product left.  `idle_keys[0, idle_len)` is
+// cleared (the key set the next product will raise; nothing of this call uses it).  Launched as a programmatic
+// dependent: it reads nothing before the kernel before it has completed.
+__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_kernel(const AcceptParams p, unsigned long long* idle_keys, int idle_len) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int i = blockIdx.x * kArgmaxThreads + threadIdx.x; i < idle_len; i += gridDim.x * kArgmaxThreads) idle_keys[i] = 0ull;
+    accept_walk_seq(p, (int)blockIdx.x);
 }
 
 // Grid of the scan for `items` (row, chunk) items on a device with `sms` multiprocessors: as many warps as give

@@ -39,8 +39,6 @@ struct owl_ctx {
     unsigned long long* part_keys = nullptr;
     unsigned long long* lm_keys = nullptr;      // two sets of one arg-max key per row for the LM-head product's epilogue
     uint32_t lm_epoch = 0;                      // calls launched so far: set (lm_epoch & 1) is in use, the other one clean
-    unsigned int* seq_counter = nullptr;
-    uint32_t accept_epoch = 0;
     long long part_keys_len = 0;
     // tensor maps over the callers' K and V caches: a few most recently used (cache pointers, geometry) pairs
     // are kept, so that a caller rotating over several caches does not pay two encodes per call
@@ -284,8 +282,6 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         alloc((void**)&ctx->part_keys, (size_t)ctx->part_keys_len * sizeof(unsigned long long));
         alloc((void**)&ctx->lm_keys, 2 * (size_t)max_dims->total_nodes * sizeof(unsigned long long));
         if (ok) ok = cudaMemset(ctx->lm_keys, 0, 2 * (size_t)max_dims->total_nodes * sizeof(unsigned long long)) == cudaSuccess;
-        alloc((void**)&ctx->seq_counter, 2 * (size_t)max_dims->batch * sizeof(unsigned int));
-        if (ok) ok = cudaMemset(ctx->seq_counter, 0, 2 * (size_t)max_dims->batch * sizeof(unsigned int)) == cudaSuccess;
     }
     if (ok) {
         ok = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess &&
@@ -331,7 +327,6 @@ int owl_destroy(owl_ctx* ctx) {
     cudaFree(ctx->sched_header);
     cudaFree(ctx->part_keys);
     cudaFree(ctx->lm_keys);
-    cudaFree(ctx->seq_counter);
     for (auto& s : ctx->stg) cudaFree(s.p);
     for (auto& ev : ctx->ev)
         if (ev) cudaEventDestroy(ev);
@@ -339,11 +334,12 @@ int owl_destroy(owl_ctx* ctx) {
     return OWL_OK;
 }
 
-static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool early);
+static void launch_scan(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool early);
+static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream);
 
 // Attention of a verify step.  `ap` non-null: the acceptance of the same step.  A small scan rides in the attention
-// kernel's spare warps and the walk in the merge kernel, two launches for the whole step; a larger one (`own_scan`) is a
-// kernel of its own between the attention pass and its merge, where it fills the SMs that the pass leaves one by one.
+// kernel's spare warps, two launches for the whole step; a larger one (`own_scan`) is a kernel of its own between the attention pass and its merge, where it fills the SMs that the pass leaves one by one.  The walk
+// rides in the merge kernel.
 static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, const void* k_cache, const void* v_cache,
                             const int32_t* block_table, const int32_t* ctx_lens, const int32_t* node_offsets,
                             const int32_t* tree_parent, void* out, float* lse, void* stream_, AcceptParams* ap,
@@ -443,11 +439,8 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     }
     ++ctx->launches;
     if (ctx->profiling) cudaEventRecord(ctx->ev[1], stream);
-    if (own_scan) {
-        if (!ctx->profiling) launch_accept(ctx, *ap, stream, true);
-        ap = ctx->profiling ? ap : nullptr;
-    }
-    const bool walk_here = ap && !own_scan;
+    if (own_scan && !ctx->profiling) launch_scan(ctx, *ap, stream, true);
+    const bool walk_here = ap && !(own_scan && ctx->profiling);
     const size_t stage_bytes = combine_smem_bytes(p.combine_group, grid + (walk_here ? (unsigned)d->batch : 0u), ctx->sm_count);
     if (walk_here)
         launch_dependent_smem(combine_sched_kernel<true>, dim3(grid + (unsigned)d->batch), dim3(kCombineWarps * 32), stage_bytes, stream,
@@ -456,7 +449,7 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
         launch_dependent_smem(combine_sched_kernel<false>, dim3(grid), dim3(kCombineWarps * 32), stage_bytes, stream, p, AcceptParams{});
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[2], stream); ctx->ev_attn_valid = true; }
-    if (own_scan && ap) launch_accept(ctx, *ap, stream, false);      // profiling: each kernel timed by itself
+    if (ap && !walk_here) launch_accept(ctx, *ap, stream);      // profiling: the halves timed apart
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_verify_attn launch");
     return OWL_OK;
@@ -513,15 +506,17 @@ static int accept_params(owl_ctx* ctx, const owl_dims* d, const float* logits, c
     return OWL_OK;
 }
 
-// The scan with its walk as a kernel of its own; the walk runs in the CTA that finishes a sequence.
-static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool early) {
-    p.seq_counter = ctx->seq_counter;
-    p.counter_stride = ctx->max_dims.batch;
-    p.epoch = ++ctx->accept_epoch;
+// The scan as a kernel of its own.
+static void launch_scan(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool early) {
     p.early = early ? 1 : 0;
+    launch_dependent_smem(argmax_partial_kernel, dim3(argmax_grid((long long)p.chunks * p.total_nodes, ctx->sm_count)), dim3(kArgmaxThreads),
+                          0, stream, p);
+    ++ctx->launches;
+}
+static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream) {
     if (ctx->profiling) cudaEventRecord(ctx->ev[3], stream);
-    launch_dependent(argmax_partial_kernel, dim3(argmax_grid((long long)p.chunks * p.total_nodes, ctx->sm_count)), dim3(kArgmaxThreads),
-                     stream, p);
+    launch_scan(ctx, p, stream, false);
+    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, static_cast<unsigned long long*>(nullptr), 0);
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[4], stream); ctx->ev_accept_valid = true; }
 }
@@ -535,7 +530,7 @@ static int tree_accept_impl(owl_ctx* ctx, const owl_dims* d, const float* logits
                                  node_argmax, p, spec_node);
     if (rc != OWL_OK) return rc;
     DeviceGuard guard(ctx->device);
-    launch_accept(ctx, p, static_cast<cudaStream_t>(stream_), false);
+    launch_accept(ctx, p, static_cast<cudaStream_t>(stream_));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_tree_accept launch");
     return OWL_OK;
@@ -672,7 +667,7 @@ int owl_lm_head_accept(owl_ctx* ctx, const owl_dims* d, int32_t hidden_dim, cons
     p.status = ctx->status;
     p.batch = d->batch; p.total_nodes = d->total_nodes; p.nodes_uniform = d->total_nodes / d->batch;
     p.max_nodes = d->max_nodes; p.vocab = d->vocab; p.path_stride = d->path_stride;
-    launch_dependent(gemm_path::accept_walk_kernel, dim3((unsigned)d->batch), dim3(kArgmaxThreads), stream, p, idle_keys,
+    launch_dependent(accept_walk_kernel, dim3((unsigned)d->batch), dim3(kArgmaxThreads), stream, p, idle_keys,
                      ctx->max_dims.total_nodes);
     ++ctx->launches;
     cudaError_t e = cudaGetLastError();
@@ -846,7 +841,7 @@ int owl_last_kernel_times(owl_ctx* ctx, void* stream_, double t[4]) {
 // those callers cannot own an owl_ctx.  For them the arg-max scratch (one 64-bit key per logits
 // row and 8192-float vocabulary chunk) and the device status word live in the fixed array below,
 // which is part of the loaded library image: every device that loads the library holds its
-// (OWL_STATIC_MAX_KEYS + 32 + 1024) * 8 bytes until the process exits, whether or not this entry point is ever called.
+// (OWL_STATIC_MAX_KEYS + 32) * 8 bytes until the process exits, whether or not this entry point is ever called.
 //
 // The array's name is only a host-side handle here; the device address handed to the kernels
 // comes from cudaGetSymbolAddress, looked up once per device with that device current.
@@ -855,20 +850,16 @@ namespace {
 
 constexpr int kStaticMaxKeys = OWL_STATIC_MAX_KEYS;            // (row, chunk) keys
 constexpr int kStaticStatusWords = 32;                         // one 256-byte line for the status word
-constexpr int kStaticCounterWords = kMaxBatch;                 // per-sequence progress counters of the scan
 constexpr int kStaticMaxDevices = 64;
 
-static __device__ __align__(256) unsigned long long g_accept_scratch[kStaticMaxKeys + kStaticStatusWords + kStaticCounterWords];
-// Every device has its own copy of the array, hence its own call counter: the counter's parity selects the set of
-// progress counters a call counts in, and the set a call clears must be the one the next call ON THAT DEVICE uses.
+static __device__ __align__(256) unsigned long long g_accept_scratch[kStaticMaxKeys + kStaticStatusWords];
+// every device has its own copy of the array
 unsigned long long* g_static_addr[kStaticMaxDevices] = {nullptr};
 bool g_static_ready[kStaticMaxDevices] = {false};
-uint32_t g_static_epoch[kStaticMaxDevices] = {0};
 std::mutex g_static_mutex;
 
-// Device address of g_accept_scratch on the current device `dev` (looked up on first use) and the number of this
-// call among the calls made on that device.
-cudaError_t static_scratch(int dev, unsigned long long** out, uint32_t* epoch) {
+// Device address of g_accept_scratch on the current device `dev` (looked up on first use).
+cudaError_t static_scratch(int dev, unsigned long long** out) {
     std::lock_guard<std::mutex> lock(g_static_mutex);
     if (!g_static_ready[dev]) {
         void* p = nullptr;
@@ -878,7 +869,6 @@ cudaError_t static_scratch(int dev, unsigned long long** out, uint32_t* epoch) {
         g_static_ready[dev] = true;
     }
     *out = g_static_addr[dev];
-    *epoch = ++g_static_epoch[dev];
     return cudaSuccess;
 }
 
@@ -899,8 +889,7 @@ extern "C" int owl_tree_accept_static(const owl_dims* d, const float* logits, co
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kStaticMaxDevices) return OWL_ERR_CUDA;
     unsigned long long* scratch = nullptr;
-    uint32_t epoch = 0;
-    if (static_scratch(dev, &scratch, &epoch) != cudaSuccess) { cudaGetLastError(); return OWL_ERR_CUDA; }
+    if (static_scratch(dev, &scratch) != cudaSuccess) { cudaGetLastError(); return OWL_ERR_CUDA; }
     // without a status word of the caller's the verdict goes to a word of the array that no call reports
     int32_t* status = device_status ? device_status : reinterpret_cast<int32_t*>(scratch + kStaticMaxKeys);
 
@@ -926,12 +915,10 @@ extern "C" int owl_tree_accept_static(const owl_dims* d, const float* logits, co
     p.max_nodes = d->max_nodes;
     p.vocab = d->vocab;
     p.path_stride = d->path_stride;
-    p.seq_counter = reinterpret_cast<unsigned int*>(scratch + kStaticMaxKeys + kStaticStatusWords);   // 2 x kMaxBatch
-    p.counter_stride = kMaxBatch;
-    p.epoch = epoch;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) { cudaGetLastError(); return OWL_ERR_CUDA; }
     argmax_partial_kernel<<<argmax_grid((long long)chunks * d->total_nodes, sms), kArgmaxThreads, 0, stream>>>(p);
+    accept_walk_kernel<<<(unsigned)p.batch, kArgmaxThreads, 0, stream>>>(p, nullptr, 0);
     if (cudaGetLastError() != cudaSuccess) return OWL_ERR_CUDA;
     return OWL_OK;
 }

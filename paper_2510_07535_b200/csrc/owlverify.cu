@@ -722,7 +722,7 @@ int owl_verify_step(owl_ctx* ctx, const owl_dims* d, const void* q, const void* 
     // merge kernel, which also walks the trees.
     AcceptParams ap;
     rc = accept_params(ctx, d, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token, node_argmax, ap,
-                       nullptr, own_scan ? 0 : kArgmaxMinChunk);   // guests: small items, so that the last ones end together
+                       nullptr, own_scan ? 0 : kArgmaxChunk);      // guests are few: what counts is the cost per item
     if (rc != OWL_OK) return rc;
     ctx->ev_accept_valid = false;
     return verify_attn_impl(ctx, d, q, k_cache, v_cache, block_table, ctx_lens, node_offsets, tree_parent, out, lse, stream_, &ap, false,

@@ -366,8 +366,7 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
 //    in; a look at an mbarrier costs 70 to 130): one per stream, on which the softmax warpgroup announces P, and
 //    one on which stream 0's warpgroup tells that it has seen the next key tile arrive (units of up to 128 rows
 //    wait for the tile itself);
-//  * the iterations in which both streams have both products to issue run in a loop of their own without
-//    per-product conditions; the first and the last ones of a segment take the general form.
+//  * one turn's text serves both streams and all tiles.
 template <bool kWide, bool kF16>
 __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t tmem) {
     constexpr unsigned kAll = 0xffffffffu;
@@ -393,124 +392,103 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
         const int T = tile1 - tile0;
         const int n_it[2] = {shared ? T : (T + 1) >> 1, shared ? T : T >> 1};
 
-        // ring slots of the K tile and of the V tile each stream needs next, as running counters
-        const uint32_t step_items = shared ? 2u : 4u;
-        uint32_t k_slot[2], v_slot[2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const uint32_t first = item_base + (shared ? 0u : 2u * (uint32_t)s);
-            k_slot[s] = first % kSlots;
-            v_slot[s] = (first + 1u) % kSlots;
-        }
-        auto advance = [&](uint32_t& slot) { slot += step_items; if (slot >= (uint32_t)kSlots) slot -= kSlots; };
-        // O_s (+)= P_s V: A from tensor memory, B = the V tile as it lies in the ring (MN-major)
-        auto issue_pv = [&](int s, uint32_t issue, uint32_t acc0) {
-            const uint32_t v_lo = (uint32_t)v_desc0 + v_slot[s] * (uint32_t)(kSlotBytes >> 4), v_hi = (uint32_t)(v_desc0 >> 32);
-            const uint32_t tO = tmem + 256 + s * 128, tP = tmem + s * 128;
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                umma_ts_lh_if(issue, tO, tP + ks * 8, v_lo + (uint32_t)(ks * 4096 >> 4), v_hi, idesc_pv, ks ? 1u : acc0);
-        };
-        // S_s = Q K^T: both operands K-major in shared memory
-        auto issue_qk = [&](int s, uint32_t issue) {
-            const uint32_t q_lo = (uint32_t)q_desc0 + (uint32_t)((shared && s) ? (kQBytes >> 4) : 0), q_hi = (uint32_t)(q_desc0 >> 32);
-            const uint32_t k_lo = (uint32_t)k_desc0 + k_slot[s] * (uint32_t)(kSlotBytes >> 4), k_hi = (uint32_t)(k_desc0 >> 32);
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    umma_ss_lh_if(issue, tmem + s * 128, q_lo + (uint32_t)((hf * 16384 + ks * 32) >> 4), q_hi,
-                                  k_lo + (uint32_t)((hf * 1024 + ks * 32) >> 4), k_hi, idesc_qk, (hf | ks) ? 1u : 0u);
-        };
-        // Before S = Q K^T of the stream's tile i + 1.  M > 128: the issue loop is what bounds the unit, and the
-        // softmax warpgroup, which has time to spare, looks at the tile's arrival barrier and passes the news on
-        // through hardware barrier 6 (about 25 clocks here).  M <= 128: the tile itself is what the warp
-        // usually waits for, and it waits on the arrival barrier directly, one wake-up instead of two.
-        auto wait_next_k = [&](int s, int i) {
-            if (shared) {
-                // (both streams read the tile: stream 1 finds what stream 0 has just made sure of)
-                if (s == 0) asm volatile("bar.sync 6, 64;" ::: "memory");
-            } else {
-                const uint32_t seq = (item_base >> 1) + (uint32_t)(2 * (i + 1) + s);
-                ok = __all_sync(kAll, mbar_wait(smem_u32(&aux->full[seq % kTilesInFlight]), (seq / kTilesInFlight) & 1u,
-                                                abort_flag)) && ok;
-            }
-        };
-        // The same two products with the k-steps in a loop, for the few iterations of the general form below (they
-        // are too rare to be worth the code size of another thirty-two unrolled instructions)
-        auto issue_pv_rolled = [&](int s, uint32_t issue, uint32_t acc0) {
-            uint64_t vdesc = v_desc0 + (uint64_t)(v_slot[s] * (uint32_t)(kSlotBytes >> 4));
-            const uint32_t tO = tmem + 256 + s * 128;
-            uint32_t tP = tmem + s * 128;
-#pragma unroll 1
-            for (int ks = 0; ks < 8; ++ks, vdesc += 4096 >> 4, tP += 8)
-                umma_ts_if(issue, tO, tP, vdesc, idesc_pv, ks ? 1u : acc0);
-        };
-        auto issue_qk_rolled = [&](int s, uint32_t issue) {
-            uint64_t qdesc = q_desc0 + (uint64_t)((shared && s) ? (kQBytes >> 4) : 0);
-            uint64_t kdesc = k_desc0 + (uint64_t)(k_slot[s] * (uint32_t)(kSlotBytes >> 4));
-#pragma unroll 1
-            for (int j = 0; j < 8; ++j) {
-                umma_ss_if(issue, tmem + s * 128, qdesc, kdesc, idesc_qk, j ? 1u : 0u);
-                // four k-steps of 32 bytes inside a 128-byte swizzle row, then the other half of the head dimension
-                qdesc += j == 3 ? (uint64_t)((16384 - 96) >> 4) : 2u;
-                kdesc += j == 3 ? (uint64_t)((1024 - 96) >> 4) : 2u;
-            }
-        };
-        // General form of one iteration: O += P V of tile i, then S = Q K^T of tile i + 1 (which overwrites the P just
-        // consumed; the tensor pipe runs them in order), each where the stream has such a tile.  i = -1 issues the
-        // first S of both streams, after this warp's own look at the arrival barrier of their first tiles.
-        auto general = [&](int i) {
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const bool last_reader = !shared || s == 1;
-                const bool do_pv = i >= 0 && i < n_it[s], do_qk = i + 1 < n_it[s];
-                if (do_pv) asm volatile("bar.sync %0, %1;" ::"r"(4 + s), "r"(p_threads) : "memory");
-                if (i < 0 && do_qk && !(shared && s == 1)) {
-                    const uint32_t seq = (item_base >> 1) + (uint32_t)s;
-                    ok = __all_sync(kAll, mbar_wait(smem_u32(&aux->full[seq % kTilesInFlight]),
-                                                    (seq / kTilesInFlight) & 1u, abort_flag)) && ok;
-                }
-                tc_fence_after();
-                uint32_t issue = (ok && do_pv) ? elected : 0u;
-                issue_pv_rolled(s, issue, i > 0 ? 1u : 0u);
-                umma_commit_if(i == n_it[s] - 1 ? issue : 0u, smem_u32(&aux->o_done[s]));   // only the segment end waits for it
-                umma_commit_if(last_reader ? issue : 0u, smem_u32(&aux->empty[v_slot[s]]));
-                if (do_pv) advance(v_slot[s]);
-                if (i >= 0 && do_qk) { wait_next_k(s, i); tc_fence_after(); }
-                issue = (ok && do_qk) ? elected : 0u;
-                issue_qk_rolled(s, issue);
-                umma_commit_if(issue, smem_u32(&aux->s_full[s]));
-                umma_commit_if(last_reader ? issue : 0u, smem_u32(&aux->empty[k_slot[s]]));
-                if (do_qk) advance(k_slot[s]);
-            }
-        };
+        // ring slots of the V tile and of the K tile that the next turn needs
+        uint32_t k_slot = item_base % kSlots, v_slot = (item_base + 1u) % kSlots;
+        // A turn: O_s += P_s V of the stream's tile i, then S_s = Q K^T of its tile i + 1 (which overwrites the P just
+        // consumed; the tensor pipe runs them in order), each where the stream has such a tile; i = -1 issues the first S
+        // of both streams.  The text of one turn serves both streams and all tiles: with the two streams unrolled (and the
+        // first and last turns in a rolled form of their own) there was twice the text to fetch into cold caches
+        // (2K step 15.5 -> 14.4 us, 32K 39.7 -> 38.3 us, round 49.3 -> 47.9 us).
 #pragma unroll 1
         for (int i = -1; i < n_it[0]; ++i) {
-            if (i < 0 || i >= n_it[1] - 1) { general(i); continue; }
-            // Steady state: both streams have both products.  (Releasing the ring slots from a softmax thread instead -
-            // a score tile's arrival covers every product issued before it - would spare this warp two commits of 60 to
-            // 100 clocks per tile, but the slots then come back late and the ring runs dry: 15 to 35 % slower.)
-            auto steady = [&]() {
-                const uint32_t issue = ok ? elected : 0u;
+            if (kWide && shared && i >= 0 && i + 1 < T) {
+                // The middle of a 256-row unit, where this warp's time is what counts: both streams have both products, and
+                // a turn has no conditions but the stream's commits (with the general turn instead 70B 660 -> 693 us;
+                // with both streams unrolled 660 -> 653 us, fp16 with 60 nodes 72.8 -> 71.0 us).
+                const uint32_t issue = ok ? elected : 0u, acc0 = i > 0 ? 1u : 0u;
+                const uint32_t v_lo = (uint32_t)v_desc0 + v_slot * (uint32_t)(kSlotBytes >> 4), v_hi = (uint32_t)(v_desc0 >> 32);
+                const uint32_t k_lo = (uint32_t)k_desc0 + k_slot * (uint32_t)(kSlotBytes >> 4), k_hi = (uint32_t)(k_desc0 >> 32);
+                const uint32_t q_hi = (uint32_t)(q_desc0 >> 32);
+                uint32_t q_lo = (uint32_t)q_desc0, tS = tmem, s_bar = smem_u32(&aux->s_full[0]);
+                const uint32_t v_empty = smem_u32(&aux->empty[0]) + v_slot * 8u, k_empty = smem_u32(&aux->empty[0]) + k_slot * 8u;
+#pragma unroll 1
+                for (uint32_t s = 0; s < 2; ++s) {
+                    asm volatile("bar.sync %0, 160;" ::"r"(4 + s) : "memory");
+                    tc_fence_after();
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
+                    for (int ks = 0; ks < 8; ++ks)
+                        umma_ts_lh_if(issue, tS + 256, tS + ks * 8, v_lo + (uint32_t)(ks * 4096 >> 4), v_hi, idesc_pv, ks ? 1u : acc0);
+                    umma_commit_if(s ? issue : 0u, v_empty);
+                    if (s == 0) asm volatile("bar.sync 6, 64;" ::: "memory");
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            umma_ss_lh_if(issue, tS, q_lo + (uint32_t)((hf * 16384 + ks * 32) >> 4), q_hi,
+                                          k_lo + (uint32_t)((hf * 1024 + ks * 32) >> 4), k_hi, idesc_qk, (hf | ks) ? 1u : 0u);
+                    umma_commit_if(issue, s_bar);
+                    umma_commit_if(s ? issue : 0u, k_empty);
+                    tS += 128; q_lo += kQBytes >> 4; s_bar += 8;
+                }
+                k_slot += 2u; if (k_slot >= (uint32_t)kSlots) k_slot -= kSlots;
+                v_slot += 2u; if (v_slot >= (uint32_t)kSlots) v_slot -= kSlots;
+                continue;
+            }
+#pragma unroll 1
+            for (uint32_t s = 0; s < 2; ++s) {
+                const int n_s = s ? n_it[1] : n_it[0];
+                const bool do_pv = i >= 0 && i < n_s, do_qk = i + 1 < n_s;
+                const bool last_reader = !shared || s == 1;
+                const uint32_t tS = tmem + s * 128;
+                if (do_pv) {
+                    // P of tile i is announced on hardware barrier 4 + s
                     asm volatile("bar.sync %0, %1;" ::"r"(4 + s), "r"(p_threads) : "memory");
                     tc_fence_after();
-                    issue_pv(s, issue, i > 0 ? 1u : 0u);
-                    if (!shared || s == 1) umma_commit_if(issue, smem_u32(&aux->empty[v_slot[s]]));
-                    advance(v_slot[s]);
-                    wait_next_k(s, i);                                      // the next K tile has landed
-                    issue_qk(s, ok ? issue : 0u);
-                    umma_commit_if(issue, smem_u32(&aux->s_full[s]));
-                    if (!shared || s == 1) umma_commit_if(issue, smem_u32(&aux->empty[k_slot[s]]));
-                    advance(k_slot[s]);
+                    const uint32_t issue = ok ? elected : 0u;
+                    // O_s (+)= P_s V: A from tensor memory, B = the V tile as it lies in the ring (MN-major)
+                    const uint32_t v_lo = (uint32_t)v_desc0 + v_slot * (uint32_t)(kSlotBytes >> 4), v_hi = (uint32_t)(v_desc0 >> 32);
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        umma_ts_lh_if(issue, tS + 256, tS + ks * 8, v_lo + (uint32_t)(ks * 4096 >> 4), v_hi, idesc_pv, ks ? 1u : (i > 0 ? 1u : 0u));
+                    umma_commit_if(i == n_s - 1 ? issue : 0u, smem_u32(&aux->o_done[0]) + s * 8u);   // only the segment end waits for it
+                    // (Releasing the ring slots from a softmax thread instead - a score tile's arrival covers every product
+                    // issued before it - spares this warp two commits per tile, but the slots come back late: 1 % slower
+                    // on 256-row units, 15 to 35 % on the bandwidth-bound ones.)
+                    umma_commit_if(last_reader ? issue : 0u, smem_u32(&aux->empty[0]) + v_slot * 8u);
                 }
-            };
-            // (The backward branch over this long unrolled body stalls the warp for some 400 clocks - the loop head has
-            // left the instruction caches by the time it is taken.  Two tiles per trip halve the count of branches but
-            // double the text; measured, neither form wins.)
-            steady();
+                if (do_qk) {
+                    // The next K tile has landed.  M > 128: the softmax warpgroup, which has time to spare, looks at the tile's
+                    // arrival barrier and passes the news on through hardware barrier 6 (about 25 clocks here, 70 to
+                    // 130 for a look at an mbarrier); stream 1 finds what stream 0 has just made sure of.  M <= 128: the tile
+                    // itself is what the warp usually waits for, on the arrival barrier directly, one wake-up instead of two.
+                    if (shared && i >= 0) {
+                        if (s == 0) asm volatile("bar.sync 6, 64;" ::: "memory");
+                    } else if (!(shared && s == 1)) {
+                        const uint32_t seq = (item_base >> 1) + (shared ? 0u : (uint32_t)(2 * (i + 1)) + s);
+                        ok = __all_sync(kAll, mbar_wait(smem_u32(&aux->full[seq % kTilesInFlight]), (seq / kTilesInFlight) & 1u,
+                                                        abort_flag)) && ok;
+                    }
+                    tc_fence_after();
+                    const uint32_t issue = ok ? elected : 0u;
+                    // S_s = Q K^T: both operands K-major in shared memory
+                    const uint32_t q_lo = (uint32_t)q_desc0 + ((shared && s) ? (uint32_t)(kQBytes >> 4) : 0u), q_hi = (uint32_t)(q_desc0 >> 32);
+                    const uint32_t k_lo = (uint32_t)k_desc0 + k_slot * (uint32_t)(kSlotBytes >> 4), k_hi = (uint32_t)(k_desc0 >> 32);
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            umma_ss_lh_if(issue, tS, q_lo + (uint32_t)((hf * 16384 + ks * 32) >> 4), q_hi,
+                                          k_lo + (uint32_t)((hf * 1024 + ks * 32) >> 4), k_hi, idesc_qk, (hf | ks) ? 1u : 0u);
+                    umma_commit_if(issue, smem_u32(&aux->s_full[0]) + s * 8u);
+                    umma_commit_if(last_reader ? issue : 0u, smem_u32(&aux->empty[0]) + k_slot * 8u);
+                }
+                // the tiles lie in the ring in the order of the turns that consume them, K and V by turns
+                if (last_reader) {
+                    k_slot += 2u;
+                    if (k_slot >= (uint32_t)kSlots) k_slot -= kSlots;
+                    if (i >= 0) { v_slot += 2u; if (v_slot >= (uint32_t)kSlots) v_slot -= kSlots; }
+                }
+            }
         }
         item_base += 2u * (uint32_t)T;
         ++seg_no;

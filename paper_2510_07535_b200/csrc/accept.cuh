@@ -162,9 +162,7 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
 // becomes rare quickly - looks for the first value that attains it.  Strict '>' and first-match keep the lowest
 // index among equal values, because a lane's indices grow along its walk; the maximum over (value, ~index) keys
 // then does not depend on how the chunk's elements are dealt out to lanes.
-// kPipelined: the next round's loads are issued before this round is reduced (twice the registers); the attention
-// kernel's guest warps, which run on 72 registers, use the plain form.
-template <bool kPipelined>
+// The next round's loads are issued before this round is reduced.
 __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, const int row, const int chunk) {
     const int lane = threadIdx.x & 31;
     const long long V = p.vocab;
@@ -209,21 +207,13 @@ __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, co
             }
         }
     };
-    if (kPipelined) {
-        float4 xa[8], xb[8];
-        if (nvec > 0) load_round(0, xa);
-        for (int v0 = 0; v0 < nvec; v0 += 2 * 32 * 8) {
-            if (v0 + 32 * 8 < nvec) load_round(v0 + 32 * 8, xb);
-            reduce_round(v0, xa);
-            if (v0 + 2 * 32 * 8 < nvec) load_round(v0 + 2 * 32 * 8, xa);
-            if (v0 + 32 * 8 < nvec) reduce_round(v0 + 32 * 8, xb);
-        }
-    } else {
-        for (int v0 = 0; v0 < nvec; v0 += 32 * 8) {
-            float4 x[8];
-            load_round(v0, x);
-            reduce_round(v0, x);
-        }
+    float4 xa[8], xb[8];
+    if (nvec > 0) load_round(0, xa);
+    for (int v0 = 0; v0 < nvec; v0 += 2 * 32 * 8) {
+        if (v0 + 32 * 8 < nvec) load_round(v0 + 32 * 8, xb);
+        reduce_round(v0, xa);
+        if (v0 + 2 * 32 * 8 < nvec) load_round(v0 + 2 * 32 * 8, xa);
+        if (v0 + 32 * 8 < nvec) reduce_round(v0 + 32 * 8, xb);
     }
     unsigned long long key = bi != 0xffffffffu ? argmax_key(bv, bi) : 0ull;
     if (lane < 8) {              // ragged ends: at most 3 + 3 elements per chunk
@@ -274,7 +264,7 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const Ac
     const long long stride = (long long)gridDim.x * kArgmaxWarps;
     for (long long it = (long long)blockIdx.x * kArgmaxWarps + warp; it < items; it += stride) {
         const int row = (int)(it / p.chunks), chunk = (int)(it - (long long)row * p.chunks);
-        argmax_scan_chunk_warp<true>(p, row, chunk);
+        argmax_scan_chunk_warp(p, row, chunk);
     }
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -964,10 +964,14 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
     }
 
     // registers move from the warpgroup of the producer / MMA warps to the two softmax warpgroups,
-    // whose threads each hold a 128-column row of S: 128 x 72 + 256 x 216 = 384 x 168, the registers the CTA was launched with
+    // whose threads each hold a 128-column row of S: 128 x 72 + 256 x 216 = 384 x 168, the registers the CTA was launched
+    // with.  The logits guests take 104 (128 x 104 + 256 x 200) to have two rounds of loads in flight instead of one: at
+    // short contexts the scan is what a step waits for (32 nodes at 9000 tokens 30.9 -> 21.9 us, 64 nodes 54.0 -> 33.9 us;
+    // 2K chain 14.4 -> 14.5, 32K 38.4 -> 38.5 us).
     uint32_t items = 0;
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if (kFused) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         if (!kManySeqs) wait_for_inputs();
         if (warp == 0) {
             if (!kManySeqs) build_walk_small(p, w);
@@ -977,10 +981,11 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         } else if (kFused) {
             const long long items = (long long)ap.total_nodes * ap.chunks;
             for (long long it = 2ll * blockIdx.x + (warp - 2); it < items; it += 2ll * gridDim.x)
-                argmax_scan_chunk_warp<false>(ap, (int)(it / ap.chunks), (int)(it % ap.chunks));
+                argmax_scan_chunk_warp(ap, (int)(it / ap.chunks), (int)(it % ap.chunks));
         }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        if (kFused) asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+        else asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
         if (!kManySeqs) wait_for_inputs();
         softmax_loop<kWide, kF16>(p, aux, smem, tmem, warp >= 8 ? 1 : 0);
     }

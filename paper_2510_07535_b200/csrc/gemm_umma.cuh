@@ -108,19 +108,25 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* tmap,
         : : "r"(dst), "l"(tmap), "r"(bar_cluster), "r"(c0), "r"(c1), "l"(policy) : "memory");
 }
 
-// The arg-max of 32 columns (rows of A) over a warp's 32 lanes (rows of B): lane j gets column j's key.  `hi` of a lane
-// without a row of B is 0, below every real value's image.
-__device__ __forceinline__ unsigned long long warp_column_argmax(const uint32_t (&v)[32], bool lane_valid, uint32_t row0) {
+__device__ __forceinline__ float redux_max_f32(float x) {       // over the warp; NaN drops out
+    float y;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+    return y;
+}
+// The arg-max of 32 columns (rows of A) over a warp's 32 lanes (rows of B, `valid` the mask of those that exist): lane j
+// gets column j's key.  NaN reads as -inf.
+__device__ __forceinline__ unsigned long long warp_column_argmax(const uint32_t (&v)[32], bool lane_valid, uint32_t valid, uint32_t row0) {
     const int lane = threadIdx.x & 31;
-    uint32_t best = 0u, who = 0u;
+    float best = -INFINITY;
+    uint32_t who = 0u;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
-        const uint32_t hi = lane_valid ? (uint32_t)(argmax_key(__uint_as_float(v[j]), 0u) >> 32) : 0u;
-        const uint32_t m = __reduce_max_sync(0xffffffffu, hi);
-        const uint32_t first = (uint32_t)__ffs((int)__ballot_sync(0xffffffffu, hi == m)) - 1u;   // lowest row of B among equals
-        if (lane == j) { best = m; who = first; }
+        const float x = lane_valid ? fmaxf(__uint_as_float(v[j]), -INFINITY) : -INFINITY;
+        const float m = redux_max_f32(x);
+        const uint32_t at = __ballot_sync(0xffffffffu, x == m);
+        if (lane == j) { best = m; who = at; }
     }
-    return best ? ((unsigned long long)best << 32) | (uint32_t)(~(row0 + who)) : 0ull;
+    return argmax_key(best, row0 + (uint32_t)__ffs((int)(who & valid)) - 1u);          // the lowest row of B among equals
 }
 
 // gridDim.x is even: CTAs 2j and 2j + 1 are pair j.
@@ -272,6 +278,7 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
             const int end = first + share < p.N ? first + share : p.N;
             const int warp_row = first + (warp & 3) * 32;               // row of B in the warp's lane 0
             const bool lane_valid = warp_row + lane < end;
+            const uint32_t valid = __ballot_sync(0xffffffffu, lane_valid);
             if (ok && warp_row < end) {
 #pragma unroll 1
                 for (int g = 0; g < kGroups; ++g) {
@@ -283,7 +290,7 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
                         tmem_ld32(tmem + lane_sel + buf * 256u + g * 256u + c4 * 32, v);
                         tmem_wait_ld();
                         if (kEpi == kEpiArgmax) {
-                            const unsigned long long key = warp_column_argmax(v, lane_valid, (uint32_t)warp_row);
+                            const unsigned long long key = warp_column_argmax(v, lane_valid, valid, (uint32_t)warp_row);
                             if (lane < left) atomicMax(&aux->best[a0 + lane], key);
                         } else if (lane_valid) {
                             float* dst = p.c + (long long)a0 * p.ldc + warp_row + lane;

@@ -164,6 +164,17 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
     if (kEpi == kEpiArgmax)
         for (int i = tid; i < kMaxRows; i += kThreads) aux->best[i] = 0ull;
     if (warp == 0 && !misaligned) { tmem_alloc_pair(smem_u32(&aux->tmem_base), 512); tmem_relinquish_pair(); }
+    if (warp == 0 && lane == 0 && !misaligned) {
+        // Ask for the ring's first fill of B to be brought to L2 under the tail of whatever precedes this kernel.  That
+        // hands nothing to this kernel yet: the copies below read L2, which holds what was written last.
+        // (cell 10 x 4096 -> 12288 75.2 -> 72.0 us, 3 x 2048 -> 5076 26.4 -> 25.5, LM head 30 x 2688 -> 32000 33.0 -> 32.2.)
+        const CUtensorMap* bmap = p.tall_rounds ? &bmap_hi : &bmap_lo;
+        const int share = (p.tall_rounds ? p.h_lo + 16 : p.h_lo) >> 1, row = pair * 2 * share + (int)rank * share;
+        const int blocks = min(p.K / kBK, stages * kQ);
+        if (row < p.N)
+            for (int kb = 0; kb < blocks; ++kb)
+                asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(bmap), "r"(kb * kBK), "r"(row) : "memory");
+    }
     // may be launched as a programmatic dependent of the kernel before it in the stream: the set-up above touched no
     // input and ran beside that kernel's tail; from here on it has completed (a no-op in an ordinary launch).  The
     // kernel after this one may queue up in turn; it waits likewise before it reads anything.

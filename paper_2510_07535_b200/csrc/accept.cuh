@@ -236,6 +236,7 @@ __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, co
 // consecutive chunks), each with eight 16-byte loads per lane in flight, so that a warp streams without the
 // per-item cost of a CTA's launch and barriers.
 constexpr int kArgmaxWarps = kArgmaxThreads / 32;
+constexpr int kScanAhead = 4096;        // floats
 constexpr int kArgmaxCtasPerSm = 2;     // what fits at the kernel's register count
 __host__ inline long long argmax_warps(int sms) { return (long long)sms * kArgmaxCtasPerSm * kArgmaxWarps; }
 
@@ -245,6 +246,18 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const Ac
     // scan need not wait: the pass lets its dependents start only once everything before it has completed, and the
     // scan reads nothing of the pass.  The CTAs then fill the SMs as their attention CTAs end (which is tens of
     // microseconds apart), and wait before they exit, so that the merge that follows finds the pass completed.
+    if (!p.early && (threadIdx.x & 31) == 0) {
+        // The warp's first rounds are asked for to L2 under the tail of whatever precedes this kernel (756 rows x 128256
+        // 61.3 -> 59.3 us per call, 60 rows 9.1 -> 8.4).  It hands nothing to this kernel yet: L2 holds what was written last.
+        const long long it = (long long)blockIdx.x * kArgmaxWarps + (threadIdx.x >> 5);
+        if (it < (long long)p.total_nodes * p.chunks) {
+            const long long row = it / p.chunks, c0 = (it - row * p.chunks) * p.chunk;
+            const long long n = min((long long)min(p.chunk, kScanAhead), (long long)p.vocab - c0);
+            const uintptr_t b = reinterpret_cast<uintptr_t>(p.logits + row * p.vocab + c0);
+            const uintptr_t lo = (b + 15) & ~(uintptr_t)15, hi = (b + 4 * n) & ~(uintptr_t)15;
+            if (hi > lo) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((uint32_t)(hi - lo)) : "memory");
+        }
+    }
     if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may queue up; it waits likewise
     const int warp = threadIdx.x >> 5;

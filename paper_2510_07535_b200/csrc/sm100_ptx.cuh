@@ -51,17 +51,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Non-blocking test of a phase (try_wait may suspend the thread for a while before it answers).
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-
 // Bounded wait.  A phase that has already completed returns true after one poll; otherwise the wait
 // returns false at once if the CTA's abort flag is up, and else spins on try_wait;
 // every 256 failed polls it looks at the abort flag and at the wall clock, and after the time limit
@@ -92,14 +81,8 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 }
 
 // ------------------------------------------------------------------------------------ TMA
-// 5-D tile load global -> shared, completion counted in bytes on an mbarrier of this CTA.
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
-                                            int c3, int c4) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-        : : "r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4) : "memory");
-}
-// Same with an L2 cache policy (from l2_policy_*).
+// 5-D tile load global -> shared, completion counted in bytes on an mbarrier of this CTA, with an L2 cache policy
+// (from l2_policy_*).
 __device__ __forceinline__ void tma_load_5d_hint(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
                                                  int c3, int c4, uint64_t policy) {
     asm volatile(
@@ -129,11 +112,6 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// One arrival on `bar` once every tcgen05.mma this thread issued before has completed.
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 
 // ------------------------------------------------------------------------------------ CTA pairs (cluster of two)
 // Two CTAs of a cluster on neighbouring SMs run one tcgen05.mma of M = 256 together (cta_group::2): each holds its
@@ -193,7 +171,7 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // D[tmem of both CTAs] (+)= A[smem of both] * B[smem of both], M = 256; issued by one thread of the even-ranked CTA.
-// Descriptors as (low, high) words, as in umma_ss_lh below.
+// Descriptors as (low, high) words, as in umma_ss_lh_if below.
 __device__ __forceinline__ void umma_ss_pair_lh(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                                 uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -233,71 +211,12 @@ __host__ __device__ constexpr uint32_t umma_idesc_16bit(int m, int n, int a_mn_m
            ((uint32_t)b_mn_major << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.
-__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        : : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]; issued by one thread.
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
-        : : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-// Same instructions with the descriptors given as (low, high) words.  Within a batch of k-steps only the
-// low word (the start address) changes, so the issuing thread has one value per operand to refresh
-// between two instructions instead of whole 64-bit descriptors.
-__device__ __forceinline__ void umma_ss_lh(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                           uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %2};\n\t"
-        "mov.b64 db, {%3, %4};\n\t"
-        "setp.ne.b32 p, %6, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}\n"
-        : : "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_ts_lh(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
-                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}\n"
-        : : "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-// The same two instructions and the commit for a warp that stays converged: every lane executes them and `issue`
-// (non-zero in the one elected lane, and only when there is work) is the guard.  With no divergent branch around
-// them the compiler may keep descriptors, addresses and loop state in uniform registers; issued from inside an
-// `if (lane == 0)` block the same sequence ran 20 % slower as soon as other warps of the SM sub-partition had
-// arithmetic to issue, and at the tensor pipe's own rate (64 clocks per 128x128x16) in this form.
-__device__ __forceinline__ void umma_ss_if(uint32_t issue, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        : : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(issue) : "memory");
-}
-__device__ __forceinline__ void umma_ts_if(uint32_t issue, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
-        : : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(issue) : "memory");
-}
-// The same two instructions with each shared-memory descriptor given as its low
-// and high 32-bit words.  Only the low word (the 14-bit start address field)
+// D[tmem] (+)= A * B, A in shared memory (ss) or tensor memory (ts), B in shared memory, for a warp that stays converged:
+// every lane executes them and `issue` (non-zero in the one elected lane, and only when there is work) is the guard.
+// With no divergent branch around them the compiler may keep descriptors, addresses and loop state in uniform
+// registers; issued from inside an `if (lane == 0)` block the same sequence ran 20 % slower as soon as other warps of the
+// SM sub-partition had arithmetic to issue, and at the tensor pipe's own rate (64 clocks per 128x128x16) in this form.
+// Descriptors come as (low, high) words.  Only the low word (the 14-bit start address field)
 // changes between the MMAs of one tile, so the issuing thread advances it with a
 // single 32-bit add instead of a 64-bit one; the operand must stay inside the
 // 256 KB window that the field can address without a carry into bit 14.
@@ -322,6 +241,7 @@ __device__ __forceinline__ void umma_ts_lh_if(uint32_t issue, uint32_t d_tmem, u
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}\n"
         : : "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(issue) : "memory");
 }
+// One arrival on `bar` once every tcgen05.mma this thread issued before has completed; guarded like the products.
 __device__ __forceinline__ void umma_commit_if(uint32_t issue, uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred q;\n\t"

@@ -1,9 +1,10 @@
 """Kernel branches at the sizes where they can go wrong, against the CPU oracle (tolerances as in test_gpu_parity)."""
+import numpy as np
 import pytest
 import torch
 
 from paper_2510_07535_b200 import OwlContext, make_dims, workloads as W
-from test_gpu_parity import check_attention
+from test_gpu_parity import check_accept, check_attention
 
 pytestmark = pytest.mark.gpu
 
@@ -38,6 +39,26 @@ def test_merge_rounds_of_partials(hkv, ctx):
     wl = W.generate(W.Spec("merge", 4 * hkv, hkv, ctx, [("tree", 9, 3)] * len(ctx), shuffle_pages=True, seed=800 + len(ctx),
                            with_logits=False))
     check_attention(wl)
+
+
+@pytest.mark.parametrize("batch,nodes", [(300, 2), (20, 40)])
+def test_more_segments_per_cta_than_announced_at_once(batch, nodes):
+    """2400 short units over 148 CTAs: 16 segments each, through the eight places the producer announces them in; and
+    160 units of 160 rows (both row blocks)."""
+    rng = np.random.default_rng(batch)
+    # at least 40 keys a row: the 1e-2 of check_attention is meant for outputs well below 1.  A row of a handful of keys is
+    # close to a single V row of N(0, 1), up to 4 in magnitude over this many, where rounding the output to bf16 alone is
+    # off by up to 2^-9 * 4 = 0.008 and the rounded softmax weights by as much again (0.0112 seen with contexts from 0).
+    ctx = [int(x) for x in rng.integers(40, 240, size=batch)]
+    hq = 8 if nodes == 2 else 32
+    wl = W.generate(W.Spec("segs", hq, 8, ctx, [("chain", nodes)] * batch, shuffle_pages=True, seed=900 + batch, with_logits=False))
+    check_attention(wl)
+
+
+@pytest.mark.parametrize("nodes,vocab", [(1, 50257), (9, 8193), (17, 20001), (33, 128256), (64, 50257)])
+def test_scan_items_of_every_size_and_walk_groups(nodes, vocab):
+    """Items of 2048 to 8192 floats with ragged rows; 4 to 32 threads per node in the walk."""
+    check_accept(W.generate(W.Spec("items", 4, 1, [20] * 3, [("chain", nodes)] * 3, seed=950 + nodes, vocab=vocab)))
 
 
 @pytest.mark.parametrize("rows,d_in", [(1, 64), (16, 192), (17, 64), (32, 320), (33, 192), (128, 192), (129, 64), (256, 192), (257, 64), (383, 192)])

@@ -15,7 +15,7 @@
 //
 // Inside a verify step with a small scan both halves run as guests of the attention kernels: the scan in warps
 // the attention pass does not use (argmax_scan_chunk_warp), the walk in extra CTAs of the merge kernel, after
-// the pass has completed; no counters are involved there.
+// the pass has completed.
 #pragma once
 
 #include "owl_common.cuh"

@@ -61,10 +61,13 @@ constexpr int kSmemBytes = kAuxOff + kAuxBytes;          // 232448 = 227 KB
 constexpr uint32_t kTmemCols = 512;
 constexpr float kLazyRescale = 8.0f;       // log2 units
 
-// A unit's tiles [tile0, tile1) that this CTA works through, as the producer announces it to the other roles.  Eight
-// places are enough: the producer is never more than four segments ahead of the slowest reader (three tiles fit the
-// ring, and a segment's products wait for its Q, which is loaded after the stores of the segment before).
+// A unit's tiles [tile0, tile1) that this CTA works through, as the producer announces it to the other roles, the
+// readers: the MMA warp and the two softmax warpgroups.  Eight places are never what holds the producer back: it is at
+// most four segments ahead of the slowest reader (three tiles fit the ring, and a segment's products wait for its Q,
+// which is loaded after the stores of the segment before).  After a wait that gave up the ring no longer paces it, so it
+// looks at `seg_reached` before it reuses a place.
 constexpr int kSegs = 8;
+constexpr int kReaders = 288;                // threads: softmax 256, MMA warp 32
 struct Segment {
     int b, h, n, L, node_base, M;
     int tiles, tile0, tile1;        // tile1 == 0: no more segments
@@ -94,6 +97,8 @@ struct Aux {
     uint64_t q_full;
     uint32_t tmem_base;
     int abort_flag;
+    int seg_reached;                 // the segment that the readers have come to: they are done with those before it
+    int seg_close;                   // no reader takes this segment or a later one (a wait for an announcement gave up)
     int seg_bad_tree;
     Segment seg[kSegs];
     int sched_b0;
@@ -272,23 +277,49 @@ __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w)
     w.cur_ok = true;
 }
 
-// The CTA's segment seg_no, once the producer has announced it (tile1 == 0: there is none).  The wait does not look at
-// the abort flag: every role must take the same segments, whatever gave up.  The producer announces all of them in any
-// case, its own waits being bounded; the limit here, ten times theirs, is never reached.
-__device__ __forceinline__ Segment next_segment(Aux* aux, uint32_t seg_no) {
-    const uint32_t bar = smem_u32(&aux->seg_full[seg_no % kSegs]), parity = (seg_no / kSegs) & 1u;
-    uint64_t t0 = 0;
-    for (uint32_t polls = 0; !mbar_try_wait(bar, parity); ++polls) {
-        if ((polls & 255u) == 255u) {
-            const uint64_t now = global_timer_ns();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > 10 * kWaitLimitNs) { Segment none{}; return none; }
+__device__ __forceinline__ void named_barrier(int id, int count) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// The readers meet on hardware barrier 3 before the first segment and at the end of each one.  The first softmax warp has
+// by then seen the announcement of the next, segment `seg_no`, for all of them: whatever gave up, they take the same
+// segments, and none begins one before the others have left the key loop of the one before it.  (That keeps the arrivals
+// of two segments on the hand-off barriers apart, whose counts differ.)  The wait does not look at the abort flag, as the
+// producer announces every segment in any case, its own waits being bounded; ten times their limit is the backstop.
+__device__ __forceinline__ void meet_before_segment(Aux* aux, uint32_t seg_no, bool leader) {
+    if (leader) {
+        const uint32_t bar = smem_u32(&aux->seg_full[seg_no % kSegs]), parity = (seg_no / kSegs) & 1u;
+        uint64_t t0 = 0;
+        for (uint32_t polls = 0; !mbar_try_wait(bar, parity); ++polls) {
+            if ((polls & 255u) == 255u) {
+                const uint64_t now = global_timer_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > 10 * kWaitLimitNs) {
+                    const_cast<volatile int&>(aux->seg_close) = (int)seg_no;
+                    const_cast<volatile int&>(aux->abort_flag) = 1;
+                    break;
+                }
+            }
         }
+        __syncwarp();
     }
-    return aux->seg[seg_no % kSegs];
+    named_barrier(3, kReaders);
+}
+// The CTA's segment seg_no; tile1 == 0: there is none.
+__device__ __forceinline__ Segment announced_segment(Aux* aux, uint32_t seg_no) {
+    Segment g = aux->seg[seg_no % kSegs];
+    if ((int)seg_no >= const_cast<volatile int&>(aux->seg_close)) g.tile1 = 0;
+    return g;
 }
 
 // ------------------------------------------------------------------------------------------ producer
+__device__ __forceinline__ bool readers_reached(Aux* aux, int seg_no) {
+    const uint64_t t0 = global_timer_ns();
+    while (const_cast<volatile int&>(aux->seg_reached) < seg_no)
+        if (global_timer_ns() - t0 > 10 * kWaitLimitNs) return false;
+    return true;
+}
+
 template <bool kWide>
 __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtensorMap* kmap, const CUtensorMap* vmap,
                                               Aux* aux, uint32_t ring, Walker w, uint32_t& items_out) {
@@ -303,6 +334,9 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
     for (uint32_t seg_no = 0;; ++seg_no) {
         Segment g;
         const bool more = w.template next<kWide>(p, g);
+        // a place is free again once the readers have come to the segment after the one that it held (not abortable:
+        // their waits are bounded; should it give up all the same, nothing is announced any more and they do likewise)
+        if (seg_no >= (uint32_t)kSegs && !readers_reached(aux, (int)seg_no - kSegs + 1)) break;
         Segment& announced = aux->seg[seg_no % kSegs];
         if (lane == 0) {
             if (!more) g.tile0 = g.tile1 = 0;
@@ -382,7 +416,8 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
     uint32_t seg_no = 0, item_base = 0;
 
     for (;;) {
-        const Segment g = next_segment(aux, seg_no);
+        meet_before_segment(aux, seg_no, false);
+        const Segment g = announced_segment(aux, seg_no);
         const int tile0 = __reduce_max_sync(kAll, g.tile0), tile1 = __reduce_max_sync(kAll, g.tile1);
         if (tile1 == 0) break;
         const bool shared = kWide && __reduce_max_sync(kAll, g.shared ? 1 : 0) != 0;
@@ -496,10 +531,6 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
 }
 
 // ------------------------------------------------------------------------------------------ softmax warpgroups
-__device__ __forceinline__ void named_barrier(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 __device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
 
 // Writes a warp's 32 rows x 32 columns (lane = row, v = its 32 fp32 values) to global memory through a
@@ -564,14 +595,17 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
     uint32_t it = 0, seg_no = 0, od_phase = 0;   // od_phase: segments of this stream that issued a product
     uint32_t tile_base = 0;                      // key tiles of the CTA's earlier segments (the ring counts them through)
 
+    const bool leader = s == 0 && wtid < 32;
+    meet_before_segment(aux, 0, leader);
     for (;;) {
-        const Segment g = next_segment(aux, seg_no);
+        const Segment g = announced_segment(aux, seg_no);
         if (g.tile1 == 0) break;
         // ---- Q rows (16-byte asynchronous copies, rows beyond M zero-filled) and, in stream 0's warpgroup, the
         // ancestor masks; every global read of the segment start is in flight at the same time
         int parent_i = -1;
         if (s == 0 && wtid < g.n) parent_i = p.tree_parent[g.node_base + wtid];
         if (seg_no > 0) named_barrier(1, 256);   // the other warpgroup may still be reading its staging area in the Q blocks
+        if (leader) const_cast<volatile int&>(aux->seg_reached) = (int)seg_no;
         {
             // shared: this warpgroup loads its own 128-row block; split: rows [64 s, 64 s + 64) of block 0
             const int blk = g.shared ? s : 0;
@@ -843,7 +877,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         // split mode: the streams exchange (m, l, lx) through the second Q block, which only the shared mode uses
         float (*ml)[128][3] = reinterpret_cast<float (*)[128][3]>(smem + kQBytes);
         if (!g.shared) { ml[s][row_local][0] = m; ml[s][row_local][1] = l; ml[s][row_local][2] = lx; }
-        named_barrier(1, 256);                 // both streams done: all MMAs of the segment have completed
+        meet_before_segment(aux, seg_no + 1, leader);    // both streams done: all MMAs of the segment have completed
         // (looking up seq_bad in global memory here stood between a unit's last product and its stores)
         const bool write_ok = !bad_tree && !*abort_flag && !const_cast<volatile int&>(aux->seg[seg_no % kSegs].bad_page);
         // only the first and the last unit of a CTA's piece can be cut: two partial slots per CTA
@@ -937,6 +971,8 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         mbar_init(smem_u32(&aux->q_full), 256);
         for (int i = 0; i < kSegs; ++i) mbar_init(smem_u32(&aux->seg_full[i]), 1);
         aux->abort_flag = 0;
+        aux->seg_reached = 0;
+        aux->seg_close = 0x7fffffff;
         aux->seg_bad_tree = 0;
         aux->sched_b0 = 0; aux->sched_tile_begin = 0;
         fence_barrier_init();

@@ -38,6 +38,10 @@ __device__ __forceinline__ void fence_barrier_init() {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_if(bool arrive, uint32_t bar) {      // without a branch
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}\n"
+                 ::"r"(bar), "r"(arrive ? 1u : 0u) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
@@ -68,6 +72,21 @@ __device__ __forceinline__ bool mbar_wait_ns(uint32_t bar, uint32_t parity, vola
             const uint64_t now = global_timer_ns();
             if (t0 == 0) t0 = now;
             else if (now - t0 > limit_ns || polls > 0x7fffff00u) { *abort_flag = 1; return false; }
+        }
+    }
+}
+// The same for an arrival that is certain to come, whatever gave up elsewhere, because whoever owes it makes it on every
+// path and waits for nothing unbounded: does not look at the abort flag, and the time limit, which it raises the flag at,
+// is a backstop beyond everything that the other side's own waits can take.
+__device__ __forceinline__ bool mbar_wait_certain(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (mbar_try_wait(bar, parity)) return true;
+    uint64_t t0 = 0;
+    for (uint32_t polls = 0;; ++polls) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((polls & 255u) == 255u) {
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > 10 * kWaitLimitNs) { *abort_flag = 1; return false; }
         }
     }
 }

@@ -284,23 +284,11 @@ __device__ __forceinline__ void named_barrier(int id, int count) {
 // The readers meet on hardware barrier 3 before the first segment and at the end of each one.  The first softmax warp has
 // by then seen the announcement of the next, segment `seg_no`, for all of them: whatever gave up, they take the same
 // segments, and none begins one before the others have left the key loop of the one before it.  (That keeps the arrivals
-// of two segments on the hand-off barriers apart, whose counts differ.)  The wait does not look at the abort flag, as the
-// producer announces every segment in any case, its own waits being bounded; ten times their limit is the backstop.
+// of two segments on the hand-off barriers apart, whose counts differ.)  The producer announces every segment in any case.
 __device__ __forceinline__ void meet_before_segment(Aux* aux, uint32_t seg_no, bool leader) {
     if (leader) {
-        const uint32_t bar = smem_u32(&aux->seg_full[seg_no % kSegs]), parity = (seg_no / kSegs) & 1u;
-        uint64_t t0 = 0;
-        for (uint32_t polls = 0; !mbar_try_wait(bar, parity); ++polls) {
-            if ((polls & 255u) == 255u) {
-                const uint64_t now = global_timer_ns();
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > 10 * kWaitLimitNs) {
-                    const_cast<volatile int&>(aux->seg_close) = (int)seg_no;
-                    const_cast<volatile int&>(aux->abort_flag) = 1;
-                    break;
-                }
-            }
-        }
+        if (!mbar_wait_certain(smem_u32(&aux->seg_full[seg_no % kSegs]), (seg_no / kSegs) & 1u, &aux->abort_flag))
+            const_cast<volatile int&>(aux->seg_close) = (int)seg_no;
         __syncwarp();
     }
     named_barrier(3, kReaders);
@@ -436,11 +424,11 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
         // (2K step 15.5 -> 14.4 us, 32K 39.7 -> 38.3 us, round 49.3 -> 47.9 us).
 #pragma unroll 1
         for (int i = -1; i < n_it[0]; ++i) {
-            if (kWide && shared && i >= 0 && i + 1 < T) {
+            if (kWide && shared && ok && i >= 0 && i + 1 < T) {
                 // The middle of a 256-row unit, where this warp's time is what counts: both streams have both products, and
                 // a turn has no conditions but the stream's commits (with the general turn instead 70B 660 -> 693 us;
                 // with both streams unrolled 660 -> 653 us, fp16 with 60 nodes 72.8 -> 71.0 us).
-                const uint32_t issue = ok ? elected : 0u, acc0 = i > 0 ? 1u : 0u;
+                const uint32_t issue = elected, acc0 = i > 0 ? 1u : 0u;
                 const uint32_t v_lo = (uint32_t)v_desc0 + v_slot * (uint32_t)(kSlotBytes >> 4), v_hi = (uint32_t)(v_desc0 >> 32);
                 const uint32_t k_lo = (uint32_t)k_desc0 + k_slot * (uint32_t)(kSlotBytes >> 4), k_hi = (uint32_t)(k_desc0 >> 32);
                 const uint32_t q_hi = (uint32_t)(q_desc0 >> 32);
@@ -514,7 +502,11 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
                         for (int ks = 0; ks < 4; ++ks)
                             umma_ss_lh_if(issue, tS, q_lo + (uint32_t)((hf * 16384 + ks * 32) >> 4), q_hi,
                                           k_lo + (uint32_t)((hf * 1024 + ks * 32) >> 4), k_hi, idesc_qk, (hf | ks) ? 1u : 0u);
+                    // S is announced on every path, by the commit or, when nothing was issued, by hand: the softmax warps
+                    // rely on it to be at most one tile ahead of this warp's bar.sync (their second arrival in one
+                    // generation of barrier 4 + s would leave this warp waiting there for good)
                     umma_commit_if(issue, smem_u32(&aux->s_full[0]) + s * 8u);
+                    mbar_arrive_if(elected != issue, smem_u32(&aux->s_full[0]) + s * 8u);
                     umma_commit_if(last_reader ? issue : 0u, smem_u32(&aux->empty[0]) + k_slot * 8u);
                 }
                 // the tiles lie in the ring in the order of the turns that consume them, K and V by turns
@@ -661,7 +653,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
 
         for (int i = 0; i < (idle ? 0 : n_it); ++i) {
             const int t = g.tile(s, i);
-            mbar_wait(smem_u32(&aux->s_full[s]), (it + i) & 1u, abort_flag);
+            mbar_wait_certain(smem_u32(&aux->s_full[s]), (it + i) & 1u, abort_flag);
             tc_fence_after();
             if ((t + 1) * kTileKeys > g.L) {
                 // The tile reaches drafted positions (or the end of the sequence): at most two tiles per unit.
@@ -850,7 +842,8 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             tc_fence_before();
             // Hand-off of P: hardware barrier 4 + s, the live warps of this warpgroup + the MMA warp.  Executed once per
             // key tile of this stream - n_it times per segment, the count of the MMA warp's bar.sync on it - on every
-            // path: nothing above leaves the loop body early, and a wait that gave up only changed what was computed.
+            // path: nothing above leaves the loop body early.  S of this tile has been announced, on every path too, so
+            // the MMA warp has passed its bar.sync for the tile before: one generation never sees two tiles' arrivals.
             asm volatile("bar.arrive %0, %1;" ::"r"(4 + s), "r"(32 * live + 32) : "memory");
             // In a unit of more than 128 rows the MMA warp polls no mbarrier between O += P V of this tile and
             // S = Q K^T of the next one: the first warp of the warpgroup looks at that tile's arrival barrier for it

@@ -1,7 +1,7 @@
-"""A model of how the attention kernel's roles agree on the segments of a CTA's piece, run under random interleavings on
-the CPU.  A wait on a tile or on a free slot may give up at any point; from then on all of those return at once.  What is
-never abortable must still end: the readers' barriers and the producer's look at `seg_reached`, and every reader must have
-taken every segment."""
+"""A model of how the attention kernel's roles agree on the segments of a CTA's piece and hand over P tile by tile, run under
+random interleavings on the CPU.  A wait on a tile or on a free slot may give up at any point; from then on all of those
+return at once.  What is never abortable must still end: the hardware barriers, the wait for a score tile and the producer's
+look at `seg_reached`, and every reader must have taken every segment."""
 import random
 import re
 from pathlib import Path
@@ -14,21 +14,29 @@ SLOTS = int(re.search(r"constexpr int kSlots = (\d+);", SOURCE).group(1))
 
 
 class Cta:
-    def __init__(self, rng, segments, paced):
-        self.rng, self.paced, self.abort = rng, paced, False
+    def __init__(self, rng, segments, paced, certain):
+        self.rng, self.paced, self.certain, self.abort = rng, paced, certain, False
         self.tiles = [rng.randint(1, 3) for _ in range(segments)] + [0]       # 0: no more segments
         self.place, self.announced = [None] * PLACES, [0] * PLACES            # contents; completed phases
         self.reached = 0
         self.loaded = self.freed = 0                                          # tiles, each of two slots
         self.q_full = 0                                                       # segments whose Q has been loaded
-        self.scores = self.weights = self.products = 0                        # tiles: S announced, P handed over, P V done
-        self.arrived, self.generation = {1: 0, 3: 0}, {1: 0, 3: 0}            # hardware barriers
+        self.live = [rng.randint(1, 4) for _ in range(segments + 1)]          # softmax warps that hand over P
+        self.scores = self.products = 0                                       # tiles: S announced, P V done
+        self.open, self.generation = {}, {1: 0, 3: 0, 4: 0}                   # hardware barriers: (arrived, expected)
 
-    def sync(self, bar, need):
+    def arrive(self, bar, warps, need):          # bar.arrive
+        got, expected = self.open.pop(bar, (0, need))
+        got += warps
+        assert expected == need and got <= need, f"barrier {bar}: {got} of {need} and {expected} warps in one generation"
+        if got == need:
+            self.generation[bar] += 1
+        else:
+            self.open[bar] = (got, need)
+
+    def sync(self, bar, need):                   # bar.sync of one warp (of one role for barriers 1 and 3)
         mine = self.generation[bar]
-        self.arrived[bar] += 1
-        if self.arrived[bar] == need:
-            self.arrived[bar], self.generation[bar] = 0, mine + 1
+        self.arrive(bar, 1, need)
         return lambda: self.generation[bar] > mine
 
     def bounded(self, condition):
@@ -67,7 +75,7 @@ class Cta:
                 first = self.products
                 yield self.bounded(lambda: self.loaded > first)
                 self.scores += 1
-                yield lambda: self.weights > first
+                yield self.sync(4, self.live[taken[-1]] + 1)
                 self.products += 1
                 self.freed = min(self.loaded, self.products)
 
@@ -87,8 +95,9 @@ class Cta:
                 self.q_full += 1
                 base = sum(self.tiles[:seg])
                 for i in range(self.tiles[seg]):
-                    yield self.bounded(lambda: self.scores > base + i)
-                    self.weights += 1
+                    announced = lambda: self.scores > base + i
+                    yield announced if self.certain else self.bounded(announced)
+                    self.arrive(4, self.live[seg], self.live[seg] + 1)
                 yield self.bounded(lambda: self.products >= base + self.tiles[seg])
             yield from self.meet(k + 1, leader)
             assert not self.paced or self.place[k % PLACES] == seg        # bad_page is read here
@@ -113,21 +122,23 @@ class Cta:
         return taken
 
 
-def segments_of(seed, segments, paced):
+def segments_of(seed, segments, paced=True, certain=True):
     rng = random.Random(seed)
-    return Cta(rng, segments, paced).run(abort_at=rng.choice([0, 10 ** 9, rng.randint(0, 12 * segments)]))
+    return Cta(rng, segments, paced, certain).run(abort_at=rng.choice([0, 10 ** 9, rng.randint(0, 12 * segments)]))
 
 
 @pytest.mark.parametrize("segments", [1, PLACES - 1, PLACES, PLACES + 1, 16, 40])
 def test_all_roles_take_the_same_segments_whatever_gives_up(segments):
     for seed in range(300):
-        assert segments_of(seed, segments, True) == [list(range(segments + 1))] * 3, seed
+        assert segments_of(seed, segments) == [list(range(segments + 1))] * 3, seed
 
 
-def test_the_model_shows_what_an_unpaced_producer_does():
+@pytest.mark.parametrize("segments,without", [(40, "paced"), (4, "certain")])
+def test_the_model_shows_what_each_rule_is_for(segments, without):
+    """A producer that nothing paces, and softmax warps that hand over P of a tile whose S was not announced."""
     def broken(seed):
         try:
-            return segments_of(seed, 40, False) != [list(range(41))] * 3
+            return segments_of(seed, segments, **{without: False}) != [list(range(segments + 1))] * 3
         except (AssertionError, IndexError):
             return True
     assert any(broken(seed) for seed in range(300))

@@ -205,6 +205,7 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
             const uint64_t keep_policy = l2_policy_evict_last();      // A is read by every pair for every tile
             uint32_t stage = 0, ph = 1;
             bool peek = true;                                         // the first pass over the ring finds it empty
+            bool going = true;      // nothing is issued any more after a wait that gave up: `issued` counts in ring order
             for (int t = 0; t < p.rounds; ++t) {
                 const int row0 = tile_row0(t), share = tile_rows(t) >> 1;
                 if (row0 >= p.N) break;
@@ -213,7 +214,8 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
                 // both CTAs' copies of a stage complete on the even CTA's barrier, which expects all their bytes
                 const uint32_t bytes = (uint32_t)(2 * kQ * (share + kGroups * a_half) * kBK * 2);
                 for (int kb = 0; kb < kblocks; kb += kQ) {
-                    if (peek || wait(empty_bar + stage * 8u, ph)) {
+                    going = going && (peek || wait(empty_bar + stage * 8u, ph));
+                    if (going) {
                         const uint32_t full = full_bar + stage * 8u, full0 = cluster_map(full, 0);
                         const uint32_t dst = ring + stage * (uint32_t)(kQ * bbytes);
                         if (rank == 0) mbar_arrive_expect_tx(full, bytes);
@@ -283,7 +285,8 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
             if (row0 >= p.N) break;
             const uint32_t buf = tcount % kBufs, acc_ph = (tcount / kBufs) & 1u;
             const int share = tile_rows(t) >> 1;
-            const bool ok = wait(smem_u32(&aux->acc_full[buf]), acc_ph);
+            // (one verdict for the warp: what follows are warp-wide instructions)
+            const bool ok = __all_sync(0xffffffffu, wait(smem_u32(&aux->acc_full[buf]), acc_ph));
             tc_fence_after();
             const int first = row0 + (int)rank * share;                 // this CTA's rows of B: [first, end)
             const int end = first + share < p.N ? first + share : p.N;
@@ -328,9 +331,10 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
     if (aux->abort_flag && warp == 0 && lane == 0) {
         if (rank == 0) {
             // both CTAs' copies complete on this CTA's barriers: give those in flight a bounded time to land before
-            // either CTA's shared memory is released (the peer leaves only after the cluster barrier below)
+            // either CTA's shared memory is released (the peer leaves only after the cluster barrier below).  The peer's
+            // producer may have gone on for longer than this one: the turn past the last is that time for its copies.
             const uint32_t first = issued > (uint32_t)stages ? issued - stages : 0u;
-            for (uint32_t it = first; it < issued; ++it) {
+            for (uint32_t it = first; it <= issued; ++it) {
                 const uint32_t bar = smem_u32(&aux->full[it % stages]), ph = (it / stages) & 1u;
                 for (int polls = 0; polls < (1 << 20) && !mbar_try_wait_cluster(bar, ph); ++polls) {}
             }

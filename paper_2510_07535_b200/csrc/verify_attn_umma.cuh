@@ -475,7 +475,9 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)
                         umma_ts_lh_if(issue, tS + 256, tS + ks * 8, v_lo + (uint32_t)(ks * 4096 >> 4), v_hi, idesc_pv, ks ? 1u : (i > 0 ? 1u : 0u));
-                    umma_commit_if(i == n_s - 1 ? issue : 0u, smem_u32(&aux->o_done[0]) + s * 8u);   // only the segment end waits for it
+                    // only the segment end waits for it; made on every path, like the announcement of S below
+                    umma_commit_if(i == n_s - 1 ? issue : 0u, smem_u32(&aux->o_done[0]) + s * 8u);
+                    mbar_arrive_if(i == n_s - 1 && elected != issue, smem_u32(&aux->o_done[0]) + s * 8u);
                     // (Releasing the ring slots from a softmax thread instead - a score tile's arrival covers every product
                     // issued before it - spares this warp two commits per tile, but the slots come back late: 1 % slower
                     // on 256-row units, 15 to 35 % on the bandwidth-bound ones.)
@@ -865,7 +867,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         // ---- segment end: every product of this stream has completed
         // (an idle warp sleeps on the hardware barrier below instead; it reads nothing)
         if (n_it > 0) {
-            if (!idle) mbar_wait(smem_u32(&aux->o_done[s]), od_phase & 1u, abort_flag);
+            if (!idle) mbar_wait_certain(smem_u32(&aux->o_done[s]), od_phase & 1u, abort_flag);
             ++od_phase;
         }
         tc_fence_after();

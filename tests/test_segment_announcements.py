@@ -105,7 +105,8 @@ class Cta:
                     announced = lambda: self.scores > base + i
                     yield announced if self.certain else self.bounded(announced)
                     self.arrive(4, self.live[seg], self.live[seg] + 1)
-                yield self.bounded(lambda: self.products >= base + self.tiles[seg])
+                finished = lambda: self.products >= base + self.tiles[seg]
+                yield finished if self.certain else self.bounded(finished)
             yield from self.meet(k + 1, leader)
             assert not self.paced or self.place[k % PLACES] == seg        # bad_page is read here
 

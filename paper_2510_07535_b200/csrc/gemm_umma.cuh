@@ -57,6 +57,10 @@ constexpr int kWindowBytes = 128 * kBK * 2;      // what an instruction reads of
 constexpr int kMaxStages = 8;
 constexpr int kAuxBytes = 4096;
 constexpr int kSmemLimit = 232448;               // 227 KB
+// A launch asks for at least this much, so that an SM never holds two of these CTAs (2 x (116 + 1) KB > 228 KB).  Each
+// takes all of its SM's tensor memory, and a pair takes that of two SMs: two pairs of different streams on the same two
+// SMs, each with one half allocated, would wait for each other for good.
+constexpr int kSmemAlone = 118784;
 constexpr int kMaxTile = 256;                    // rows of B per tile, both CTAs
 constexpr int kMaxRows = 384;                    // rows of A
 constexpr int kGroupRows = 256;                  // rows of A in one column group; above, two groups
@@ -92,7 +96,26 @@ __host__ inline int ring_stages(int groups, int block_bytes) {
 }
 // (the pad behind the ring: the window of the last stage may reach one window past it)
 __host__ inline int smem_bytes(int groups, int stages, int block_bytes) {
-    return kAuxBytes + stages * stage_kblocks(groups) * block_bytes + kWindowBytes;
+    const int used = kAuxBytes + stages * stage_kblocks(groups) * block_bytes + kWindowBytes;
+    return used > kSmemAlone ? used : kSmemAlone;
+}
+
+// How a product of M rows of A and N rows of B is laid out on `pairs` CTA pairs: the fields of GemmParams that follow from
+// the sizes.  Every pair gets the same number of 16-row units of B, cut into as few tiles as the height limit allows.
+__host__ inline int column_groups(int M) { return M <= kGroupRows ? 1 : 2; }
+__host__ inline int product_pairs(int N, int sms) { return (N + 15) / 16 < sms / 2 ? (N + 15) / 16 : sms / 2; }
+__host__ inline GemmParams product_plan(int M, int N, int K, int pairs) {
+    const int groups = column_groups(M);
+    GemmParams g{};
+    g.M = M; g.N = N; g.K = K;
+    g.group_rows = (M + 16 * groups - 1) / (16 * groups) * 16;
+    const int units = (N + 15) / 16, per_pair = (units + pairs - 1) / pairs;
+    g.rounds = (per_pair + kMaxTile / 16 - 1) / (kMaxTile / 16);
+    g.h_lo = per_pair / g.rounds * 16;
+    g.tall_rounds = per_pair % g.rounds;
+    g.block_bytes = (g.h_lo + (g.tall_rounds ? 16 : 0) + groups * g.group_rows) / 2 * kBK * 2;
+    g.stages = ring_stages(groups, g.block_bytes);
+    return g;
 }
 
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {

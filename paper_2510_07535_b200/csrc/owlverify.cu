@@ -182,22 +182,11 @@ template <int kEpi>
 int launch_gemm(owl_ctx* ctx, const void* a, const void* b, int M, int N, int K, unsigned long long* row_key, float* c,
                 long long ldc, cudaStream_t stream) {
     using namespace gemm_path;
-    const int groups = M <= kGroupRows ? 1 : 2;
-    GemmParams g{};
-    g.M = M; g.N = N; g.K = K;
-    g.group_rows = (M + 16 * groups - 1) / (16 * groups) * 16;
+    const int groups = column_groups(M), pairs = product_pairs(N, ctx->sm_count);
+    GemmParams g = product_plan(M, N, K, pairs);
+    const int h_hi = g.h_lo + (g.tall_rounds ? 16 : 0);
     g.status = ctx->status;
     g.row_key = row_key; g.c = c; g.ldc = ldc;
-    // every pair gets the same number of 16-row units of B, cut into as few tiles as the height limit allows
-    const int units = (N + 15) / 16, max_pairs = ctx->sm_count / 2;
-    const int pairs = units < max_pairs ? units : max_pairs;
-    const int per_pair = (units + pairs - 1) / pairs;
-    g.rounds = (per_pair + kMaxTile / 16 - 1) / (kMaxTile / 16);
-    g.h_lo = per_pair / g.rounds * 16;
-    g.tall_rounds = per_pair % g.rounds;
-    const int h_hi = g.h_lo + (g.tall_rounds ? 16 : 0);
-    g.block_bytes = (h_hi + groups * g.group_rows) / 2 * kBK * 2;
-    g.stages = ring_stages(groups, g.block_bytes);
     CUtensorMap amap, bmap_hi, bmap_lo;
     const int ra = make_operand_map(ctx->encode, &amap, a, M, K, g.group_rows / 2);
     int rb = make_operand_map(ctx->encode, &bmap_lo, b, N, K, g.h_lo / 2);

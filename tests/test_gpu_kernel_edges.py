@@ -80,3 +80,30 @@ def test_product_row_padding_and_odd_k_blocks(rows, d_in):
     bound = d_in * 2.0 ** -24 * (h.double().abs() @ w.double().abs().t())
     assert bool(((ws.cpu().double() - ref).abs() <= bound).all())
     ctx.close()
+
+
+def test_small_products_on_two_streams():
+    """Products that take a fraction of an SM's shared memory each, of two contexts on two streams at once: every one has to
+    have its SMs' tensor memory to itself."""
+    rows, d_in, d = 8, 256, 512
+    g = torch.Generator().manual_seed(1)
+    h = torch.randn(rows, d_in, generator=g).bfloat16()
+    w = torch.randn(4 * d, d_in, generator=g).bfloat16()
+    hc, wc, emb = h.cuda(), w.cuda(), torch.zeros(rows, d, dtype=torch.bfloat16, device="cuda")
+    sides = []
+    for _ in range(2):
+        sides.append((torch.cuda.Stream(), OwlContext(make_dims(batch=1, total_nodes=1, max_nodes=1)), torch.zeros(rows, d, device="cuda"),
+                      torch.empty(rows, d, device="cuda"), torch.full((rows, 4 * d), float("nan"), device="cuda")))
+    torch.cuda.synchronize()
+    for _ in range(50):
+        for stream, ctx, z, hf, ws in sides:
+            with torch.cuda.stream(stream):
+                ctx.owl_lstm_cell(hc, emb, wc, 0.0, z, hf, None, ws)
+    torch.cuda.synchronize()
+    ref = h.double() @ w.double().t()
+    bound = d_in * 2.0 ** -24 * (h.double().abs() @ w.double().abs().t())       # fp32 accumulation of d_in exact products
+    for stream, ctx, _, _, ws in sides:
+        with torch.cuda.stream(stream):
+            assert ctx.owl_get_status() == 0
+        assert bool(((ws.cpu().double() - ref).abs() <= bound).all())
+        ctx.close()

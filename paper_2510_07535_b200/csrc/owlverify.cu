@@ -33,7 +33,6 @@ struct owl_ctx {
     int32_t* status = nullptr;
     unsigned long long* selftest_ns = nullptr;
     int32_t* seq_bad = nullptr;
-    unsigned int* commit_done = nullptr;        // CommitParams::seq_done
     long long* sched_seq_begin = nullptr;
     SchedHeader* sched_header = nullptr;
     unsigned long long* part_keys = nullptr;
@@ -261,7 +260,6 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     alloc((void**)&ctx->status, sizeof(int32_t));
     alloc((void**)&ctx->selftest_ns, 2 * sizeof(unsigned long long));
     alloc((void**)&ctx->seq_bad, (size_t)max_dims->batch * sizeof(int32_t));
-    alloc((void**)&ctx->commit_done, kMaxBatch * sizeof(unsigned int));      // owl_kv_commit takes any batch
     alloc((void**)&ctx->sched_seq_begin, ((size_t)max_dims->batch + 1) * sizeof(long long));
     alloc((void**)&ctx->sched_header, sizeof(SchedHeader));
     if (acc) {
@@ -274,8 +272,7 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     }
     if (ok) {
         ok = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess &&
-             cudaMemset(ctx->seq_bad, 0, (size_t)max_dims->batch * sizeof(int32_t)) == cudaSuccess &&
-             cudaMemset(ctx->commit_done, 0, kMaxBatch * sizeof(unsigned int)) == cudaSuccess;
+             cudaMemset(ctx->seq_bad, 0, (size_t)max_dims->batch * sizeof(int32_t)) == cudaSuccess;
     }
     for (int i = 0; ok && i < 6; ++i) ok = cudaEventCreate(&ctx->ev[i]) == cudaSuccess;
     if (ok && attn) {
@@ -311,7 +308,6 @@ int owl_destroy(owl_ctx* ctx) {
     cudaFree(ctx->status);
     cudaFree(ctx->selftest_ns);
     cudaFree(ctx->seq_bad);
-    cudaFree(ctx->commit_done);
     cudaFree(ctx->sched_seq_begin);
     cudaFree(ctx->sched_header);
     cudaFree(ctx->part_keys);
@@ -619,8 +615,20 @@ int owl_kv_commit(owl_ctx* ctx, const owl_dims* d, void* k_cache, void* v_cache,
     p.max_nodes = d->max_nodes; p.num_kv_heads = d->num_kv_heads;
     p.page_size = d->page_size; p.page_shift = log2_exact(d->page_size);
     p.max_pages_per_seq = d->max_pages_per_seq; p.num_pages = d->num_pages; p.path_stride = d->path_stride;
-    p.seq_done = ctx->commit_done;
-    launch_dependent(kv_commit_kernel, dim3(2u * (unsigned)d->num_kv_heads, (unsigned)d->batch), dim3(kCommitThreads), stream, p);
+    const unsigned cluster = d->num_kv_heads < kCommitMaxCluster ? (unsigned)d->num_kv_heads : (unsigned)kCommitMaxCluster;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster, (unsigned)d->batch);
+    cfg.blockDim = dim3(kCommitThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, kv_commit_kernel, p);
     ++ctx->launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_kv_commit launch");

@@ -101,12 +101,12 @@ struct CommitParams {
     const int32_t* accept_len;
     const int32_t* accept_path;
     int32_t* status;
-    unsigned int* seq_done;        // [kMaxBatch], 0 between calls: CTAs of the sequence that have read its length
     int32_t batch, total_nodes, nodes_uniform, max_nodes, num_kv_heads;
     int32_t page_size, page_shift, max_pages_per_seq, num_pages, path_stride;
 };
 
-constexpr int kCommitThreads = 256;
+constexpr int kCommitThreads = 256;      // half of them move K, half V
+constexpr int kCommitMaxCluster = 8;     // CTAs of a sequence
 
 // What every CTA of sequence b decides alike, from the inputs alone: 0 = commit, else the error code.
 // The accepted path must be a root path in node order (path[0] = 0, strictly increasing, below n) and every page
@@ -138,42 +138,44 @@ __device__ __forceinline__ int commit_verdict(const CommitParams& p, int b, int&
     return *s_flag;
 }
 
-// grid (2 * Hkv, B): blockIdx.x = 2 * head + (0: K, 1: V).  Every source row is read into shared memory before any
-// destination is written, because a position can be the source of one move and the destination of a later one.
-// The committed length grows by accept_len once all CTAs of the sequence have read the old one: each counts itself in
-// after that and the last one writes (and the counter wraps to zero for the next call).
+// grid (C, B) in clusters of (C, 1), C = min(Hkv, 8): a sequence's heads are dealt out to its cluster's CTAs.  Every source
+// row is read into shared memory before any destination is written, because a position can be the source of one move and
+// the destination of a later one.  The committed length grows by accept_len once all CTAs of the sequence have read the old
+// one: the cluster's barrier says so, and nothing is kept from one call for the next (a counter per sequence in the
+// context did the same for one stream at a time; a second kernel for the lengths is one more launch in the chain).
 __global__ void __launch_bounds__(kCommitThreads) kv_commit_kernel(const CommitParams p) {
     // may be launched as a programmatic dependent: nothing is read before the kernel before it in the stream has
     // completed (a no-op in an ordinary launch); the kernel after this one may queue up and waits likewise
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ uint4 s_rows[kMaxNodes * 16];       // up to 64 rows of 128 bf16
+    __shared__ uint4 s_rows[2][kMaxNodes * 16];    // up to 64 rows of 128 bf16 each of K and V
     __shared__ int s_path[kMaxNodes];
     __shared__ int s_flag;
-    const int b = blockIdx.y, h = blockIdx.x >> 1;
+    const int b = blockIdx.y;
     int L, n, a;
     const int verdict = commit_verdict(p, b, L, n, a, s_path, &s_flag);
-    if (verdict != 0) {
+    if (verdict != 0) {                            // in every CTA of the cluster
         if (threadIdx.x == 0 && blockIdx.x == 0) report(p.status, verdict);
         return;
     }
-    if (threadIdx.x == 0) {
-        // every thread's read of the length came before the barriers of commit_verdict
-        __threadfence();
-        if (atomicInc(p.seq_done + b, gridDim.x - 1u) == gridDim.x - 1u) p.ctx_lens[b] = L + a;
-    }
-    __nv_bfloat16* cache = (blockIdx.x & 1) ? p.v_cache : p.k_cache;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // this CTA has read the length
+    const int kv = threadIdx.x / (kCommitThreads / 2), first = (threadIdx.x % (kCommitThreads / 2)) >> 4, piece = threadIdx.x & 15;
+    constexpr int kStep = kCommitThreads / 32;     // rows per turn of a half
+    __nv_bfloat16* cache = kv ? p.v_cache : p.k_cache;
     const int32_t* table = p.block_table + (long long)b * p.max_pages_per_seq;
-    auto row_ptr = [&](int pos) {
-        const long long page = table[pos >> p.page_shift];
-        return reinterpret_cast<uint4*>(cache + ((page * p.num_kv_heads + h) * p.page_size + (pos & (p.page_size - 1))) * kHeadDim);
-    };
-    const int piece = threadIdx.x & 15;
-    for (int k = threadIdx.x >> 4; k < a; k += kCommitThreads / 16)
-        if (s_path[k] != k) s_rows[k * 16 + piece] = row_ptr(L + s_path[k])[piece];
-    __syncthreads();
-    for (int k = threadIdx.x >> 4; k < a; k += kCommitThreads / 16)
-        if (s_path[k] != k) row_ptr(L + k)[piece] = s_rows[k * 16 + piece];
+    for (int h = blockIdx.x; h < p.num_kv_heads; h += gridDim.x) {
+        auto row_ptr = [&](int pos) {
+            const long long page = table[pos >> p.page_shift];
+            return reinterpret_cast<uint4*>(cache + ((page * p.num_kv_heads + h) * p.page_size + (pos & (p.page_size - 1))) * kHeadDim);
+        };
+        for (int k = first; k < a; k += kStep)
+            if (s_path[k] != k) s_rows[kv][k * 16 + piece] = row_ptr(L + s_path[k])[piece];
+        __syncthreads();
+        for (int k = first; k < a; k += kStep)         // (a thread takes back what it put there itself)
+            if (s_path[k] != k) row_ptr(L + k)[piece] = s_rows[kv][k * 16 + piece];
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.ctx_lens[b] = L + a;
 }
 
 }  // namespace owl

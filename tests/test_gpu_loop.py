@@ -161,6 +161,53 @@ def test_kv_commit_matches_oracle_bit_for_bit(page):
         ctx.close()
 
 
+@pytest.mark.parametrize("hkv", [3, 12, 16])
+def test_kv_commit_with_heads_dealt_out_unevenly(hkv):
+    """Heads that are fewer than, or no multiple of, the CTAs of a sequence."""
+    rng = np.random.default_rng(70 + hkv)
+    offs, lens, table, k, v, alen, path = _commit_case(rng, 4, hkv, 16)
+    d = make_dims(batch=4, total_nodes=int(offs[-1]), max_nodes=int(np.diff(offs).max()), num_kv_heads=hkv, page_size=16,
+                  max_pages_per_seq=table.shape[1], num_pages=k.shape[0])
+    ctx = OwlContext(make_dims(batch=4, total_nodes=int(offs[-1]), max_nodes=64))
+    kd, vd, ld = dev_bf16(k), dev_bf16(v), dev_i32(lens)
+    ctx.owl_kv_commit(d, kd, vd, dev_i32(table), ld, dev_i32(offs), dev_i32(alen), dev_i32(path))
+    assert ctx.owl_get_status() == 0
+    oracle.kv_commit(k, v, table, lens, offs, alen, path)
+    np.testing.assert_array_equal(ld.cpu().numpy(), lens)
+    assert np.array_equal(bits_of(kd), k) and np.array_equal(bits_of(vd), v)
+    ctx.close()
+
+
+def test_kv_commits_of_one_context_on_two_streams():
+    """The commit keeps nothing in the context, so two streams that commit different batches through one (its status word
+    apart) do not meddle with each other: every length grows by its own accept_len, every time."""
+    rng = np.random.default_rng(80)
+    ctx = OwlContext(make_dims(batch=1, total_nodes=64, max_nodes=64))
+    B, n, page, rounds = 64, 4, 16, 20
+    sides = []
+    for hkv in (2, 8):
+        lens = rng.integers(0, 50, size=B).astype(np.int32)
+        alen = rng.integers(1, n + 1, size=B).astype(np.int32)
+        path = np.full((B, 64), -1, np.int32)
+        for b in range(B):
+            path[b, :alen[b]] = np.concatenate([[0], 1 + np.sort(rng.choice(n - 1, alen[b] - 1, replace=False))])
+        pages = (50 + (rounds + 1) * n) // page + 1
+        d = make_dims(batch=B, total_nodes=B * n, max_nodes=n, num_kv_heads=hkv, page_size=page, max_pages_per_seq=pages, num_pages=B * pages)
+        k, v = (torch.zeros(B * pages, hkv, page, 128, dtype=torch.bfloat16, device=DEV) for _ in range(2))
+        sides.append((torch.cuda.Stream(), d, k, v, dev_i32(np.arange(B * pages).reshape(B, pages)), dev_i32(lens), dev_i32(alen),
+                      dev_i32(path), lens + rounds * alen))
+    torch.cuda.synchronize()
+    for _ in range(rounds):
+        for stream, d, k, v, table, lens, alen, path, _ in sides:
+            with torch.cuda.stream(stream):
+                ctx.owl_kv_commit(d, k, v, table, lens, None, alen, path)
+    torch.cuda.synchronize()
+    assert ctx.owl_get_status() == 0
+    for *_, lens, alen, path, want in sides:
+        np.testing.assert_array_equal(lens.cpu().numpy(), want)
+    ctx.close()
+
+
 def test_kv_commit_hand_worked_and_errors(golden_dir):
     g = json.load(open(os.path.join(golden_dir, "kv_commit_cases.json")))
     rng = np.random.default_rng(60)

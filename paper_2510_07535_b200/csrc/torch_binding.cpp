@@ -6,6 +6,7 @@
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <utility>
@@ -69,10 +70,11 @@ bool dims_of(PyObject* o, owl_dims* out) {
     return ok;
 }
 
+// (the low 32 bits of any integer, as ctypes' c_int32 takes it)
 bool int_of(PyObject* o, int* out) {
-    const long v = PyLong_AsLong(o);
-    *out = (int)v;
-    return !(v == -1 && PyErr_Occurred());
+    const unsigned long v = PyLong_AsUnsignedLongMask(o);
+    *out = (int)(unsigned)v;
+    return !(v == (unsigned long)-1 && PyErr_Occurred());
 }
 
 // What the calls on a context begin with: (handle, device, ...)
@@ -221,7 +223,16 @@ OWL_CALL(tree_accept_static) {
     return unlocked([&] { return owl_tree_accept_static(&d, static_cast<float*>(p[0]), i(1), i(2), i(3), i(4), i(5), i(6), i(7), i(8), stream); });
 }
 
-#define OWL_METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
+// torch throws: from a tensor that has no storage or no strides, or where there is no device.  In Python that is an
+// ordinary exception.
+template <PyObject* (*kCall)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
+    HANDLE_TH_ERRORS
+    return kCall(self, args, nargs);
+    END_HANDLE_TH_ERRORS
+}
+
+#define OWL_METHOD(name) {#name, (PyCFunction)(void (*)(void))guarded<name>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {OWL_METHOD(verify_attn), OWL_METHOD(verify_attn_f16), OWL_METHOD(tree_accept), OWL_METHOD(tree_accept_spec),
                          OWL_METHOD(verify_step), OWL_METHOD(kv_commit), OWL_METHOD(prepare_spec_tree), OWL_METHOD(prepare_hybrid),
                          OWL_METHOD(lm_head_accept), OWL_METHOD(lstm_cell), OWL_METHOD(tree_accept_static), {nullptr, nullptr, 0, nullptr}};

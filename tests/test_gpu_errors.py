@@ -44,6 +44,18 @@ def test_host_detected_errors():
     ctx.close()
 
 
+def test_tensors_without_strides_or_storage_raise():
+    """A sparse tensor has no strides to check and no data pointer to hand over: an exception of the call, nothing launched."""
+    wl = _wl()
+    dw = DeviceWorkload.upload(wl)
+    ctx = OwlContext(dims_of(wl))
+    n0 = ctx.launch_count()
+    with pytest.raises((RuntimeError, TypeError)):
+        DeviceWorkload.attn(dataclass_replace(dw, lse=torch.eye(4, device="cuda").to_sparse()), ctx)
+    assert ctx.launch_count() == n0 and ctx.owl_get_status() == 0
+    ctx.close()
+
+
 def dataclass_replace(dw, **kw):
     import dataclasses
     return dataclasses.replace(dw, **kw)

@@ -9,6 +9,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <cstring>
 #include <utility>
 
 #include "../../include/owlverify.h"
@@ -59,11 +60,12 @@ bool tensors(PyObject* const* args, const Spec* spec, size_t count, int device, 
     return true;
 }
 
-// owl_dims out of the ctypes structure (any object with a buffer of that size)
+// owl_dims out of the ctypes structure, known by the layout that its buffer states (raw bytes of that size are refused)
 bool dims_of(PyObject* o, owl_dims* out) {
     Py_buffer view;
-    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return false;
-    const bool ok = view.len == (Py_ssize_t)sizeof(owl_dims);
+    if (PyObject_GetBuffer(o, &view, PyBUF_FORMAT) != 0) return false;
+    static const char kLayout[] = "T{<i:batch:<i:total_nodes:";
+    const bool ok = view.len == (Py_ssize_t)sizeof(owl_dims) && view.format && strncmp(view.format, kLayout, sizeof kLayout - 1) == 0;
     if (ok) memcpy(out, view.buf, sizeof *out);
     else PyErr_SetString(PyExc_TypeError, "dims: not an OwlDims");
     PyBuffer_Release(&view);

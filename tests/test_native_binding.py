@@ -24,6 +24,7 @@ def native():
 @pytest.mark.parametrize("args,message", [
     ((0, 0), "expected 10 arguments"),
     ((0, 0, b"short") + (None,) * 7, "OwlDims"),
+    ((0, 0, bytes(pkg.OwlDims(1, 1, 1))) + (None,) * 7, "OwlDims"),
     ((0, 0, pkg.OwlDims(), [1.0]) + (None,) * 6, "k_cache: expected a tensor"),
     ((0, 0, pkg.OwlDims(), torch.zeros(4, dtype=torch.bfloat16)) + (None,) * 6, "k_cache: expected contiguous torch.bfloat16 tensor on cuda:0"),
     ((None, 0, pkg.OwlDims()) + (None,) * 7, ""),

@@ -915,7 +915,7 @@ extern "C" int owl_tree_accept_static(const owl_dims* d, const float* logits, co
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) { cudaGetLastError(); return OWL_ERR_CUDA; }
     argmax_partial_kernel<<<argmax_grid((long long)chunks * d->total_nodes, sms), kArgmaxThreads, 0, stream>>>(p);
-    accept_walk_kernel<<<(unsigned)p.batch, kArgmaxThreads, 0, stream>>>(p, nullptr, 0);
+    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, static_cast<unsigned long long*>(nullptr), 0);
     if (cudaGetLastError() != cudaSuccess) return OWL_ERR_CUDA;
     return OWL_OK;
 }

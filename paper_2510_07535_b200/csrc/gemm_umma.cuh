@@ -5,8 +5,9 @@
 //   drafter     A = h [rows, d_in], B = [W^f; W^i; W^o; W^c] ([4d, d_in]), Eq. 2; the epilogue stores fp32.
 // M is small (up to 384 rows), N is huge: B is read from HBM exactly once, A comes again and again out of L2.
 //
-// The WEIGHTS are the instruction's M operand: the accumulator is C^T, one row of B per lane of tensor memory, one row of
-// A (rounded up to 16) per column.  What bounds the product is B's bytes and, run in a loop, the board's power.  With A as
+// The WEIGHTS are the instruction's M operand wherever a tile has more rows of B than there are rows of A (the other way
+// round, kRowsOnLanes, is below): the accumulator is C^T, one row of B per lane of tensor memory, one row of A (rounded up
+// to 16) per column.  What bounds the product is B's bytes and, run in a loop, the board's power.  With A as
 // the M operand every instruction multiplied 128 rows however few exist: at 30 rows and 6 TB/s the tensor cores did the
 // work of an 800 TFLOP/s product, three quarters of it on rows that nobody reads, and the power cap took the SM clock from
 // 1965 to 1140 MHz, which slows the memory system as well.
@@ -24,6 +25,11 @@
 // Measured (128256 x 4096 weights, us in a loop at the power cap; before = A as the M operand): 16 rows 192 -> 161, 32 rows
 // 195 -> 158, 64 rows 205 -> 163, 96 rows 195 -> 172, 128 rows 203 -> 183, 144 rows 281 -> 216, 192 rows 279 -> 233,
 // 256 rows 286 -> 273.  One CTA per SM instead of pairs: 162 / 163 / 175 / 185 / 193 us at 16 / 32 / 64 / 96 / 128 rows.
+//
+// kRowsOnLanes: few weights and many rows (weights of a few MB cut over 74 pairs make tiles of 16 to 100 rows of B, and
+// 256 rows of A as columns then keep the tensor cores busy for far longer than the bytes take).  The same stages, with the
+// roles of the two operands swapped in the instruction: one row of A per lane, the tile's rows of B as columns; a thread
+// of the epilogue owns a row of A for the whole kernel.  (rows_on_lanes has the rule and the figures.)
 //
 // Balance.  Every pair gets ceil(N / 16 / pairs) units of 16 rows of B, cut into as few tiles of at most 256 as
 // possible, the tiles of one round equally high on every pair (heights differ by at most 16 between rounds).
@@ -50,6 +56,7 @@ namespace gemm_path {
 using namespace sm100;
 
 enum Epilogue { kEpiArgmax = 0, kEpiStore = 1 };
+constexpr uint32_t kNobody = 0xffffffffu;
 
 constexpr int kBK = 64;                          // a k-block: one 128-byte swizzle row per operand row
 constexpr int kThreads = 256;
@@ -102,6 +109,14 @@ __host__ inline int smem_bytes(int groups, int stages, int block_bytes) {
 
 // How a product of M rows of A and N rows of B is laid out on `pairs` CTA pairs: the fields of GemmParams that follow from
 // the sizes.  Every pair gets the same number of 16-row units of B, cut into as few tiles as the height limit allows.
+// Which operand takes the lanes: the one of which a tile has more rows, since an instruction takes as long as it has
+// columns.  Measured with rows of B / rows of A on the lanes, us, weights not in L2, tile height h against a group's rows r:
+// argmax, K 1024 -> 5000 (h 80) at r 64: 10.5 / 10.8, 112: 11.9 / 10.9, 208: 14.5 / 11.3, 256: 15.5 / 12.5, 2 x 192:
+// 20.8 / 17.6; K 2112 -> 32000 (h 224) at r 112: 27.1 / 30.6, 208: 33.0 / 33.2, 256: 35.9 / 33.5, 2 x 192: 51.3 / 57.0.
+// Store, 1024 -> 4736 (h 64) at r 48: 19.3 / 19.4, 64: 22.9 / 20.1, 208: 46.4 / 45.4, 2 x 192: 86.9 / 78.0.
+__host__ inline bool rows_on_lanes(const GemmParams& g, Epilogue epi) {
+    return epi == kEpiStore ? g.h_lo <= g.group_rows : g.h_lo < g.group_rows;
+}
 __host__ inline int column_groups(int M) { return M <= kGroupRows ? 1 : 2; }
 __host__ inline int product_pairs(int N, int sms) { return (N + 15) / 16 < sms / 2 ? (N + 15) / 16 : sms / 2; }
 __host__ inline GemmParams product_plan(int M, int N, int K, int pairs) {
@@ -152,8 +167,23 @@ __device__ __forceinline__ unsigned long long warp_column_argmax(const uint32_t 
     return argmax_key(best, row0 + (uint32_t)__ffs((int)(who & valid)) - 1u);          // the lowest row of B among equals
 }
 
+// The arg-max of a row's columns [0, count) of 32, this lane's, folded into its best so far; `col0` is the first one's index.
+// NaN reads as -inf.  Columns come in ascending order: a later one wins only if it is larger.
+__device__ __forceinline__ void lane_row_argmax(const uint32_t (&v)[32], int count, uint32_t col0, float& best, uint32_t& who) {
+    float m = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+        if (j < count) m = fmaxf(m, __uint_as_float(v[j]));
+    if (who == kNobody || m > best) {
+        best = m;
+#pragma unroll
+        for (int j = 31; j >= 0; --j)
+            if (j < count && fmaxf(__uint_as_float(v[j]), -INFINITY) == m) who = col0 + j;
+    }
+}
+
 // gridDim.x is even: CTAs 2j and 2j + 1 are pair j.
-template <int kEpi, int kGroups>
+template <int kEpi, int kGroups, bool kRowsOnLanes>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap_hi,
                  const __grid_constant__ CUtensorMap bmap_lo) {
@@ -184,7 +214,7 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
         tma_prefetch_desc(&bmap_hi);
         tma_prefetch_desc(&bmap_lo);
     }
-    if (kEpi == kEpiArgmax)
+    if (kEpi == kEpiArgmax && !kRowsOnLanes)
         for (int i = tid; i < kMaxRows; i += kThreads) aux->best[i] = 0ull;
     if (warp == 0 && !misaligned) { tmem_alloc_pair(smem_u32(&aux->tmem_base), 512); tmem_relinquish_pair(); }
     if (warp == 0 && lane == 0 && !misaligned) {
@@ -262,7 +292,6 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
-            const uint32_t idesc = umma_idesc_16bit(256, p.group_rows, 0, 0, false);
             const uint64_t desc0 = umma_smem_desc_sw128(ring, 16, 1024);     // operands differ in the start address only
             const uint32_t desc_hi = (uint32_t)(desc0 >> 32), desc_lo = (uint32_t)desc0;
             uint32_t stage = 0, ph = 0, tcount = 0;
@@ -272,6 +301,7 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
                 const uint32_t buf = tcount % kBufs, acc_ph = (tcount / kBufs) & 1u;
                 const uint32_t a_off = (uint32_t)(tile_rows(t) >> 1) * (kBK * 2) >> 4, a_step = (uint32_t)a_half * (kBK * 2) >> 4;
                 const uint32_t d = tmem + buf * 256u;
+                const uint32_t idesc = umma_idesc_16bit(256, kRowsOnLanes ? tile_rows(t) : p.group_rows, 0, 0, false);
                 bool ok = wait(smem_u32(&aux->acc_empty[buf]), acc_ph ^ 1u);      // both epilogues have read this buffer
                 for (int kb = 0; kb < kblocks; kb += kQ) {
                     ok = (peek || wait(full_bar + stage * 8u, ph)) && ok;
@@ -286,9 +316,10 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
 #pragma unroll
                             for (int g = 0; g < kGroups; ++g) {
                                 const uint32_t a_lo = b_lo + a_off + g * a_step;
+                                const uint32_t lanes_lo = kRowsOnLanes ? a_lo : b_lo, columns_lo = kRowsOnLanes ? b_lo : a_lo;
 #pragma unroll
                                 for (int ks = 0; ks < kBK / 16; ++ks)    // 32 bytes along K inside the 128-byte swizzle row
-                                    umma_ss_pair_lh(d + g * 256u, b_lo + ks * 2, desc_hi, a_lo + ks * 2, desc_hi, idesc,
+                                    umma_ss_pair_lh(d + g * 256u, lanes_lo + ks * 2, desc_hi, columns_lo + ks * 2, desc_hi, idesc,
                                                     (q | ks) ? 1u : (kb ? 1u : 0u));
                             }
                         }
@@ -302,6 +333,14 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
     } else if (warp >= 4) {
         const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
         const int chunks = (p.group_rows + 31) / 32;
+        // kRowsOnLanes: this lane's row of A in each group, and its best so far
+        const int my_row = (int)rank * a_half + (warp & 3) * 32 + lane;
+        const bool warp_has_rows = (warp & 3) * 32 < a_half, row_on_lane = (warp & 3) * 32 + lane < a_half;
+        const bool c_aligned = (reinterpret_cast<uintptr_t>(p.c) & 15) == 0 && (p.ldc & 3) == 0;
+        float best[kGroups];
+        uint32_t who[kGroups];
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) { best[g] = -INFINITY; who[g] = kNobody; }
         uint32_t tcount = 0;
         for (int t = 0; t < p.rounds; ++t, ++tcount) {
             const int row0 = tile_row0(t);
@@ -316,7 +355,35 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
             const int warp_row = first + (warp & 3) * 32;               // row of B in the warp's lane 0
             const bool lane_valid = warp_row + lane < end;
             const uint32_t valid = __ballot_sync(0xffffffffu, lane_valid);
-            if (ok && warp_row < end) {
+            if (kRowsOnLanes) {
+                const int cols = min(tile_rows(t), p.N - row0);               // rows of B that exist: the columns here
+                if (ok && warp_has_rows) {
+#pragma unroll
+                    for (int g = 0; g < kGroups; ++g) {
+                        const int row = g * p.group_rows + my_row;
+#pragma unroll 1
+                        for (int c0 = 0; c0 < cols; c0 += 32) {
+                            uint32_t v[32];
+                            tmem_ld32(tmem + lane_sel + buf * 256u + g * 256u + c0, v);
+                            tmem_wait_ld();
+                            if (kEpi == kEpiArgmax) {
+                                lane_row_argmax(v, cols - c0, (uint32_t)(row0 + c0), best[g], who[g]);
+                            } else if (row_on_lane && row < p.M) {
+                                float* dst = p.c + (long long)row * p.ldc + row0 + c0;
+                                if (c_aligned && cols - c0 >= 32) {
+#pragma unroll
+                                    for (int j = 0; j < 32; j += 4)
+                                        *reinterpret_cast<uint4*>(dst + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                                } else {
+#pragma unroll
+                                    for (int j = 0; j < 32; ++j)
+                                        if (c0 + j < cols) dst[j] = __uint_as_float(v[j]);
+                                }
+                            }
+                        }
+                    }
+                }
+            } else if (ok && warp_row < end) {
 #pragma unroll 1
                 for (int g = 0; g < kGroups; ++g) {
 #pragma unroll 1
@@ -342,7 +409,12 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
             // unconditional: the issuing thread's wait on the even CTA's barrier must end
             mbar_arrive_cluster(cluster_map(smem_u32(&aux->acc_empty[buf]), 0));
         }
-        if (kEpi == kEpiArgmax) {
+        if (kEpi == kEpiArgmax && kRowsOnLanes) {
+#pragma unroll
+            for (int g = 0; g < kGroups; ++g)
+                if (row_on_lane && g * p.group_rows + my_row < p.M && who[g] != kNobody)
+                    atomicMax(p.row_key + g * p.group_rows + my_row, argmax_key(best[g], who[g]));
+        } else if (kEpi == kEpiArgmax) {
             asm volatile("bar.sync 1, 128;" ::: "memory");              // the four epilogue warps
             for (int i = tid - 128; i < p.M; i += 128)
                 if (aux->best[i]) atomicMax(p.row_key + i, aux->best[i]);

@@ -194,7 +194,9 @@ int launch_gemm(owl_ctx* ctx, const void* a, const void* b, int M, int N, int K,
         snprintf(ctx->err, sizeof ctx->err, "cuTensorMapEncodeTiled failed (%d, %d): operands must be 16-byte aligned", ra, rb);
         return OWL_ERR_CUDA;
     }
-    launch_dependent_smem(groups == 1 ? gemm_umma_kernel<kEpi, 1> : gemm_umma_kernel<kEpi, 2>, dim3(2u * (unsigned)pairs),
+    auto* kernel = rows_on_lanes(g, (Epilogue)kEpi) ? (groups == 1 ? gemm_umma_kernel<kEpi, 1, true> : gemm_umma_kernel<kEpi, 2, true>)
+                                    : (groups == 1 ? gemm_umma_kernel<kEpi, 1, false> : gemm_umma_kernel<kEpi, 2, false>);
+    launch_dependent_smem(kernel, dim3(2u * (unsigned)pairs),
                           dim3(kThreads), (size_t)smem_bytes(groups, g.stages, g.block_bytes), stream, g, amap, bmap_hi, bmap_lo);
     ++ctx->launches;
     return OWL_OK;
@@ -288,8 +290,10 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         auto full_smem = [](auto* kernel) {
             return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) == cudaSuccess;
         };
-        ok = full_smem(gemm_umma_kernel<kEpiArgmax, 1>) && full_smem(gemm_umma_kernel<kEpiArgmax, 2>) &&
-             full_smem(gemm_umma_kernel<kEpiStore, 1>) && full_smem(gemm_umma_kernel<kEpiStore, 2>);
+        ok = full_smem(gemm_umma_kernel<kEpiArgmax, 1, false>) && full_smem(gemm_umma_kernel<kEpiArgmax, 2, false>) &&
+             full_smem(gemm_umma_kernel<kEpiStore, 1, false>) && full_smem(gemm_umma_kernel<kEpiStore, 2, false>) &&
+             full_smem(gemm_umma_kernel<kEpiArgmax, 1, true>) && full_smem(gemm_umma_kernel<kEpiArgmax, 2, true>) &&
+             full_smem(gemm_umma_kernel<kEpiStore, 1, true>) && full_smem(gemm_umma_kernel<kEpiStore, 2, true>);
     }
     if (!ok || cudaDeviceSynchronize() != cudaSuccess) {
         cudaGetLastError();

@@ -104,6 +104,48 @@ def test_lm_head_accept_small(trees, K, V):
     ctx.close()
 
 
+@pytest.mark.parametrize("trees,K,V", [
+    ([("tree", 64, 8)] * 5, 4096, 12000),                           # 320 rows at a real hidden width: 64 stages of one k-block through a ring of seven
+    ([("tree", 64, 8)] * 2, 1024, 5000),                            # rows of A on the lanes (tiles of 80 weight rows): 128 rows
+    ([("tree", 64, 8)] * 4, 448, 40000),                            # ... 256 rows, three rounds, seven k-blocks
+    ([("tree", 64, 8)] * 4 + [("chain", 1)], 192, 5000),            # ... 257 rows in two groups
+    ([("tree", 64, 8)] * 6, 1024, 2000),                            # ... 384 rows, tiles of 32
+])
+def test_lm_head_accept_in_both_operand_orders(trees, K, V):
+    ctx = OwlContext(make_dims(batch=8, total_nodes=384, max_nodes=64, vocab=V))
+    alen = _lm_head_case(ctx, 2000 + K + V, trees, K, V)
+    assert alen.max() > 1
+    ctx.close()
+
+
+def test_rows_on_lanes_ties_infinities_and_nan():
+    """100 rows against 5000 weight rows: the arg-max of equal logits is the lowest index (equal weight rows in one tile, in
+    two tiles of a pair's CTAs and in tiles of different pairs), -inf everywhere gives 0, and NaN never wins."""
+    N, K, V = 100, 64, 5000
+    hidden = torch.zeros(N, K, device=DEV, dtype=torch.bfloat16)
+    weight = torch.zeros(V, K, device=DEV, dtype=torch.bfloat16)
+    hidden[:, 0] = 1.0
+    weight[:, 0] = -1.0
+    want = []
+    for i in range(N - 2):                              # row i looks at feature 1 + i % 32: equal logits at three columns
+        f, cols = 1 + i % 32, sorted({7 + 5 * (i % 32), 47 + 5 * (i % 32), 2600 + 61 * (i % 32)})
+        hidden[i, f] = 2.0
+        weight[cols, f] = 3.0
+        want.append(cols[0])
+    weight[3, 40], hidden[10, 40] = float("nan"), 1.0   # column 3 is NaN for every row
+    hidden[N - 2, 0] = float("inf")
+    want += [0, 0]                                      # -inf (and NaN in column 3) everywhere; all -1: the first
+    d = make_dims(batch=N, total_nodes=N, max_nodes=1, vocab=V)
+    ctx = OwlContext(d)
+    outs = [torch.zeros(N, dtype=torch.int32, device=DEV), torch.zeros(N, 64, dtype=torch.int32, device=DEV)] + \
+           [torch.zeros(N, dtype=torch.int32, device=DEV) for _ in range(2)]
+    tok = torch.zeros(N, dtype=torch.int32, device=DEV)
+    ctx.owl_lm_head_accept(d, hidden, weight, tok, None, tok - 1, *outs)
+    assert ctx.owl_get_status() == 0
+    assert outs[3].cpu().tolist() == want
+    ctx.close()
+
+
 def test_lm_head_accept_calls_of_different_sizes_on_one_context():
     """The row keys live in two sets that alternate between calls, each cleared as a whole by the call before: a
     200-row call, an 8-row call, a 200-row call and a 23-row call through one context (two launches each inside

@@ -5,6 +5,7 @@ import torch
 
 from paper_2510_07535_b200 import OwlContext, make_dims, workloads as W
 from test_gpu_parity import check_accept, check_attention
+from test_product_plan import ROWS_ON_LANES, SEVERAL_TILES
 
 pytestmark = pytest.mark.gpu
 
@@ -64,7 +65,7 @@ def test_scan_items_of_every_size_and_walk_groups(nodes, vocab):
 @pytest.mark.parametrize("rows,d_in", [(1, 64), (16, 192), (17, 64), (32, 320), (33, 192), (128, 192), (129, 64), (256, 192), (257, 64), (383, 192)])
 def test_product_row_padding_and_odd_k_blocks(rows, d_in):
     """The weight-streaming product behind the drafter cell, element by element: rows around the padding to 16 and the
-    switch to two column groups (257), one, three and five k-blocks (a stage holds two), several tiles per CTA pair.
+    switch to two column groups (257), one, three and five k-blocks (a stage holds two); one tile per CTA pair.
     Bound: fp32 accumulation of K exact products, K 2^-24 sum_k |h_k| |w_k| per element."""
     d = 4096 + 20
     g = torch.Generator().manual_seed(rows)
@@ -79,6 +80,29 @@ def test_product_row_padding_and_odd_k_blocks(rows, d_in):
     ref = h.double() @ w.double().t()
     bound = d_in * 2.0 ** -24 * (h.double().abs() @ w.double().abs().t())
     assert bool(((ws.cpu().double() - ref).abs() <= bound).all())
+    ctx.close()
+
+
+@pytest.mark.parametrize("rows,d_in,d", SEVERAL_TILES + ROWS_ON_LANES)
+def test_product_over_several_tiles_and_in_both_operand_orders(rows, d_in, d):
+    """Element by element at the shapes that test_product_plan.py describes.  Bound: fp32 accumulation of K exact products,
+    K 2^-24 sum_k |h_k| |w_k| per element."""
+    g = torch.Generator(device="cuda").manual_seed(rows + d)
+    h = torch.randn(rows, d_in, generator=g, device="cuda").bfloat16()
+    w = torch.randn(4 * d, d_in, generator=g, device="cuda").bfloat16()
+    emb = torch.zeros(rows, d, dtype=torch.bfloat16, device="cuda")
+    z, hf = torch.zeros(rows, d, device="cuda"), torch.empty(rows, d, device="cuda")
+    scratch = torch.full((4 * rows * d + 4,), float("nan"), device="cuda")
+    ctx = OwlContext(make_dims(batch=1, total_nodes=1, max_nodes=1))
+    ref = h.double() @ w.double().t()
+    bound = d_in * 2.0 ** -24 * (h.double().abs() @ w.double().abs().t())
+    for first in (0, 1):                                   # scratch that is aligned to 16 bytes, and to 4 only
+        ws = scratch[first:first + 4 * rows * d].view(rows, 4 * d)
+        ws.fill_(float("nan"))
+        ctx.owl_lstm_cell(h, emb, w, 0.0, z, hf, None, ws)
+        assert ctx.owl_get_status() == 0
+        assert bool(((ws.double() - ref).abs() <= bound).all())
+        assert torch.isnan(scratch[first + 4 * rows * d:]).all()
     ctx.close()
 
 

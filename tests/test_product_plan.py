@@ -7,7 +7,8 @@ import pytest
 
 from paper_2510_07535_b200 import build as owl_build
 
-FIELDS = ("rounds", "tall_rounds", "h_lo", "group_rows", "stages", "kblocks_per_stage", "smem")
+FIELDS = ("rounds", "tall_rounds", "h_lo", "group_rows", "stages", "kblocks_per_stage", "smem", "rows_on_lanes_argmax",
+          "rows_on_lanes_store")
 PROGRAM = r"""
 #include <cstdio>
 #include "gemm_umma.cuh"
@@ -17,8 +18,8 @@ int main() {
     while (scanf("%d %d %d %d", &M, &N, &K, &sms) == 4) {
         const int groups = column_groups(M);
         const GemmParams g = product_plan(M, N, K, product_pairs(N, sms));
-        printf("%d %d %d %d %d %d %d\n", g.rounds, g.tall_rounds, g.h_lo, g.group_rows, g.stages, stage_kblocks(groups),
-               smem_bytes(groups, g.stages, g.block_bytes));
+        printf("%d %d %d %d %d %d %d %d %d\n", g.rounds, g.tall_rounds, g.h_lo, g.group_rows, g.stages, stage_kblocks(groups),
+               smem_bytes(groups, g.stages, g.block_bytes), rows_on_lanes(g, kEpiArgmax), rows_on_lanes(g, kEpiStore));
     }
 }
 """
@@ -47,3 +48,22 @@ def test_an_sm_never_holds_two_ctas(plans):
     for shape, p in zip(shapes, plans(shapes)):
         assert 2 * (p["smem"] + 1024) > 228 * 1024 and p["smem"] <= 227 * 1024, (shape, p)
         assert p["stages"] >= 2 and p["h_lo"] + (16 if p["tall_rounds"] else 0) <= 256, (shape, p)
+
+
+# (rows of A, K, d) of cell calls: products of 4d weight rows that test_gpu_kernel_edges.py checks element by element
+SEVERAL_TILES = [(10, 1088, 12288 + 252), (130, 1088, 12288 + 252), (200, 1088, 12288 + 252), (257, 1088, 12288 + 252), (384, 1024, 12288 + 252)]
+ROWS_ON_LANES = [(64, 1088, 1184), (100, 448, 1184), (256, 1088, 1184), (256, 1088, 12288 + 252), (257, 1088, 1184), (384, 1024, 1184),
+                 (384, 960, 2048), (33, 64, 4)]
+
+
+def test_the_shapes_of_the_gpu_tests_have_what_they_are_there_for(plans):
+    """Three rounds of tiles and more, the last ones lower, a ring that wraps within a tile, an odd number of k-blocks; and the
+    swapped operand order at one and at two groups, at one round and at several."""
+    for (m, k, d), p in zip(SEVERAL_TILES, plans([(m, 4 * d, k) for m, k, d in SEVERAL_TILES])):
+        assert p["rounds"] >= 3 and 0 < p["tall_rounds"] < p["rounds"], p
+        assert -(-(k // 64) // p["kblocks_per_stage"]) > p["stages"], p
+        assert not p["rows_on_lanes_store"], p
+    assert any((k // 64) % 2 for _, k, _ in SEVERAL_TILES) and {m > 256 for m, _, _ in SEVERAL_TILES} == {True, False}
+    lanes = plans([(m, 4 * d, k) for m, k, d in ROWS_ON_LANES])
+    assert all(p["rows_on_lanes_store"] for p in lanes)
+    assert {(p["kblocks_per_stage"], p["rounds"] > 1) for p in lanes} >= {(2, False), (2, True), (1, False)}

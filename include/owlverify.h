@@ -280,9 +280,10 @@ double owl_lstm_alpha(int32_t n_depth, int32_t d);
  * two calls, results bit for bit those of the two calls.  The two halves do not depend on each other (the
  * logits are an input), so a small acceptance (total_nodes * ceil(vocab / 8192) <= 1024) costs no launch
  * of its own: spare warps of the attention kernel scan the logits while K/V stream in, and the kernel
- * that merges the attention partials also walks the trees.  Larger scans follow the attention pass as a
- * kernel of their own.  Everything runs on `stream`, in stream order.  Asynchronous; errors as in the
- * two calls (argument errors of either half are reported before anything is launched).
+ * that merges the attention partials also walks the trees.  A larger scan is a kernel of its own between
+ * the attention pass and that merge; it reads nothing of the pass and runs beside its end.  Everything
+ * runs on `stream`, after what was queued there before.  Asynchronous; errors as in the two calls
+ * (argument errors of either half are reported before anything is launched).
  */
 int owl_verify_step(owl_ctx* ctx, const owl_dims* dims, const void* q, const void* k_cache, const void* v_cache,
                     const int32_t* block_table, const int32_t* ctx_lens, const int32_t* node_offsets,
@@ -317,7 +318,8 @@ int owl_verify_step_host(owl_ctx* ctx, const owl_dims* dims, const void* q_h, co
  * cudaMalloc - and the device-wide synchronisation it can imply - is forbidden.  Such callers
  * cannot use owl_create, which allocates a workspace.  This call takes no context and allocates
  * nothing, neither with cudaMalloc nor through any library: its scratch (one 64-bit arg-max key
- * per logits row and 8192-float vocabulary chunk, the status word) is a fixed array inside the library image.  The price: every GPU on which the library is loaded holds that array,
+ * per logits row and 8192-float vocabulary chunk, the status word) is a fixed array inside the library
+ * image.  The price: every GPU on which the library is loaded holds that array,
  * (OWL_STATIC_MAX_KEYS + 32) * 8 bytes = 128.25 KiB, until the process exits.
  *
  * Limit: total_nodes * ceil(vocab / 8192) <= OWL_STATIC_MAX_KEYS (e.g. 1024 nodes at a 128256-entry

@@ -233,14 +233,14 @@ __device__ __forceinline__ void argmax_scan_chunk_warp(const AcceptParams& p, co
 }
 
 // Persistent scan: the grid's warps take the (row, vocabulary chunk) items in turn (consecutive warps read
-// consecutive chunks), each with eight 16-byte loads per lane in flight, so that a warp streams without the
-// per-item cost of a CTA's launch and barriers.
+// consecutive chunks), each with up to two rounds of eight 16-byte loads per lane in flight, so that a warp streams
+// without the per-item cost of a CTA's launch and barriers.
 constexpr int kArgmaxWarps = kArgmaxThreads / 32;
 constexpr int kScanAhead = 4096;        // floats
-constexpr int kArgmaxCtasPerSm = 2;     // what fits at the kernel's register count
+constexpr int kArgmaxCtasPerSm = 2;     // what fits at the kernel's register count; argmax_grid counts on it
 __host__ inline long long argmax_warps(int sms) { return (long long)sms * kArgmaxCtasPerSm * kArgmaxWarps; }
 
-__global__ void __launch_bounds__(kArgmaxThreads) argmax_partial_kernel(const AcceptParams p) {
+__global__ void __launch_bounds__(kArgmaxThreads, kArgmaxCtasPerSm) argmax_partial_kernel(const AcceptParams p) {
     // may be launched as a programmatic dependent of the kernel before it in the stream: nothing is read
     // before that kernel has completed (a no-op in an ordinary launch).  After the attention pass of the same step the
     // scan need not wait: the pass lets its dependents start only once everything before it has completed, and the

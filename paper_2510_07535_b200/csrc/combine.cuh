@@ -48,7 +48,7 @@ inline size_t combine_smem_bytes(int group, unsigned ctas, int sms) {
 // kFused (verify step): the grid has one more CTA per sequence after the row CTAs; each of those runs one
 // sequence's acceptance walk over the arg-max keys that the pass's spare warps left (`ap`).
 //
-// p.combine_group: partials fetched per round, at most 32 (combine_group below).  A round's rows go through a
+// p.combine_group: partials fetched per round, at most 32 (combine_group above).  A round's rows go through a
 // warp-private stage in shared memory of that many rows, which is what limits the CTAs per SM.
 //
 // The stage is there for the sake of the code's length, not of the data: with the rows in registers the fetch and

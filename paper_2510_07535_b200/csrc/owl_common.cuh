@@ -170,8 +170,8 @@ __device__ __forceinline__ bool seq_shape_ok(const AttnParams& p, int b, int n, 
 }
 
 // Schedule of a batch of at most 32 sequences, derived by one warp on its own: lane b holds sequence b, prefix sums
-// by shuffle, no shared memory.  The split-KV pass (every warp of it) and the merge that follows it call the same
-// function on the same inputs, so the merge needs nothing from the pass but its partials.
+// by shuffle, no shared memory.  The split-KV pass (its producer warp) and the merge that follows it (every warp) call the
+// same function on the same inputs, so the merge needs nothing from the pass but its partials.
 constexpr int kSchedTileKeys = 128;      // key tile of the split-KV pass
 struct WarpSchedule {
     int n, L, node_base, tiles;          // this lane's sequence (tiles = 0 if it is not schedulable)

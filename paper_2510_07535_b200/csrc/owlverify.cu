@@ -327,8 +327,9 @@ static void launch_scan(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool
 static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream);
 
 // Attention of a verify step.  `ap` non-null: the acceptance of the same step.  A small scan rides in the attention
-// kernel's spare warps, two launches for the whole step; a larger one (`own_scan`) is a kernel of its own between the attention pass and its merge, where it fills the SMs that the pass leaves one by one.  The walk
-// rides in the merge kernel.
+// kernel's spare warps, two launches for the whole step; a larger one (`own_scan`) is a kernel of its own between the
+// attention pass and its merge, where it fills the SMs that the pass leaves one by one, three launches.  The walk rides
+// in the merge kernel either way.
 static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, const void* k_cache, const void* v_cache,
                             const int32_t* block_table, const int32_t* ctx_lens, const int32_t* node_offsets,
                             const int32_t* tree_parent, void* out, float* lse, void* stream_, AcceptParams* ap,
@@ -458,7 +459,7 @@ int owl_verify_attn_f16(owl_ctx* ctx, const owl_dims* d, const void* q, const vo
                             nullptr, true);
 }
 
-// Argument checks of the acceptance and its kernel parameters (everything but the counters of the stand-alone kernel).
+// Argument checks of the acceptance and its kernel parameters.
 static int accept_params(owl_ctx* ctx, const owl_dims* d, const float* logits, const int32_t* draft_tokens,
                          const int32_t* node_offsets, const int32_t* tree_parent, int32_t* accept_len,
                          int32_t* accept_path, int32_t* bonus_token, int32_t* node_argmax, AcceptParams& p,

@@ -422,14 +422,15 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
         // A turn: O_s += P_s V of the stream's tile i, then S_s = Q K^T of its tile i + 1 (which overwrites the P just
         // consumed; the tensor pipe runs them in order), each where the stream has such a tile; i = -1 issues the first S
         // of both streams.  The text of one turn serves both streams and all tiles: with the two streams unrolled (and the
-        // first and last turns in a rolled form of their own) there was twice the text to fetch into cold caches
-        // (2K step 15.5 -> 14.4 us, 32K 39.7 -> 38.3 us, round 49.3 -> 47.9 us).
+        // first and last turns in a rolled form of their own) there was twice the text to fetch into cold caches, and a 2K
+        // step took 15.4 us instead of 14.4, 32K 39.6 instead of 38.3, 4 x 128K 641 instead of 629.
 #pragma unroll 1
         for (int i = -1; i < n_it[0]; ++i) {
             if (kWide && shared && ok && i >= 0 && i + 1 < T) {
                 // The middle of a 256-row unit, where this warp's time is what counts: both streams have both products, and
-                // a turn has no conditions but the stream's commits (with the general turn instead 70B 660 -> 693 us;
-                // with both streams unrolled 660 -> 653 us, fp16 with 60 nodes 72.8 -> 71.0 us).
+                // a turn has no conditions but the stream's commits.  With the general turn here as well the 70B step took
+                // 693 us instead of 660; with this one unrolled over the streams 653, which the next pass's cold fetches
+                // of the longer text cost the short cases again.
                 const uint32_t issue = elected, acc0 = i > 0 ? 1u : 0u;
                 const uint32_t v_lo = (uint32_t)v_desc0 + v_slot * (uint32_t)(kSlotBytes >> 4), v_hi = (uint32_t)(v_desc0 >> 32);
                 const uint32_t k_lo = (uint32_t)k_desc0 + k_slot * (uint32_t)(kSlotBytes >> 4), k_hi = (uint32_t)(k_desc0 >> 32);

@@ -105,7 +105,7 @@ def test_lm_head_accept_small(trees, K, V):
 
 
 @pytest.mark.parametrize("trees,K,V", [
-    ([("tree", 64, 8)] * 5, 4096, 12000),                           # 320 rows at a real hidden width: 64 stages of one k-block through a ring of seven
+    ([("tree", 64, 8)] * 5, 4096, 12000),                           # 320 rows at a real hidden width: 64 stages of one k-block through a ring of six
     ([("tree", 64, 8)] * 2, 1024, 5000),                            # rows of A on the lanes (tiles of 80 weight rows): 128 rows
     ([("tree", 64, 8)] * 4, 448, 40000),                            # ... 256 rows, three rounds, seven k-blocks
     ([("tree", 64, 8)] * 4 + [("chain", 1)], 192, 5000),            # ... 257 rows in two groups

@@ -715,13 +715,14 @@ int owl_verify_step(owl_ctx* ctx, const owl_dims* d, const void* q, const void* 
     if (!ctx) return OWL_ERR_INVALID_ARG;
     int rc = check_dims(d, true, true);
     if (rc != OWL_OK) return rc;
-    // A scan of up to about a thousand (row, chunk) items - a few per spare warp - rides inside the attention kernel;
-    // a larger one slows the attention down by more than its own kernel costs (measured: 4 x 64 nodes of a 128K
-    // vocabulary, 570 -> 605 us), so it follows as a kernel of its own in stream order.
+    // A scan of up to 1024 (row, 8192-float chunk) items, three to four per spare warp, rides inside the attention kernel; a
+    // larger one is a kernel of its own between the attention pass and the merge.  One sequence, 128256 tokens, us per
+    // step as guests / as a kernel at contexts of 1K, 3K, 9K, 32K: 8 nodes 12.1 / 12.4, 15.2 / 15.8, 18.7 / 19.6, 32.6 / 33.4;
+    // 32 nodes 15.1 / 16.6, 18.5 / 19.6, 21.5 / 22.9, 35.7 / 36.9; 64 nodes (1024 items) 26.9 / 25.4,
+    // 30.2 / 28.9, 32.7 / 33.1, 49.1 / 51.3: there the line goes through, by the scan's size alone.  Beyond it guests slow the
+    // attention down (4 x 64 nodes at 128K: by 35 us).
     const long long scan_items = (long long)d->total_nodes * ((d->vocab + kArgmaxChunk - 1) / kArgmaxChunk);
     const bool own_scan = scan_items > 1024;
-    // Two launches: the attention kernel, whose two spare warps per CTA scan the logits while K/V stream in, and the
-    // merge kernel, which also walks the trees.
     AcceptParams ap;
     rc = accept_params(ctx, d, logits, draft_tokens, node_offsets, tree_parent, accept_len, accept_path, bonus_token, node_argmax, ap,
                        nullptr, own_scan ? 0 : kArgmaxChunk);      // guests are few: what counts is the cost per item

@@ -310,14 +310,13 @@ __device__ __forceinline__ bool readers_reached(Aux* aux, int seg_no) {
 
 template <bool kWide>
 __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtensorMap* kmap, const CUtensorMap* vmap,
-                                              Aux* aux, uint32_t ring, Walker w, uint32_t& items_out) {
+                                              Aux* aux, uint32_t ring, Walker w) {
     const int lane = threadIdx.x & 31;
     volatile int* abort_flag = &aux->abort_flag;
     const int ppt = kTileKeys >> p.page_shift;               // pages (= TMA boxes) per tile
     const uint32_t box_bytes = (uint32_t)p.page_size * 256u;
     const int oob = p.num_pages * p.num_kv_heads;            // a coordinate past the end: the box reads zeros
     uint32_t item = 0;
-    bool going = true;
     // K/V are read once: let them leave L2 first, so that Q, the partials, the tables and the code stay
     const uint64_t stream_policy = l2_policy_evict_first();
     for (uint32_t seg_no = 0;; ++seg_no) {
@@ -360,22 +359,20 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
             for (int kv = 0; kv < 2; ++kv) {
                 const uint32_t slot = item % kSlots, ph = (item / kSlots) & 1u;
                 const uint32_t full = smem_u32(&aux->full[(item >> 1) % kTilesInFlight]);
-                // A lane that has given up once issues nothing any more, so its `item` counts, in order, what it has issued
-                // (the drain at the kernel's end goes by it); the lanes meet on every path.  (A vote for one verdict costs
-                // 16 mixed sequences 1.5 %.)
-                going = going && mbar_wait(smem_u32(&aux->empty[slot]), ph ^ 1u, abort_flag);
+                // A slot whose wait gave up is left out, but `item` goes by the tiles all the same: K and V keep their slots, and
+                // the lanes, which may disagree about a wait that gives up, keep step.
+                const bool ok = mbar_wait(smem_u32(&aux->empty[slot]), ph ^ 1u, abort_flag);
                 // the tile's barrier expects K and V together (announced with K; V follows as its slot frees up)
-                if (going && lane == 0 && kv == 0) mbar_arrive_expect_tx(full, 2u * (uint32_t)kSlotBytes);
+                if (ok && lane == 0 && kv == 0) mbar_arrive_expect_tx(full, 2u * (uint32_t)kSlotBytes);
                 __syncwarp();
-                if (going && lane < ppt)
+                if (ok && lane < ppt)
                     tma_load_5d_hint(ring + slot * kSlotBytes + lane * box_bytes, kv ? vmap : kmap, full, 0, 0, 0, 0, c_cur,
                                      stream_policy);
-                item += going ? 1u : 0u;
+                ++item;
                 __syncwarp();
             }
         }
     }
-    items_out = item;
 }
 
 // ------------------------------------------------------------------------------------------ MMA issuer
@@ -478,7 +475,7 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
                         umma_ts_lh_if(issue, tS + 256, tS + ks * 8, v_lo + (uint32_t)(ks * 4096 >> 4), v_hi, idesc_pv, ks ? 1u : (i > 0 ? 1u : 0u));
                     // only the segment end waits for it; made on every path, like the announcement of S below
                     umma_commit_if(i == n_s - 1 ? issue : 0u, smem_u32(&aux->o_done[0]) + s * 8u);
-                    mbar_arrive_if(i == n_s - 1 && elected != issue, smem_u32(&aux->o_done[0]) + s * 8u);
+                    if (!ok && i == n_s - 1 && elected) mbar_arrive(smem_u32(&aux->o_done[0]) + s * 8u);
                     // (Releasing the ring slots from a softmax thread instead - a score tile's arrival covers every product
                     // issued before it - spares this warp two commits per tile, but the slots come back late: 1 % slower
                     // on 256-row units, 15 to 35 % on the bandwidth-bound ones.)
@@ -511,7 +508,7 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
                     // rely on it to be at most one tile ahead of this warp's bar.sync (their second arrival in one
                     // generation of barrier 4 + s would leave this warp waiting there for good)
                     umma_commit_if(issue, smem_u32(&aux->s_full[0]) + s * 8u);
-                    mbar_arrive_if(elected != issue, smem_u32(&aux->s_full[0]) + s * 8u);
+                    if (!ok && elected) mbar_arrive(smem_u32(&aux->s_full[0]) + s * 8u);
                     umma_commit_if(last_reader ? issue : 0u, smem_u32(&aux->empty[0]) + k_slot * 8u);
                 }
                 // the tiles lie in the ring in the order of the turns that consume them, K and V by turns
@@ -1002,14 +999,13 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
     // with.  The logits guests take 104 (128 x 104 + 256 x 200) to have two rounds of loads in flight instead of one: at
     // short contexts the scan is what a step waits for (32 nodes at 9000 tokens 30.9 -> 21.9 us, 64 nodes 54.0 -> 33.9 us;
     // 2K chain 14.4 -> 14.5, 32K 38.4 -> 38.5 us).
-    uint32_t items = 0;
     if (warp < 4) {
         if (kFused) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         if (!kManySeqs) wait_for_inputs();
         if (warp == 0) {
             if (!kManySeqs) build_walk_small(p, w);
-            producer_loop<kWide>(p, &kmap, &vmap, aux, smem_base + kRingOff, w, items);
+            producer_loop<kWide>(p, &kmap, &vmap, aux, smem_base + kRingOff, w);
         } else if (warp == 1) {
             mma_loop<kWide, kF16>(aux, smem_base, tmem);
         } else if (kFused) {
@@ -1028,13 +1024,10 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
     __syncthreads();
     if (warp == 0) {
         if (aux->abort_flag) {
-            // give the copies still in flight a bounded time to land before the CTA's shared memory is released
-            const uint32_t tiles_issued = (items + 1u) >> 1;
-            const uint32_t first = tiles_issued > (uint32_t)kTilesInFlight ? tiles_issued - kTilesInFlight : 0u;
-            for (uint32_t it = first; it < tiles_issued; ++it) {
-                const uint32_t bar = smem_u32(&aux->full[it % kTilesInFlight]), ph = (it / kTilesInFlight) & 1u;
-                for (int polls = 0; polls < (1 << 20) && !mbar_try_wait(bar, ph); ++polls) {}
-            }
+            // Copies may still be in flight, and which barriers they complete on is not certain any more: a thousand times
+            // what a copy takes, before the CTA's shared memory is released.
+            const uint64_t t0 = global_timer_ns();
+            for (int polls = 0; polls < (1 << 22) && global_timer_ns() - t0 < 2000000ull; ++polls) {}
             if (lane == 0) report(p.status, kErrTimeout);
         }
         tc_fence_after();

@@ -1,8 +1,7 @@
 """A model of how the attention kernel's roles agree on the segments of a CTA's piece and hand over P tile by tile, run under
 random interleavings on the CPU.  A wait on a tile or on a free slot may give up at any point; from then on all of those
 return at once.  What is never abortable must still end: the hardware barriers, the wait for a score tile and the producer's
-look at `seg_reached`; every reader must have taken every segment; and the copies that the producer has issued must be
-the first ones in order, which is what the drain at the kernel's end takes them for."""
+look at `seg_reached`; every reader must have taken every segment; and a copy goes to the ring slot of its own tile and kind."""
 import random
 import re
 from pathlib import Path
@@ -15,12 +14,12 @@ SLOTS = int(re.search(r"constexpr int kSlots = (\d+);", SOURCE).group(1))
 
 
 class Cta:
-    def __init__(self, rng, segments, paced, certain, final):
-        self.rng, self.paced, self.certain, self.final, self.abort = rng, paced, certain, final, False
+    def __init__(self, rng, segments, paced, certain, by_tile):
+        self.rng, self.paced, self.certain, self.by_tile, self.abort = rng, paced, certain, by_tile, False
         self.tiles = [rng.randint(1, 3) for _ in range(segments)] + [0]       # 0: no more segments
         self.place, self.announced = [None] * PLACES, [0] * PLACES            # contents; completed phases
         self.reached = 0
-        self.issued = self.freed = 0                                          # slots copied to; tiles (two slots) consumed
+        self.copied, self.freed = set(), 0                                    # items (K, V, K, V, ...) copied; tiles consumed
         self.q_full = 0                                                       # segments whose Q has been loaded
         self.live = [rng.randint(1, 4) for _ in range(segments + 1)]          # softmax warps that hand over P
         self.scores = self.products = 0                                       # tiles: S announced, P V done
@@ -47,7 +46,7 @@ class Cta:
         return lambda: self.announced[k % PLACES] % 2 != (k // PLACES) % 2
 
     def producer(self):
-        going, slot = True, 0                    # of the sequence K, V, K, V, ...
+        item, wanted = 0, 0                      # the ring's count; of the sequence K, V, K, V, ...
         for k, tiles in enumerate(self.tiles):
             if self.paced and k >= PLACES:
                 yield lambda: self.reached >= k - PLACES + 1
@@ -55,14 +54,14 @@ class Cta:
             yield None
             self.announced[k % PLACES] += 1
             for _ in range(2 * tiles):
-                free = lambda: self.issued - 2 * self.freed < SLOTS
-                if going or not self.final:
-                    yield self.bounded(free)
-                    going = free()
-                if going:
-                    assert self.issued == slot, "a copy after one that was left out"
-                    self.issued += 1
-                slot += 1
+                free = lambda: item - 2 * self.freed < SLOTS
+                yield self.bounded(free)
+                if free():
+                    assert item % 2 == wanted % 2, "K in a slot of V"
+                    self.copied.add(item)
+                if free() or self.by_tile:
+                    item += 1
+                wanted += 1
 
     def meet(self, k, leader):                   # meet_before_segment
         if self.paced:
@@ -80,11 +79,11 @@ class Cta:
             yield self.bounded(lambda: self.q_full > k)
             for _ in range(self.tiles[taken[-1]]):
                 first = self.products
-                yield self.bounded(lambda: self.issued >= 2 * first + 2)
+                yield self.bounded(lambda: {2 * first, 2 * first + 1} <= self.copied)
                 self.scores += 1
                 yield self.sync(4, self.live[taken[-1]] + 1)
                 self.products += 1
-                self.freed = min(self.issued // 2, self.products)
+                self.freed = self.products
 
     def softmax(self, taken, leader):
         """One stream's warpgroup; the second one here only loads Q and sleeps through the tiles."""
@@ -130,9 +129,9 @@ class Cta:
         return taken
 
 
-def segments_of(seed, segments, paced=True, certain=True, final=True):
+def segments_of(seed, segments, paced=True, certain=True, by_tile=True):
     rng = random.Random(seed)
-    return Cta(rng, segments, paced, certain, final).run(abort_at=rng.choice([0, 10 ** 9, rng.randint(0, 12 * segments)]))
+    return Cta(rng, segments, paced, certain, by_tile).run(abort_at=rng.choice([0, 10 ** 9, rng.randint(0, 12 * segments)]))
 
 
 @pytest.mark.parametrize("segments", [1, PLACES - 1, PLACES, PLACES + 1, 16, 40])
@@ -141,10 +140,10 @@ def test_all_roles_take_the_same_segments_whatever_gives_up(segments):
         assert segments_of(seed, segments) == [list(range(segments + 1))] * 3, seed
 
 
-@pytest.mark.parametrize("segments,without", [(40, "paced"), (4, "certain"), (4, "final")])
+@pytest.mark.parametrize("segments,without", [(40, "paced"), (4, "certain"), (4, "by_tile")])
 def test_the_model_shows_what_each_rule_is_for(segments, without):
     """A producer that nothing paces, softmax warps that hand over P of a tile whose S was not announced, a producer that
-    copies on after a wait of its own gave up."""
+    counts only what it has copied."""
     def broken(seed):
         try:
             return segments_of(seed, segments, **{without: False}) != [list(range(segments + 1))] * 3

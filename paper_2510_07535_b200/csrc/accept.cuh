@@ -66,6 +66,17 @@ struct AcceptParams {
     int32_t chunk, chunks;           // floats per item, items per row
 };
 
+// The LM-head product's row keys only ever grow (atomicMax) and must start from 0, below every real key.  Two sets of
+// `stride` keys alternate between calls: a call's product raises one, its walk reads that one and clears the other as a
+// whole, so that no memset stands in front of a product.  Which set is a call's own is counted on the device - a call
+// replayed from a graph has its host side behind it: the product reads call[0] and leaves what it read in call[1], the
+// walk goes by call[1] and moves call[0] on.  (Two words, because a walk's CTAs read the number while one of them moves it.)
+struct KeySets {
+    unsigned long long* keys;        // [2, stride]; null: the walk's keys are AcceptParams::part_keys
+    uint32_t* call;
+    int32_t stride;
+};
+
 __device__ __forceinline__ unsigned long long argmax_key(float x, uint32_t idx) {
     if (x != x) x = -INFINITY;   // NaN never wins
     x += 0.0f;                   // -0.0 -> +0.0
@@ -282,14 +293,22 @@ __global__ void __launch_bounds__(kArgmaxThreads, kArgmaxCtasPerSm) argmax_parti
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// One sequence's acceptance walk per CTA over the keys the scan or the LM-head product left.  `idle_keys[0, idle_len)` is
-// cleared (the key set the next product will raise; nothing of this call uses it).  Launched as a programmatic
-// dependent: it reads nothing before the kernel before it has completed.
-__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_kernel(const AcceptParams p, unsigned long long* idle_keys, int idle_len) {
+// One sequence's acceptance walk per CTA over the keys the scan or the LM-head product (`sets`) left.  Launched as a
+// programmatic dependent: it reads nothing before the kernel before it has completed.
+__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_kernel(AcceptParams p, const KeySets sets) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    for (int i = blockIdx.x * kArgmaxThreads + threadIdx.x; i < idle_len; i += gridDim.x * kArgmaxThreads) idle_keys[i] = 0ull;
+    uint32_t call = 0u;
+    if (sets.keys) {
+        call = __ldcg(sets.call + 1);
+        p.part_keys = sets.keys + (size_t)(call & 1u) * sets.stride;
+    }
     accept_walk_seq(p, (int)blockIdx.x);
+    if (sets.keys) {
+        unsigned long long* idle = sets.keys + (size_t)((call + 1u) & 1u) * sets.stride;
+        for (int i = blockIdx.x * kArgmaxThreads + threadIdx.x; i < sets.stride; i += gridDim.x * kArgmaxThreads) idle[i] = 0ull;
+        if (blockIdx.x == 0 && threadIdx.x == 0) sets.call[0] = call + 1u;
+    }
 }
 
 // Grid of the scan for `items` (row, chunk) items on a device with `sms` multiprocessors: as many warps as give

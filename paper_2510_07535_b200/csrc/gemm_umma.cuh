@@ -81,7 +81,7 @@ struct GemmParams {
     int tall_rounds;                // rounds [0, tall_rounds) are h_lo + 16 rows of B high, the others h_lo
     int h_lo;                       // multiple of 16, <= 256
     int32_t* status;
-    unsigned long long* row_key;    // kEpiArgmax: [M] keys (value, ~column), raised by atomicMax; cleared by the caller
+    KeySets sets;                   // kEpiArgmax: keys (value, ~column) of the rows, raised by atomicMax
     float* c;                       // kEpiStore: fp32 [M, ldc]
     long long ldc;
 };
@@ -337,6 +337,13 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
         const int my_row = (int)rank * a_half + (warp & 3) * 32 + lane;
         const bool warp_has_rows = (warp & 3) * 32 < a_half, row_on_lane = (warp & 3) * 32 + lane < a_half;
         const bool c_aligned = (reinterpret_cast<uintptr_t>(p.c) & 15) == 0 && (p.ldc & 3) == 0;
+        // this call's set of keys (the dependency wait lies before: the walk before this call has moved the number on)
+        unsigned long long* row_key = nullptr;
+        if (kEpi == kEpiArgmax) {
+            const uint32_t call = __ldcg(p.sets.call);
+            row_key = p.sets.keys + (size_t)(call & 1u) * p.sets.stride;
+            if (blockIdx.x == 0 && tid == 128) p.sets.call[1] = call;
+        }
         float best[kGroups];
         uint32_t who[kGroups];
 #pragma unroll
@@ -413,11 +420,11 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
 #pragma unroll
             for (int g = 0; g < kGroups; ++g)
                 if (row_on_lane && g * p.group_rows + my_row < p.M && who[g] != kNobody)
-                    atomicMax(p.row_key + g * p.group_rows + my_row, argmax_key(best[g], who[g]));
+                    atomicMax(row_key + g * p.group_rows + my_row, argmax_key(best[g], who[g]));
         } else if (kEpi == kEpiArgmax) {
             asm volatile("bar.sync 1, 128;" ::: "memory");              // the four epilogue warps
             for (int i = tid - 128; i < p.M; i += 128)
-                if (aux->best[i]) atomicMax(p.row_key + i, aux->best[i]);
+                if (aux->best[i]) atomicMax(row_key + i, aux->best[i]);
         }
     }
 

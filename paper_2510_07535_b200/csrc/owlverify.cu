@@ -36,8 +36,7 @@ struct owl_ctx {
     long long* sched_seq_begin = nullptr;
     SchedHeader* sched_header = nullptr;
     unsigned long long* part_keys = nullptr;
-    unsigned long long* lm_keys = nullptr;      // two sets of one arg-max key per row for the LM-head product's epilogue
-    uint32_t lm_epoch = 0;                      // calls launched so far: set (lm_epoch & 1) is in use, the other one clean
+    unsigned long long* lm_keys = nullptr;      // KeySets: two sets of one arg-max key per row, then the call numbers
     long long part_keys_len = 0;
     // tensor maps over the callers' K and V caches: a few most recently used (cache pointers, geometry) pairs
     // are kept, so that a caller rotating over several caches does not pay two encodes per call
@@ -178,14 +177,14 @@ __global__ void selftest_wait_kernel(int32_t* status, unsigned long long limit_n
 
 // C[M, N] = A[M, K] B[N, K]^T on the tensor cores with one of the two epilogues (gemm_umma.cuh).
 template <int kEpi>
-int launch_gemm(owl_ctx* ctx, const void* a, const void* b, int M, int N, int K, unsigned long long* row_key, float* c,
-                long long ldc, cudaStream_t stream) {
+int launch_gemm(owl_ctx* ctx, const void* a, const void* b, int M, int N, int K, const KeySets& sets, float* c, long long ldc,
+                cudaStream_t stream) {
     using namespace gemm_path;
     const int groups = column_groups(M), pairs = product_pairs(N, ctx->sm_count);
     GemmParams g = product_plan(M, N, K, pairs);
     const int h_hi = g.h_lo + (g.tall_rounds ? 16 : 0);
     g.status = ctx->status;
-    g.row_key = row_key; g.c = c; g.ldc = ldc;
+    g.sets = sets; g.c = c; g.ldc = ldc;
     CUtensorMap amap, bmap_hi, bmap_lo;
     const int ra = make_operand_map(ctx->encode, &amap, a, M, K, g.group_rows / 2);
     int rb = make_operand_map(ctx->encode, &bmap_lo, b, N, K, g.h_lo / 2);
@@ -269,8 +268,9 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         ctx->part_keys_len = (long long)max_dims->total_nodes * ((max_dims->vocab + kArgmaxChunk - 1) / kArgmaxChunk) *
                              (kArgmaxChunk / kArgmaxMinChunk);
         alloc((void**)&ctx->part_keys, (size_t)ctx->part_keys_len * sizeof(unsigned long long));
-        alloc((void**)&ctx->lm_keys, 2 * (size_t)max_dims->total_nodes * sizeof(unsigned long long));
-        if (ok) ok = cudaMemset(ctx->lm_keys, 0, 2 * (size_t)max_dims->total_nodes * sizeof(unsigned long long)) == cudaSuccess;
+        const size_t lm_bytes = (2 * (size_t)max_dims->total_nodes + 1) * sizeof(unsigned long long);
+        alloc((void**)&ctx->lm_keys, lm_bytes);
+        if (ok) ok = cudaMemset(ctx->lm_keys, 0, lm_bytes) == cudaSuccess;
     }
     if (ok) {
         ok = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess &&
@@ -506,7 +506,7 @@ static void launch_scan(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool
 static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream) {
     if (ctx->profiling) cudaEventRecord(ctx->ev[3], stream);
     launch_scan(ctx, p, stream, false);
-    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, static_cast<unsigned long long*>(nullptr), 0);
+    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, KeySets{});
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[4], stream); ctx->ev_accept_valid = true; }
 }
@@ -653,28 +653,21 @@ int owl_lm_head_accept(owl_ctx* ctx, const owl_dims* d, int32_t hidden_dim, cons
     if (!ctx->lm_keys || d->batch > ctx->max_dims.batch || d->total_nodes > ctx->max_dims.total_nodes) return OWL_ERR_TOO_LARGE;
     DeviceGuard guard(ctx->device);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    // The keys only ever grow (atomicMax) and must start from 0, below every real key.  Two sets alternate between
-    // calls: this call's set was cleared, as a whole, by the walk kernel of the call before it (by owl_create for the
-    // first two), and this call's walk kernel clears the other one - no memset in front of the product, which can
-    // then queue up behind whatever kernel precedes it.  The call number moves on only once both kernels are launched.
-    unsigned long long* keys = ctx->lm_keys + (size_t)(ctx->lm_epoch & 1u) * ctx->max_dims.total_nodes;
-    unsigned long long* idle_keys = ctx->lm_keys + (size_t)((ctx->lm_epoch + 1u) & 1u) * ctx->max_dims.total_nodes;
-    rc = launch_gemm<gemm_path::kEpiArgmax>(ctx, hidden, weight, d->total_nodes, d->vocab, hidden_dim, keys, nullptr, 0, stream);
+    const int32_t stride = ctx->max_dims.total_nodes;
+    const KeySets sets{ctx->lm_keys, reinterpret_cast<uint32_t*>(ctx->lm_keys + 2 * (size_t)stride), stride};
+    rc = launch_gemm<gemm_path::kEpiArgmax>(ctx, hidden, weight, d->total_nodes, d->vocab, hidden_dim, sets, nullptr, 0, stream);
     if (rc != OWL_OK) return rc;
     AcceptParams p{};
     p.draft_tokens = draft_tokens; p.node_offsets = node_offsets; p.tree_parent = tree_parent;
     p.accept_len = accept_len; p.accept_path = accept_path; p.bonus_token = bonus_token; p.node_argmax = node_argmax;
-    p.part_keys = keys;
     p.chunks = 1;
     p.status = ctx->status;
     p.batch = d->batch; p.total_nodes = d->total_nodes; p.nodes_uniform = d->total_nodes / d->batch;
     p.max_nodes = d->max_nodes; p.vocab = d->vocab; p.path_stride = d->path_stride;
-    launch_dependent(accept_walk_kernel, dim3((unsigned)d->batch), dim3(kArgmaxThreads), stream, p, idle_keys,
-                     ctx->max_dims.total_nodes);
+    launch_dependent(accept_walk_kernel, dim3((unsigned)d->batch), dim3(kArgmaxThreads), stream, p, sets);
     ++ctx->launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_lm_head_accept launch");
-    ++ctx->lm_epoch;
     return OWL_OK;
 }
 
@@ -694,7 +687,7 @@ int owl_lstm_cell(owl_ctx* ctx, int32_t rows, int32_t d_in, int32_t d, const voi
         return OWL_ERR_UNSUPPORTED;
     DeviceGuard guard(ctx->device);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    int rc = launch_gemm<gemm_path::kEpiStore>(ctx, h, w, rows, 4 * d, d_in, nullptr, workspace, 4ll * d, stream);
+    int rc = launch_gemm<gemm_path::kEpiStore>(ctx, h, w, rows, 4 * d, d_in, KeySets{}, workspace, 4ll * d, stream);
     if (rc != OWL_OK) return rc;
     CellParams c{};
     c.s = workspace; c.emb = static_cast<const __nv_bfloat16*>(emb);
@@ -921,7 +914,7 @@ extern "C" int owl_tree_accept_static(const owl_dims* d, const float* logits, co
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) { cudaGetLastError(); return OWL_ERR_CUDA; }
     argmax_partial_kernel<<<argmax_grid((long long)chunks * d->total_nodes, sms), kArgmaxThreads, 0, stream>>>(p);
-    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, static_cast<unsigned long long*>(nullptr), 0);
+    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, KeySets{});
     if (cudaGetLastError() != cudaSuccess) return OWL_ERR_CUDA;
     return OWL_OK;
 }

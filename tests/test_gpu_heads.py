@@ -157,6 +157,43 @@ def test_lm_head_accept_calls_of_different_sizes_on_one_context():
     ctx.close()
 
 
+@pytest.mark.parametrize("captured", [1, 2, 3])
+def test_lm_head_accept_replayed_from_a_graph_on_new_inputs(captured):
+    """A graph of one, two or three calls, replayed on hidden states that shrink from replay to replay (whatever is left of
+    an earlier replay's arg-max keys would win), between calls made directly on the same context."""
+    N, K, V = 12, 128, 3000
+    d = make_dims(batch=2, total_nodes=N, max_nodes=6, vocab=V)
+    ctx = OwlContext(d)
+    par, tok = dev_i32(np.tile(W.chain_parents(6), 2)), torch.zeros(N, dtype=torch.int32, device=DEV)
+    g = torch.Generator(device=DEV).manual_seed(7)
+    weight = torch.randn(V, K, generator=g, device=DEV, dtype=torch.bfloat16)
+    fresh = [torch.randn(N, K, generator=g, device=DEV).mul_(4.0 ** -r).to(torch.bfloat16) for r in range(8)]
+    hidden = fresh[0].clone()
+    outs = [[torch.zeros(2, dtype=torch.int32, device=DEV), torch.zeros(2, 64, dtype=torch.int32, device=DEV),
+             torch.zeros(2, dtype=torch.int32, device=DEV), torch.zeros(N, dtype=torch.int32, device=DEV)] for _ in range(captured)]
+    call = lambda o: ctx.owl_lm_head_accept(d, hidden, weight, tok, None, par, *o)
+    call(outs[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for o in outs:
+            call(o)
+    for r, h in enumerate(fresh):
+        hidden.copy_(h)
+        want = torch.argmax(h.double() @ weight.double().t(), dim=1).int()
+        for o in outs:
+            o[3].fill_(-1)
+        graph.replay()
+        assert all(torch.equal(o[3], want) for o in outs), r
+        if r % 3 == 1:
+            outs[0][3].fill_(-1)
+            call(outs[0])
+            assert torch.equal(outs[0][3], want), r
+    assert ctx.owl_get_status() == 0
+    del graph
+    ctx.close()
+
+
 def test_lm_head_accept_full_vocabulary():
     """The 8B shape's head: hidden 4096, vocabulary 128256 (1002 column tiles over 148 CTAs), a 32-node tree."""
     ctx = OwlContext(make_dims(batch=1, total_nodes=32, max_nodes=32, vocab=W.VOCAB))

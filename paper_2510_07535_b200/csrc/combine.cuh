@@ -135,7 +135,6 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
         if (!small || row_id != first) locate(row_id);
         if (tiles == 0) continue;
         if (c0 == c1) continue;  // a single CTA saw every key of this unit and wrote the result itself
-        const int bad_epoch = __ldcg(p.seq_bad + b);   // (its round trip overlaps the partial loads below)
         const int count = c1 - c0 + 1;
 
         // Partials are taken `group` at a time: lane j (< group) owns partial base + j.  The row loads do
@@ -143,6 +142,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
         // online (running maximum).
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         float sum = 0.f, mx = -INFINITY;
+        bool bad = false;
         for (int base = 0; base < count; base += group) {
             const int mine = base + lane;
             const bool have = lane < group && mine < count;
@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(p.part_o + pj * kHeadDim + lane * 4) : "memory");
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
+            bad = __any_sync(0xffffffffu, __float_as_uint(my_lse) == kBadPartial) || bad;
             float gmx = my_lse;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, o));
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
         }
-        if (bad_epoch == p.epoch) continue;            // the pass found a bad tree or page in this sequence: no output
+        if (bad) continue;                             // the pass found a bad tree or page in this sequence: no output
         const float inv = sum > 0.f ? 1.f / sum : 0.f;
         uint2 pk;
         if (p.f16) {

@@ -20,6 +20,11 @@ constexpr int kErrTimeout = -6;
 
 struct SchedHeader;
 
+// In the place of a partial's LSE: the pass met a malformed tree or a page out of range, the row stays unwritten.  A NaN that
+// no arithmetic produces.  (It travels with the partial, so nothing is left over from one call for the next, and no call
+// number has to tell the calls apart - a call replayed from a graph would carry the same one every time.)
+constexpr uint32_t kBadPartial = 0x7fb0bad0u;
+
 // Problem description handed to every kernel of the attention path.
 struct AttnParams {
     const __nv_bfloat16* q;
@@ -32,12 +37,10 @@ struct AttnParams {
     __nv_bfloat16* out;
     float* lse;                   // may be null
     float* part_o;                // [slots, rows_per_slot, D] fp32, normalised partial outputs
-    float* part_lse;              // [slots, rows_per_slot] fp32, natural-log partial LSE (-inf if empty)
+    float* part_lse;              // [slots, rows_per_slot] fp32, natural-log partial LSE (-inf if empty; kBadPartial)
     int32_t* status;              // device status word (0 = ok, first error wins)
-    int32_t* seq_bad;             // [B] epoch of the call in which the sequence was found malformed
     long long* sched_seq_begin;   // [B + 1] first flat tile of every sequence (written by CTA 0 of the pass)
     SchedHeader* sched_header;
-    int32_t epoch;
     int32_t batch, total_nodes, nodes_uniform, max_nodes;
     int32_t num_q_heads, num_kv_heads, group;  // group = Hq / Hkv
     int32_t page_size, page_shift, max_pages_per_seq, num_pages;

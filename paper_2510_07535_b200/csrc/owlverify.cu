@@ -32,7 +32,6 @@ struct owl_ctx {
     float* part_lse = nullptr;
     int32_t* status = nullptr;
     unsigned long long* selftest_ns = nullptr;
-    int32_t* seq_bad = nullptr;
     long long* sched_seq_begin = nullptr;
     SchedHeader* sched_header = nullptr;
     unsigned long long* part_keys = nullptr;
@@ -50,7 +49,6 @@ struct owl_ctx {
         uint64_t used = 0;
     } maps[kMapCacheEntries];
     uint64_t map_clock = 0;
-    int32_t epoch = 0;
     int64_t launches = 0;
     bool profiling = false;
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -260,7 +258,6 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     }
     alloc((void**)&ctx->status, sizeof(int32_t));
     alloc((void**)&ctx->selftest_ns, 2 * sizeof(unsigned long long));
-    alloc((void**)&ctx->seq_bad, (size_t)max_dims->batch * sizeof(int32_t));
     alloc((void**)&ctx->sched_seq_begin, ((size_t)max_dims->batch + 1) * sizeof(long long));
     alloc((void**)&ctx->sched_header, sizeof(SchedHeader));
     if (acc) {
@@ -273,8 +270,7 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         if (ok) ok = cudaMemset(ctx->lm_keys, 0, lm_bytes) == cudaSuccess;
     }
     if (ok) {
-        ok = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess &&
-             cudaMemset(ctx->seq_bad, 0, (size_t)max_dims->batch * sizeof(int32_t)) == cudaSuccess;
+        ok = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess;
     }
     for (int i = 0; ok && i < 6; ++i) ok = cudaEventCreate(&ctx->ev[i]) == cudaSuccess;
     if (ok && attn) {
@@ -311,7 +307,6 @@ int owl_destroy(owl_ctx* ctx) {
     cudaFree(ctx->part_lse);
     cudaFree(ctx->status);
     cudaFree(ctx->selftest_ns);
-    cudaFree(ctx->seq_bad);
     cudaFree(ctx->sched_seq_begin);
     cudaFree(ctx->sched_header);
     cudaFree(ctx->part_keys);
@@ -359,10 +354,8 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     p.part_o = ctx->part_o;
     p.part_lse = ctx->part_lse;
     p.status = ctx->status;
-    p.seq_bad = ctx->seq_bad;
     p.sched_seq_begin = ctx->sched_seq_begin;
     p.sched_header = ctx->sched_header;
-    p.epoch = ++ctx->epoch;
     p.batch = d->batch;
     p.total_nodes = d->total_nodes;
     p.nodes_uniform = d->total_nodes / d->batch;

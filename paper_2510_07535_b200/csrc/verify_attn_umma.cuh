@@ -177,7 +177,6 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
             tmin = min(tmin, tiles); tmax = max(tmax, tiles);
         } else {
             report(p.status, seq_tree_shape_ok(p, b, n) ? kErrBadPage : kErrBadTree);
-            p.seq_bad[b] = p.epoch;
         }
     }
     long long inc_t = my_tiles;
@@ -246,7 +245,6 @@ __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w)
     const int n = ws.n, L = ws.L, node_base = ws.node_base, tiles = ws.tiles;
     if (lane < p.batch && !ws.ok) {
         report(p.status, seq_tree_shape_ok(p, lane, n) ? kErrBadPage : kErrBadTree);
-        p.seq_bad[lane] = p.epoch;
     }
     Partition part;
     part.init(ws.total, gridDim.x, ws.units, ws.uniform_tiles);
@@ -345,7 +343,6 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
                 if ((unsigned)pg < (unsigned)p.num_pages) c = pg * p.num_kv_heads + g.h;
                 else {
                     report(p.status, kErrBadPage);
-                    p.seq_bad[g.b] = p.epoch;                 // for the merge
                     const_cast<volatile int&>(announced.bad_page) = 1;
                 }
             }
@@ -628,7 +625,6 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
                 if (bad) {
                     atomicExch(&aux->seg_bad_tree, 1);
                     report(p.status, kErrBadTree);
-                    p.seq_bad[g.b] = p.epoch;
                 }
                 aux->parent[wtid] = bad ? (short)-1 : (short)parent_i;
             }
@@ -873,8 +869,8 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         float (*ml)[128][3] = reinterpret_cast<float (*)[128][3]>(smem + kQBytes);
         if (!g.shared) { ml[s][row_local][0] = m; ml[s][row_local][1] = l; ml[s][row_local][2] = lx; }
         meet_before_segment(aux, seg_no + 1, leader);    // both streams done: all MMAs of the segment have completed
-        // (looking up seq_bad in global memory here stood between a unit's last product and its stores)
-        const bool write_ok = !bad_tree && !*abort_flag && !const_cast<volatile int&>(aux->seg[seg_no % kSegs].bad_page);
+        const bool bad = bad_tree || const_cast<volatile int&>(aux->seg[seg_no % kSegs].bad_page);
+        const bool write_ok = !bad && !*abort_flag;
         // only the first and the last unit of a CTA's piece can be cut: two partial slots per CTA
         const long long part_row = (2ll * blockIdx.x + (seg_no > 0 ? 1 : 0)) * p.rows_per_slot + rr;
         const long long out_row = rr < g.M ? (long long)(g.node_base + rr / G) * p.num_q_heads + g.h * G + rr % G : 0;
@@ -929,6 +925,8 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         if (row_ok && write_lse) {
             if (whole) { if (p.lse) p.lse[out_row] = lse; }
             else p.part_lse[part_row] = lse;
+        } else if (bad && write_lse && !whole && rr < g.M) {
+            p.part_lse[part_row] = __uint_as_float(kBadPartial);      // the merge leaves the row alone
         }
         tc_fence_before();
         tile_base += (uint32_t)(g.tile1 - g.tile0);

@@ -211,3 +211,33 @@ def test_inconsistent_node_offsets_are_reported_and_leave_no_trace():
             assert ctx.owl_get_status() == 0
             _accept_equals_oracle(dw, wl)
     ctx.close()
+
+
+@pytest.mark.parametrize("fault", ["page", "tree"])
+def test_a_graph_replayed_after_a_malformed_batch_writes_again(fault):
+    """One replay on a batch whose sequence 1 has a page out of range, or a malformed tree, leaves that sequence's outputs
+    alone; the next replay, on the mended batch, writes all of them.  (Long contexts, so that units are cut and merged.)"""
+    wl = W.generate(W.Spec("replay", 8, 2, [5000, 7000], [("tree", 8, 3), ("chain", 4)], shuffle_pages=True, seed=8, with_logits=False))
+    dw = DeviceWorkload.upload(wl)
+    ctx = OwlContext(dims_of(wl))
+    dw.attn(ctx)
+    want, want_lse = dw.out.clone(), dw.lse.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dw.attn(ctx)
+    t, at, bad = (dw.block_table.view(-1), int(dw.block_table.shape[1]) + 200, 10 ** 6) if fault == "page" else \
+                 (dw.tree_parent, int(wl.node_offsets[1]) + 1, 3)
+    good, first = int(t[at]), int(wl.node_offsets[1])
+    t[at] = bad
+    dw.out.fill_(7.0)
+    dw.lse.fill_(7.0)
+    graph.replay()
+    assert ctx.owl_get_status() == (-5 if fault == "page" else -4)
+    assert torch.equal(dw.out[:first], want[:first]) and torch.equal(dw.lse[:first], want_lse[:first])
+    assert bool((dw.out[first:] == 7).all()) and bool((dw.lse[first:] == 7).all())
+    t[at] = good
+    graph.replay()
+    assert ctx.owl_get_status() == 0
+    assert torch.equal(dw.out, want) and torch.equal(dw.lse, want_lse)
+    del graph
+    ctx.close()

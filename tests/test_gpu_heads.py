@@ -83,19 +83,19 @@ def _lm_head_case(ctx, seed, trees, K, V, plant=0.7):
 
 
 @pytest.mark.parametrize("trees,K,V", [
-    ([("chain", 8)], 128, 1000),                                    # one row block, ragged last vocabulary tile
-    ([("tree", 20, 4), ("chain", 3)], 64, 129),                     # a single k-block; a tile of one column
-    ([("tree", 64, 8)] * 3 + [("chain", 8)], 256, 5000),            # 200 rows: two row blocks, double-buffered accumulators
-    ([("tree", 64, 8)] * 5, 512, 3000),                             # 320 rows: three row blocks, one accumulator buffer
-    ([("tree", 32, 6)], 4096, 20000),                               # the real hidden width: 64 k-blocks per tile
-    ([("tree", 64, 8)] * 3, 64, 40000),                             # two row blocks, two rounds of tiles (144 + 128 columns)
-    ([("tree", 64, 8)] * 5, 64, 20000),                             # three row blocks, two rounds (80 + 64 columns)
-    ([("chain", 5)], 64, 16),                                       # the whole vocabulary is one 16-column tile on one CTA
-    ([("tree", 64, 8)] * 2 + [("chain", 2)], 128, 16),              # 130 rows on a CTA pair: one stage per tile, one 16-column tile
-    ([("tree", 64, 8)] * 4, 128, 1000),                             # 256 rows on CTA pairs: 63 pairs with a 16-column tile each
-    ([("tree", 40, 6)] * 4, 384, 40000),                            # 160 rows on 74 pairs: two rounds (144 + 128 columns), three stages per tile
-    ([("tree", 64, 8)] * 6, 128, 40000),                            # 384 rows: three row blocks, K a multiple of 128
-    ([("tree", 64, 8)] * 4 + [("chain", 1)], 256, 2000),            # 257 rows: one row in the third row block
+    ([("chain", 8)], 128, 1000),                                    # 8 rows, tiles of 16 weight rows, the last one ragged
+    ([("tree", 20, 4), ("chain", 3)], 64, 129),                     # a single k-block; a tile of one weight row
+    ([("tree", 64, 8)] * 3 + [("chain", 8)], 256, 5000),            # 200 rows on the lanes, one tile of 80 weight rows
+    ([("tree", 64, 8)] * 5, 512, 3000),                             # 320 rows in two groups on the lanes, tiles of 48
+    ([("tree", 32, 6)], 4096, 20000),                               # the real hidden width: 64 k-blocks, two rounds (144 + 128)
+    ([("tree", 64, 8)] * 3, 64, 40000),                             # 192 rows on the lanes, three rounds (192 + 2 x 176), half of each stage past K
+    ([("tree", 64, 8)] * 5, 64, 20000),                             # 320 rows in two groups, two rounds (144 + 128), one accumulator buffer
+    ([("chain", 5)], 64, 16),                                       # the whole vocabulary is one tile of 16 on one CTA pair
+    ([("tree", 64, 8)] * 2 + [("chain", 2)], 128, 16),              # 130 rows on the lanes of one CTA pair: one stage, one tile of 16
+    ([("tree", 64, 8)] * 4, 128, 1000),                             # 256 rows on the lanes: 63 pairs with a tile of 16 each
+    ([("tree", 40, 6)] * 4, 384, 40000),                            # 160 rows, weights on the lanes: three rounds (192 + 2 x 176), three stages per tile
+    ([("tree", 64, 8)] * 6, 128, 40000),                            # 384 rows in two groups on the lanes, three rounds, two stages per tile
+    ([("tree", 64, 8)] * 4 + [("chain", 1)], 256, 2000),            # 257 rows: two groups of 144
 ])
 def test_lm_head_accept_small(trees, K, V):
     ctx = OwlContext(make_dims(batch=8, total_nodes=384, max_nodes=64, vocab=V))
@@ -195,15 +195,15 @@ def test_lm_head_accept_replayed_from_a_graph_on_new_inputs(captured):
 
 
 def test_lm_head_accept_full_vocabulary():
-    """The 8B shape's head: hidden 4096, vocabulary 128256 (1002 column tiles over 148 CTAs), a 32-node tree."""
+    """The 8B shape's head: hidden 4096, vocabulary 128256 (7 rounds of tiles over 74 CTA pairs), a 32-node tree."""
     ctx = OwlContext(make_dims(batch=1, total_nodes=32, max_nodes=32, vocab=W.VOCAB))
     _lm_head_case(ctx, 77, [("tree", 32, 6)], 4096, W.VOCAB)
     ctx.close()
 
 
 def test_lm_head_accept_full_vocabulary_on_cta_pairs():
-    """Four 64-node trees (256 rows, two row blocks): the product runs on CTA pairs, seven rounds of 256- and 240-column
-    tiles over 74 pairs, both accumulator buffers in turn."""
+    """Four 64-node trees (256 rows, on the lanes): seven rounds of tiles of 256 and 240 weight rows over 74 CTA pairs, both
+    accumulator buffers in turn."""
     ctx = OwlContext(make_dims(batch=4, total_nodes=256, max_nodes=64, vocab=W.VOCAB))
     _lm_head_case(ctx, 78, [("tree", 64, 8)] * 4, 4096, W.VOCAB)
     ctx.close()
@@ -263,14 +263,14 @@ def _cell_case(ctx, seed, M, d_in, d, affine, steps=1, z_mean=0.0):
 
 @pytest.mark.parametrize("M,d_in,d,affine", [
     (1, 64, 64, False),
-    (5, 128, 260, True),            # d no multiple of the column tile: ragged last tile of the product
-    (130, 256, 512, True),          # two row blocks
-    (300, 64, 128, False),          # three row blocks
+    (5, 128, 260, True),            # 1040 weight rows: 65 pairs with a tile of 16 each
+    (130, 256, 512, True),          # rows on the lanes
+    (300, 64, 128, False),          # two groups of rows on the lanes
     (2, 64, 4, True),               # fewer columns than CTAs in a row's cluster: half of them hold none
-    (1, 64, 16384, True),           # the widest cell: four columns per thread, two rounds of product tiles
-    (256, 128, 4096, False),        # two full row blocks on CTA pairs, store epilogue, four rounds of 224 / 208 columns
-    (129, 384, 36, True),           # one row in the second row block; 144 columns in all
-    (300, 256, 512, True),          # three row blocks, store epilogue, K a multiple of 128
+    (1, 64, 16384, True),           # the widest cell: four columns per thread, four rounds of product tiles
+    (256, 128, 4096, False),        # all 128 lanes of both CTAs hold rows; a tile of 224
+    (129, 384, 36, True),           # rows on the lanes; 144 weight rows in all
+    (300, 256, 512, True),          # two groups of rows on the lanes, tiles of 32
 ])
 def test_lstm_cell_small(M, d_in, d, affine):
     ctx = OwlContext(make_dims(batch=1, total_nodes=1, max_nodes=1))

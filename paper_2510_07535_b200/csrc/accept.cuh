@@ -72,7 +72,7 @@ struct AcceptParams {
 // replayed from a graph has its host side behind it: the product reads call[0] and leaves what it read in call[1], the
 // walk goes by call[1] and moves call[0] on.  (Two words, because a walk's CTAs read the number while one of them moves it.)
 struct KeySets {
-    unsigned long long* keys;        // [2, stride]; null: the walk's keys are AcceptParams::part_keys
+    unsigned long long* keys;        // [2, stride]
     uint32_t* call;
     int32_t stride;
 };
@@ -293,22 +293,24 @@ __global__ void __launch_bounds__(kArgmaxThreads, kArgmaxCtasPerSm) argmax_parti
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// One sequence's acceptance walk per CTA over the keys the scan or the LM-head product (`sets`) left.  Launched as a
-// programmatic dependent: it reads nothing before the kernel before it has completed.
-__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_kernel(AcceptParams p, const KeySets sets) {
+// One sequence's acceptance walk per CTA over the keys the scan left.  Launched as a programmatic dependent: it reads
+// nothing before the kernel before it has completed.
+__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_kernel(const AcceptParams p) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    uint32_t call = 0u;
-    if (sets.keys) {
-        call = __ldcg(sets.call + 1);
-        p.part_keys = sets.keys + (size_t)(call & 1u) * sets.stride;
-    }
     accept_walk_seq(p, (int)blockIdx.x);
-    if (sets.keys) {
-        unsigned long long* idle = sets.keys + (size_t)((call + 1u) & 1u) * sets.stride;
-        for (int i = blockIdx.x * kArgmaxThreads + threadIdx.x; i < sets.stride; i += gridDim.x * kArgmaxThreads) idle[i] = 0ull;
-        if (blockIdx.x == 0 && threadIdx.x == 0) sets.call[0] = call + 1u;
-    }
+}
+// The same over the keys of the LM-head product (a kernel of its own, so that the short acceptances do not carry the choice
+// of the set).
+__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_sets_kernel(AcceptParams p, const KeySets sets) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t call = __ldcg(sets.call + 1);
+    p.part_keys = sets.keys + (size_t)(call & 1u) * sets.stride;
+    accept_walk_seq(p, (int)blockIdx.x);
+    unsigned long long* idle = sets.keys + (size_t)((call + 1u) & 1u) * sets.stride;
+    for (int i = blockIdx.x * kArgmaxThreads + threadIdx.x; i < sets.stride; i += gridDim.x * kArgmaxThreads) idle[i] = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0) sets.call[0] = call + 1u;
 }
 
 // Grid of the scan for `items` (row, chunk) items on a device with `sms` multiprocessors: as many warps as give

@@ -499,7 +499,7 @@ static void launch_scan(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream, bool
 static void launch_accept(owl_ctx* ctx, AcceptParams& p, cudaStream_t stream) {
     if (ctx->profiling) cudaEventRecord(ctx->ev[3], stream);
     launch_scan(ctx, p, stream, false);
-    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, KeySets{});
+    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p);
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[4], stream); ctx->ev_accept_valid = true; }
 }
@@ -657,7 +657,7 @@ int owl_lm_head_accept(owl_ctx* ctx, const owl_dims* d, int32_t hidden_dim, cons
     p.status = ctx->status;
     p.batch = d->batch; p.total_nodes = d->total_nodes; p.nodes_uniform = d->total_nodes / d->batch;
     p.max_nodes = d->max_nodes; p.vocab = d->vocab; p.path_stride = d->path_stride;
-    launch_dependent(accept_walk_kernel, dim3((unsigned)d->batch), dim3(kArgmaxThreads), stream, p, sets);
+    launch_dependent(accept_walk_sets_kernel, dim3((unsigned)d->batch), dim3(kArgmaxThreads), stream, p, sets);
     ++ctx->launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "owl_lm_head_accept launch");
@@ -907,7 +907,7 @@ extern "C" int owl_tree_accept_static(const owl_dims* d, const float* logits, co
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) { cudaGetLastError(); return OWL_ERR_CUDA; }
     argmax_partial_kernel<<<argmax_grid((long long)chunks * d->total_nodes, sms), kArgmaxThreads, 0, stream>>>(p);
-    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p, KeySets{});
+    launch_dependent(accept_walk_kernel, dim3((unsigned)p.batch), dim3(kArgmaxThreads), stream, p);
     if (cudaGetLastError() != cudaSuccess) return OWL_ERR_CUDA;
     return OWL_OK;
 }

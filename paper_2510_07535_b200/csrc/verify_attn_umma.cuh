@@ -299,11 +299,15 @@ __device__ __forceinline__ Segment announced_segment(Aux* aux, uint32_t seg_no) 
 }
 
 // ------------------------------------------------------------------------------------------ producer
+// One verdict for the producer warp, whose lanes must take the same way out.
 __device__ __forceinline__ bool readers_reached(Aux* aux, int seg_no) {
-    const uint64_t t0 = global_timer_ns();
-    while (const_cast<volatile int&>(aux->seg_reached) < seg_no)
-        if (global_timer_ns() - t0 > 10 * kWaitLimitNs) return false;
-    return true;
+    volatile int* reached = &aux->seg_reached;
+    bool ok = *reached >= seg_no;
+    if (!ok) {
+        const uint64_t t0 = global_timer_ns();
+        while (!(ok = *reached >= seg_no) && global_timer_ns() - t0 <= 10 * kWaitLimitNs) {}
+    }
+    return __all_sync(0xffffffffu, ok);
 }
 
 template <bool kWide>

@@ -1,6 +1,5 @@
 // LSE merge of the split-KV partials: for every output row whose keys were processed by more than
 // one CTA, out = sum_s exp(lse_s - lse) o_s with lse = ln sum_s exp(lse_s); rounded to bf16.
-// One warp per output row (packed node, query head); each lane owns 4 of the 128 output channels.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -12,6 +11,7 @@ namespace owl {
 
 constexpr int kCombineWarps = 8;
 constexpr int kCombineCtasPerSm = 4;
+constexpr int kCombineRows = 8;            // a unit's rows that a CTA merges at a time
 
 // Partials per round of the merge, for `units` units (sequence, KV head) cut by `ctas` CTAs: as many as a unit of
 // average length is cut into, plus one at either end, so that its rows take one memory round trip; longer units take
@@ -21,7 +21,7 @@ inline int combine_group(long long units, int ctas) {
     const long long g = (ctas + units - 1) / units + 2;
     return (int)(g < 4 ? 4 : g < 32 ? g : 32);
 }
-inline size_t combine_stage_bytes(int group) { return (size_t)kCombineWarps * group * 32 * sizeof(float4); }
+inline size_t combine_stage_bytes(int group) { return (size_t)kCombineWarps * group * 34 * sizeof(float4); }
 inline int combine_ctas_per_sm(int group) {
     const int fit = (int)((227u << 10) / (combine_stage_bytes(group) + 1024));
     return fit < kCombineCtasPerSm ? fit : kCombineCtasPerSm;
@@ -35,30 +35,32 @@ inline size_t combine_smem_bytes(int group, unsigned ctas, int sms) {
     return stage > spread ? stage : spread;
 }
 
-// One warp per output row finds the CTAs whose pieces cut the row's unit
-// and merges their partials in CTA order.  A CTA stores at most two partials: slot 2c if its piece starts inside
-// the unit, else 2c + 1.
+// A block of eight of a unit's packed rows per CTA and turn, 16 of the 128 channels per warp: lane = (row, four
+// channels).  The warp finds the CTAs whose pieces cut the unit and merges their partials in CTA order.  A CTA stores at
+// most two partials: slot 2c if its piece starts inside the unit, else 2c + 1.
+//
+// Partials lie as the attention kernel's lanes, one row each, can store them straight from registers in whole lines:
+// [slot][32 groups of four channels][256 rows][4].  Eight neighbouring rows are then a line of 128 bytes here too.
+// (With the rows of a partial one after the other the pass had to turn every 32 x 32 piece over in shared memory: its
+// epilogue took 1.9 us instead of 1.0 at 2K context, 3.5 instead of 3.0 for 240 rows at 47K.)
 //
 // The kernel is launched as a programmatic dependent of that pass and its time after the pass has ended is pure
 // latency, so everything that needs no output of the pass comes before the wait: for batches of at most 32
 // sequences the warp derives the schedule from the inputs exactly as the pass did (warp_schedule) and knows its
-// row's partial slots when the wait returns; what is left is one round of loads.  Larger batches read the
+// block's partial slots when the wait returns; what is left is one round of loads.  Larger batches read the
 // schedule the pass left in global memory (first flat tile of every sequence, totals, choice of partition).
 //
 // kFused (verify step): the grid has one more CTA per sequence after the row CTAs; each of those runs one
 // sequence's acceptance walk over the arg-max keys that the pass's spare warps left (`ap`).
 //
 // p.combine_group: partials fetched per round, at most 32 (combine_group above).  A round's rows go through a
-// warp-private stage in shared memory of that many rows, which is what limits the CTAs per SM.
+// warp-private stage in shared memory of that many pieces, which is what limits the CTAs per SM.
 //
 // The stage is there for the sake of the code's length, not of the data: with the rows in registers the fetch and
 // the fold were two loops unrolled 32 times, some 450 instructions that a warp with one row executes exactly once,
-// at the pace of instruction fetches from L2.  Copied with cp.async in a short rolled loop and folded in another,
-// the same work is two dozen instructions executed from the instruction cache after their first trip (attention +
-// merge call at 32K context 37.5 -> 36.8 us, with 8192 output rows 586 -> 578 us).
+// at the pace of instruction fetches from L2.
 template <bool kFused>
 __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine_sched_kernel(const AttnParams p, const AcceptParams ap) {
-    const long long rows = (long long)p.total_nodes * p.num_q_heads;
     const unsigned row_ctas = (unsigned)p.combine_row_ctas;
     if (kFused) {
         if (blockIdx.x >= row_ctas) {
@@ -69,13 +71,19 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             return;
         }
     }
-    // The row CTAs are persistent: a warp derives the schedule once and then takes rows first, first + stride, ...
-    // (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived 8192 times).
+    // The row CTAs are persistent: a warp derives the schedule once and then takes blocks first, first + row_ctas, ...
+    // (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived 8192 times).  Blocks are
+    // numbered unit by unit for the first eight rows of all units, then for the second eight and so on, up to the rows of
+    // the most nodes a sequence may have: what shorter sequences lack lies at the end.
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    extern __shared__ float4 combine_stage[];          // [warps][group][32]: a round's partial rows, warp-private
+    const int r = lane & 7, chunk = warp * 4 + (lane >> 3);      // row of the block; group of four channels
+    extern __shared__ float4 combine_stage[];          // per warp: [group][32] pieces of the partials, [group][8] LSEs
     const int group = p.combine_group;
-    float4* stage = combine_stage + warp * group * 32;
-    const long long first = (long long)blockIdx.x * kCombineWarps + warp, stride = (long long)row_ctas * kCombineWarps;
+    float4* stage = combine_stage + warp * group * 34;
+    float* lse_stage = reinterpret_cast<float*>(stage + group * 32);
+    const uint32_t stage_u32 = (uint32_t)__cvta_generic_to_shared(stage + lane);
+    const unsigned units = (unsigned)(p.batch * p.num_kv_heads);
+    const unsigned blocks = units * (unsigned)((p.group * p.max_nodes + kCombineRows - 1) / kCombineRows);
     const bool small = p.batch <= 32;
     WarpSchedule ws{};
     Partition part;
@@ -83,47 +91,39 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
         ws = warp_schedule(p);
         part.init(ws.total, p.num_ctas, ws.units, ws.uniform_tiles);
     }
-    // per row: its sequence, the CTAs c0..c1 whose pieces cut the row's unit, and the slot row of the partial this
-    // lane fetches first
-    int n = 0, hq = 0, b = 0, node_base = 0, tiles = 0, lrow = 0, c0 = 0, c1 = 0;
-    long long seq_begin = 0, t0 = 0, prow_first = 0;
-    auto row_of = [&](int c) -> long long { return (2ll * c + (part.begin(c) < t0 ? 1 : 0)) * p.rows_per_slot + lrow; };
-    auto plan = [&]() {
-        if (tiles == 0) return;
-        const int G = p.group;
-        lrow = (n - node_base) * G + hq % G;
-        t0 = seq_begin + (long long)(hq / G) * (tiles + part.pen);
-        c0 = part.owner(t0 + part.pen);
-        c1 = part.owner(t0 + part.pen + tiles - 1);
-        prow_first = row_of(c0 + min(lane, c1 - c0));
-    };
-    auto locate = [&](long long row_id) {       // every lane of the warp, same row
-        n = (int)(row_id / p.num_q_heads);
-        hq = (int)(row_id - (long long)n * p.num_q_heads);
+    // per block: its unit's row count, the first partial's slot and the number of partials (0: nothing to merge)
+    int M = 0, h = 0, row = 0, node_base = 0, slot = 0, count = 0;
+    auto locate = [&](unsigned id) {       // every lane of the warp, same block
+        const unsigned k = id / units, u = id - k * units, b = u / (unsigned)p.num_kv_heads;
+        h = (int)(u - b * (unsigned)p.num_kv_heads);
+        row = (int)k * kCombineRows + r;
+        int n, tiles;
+        long long seq_begin;
         if (small) {
-            const unsigned hit = __ballot_sync(0xffffffffu, lane < p.batch && ws.tiles > 0 && n >= ws.node_base && n < ws.node_base + ws.n);
-            b = hit ? __ffs(hit) - 1 : 0;
+            n = __shfl_sync(0xffffffffu, ws.n, b);
             node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
-            tiles = hit ? __shfl_sync(0xffffffffu, ws.tiles, b) : 0;
+            tiles = __shfl_sync(0xffffffffu, ws.tiles, b);
             seq_begin = __shfl_sync(0xffffffffu, ws.excl_t + (long long)part.pen * ws.excl_u, b);
         } else {
-            int lo = 0, hi = p.batch;  // largest b with node_offsets[b] <= n
-            if (p.node_offsets) {
-                while (hi - lo > 1) { int mid = (lo + hi) >> 1; if (p.node_offsets[mid] <= n) lo = mid; else hi = mid; }
-                b = lo;
-            } else {
-                b = n / p.nodes_uniform;
-            }
             const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
-            node_base = seq_node_base(p, b);
+            n = seq_nodes(p, (int)b);
+            node_base = seq_node_base(p, (int)b);
             seq_begin = sb;
             tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
         }
-        plan();
+        count = 0;
+        M = n * p.group;
+        if (tiles == 0 || (int)k * kCombineRows >= M) return;      // not scheduled, or no such rows
+        const long long t0 = seq_begin + (long long)h * (tiles + part.pen);
+        const int c0 = part.owner(t0 + part.pen), c1 = part.owner(t0 + part.pen + tiles - 1);
+        if (c0 == c1) return;              // a single CTA saw every key of this unit and wrote the result itself
+        // the unit's first CTA may have come from another unit; the others' pieces start in this one
+        slot = 2 * c0 + (part.begin(c0) < t0 ? 1 : 0);
+        count = c1 - c0 + 1;
     };
     // latency after the pass has ended is what this kernel costs: whatever needs no output of the pass comes before
-    // the wait - for batches of at most 32 sequences the whole plan of the warp's first row
-    if (small && first < rows) locate(first);
+    // the wait - for batches of at most 32 sequences the whole plan of the first block
+    if (small) locate(blockIdx.x);
     // from here on the split-KV pass has completed and its writes are visible (a no-op in an ordinary launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel in the stream may queue up
@@ -131,56 +131,66 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
         const SchedHeader hdr = *p.sched_header;      // larger batches read the schedule the pass left
         part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
     }
-    for (long long row_id = first; row_id < rows; row_id += stride) {
-        if (!small || row_id != first) locate(row_id);
-        if (tiles == 0) continue;
-        if (c0 == c1) continue;  // a single CTA saw every key of this unit and wrote the result itself
-        const int count = c1 - c0 + 1;
-
-        // Partials are taken `group` at a time: lane j (< group) owns partial base + j.  The row loads do
-        // not depend on the LSE values, so both go out together: one memory round trip per group.  Groups are folded
-        // online (running maximum).
+    for (unsigned id = blockIdx.x; id < blocks; id += row_ctas) {
+        if (!small || id != blockIdx.x) locate(id);
+        if (count == 0) continue;
+        // Partials are taken `group` at a time, their LSEs with them: one memory round trip per group.  Groups are folded
+        // online (running maximum, each lane its own row's).
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         float sum = 0.f, mx = -INFINITY;
         bool bad = false;
+        // slots of neighbouring CTAs lie two apart; only the first CTA's partial may be its second
+        const float4* src = reinterpret_cast<const float4*>(p.part_o) + (slot * 32ll + chunk) * kMaxRows + row;
+        const float4* next = src + (slot & 1 ? 32 : 64) * kMaxRows;
         for (int base = 0; base < count; base += group) {
-            const int mine = base + lane;
-            const bool have = lane < group && mine < count;
-            const long long prow = base == 0 ? prow_first : row_of(c0 + (have ? mine : 0));
-            const float my_lse = have ? __ldcg(p.part_lse + prow) : -INFINITY;
             const int cnt = count - base < group ? count - base : group;
-            if (base > 0) __syncwarp();                  // the stage's rows of the round before have been folded
-#pragma unroll 1
-            for (int j = 0; j < cnt; ++j) {
-                const long long pj = __shfl_sync(0xffffffffu, prow, j);
-                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage + j * 32 + lane);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(p.part_o + pj * kHeadDim + lane * 4) : "memory");
+            if (base > 0) __syncwarp();                  // the stage's weights of the round before have been read
+            for (int j = lane; j < 2 * cnt; j += 32) {   // eight rows' LSEs: two pieces of 16 bytes
+                const int at = base + (j >> 1), sl = at == 0 ? slot : (slot & ~1) + 2 * at;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(lse_stage + j * 4)),
+                             "l"(p.part_lse + (long long)sl * kMaxRows + (row - r) + (j & 1) * 4) : "memory");
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
-            bad = __any_sync(0xffffffffu, __float_as_uint(my_lse) == kBadPartial) || bad;
-            float gmx = my_lse;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, o));
-            const float mx_new = fmaxf(mx, gmx);
-            if (mx_new > -INFINITY) {
-                const float rescale = mx > -INFINITY ? __expf(mx - mx_new) : 0.f;
-                acc.x *= rescale; acc.y *= rescale; acc.z *= rescale; acc.w *= rescale;
-                sum *= rescale;
-                const float w = have ? __expf(my_lse - mx_new) : 0.f;     // -inf partial: weight 0
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll 1
-                for (int j = 0; j < cnt; ++j) {
-                    const float wj = __shfl_sync(0xffffffffu, w, j);
-                    const float4 v = stage[j * 32 + lane];                 // this lane's own copy: no barrier needed
-                    acc.x += wj * v.x; acc.y += wj * v.y; acc.z += wj * v.z; acc.w += wj * v.w;
-                    sum += wj;
-                }
-                mx = mx_new;
-            } else {
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll 4
+            for (int j = 0; j < cnt; ++j) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_u32 + (uint32_t)j * 512u), "l"(src) : "memory");
+                src = next;
+                next += 64 * kMaxRows;
+            }
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            // the row's four lanes share its weights out, which take the place of the LSEs
+            float mx_new = mx;
+            for (int j = lane >> 3; j < cnt; j += 4) {
+                const float l = lse_stage[j * 8 + r];
+                bad = bad || (row < M && __float_as_uint(l) == kBadPartial);
+                mx_new = fmaxf(mx_new, l);
+            }
+            mx_new = fmaxf(mx_new, __shfl_xor_sync(0xffffffffu, mx_new, 8));
+            mx_new = fmaxf(mx_new, __shfl_xor_sync(0xffffffffu, mx_new, 16));
+            float round_sum = 0.f;
+            for (int j = lane >> 3; j < cnt; j += 4) {
+                const float l = lse_stage[j * 8 + r], w = l > -INFINITY ? __expf(l - mx_new) : 0.f;     // an empty partial has no weight
+                lse_stage[j * 8 + r] = w;
+                round_sum += w;
+            }
+            round_sum += __shfl_xor_sync(0xffffffffu, round_sum, 8);
+            round_sum += __shfl_xor_sync(0xffffffffu, round_sum, 16);
+            const float rescale = mx > -INFINITY ? __expf(mx - mx_new) : 0.f;
+            acc.x *= rescale; acc.y *= rescale; acc.z *= rescale; acc.w *= rescale;
+            sum = sum * rescale + round_sum;
+            mx = mx_new;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+#pragma unroll 4
+            for (int j = 0; j < cnt; ++j) {
+                const float w = lse_stage[j * 8 + r];
+                const float4 v = stage[j * 32 + lane];             // this lane's own copy
+                acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
             }
         }
-        if (bad) continue;                             // the pass found a bad tree or page in this sequence: no output
+        // a bad tree or page in the unit's sequence: no output (the same for all of its rows; rows past the last hold nothing)
+        if (__any_sync(0xffffffffu, bad) || row >= M) continue;
         const float inv = sum > 0.f ? 1.f / sum : 0.f;
         uint2 pk;
         if (p.f16) {
@@ -192,8 +202,10 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             pk.x = *reinterpret_cast<uint32_t*>(&lo2);
             pk.y = *reinterpret_cast<uint32_t*>(&hi2);
         }
-        *reinterpret_cast<uint2*>(p.out + row_id * kHeadDim + lane * 4) = pk;
-        if (p.lse && lane == 0) p.lse[row_id] = sum > 0.f ? mx + logf(sum) : -INFINITY;
+        const int node = row / p.group;
+        const long long out_row = (long long)(node_base + node) * p.num_q_heads + h * p.group + (row - node * p.group);
+        *reinterpret_cast<uint2*>(p.out + out_row * kHeadDim + chunk * 4) = pk;
+        if (p.lse && chunk == 0) p.lse[out_row] = sum > 0.f ? mx + logf(sum) : -INFINITY;
     }
 }
 

@@ -36,15 +36,14 @@ struct AttnParams {
     const int32_t* tree_parent;
     __nv_bfloat16* out;
     float* lse;                   // may be null
-    float* part_o;                // [slots, rows_per_slot, D] fp32, normalised partial outputs
-    float* part_lse;              // [slots, rows_per_slot] fp32, natural-log partial LSE (-inf if empty; kBadPartial)
+    float* part_o;                // [slots, D / 4, kMaxRows, 4] fp32, normalised partial outputs
+    float* part_lse;              // [slots, kMaxRows] fp32, natural-log partial LSE (-inf if empty; kBadPartial)
     int32_t* status;              // device status word (0 = ok, first error wins)
     long long* sched_seq_begin;   // [B + 1] first flat tile of every sequence (written by CTA 0 of the pass)
     SchedHeader* sched_header;
     int32_t batch, total_nodes, nodes_uniform, max_nodes;
     int32_t num_q_heads, num_kv_heads, group;  // group = Hq / Hkv
     int32_t page_size, page_shift, max_pages_per_seq, num_pages;
-    int32_t rows_per_slot;        // row stride of one partial slot
     int32_t num_ctas;             // CTAs of the split-KV pass (the flat tile range is cut into this many pieces)
     int32_t combine_group;        // partials per round of the merge kernel, 4..32
     int32_t combine_row_ctas;     // CTAs of the merge kernel that take output rows (persistent, eight warps each)

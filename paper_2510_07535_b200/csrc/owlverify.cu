@@ -26,7 +26,6 @@ struct owl_ctx {
     int sm_count = 0;
     owl_dims max_dims{};
     int num_ctas = 0;
-    int rows_per_slot = 0;
     long long slots = 0;
     float* part_o = nullptr;
     float* part_lse = nullptr;
@@ -251,10 +250,9 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         if (ok && (e = cudaMalloc(p, bytes ? bytes : 16)) != cudaSuccess) ok = false;
     };
     if (attn) {
-        ctx->rows_per_slot = umma_path::kRows;
         ctx->slots = 2ll * ctx->num_ctas;      // a CTA stores at most two partials per call
-        alloc((void**)&ctx->part_o, (size_t)ctx->slots * ctx->rows_per_slot * kHeadDim * sizeof(float));
-        alloc((void**)&ctx->part_lse, (size_t)ctx->slots * ctx->rows_per_slot * sizeof(float));
+        alloc((void**)&ctx->part_o, (size_t)ctx->slots * kMaxRows * kHeadDim * sizeof(float));
+        alloc((void**)&ctx->part_lse, (size_t)ctx->slots * kMaxRows * sizeof(float));
     }
     alloc((void**)&ctx->status, sizeof(int32_t));
     alloc((void**)&ctx->selftest_ns, 2 * sizeof(unsigned long long));
@@ -367,7 +365,6 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     p.page_shift = log2_exact(d->page_size);
     p.max_pages_per_seq = d->max_pages_per_seq;
     p.num_pages = d->num_pages;
-    p.rows_per_slot = ctx->rows_per_slot;
     p.num_ctas = ctx->num_ctas;
     p.sm_scale = d->sm_scale;
     p.f16 = fp16 ? 1 : 0;
@@ -397,10 +394,9 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     }
 
     if (ctx->profiling) cudaEventRecord(ctx->ev[0], stream);
-    const long long rows = (long long)d->total_nodes * d->num_q_heads;
-    // one warp per row while all CTAs are resident at once; beyond that the merge kernel's warps stride over the rows
+    // one CTA per block of rows while all are resident at once; beyond that the merge kernel's CTAs stride over the blocks
     p.combine_group = combine_group((long long)d->batch * d->num_kv_heads, ctx->num_ctas);
-    const long long want_ctas = (rows + kCombineWarps - 1) / kCombineWarps;
+    const long long want_ctas = (long long)d->batch * d->num_kv_heads * ((G * d->max_nodes + kCombineRows - 1) / kCombineRows);
     const long long most_ctas = (long long)ctx->sm_count * combine_ctas_per_sm(p.combine_group);
     const unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas : most_ctas);
     p.combine_row_ctas = (int32_t)grid;

@@ -48,7 +48,7 @@ namespace umma_path {
 using namespace sm100;
 
 constexpr int kTileKeys = 128;
-constexpr int kRows = 256;                 // packed rows per unit (two streams of 128)
+constexpr int kRows = kMaxRows;                 // packed rows per unit (two streams of 128)
 constexpr int kThreads = 384;
 constexpr int kSlots = 5;                  // ring of K / V tiles
 constexpr int kSlotBytes = kTileKeys * kHeadDim * 2;     // 32 KB
@@ -528,11 +528,9 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
 // ------------------------------------------------------------------------------------------ softmax warpgroups
 __device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
 
-// Writes a warp's 32 rows x 32 columns (lane = row, v = its 32 fp32 values) to global memory through a
-// per-warp staging area in shared memory, so that every store instruction covers whole 64- or 128-byte
-// row segments instead of 32 scattered 16-byte pieces.  `out_row` / `row_ok` are the lane's own row;
-// the other rows' values come by shuffle.  kFinal: bf16 into `out`; else fp32 into the partial slot,
-// whose rows are consecutive (part_row0 = row of lane 0).
+// Writes a warp's 32 rows x 32 columns (lane = row, v = its 32 fp32 values) to `out` as 16-bit values, through a per-warp
+// staging area in shared memory, so that every store instruction covers whole 64-byte row segments instead of 32 scattered
+// pieces.  `out_row` / `row_ok` are the lane's own row; the other rows' values come by shuffle.
 constexpr int kStageStride = 36;                     // floats per staged row: 16-byte aligned, conflict-free
 constexpr int kStageBytesPerWarp = 32 * kStageStride * 4;
 // Two floats to two 16-bit values of the cache's element type (x in the low half), round to nearest even.
@@ -543,9 +541,9 @@ __device__ __forceinline__ uint32_t pack2_16bit(float x, float y) {
     return *reinterpret_cast<uint32_t*>(&b);
 }
 
-template <bool kFinal, bool kF16>
-__device__ __forceinline__ void store_rows32(const AttnParams& p, float* stage, long long out_row, bool row_ok,
-                                             long long part_row0, int col, const float (&v)[32]) {
+template <bool kF16>
+__device__ __forceinline__ void store_rows32(const AttnParams& p, float* stage, long long out_row, bool row_ok, int col,
+                                             const float (&v)[32]) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
 #pragma unroll
@@ -553,27 +551,17 @@ __device__ __forceinline__ void store_rows32(const AttnParams& p, float* stage, 
         *reinterpret_cast<float4*>(stage + lane * kStageStride + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
     __syncwarp();
     // (rolled: this code runs a few times per launch, with cold instruction caches, where its length counts)
-    if (kFinal) {
 #pragma unroll 1
-        for (int k = 0; k < 4; ++k) {                 // 8 rows x 64 bytes per instruction
-            const int row = 8 * k + (lane >> 2), piece = lane & 3;
-            const long long orow = __shfl_sync(0xffffffffu, out_row, row);
-            const bool ok = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, row) != 0;
-            const float4 a = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 8);
-            const float4 b2 = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 8 + 4);
-            uint4 u;
-            u.x = pack2_16bit<kF16>(a.x, a.y); u.y = pack2_16bit<kF16>(a.z, a.w);
-            u.z = pack2_16bit<kF16>(b2.x, b2.y); u.w = pack2_16bit<kF16>(b2.z, b2.w);
-            if (ok) *reinterpret_cast<uint4*>(p.out + orow * kHeadDim + col + piece * 8) = u;
-        }
-    } else {
-#pragma unroll 2
-        for (int k = 0; k < 8; ++k) {                 // 4 rows x 128 bytes per instruction
-            const int row = 4 * k + (lane >> 3), piece = lane & 7;
-            const bool ok = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, row) != 0;
-            const float4 a = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 4);
-            if (ok) *reinterpret_cast<float4*>(p.part_o + (part_row0 + row) * kHeadDim + col + piece * 4) = a;
-        }
+    for (int k = 0; k < 4; ++k) {                 // 8 rows x 64 bytes per instruction
+        const int row = 8 * k + (lane >> 2), piece = lane & 3;
+        const long long orow = __shfl_sync(0xffffffffu, out_row, row);
+        const bool ok = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, row) != 0;
+        const float4 a = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 8);
+        const float4 b2 = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 8 + 4);
+        uint4 u;
+        u.x = pack2_16bit<kF16>(a.x, a.y); u.y = pack2_16bit<kF16>(a.z, a.w);
+        u.z = pack2_16bit<kF16>(b2.x, b2.y); u.w = pack2_16bit<kF16>(b2.z, b2.w);
+        if (ok) *reinterpret_cast<uint4*>(p.out + orow * kHeadDim + col + piece * 8) = u;
     }
 }
 
@@ -876,14 +864,15 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         const bool bad = bad_tree || const_cast<volatile int&>(aux->seg[seg_no % kSegs].bad_page);
         const bool write_ok = !bad && !*abort_flag;
         // only the first and the last unit of a CTA's piece can be cut: two partial slots per CTA
-        const long long part_row = (2ll * blockIdx.x + (seg_no > 0 ? 1 : 0)) * p.rows_per_slot + rr;
+        const long long part_row = (2ll * blockIdx.x + (seg_no > 0 ? 1 : 0)) * kRows + rr;
         const long long out_row = rr < g.M ? (long long)(g.node_base + rr / G) * p.num_q_heads + g.h * G + rr % G : 0;
         const bool row_ok = write_ok && rr < g.M;
         const bool whole = g.whole();
         // staging for coalesced stores: the Q blocks are idle now (every MMA of the segment is done); stream 1's
         // area starts after the (m, l, lx) exchange
         float* stage = reinterpret_cast<float*>(smem + s * (kQBytes + 4096) + ((threadIdx.x >> 5) & 3) * kStageBytesPerWarp);
-        const long long part_row0 = part_row - (threadIdx.x & 31);
+        // a partial: [32 groups of four channels][kRows rows][4], so that a warp, one row per lane, stores whole lines
+        float4* part = reinterpret_cast<float4*>(p.part_o) + (part_row - rr) * 32 + rr;
         // One loop writes both modes.  shared: this warpgroup's own rows, all 128 columns of its O, weight 1 / l.
         // split: the two streams hold the same rows over disjoint key tiles; they are merged by their maxima and
         // sums, and this warpgroup writes columns [64 s, 64 s + 64) of the merged rows.
@@ -923,8 +912,12 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
                 v[j] = __uint_as_float(oa[j]) * wa;           // rows that saw no key have O = 0 and weight 0
                 if (use_b) v[j] = fmaf(__uint_as_float(ob[j]), wb, v[j]);
             }
-            if (whole) store_rows32<true, kF16>(p, stage, out_row, row_ok, part_row0, c4 * 32, v);
-            else store_rows32<false, kF16>(p, stage, out_row, row_ok, part_row0, c4 * 32, v);
+            if (whole) store_rows32<kF16>(p, stage, out_row, row_ok, c4 * 32, v);
+            else if (row_ok) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    part[(c4 * 8 + j) * kRows] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            }
         }
         if (row_ok && write_lse) {
             if (whole) { if (p.lse) p.lse[out_row] = lse; }

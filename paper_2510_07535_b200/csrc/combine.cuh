@@ -84,55 +84,48 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
     const uint32_t stage_u32 = (uint32_t)__cvta_generic_to_shared(stage + lane);
     const unsigned units = (unsigned)(p.batch * p.num_kv_heads);
     const unsigned blocks = units * (unsigned)((p.group * p.max_nodes + kCombineRows - 1) / kCombineRows);
-    const bool small = p.batch <= 32;
     WarpSchedule ws{};
-    Partition part;
-    if (small) {
-        ws = warp_schedule(p);
-        part.init(ws.total, p.num_ctas, ws.units, ws.uniform_tiles);
-    }
     // per block: its unit's row count, the first partial's slot and the number of partials (0: nothing to merge)
     int M = 0, h = 0, row = 0, node_base = 0, slot = 0, count = 0;
-    auto locate = [&](unsigned id) {       // every lane of the warp, same block
-        const unsigned k = id / units, u = id - k * units, b = u / (unsigned)p.num_kv_heads;
-        h = (int)(u - b * (unsigned)p.num_kv_heads);
+    auto plan = [&](unsigned k, int n, int tiles, auto t0, const auto& part) {
         row = (int)k * kCombineRows + r;
-        int n, tiles;
-        long long seq_begin;
-        if (small) {
-            n = __shfl_sync(0xffffffffu, ws.n, b);
-            node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
-            tiles = __shfl_sync(0xffffffffu, ws.tiles, b);
-            seq_begin = __shfl_sync(0xffffffffu, ws.excl_t + (long long)part.pen * ws.excl_u, b);
-        } else {
-            const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
-            n = seq_nodes(p, (int)b);
-            node_base = seq_node_base(p, (int)b);
-            seq_begin = sb;
-            tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
-        }
-        count = 0;
         M = n * p.group;
+        count = 0;
         if (tiles == 0 || (int)k * kCombineRows >= M) return;      // not scheduled, or no such rows
-        const long long t0 = seq_begin + (long long)h * (tiles + part.pen);
         const int c0 = part.owner(t0 + part.pen), c1 = part.owner(t0 + part.pen + tiles - 1);
         if (c0 == c1) return;              // a single CTA saw every key of this unit and wrote the result itself
         // the unit's first CTA may have come from another unit; the others' pieces start in this one
         slot = 2 * c0 + (part.begin(c0) < t0 ? 1 : 0);
         count = c1 - c0 + 1;
     };
+    auto locate = [&](unsigned id) {       // every lane of the warp, same block
+        const unsigned k = id / units, u = id - k * units, b = u / (unsigned)p.num_kv_heads;
+        h = (int)(u - b * (unsigned)p.num_kv_heads);
+        if (p.small) {
+            const int n = __shfl_sync(0xffffffffu, ws.n, b), tiles = __shfl_sync(0xffffffffu, ws.tiles, b);
+            node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
+            plan(k, n, tiles, __shfl_sync(0xffffffffu, ws.begin, b) + h * (tiles + ws.part.pen), ws.part);
+        } else {
+            Partition<long long> part;
+            const SchedHeader hdr = *p.sched_header;      // larger batches read the schedule the pass left
+            part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
+            const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
+            node_base = seq_node_base(p, (int)b);
+            const int tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
+            plan(k, seq_nodes(p, (int)b), tiles, sb + (long long)h * (tiles + part.pen), part);
+        }
+    };
     // latency after the pass has ended is what this kernel costs: whatever needs no output of the pass comes before
     // the wait - for batches of at most 32 sequences the whole plan of the first block
-    if (small) locate(blockIdx.x);
+    if (p.small) {
+        ws = warp_schedule(p);
+        locate(blockIdx.x);
+    }
     // from here on the split-KV pass has completed and its writes are visible (a no-op in an ordinary launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel in the stream may queue up
-    if (!small) {
-        const SchedHeader hdr = *p.sched_header;      // larger batches read the schedule the pass left
-        part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
-    }
     for (unsigned id = blockIdx.x; id < blocks; id += row_ctas) {
-        if (!small || id != blockIdx.x) locate(id);
+        if (!p.small || id != blockIdx.x) locate(id);
         if (count == 0) continue;
         // Partials are taken `group` at a time, their LSEs with them: one memory round trip per group.  Groups are folded
         // online (running maximum, each lane its own row's).
@@ -202,7 +195,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             pk.x = *reinterpret_cast<uint32_t*>(&lo2);
             pk.y = *reinterpret_cast<uint32_t*>(&hi2);
         }
-        const int node = row / p.group;
+        const int node = (int)row_node(p, row);
         const long long out_row = (long long)(node_base + node) * p.num_q_heads + h * p.group + (row - node * p.group);
         *reinterpret_cast<uint2*>(p.out + out_row * kHeadDim + chunk * 4) = pk;
         if (p.lse && chunk == 0) p.lse[out_row] = sum > 0.f ? mx + logf(sum) : -INFINITY;

@@ -43,13 +43,19 @@ struct AttnParams {
     SchedHeader* sched_header;
     int32_t batch, total_nodes, nodes_uniform, max_nodes;
     int32_t num_q_heads, num_kv_heads, group;  // group = Hq / Hkv
+    uint32_t group_magic;         // 65536 / group + 1 (row_node)
     int32_t page_size, page_shift, max_pages_per_seq, num_pages;
+    int32_t small;                // the schedule is derived by single warps in 32-bit arithmetic (small_schedule)
     int32_t num_ctas;             // CTAs of the split-KV pass (the flat tile range is cut into this many pieces)
     int32_t combine_group;        // partials per round of the merge kernel, 4..32
     int32_t combine_row_ctas;     // CTAs of the merge kernel that take output rows (persistent, eight warps each)
     int32_t f16;                  // q / caches / out are fp16 instead of bf16 (same size; typed as bf16 pointers here)
     float sm_scale;
 };
+
+// Node of a unit's packed row, row < kMaxRows.  (group * magic = 65536 + e with 1 <= e <= group, so the product is
+// row / group + row * e / (65536 group), too high by less than 1 / group while row * group < 65536.)
+__device__ __forceinline__ unsigned row_node(const AttnParams& p, unsigned row) { return (row * p.group_magic) >> 16; }
 
 // 2^x by the special-function unit (ex2.approx, denormals flushed); ex2(-inf) = 0.
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -78,71 +84,70 @@ __device__ __forceinline__ void report(int32_t* status, int code) { atomicCAS(st
 //            crosses a unit boundary (and there are no gaps).  Chosen when its largest piece is smaller than the flat one.
 // ---------------------------------------------------------------------------------------------
 constexpr int kBoundaryPenaltyTiles = 5;
+// T: places on the line.  int where the host has made sure that the line is short (small_schedule).  Every CTA derives its
+// piece once, on its critical path, where the code is not in the instruction caches and one instruction waits for the one
+// before: instructions are time there.
+template <typename T>
 struct Partition {
-    long long total, q;           // length of the line, of a piece
+    static constexpr bool kShort = sizeof(T) == 4;
+    T total, q;                   // length of the line, of a piece
     int rem, ctas;
     int unit_tiles, base, urem;   // aligned mode iff unit_tiles > 0
     int pen;                      // gap in front of a unit's tiles
-    // (Every CTA runs this once, on its critical path and with cold instruction caches, where each instruction costs
-    // tens of nanoseconds: one 32-bit division where the numbers allow it instead of 64-bit ones.)
-    __device__ __host__ void init(long long tiles, int ctas_, int units, int uniform_tiles) {
+    __device__ __host__ void init(T tiles, int ctas_, int units, int uniform_tiles) {
         ctas = ctas_;
         pen = kBoundaryPenaltyTiles;
-        total = tiles + (long long)pen * units;
-        if (total >= 0 && total <= 0x7fffffffll) {
+        total = tiles + (T)pen * units;
+        if (kShort || (total >= 0 && total <= 0x7fffffffll)) {
             const unsigned qq = (unsigned)total / (unsigned)ctas_;
-            q = qq; rem = (int)((unsigned)total - qq * (unsigned)ctas_);
+            q = (T)qq; rem = (int)((unsigned)total - qq * (unsigned)ctas_);
         } else {
             q = total / ctas_; rem = (int)(total % ctas_);
         }
         unit_tiles = 0; base = 0; urem = 0;
         if (uniform_tiles > 0 && units > 1 && units <= ctas_) {
-            const int b = ctas_ / units;
-            if ((uniform_tiles + b - 1) / b < q + (rem ? 1 : 0)) {
-                unit_tiles = uniform_tiles; base = b; urem = ctas_ - b * units;
+            const unsigned b = (unsigned)ctas_ / (unsigned)units;
+            if ((T)(((unsigned)uniform_tiles + b - 1u) / b) < q + (rem ? 1 : 0)) {
+                unit_tiles = uniform_tiles; base = (int)b; urem = ctas_ - (int)b * units;
                 total = tiles; pen = 0;
             }
         }
     }
     // [begin(c), begin(c + 1)) with one set of divisions (the pieces of a unit tile it exactly, so a piece's end is
     // its begin plus its length in either mode)
-    __device__ __host__ void range(int c, long long& t_begin, long long& t_end) const {
+    __device__ __host__ void range(int c, T& t_begin, T& t_end) const {
         if (unit_tiles == 0) {
-            t_begin = (long long)c * q + (c < rem ? c : rem);
+            t_begin = (T)c * q + (c < rem ? c : rem);
             t_end = t_begin + q + (c < rem ? 1 : 0);
             return;
         }
         const int big = urem * (base + 1);
         int u, k, cu;
-        if (c < big) { u = c / (base + 1); k = c - u * (base + 1); cu = base + 1; }
-        else { u = urem + (c - big) / base; k = (c - big) - (u - urem) * base; cu = base; }
-        const int qq = unit_tiles / cu, rr = unit_tiles - qq * cu;
-        t_begin = (long long)u * unit_tiles + (long long)k * qq + (k < rr ? k : rr);
+        if (c < big) { u = (int)((unsigned)c / (unsigned)(base + 1)); k = c - u * (base + 1); cu = base + 1; }
+        else { u = urem + (int)((unsigned)(c - big) / (unsigned)base); k = (c - big) - (u - urem) * base; cu = base; }
+        const int qq = (int)((unsigned)unit_tiles / (unsigned)cu), rr = unit_tiles - qq * cu;
+        t_begin = (T)u * unit_tiles + (T)k * qq + (k < rr ? k : rr);
         t_end = t_begin + qq + (k < rr ? 1 : 0);
     }
-    __device__ __host__ long long begin(int c) const {
-        if (unit_tiles == 0) return (long long)c * q + (c < rem ? c : rem);
-        const int big = urem * (base + 1);
-        int u, k, cu;
-        if (c < big) { u = c / (base + 1); k = c - u * (base + 1); cu = base + 1; }
-        else { u = urem + (c - big) / base; k = (c - big) - (u - urem) * base; cu = base; }
-        const int qq = unit_tiles / cu, rr = unit_tiles % cu;
-        return (long long)u * unit_tiles + (long long)k * qq + (k < rr ? k : rr);
+    __device__ __host__ T begin(int c) const {
+        T t_begin, t_end;
+        range(c, t_begin, t_end);
+        return t_begin;
     }
-    __device__ __host__ int owner(long long t) const {        // of a place on the line
+    __device__ __host__ int owner(T t) const {        // of a place on the line
         if (unit_tiles == 0) {
-            long long big = (long long)rem * (q + 1);
-            if (total <= 0x7fffffffll) {      // the usual case: 32-bit divisions
+            const T big = (T)rem * (q + 1);
+            if (kShort || total <= 0x7fffffffll) {
                 const unsigned tt = (unsigned)t, qq = (unsigned)q, bb = (unsigned)big;
                 return tt < bb ? (int)(tt / (qq + 1u)) : rem + (int)((tt - bb) / qq);
             }
             return t < big ? (int)(t / (q + 1)) : rem + (int)((t - big) / q);
         }
-        const int u = total <= 0x7fffffffll ? (int)((unsigned)t / (unsigned)unit_tiles) : (int)(t / unit_tiles);
-        const int local = (int)(t - (long long)u * unit_tiles);
-        const int cu = base + (u < urem ? 1 : 0), c0 = u * base + (u < urem ? u : urem);
-        const int qq = unit_tiles / cu, rr = unit_tiles % cu, bigl = rr * (qq + 1);
-        return c0 + (local < bigl ? local / (qq + 1) : rr + (local - bigl) / qq);
+        const int u = kShort || total <= 0x7fffffffll ? (int)((unsigned)t / (unsigned)unit_tiles) : (int)(t / unit_tiles);
+        const unsigned local = (unsigned)(t - (T)u * unit_tiles), cu = (unsigned)(base + (u < urem ? 1 : 0));
+        const int c0 = u * base + (u < urem ? u : urem);
+        const unsigned qq = (unsigned)unit_tiles / cu, rr = (unsigned)unit_tiles - qq * cu, bigl = rr * (qq + 1u);
+        return c0 + (int)(local < bigl ? local / (qq + 1u) : rr + (local - bigl) / qq);
     }
 };
 
@@ -161,12 +166,11 @@ __device__ __forceinline__ int seq_node_base(const AttnParams& p, int b) {
 }
 
 // A sequence is schedulable when its node count and lengths are inside the interface's limits.
-__device__ __forceinline__ bool seq_tree_shape_ok(const AttnParams& p, int b, int n) {
-    const int base = seq_node_base(p, b);
+__device__ __forceinline__ bool seq_tree_shape_ok(const AttnParams& p, int base, int n) {
     return n >= 1 && n <= p.max_nodes && base >= 0 && base + n <= p.total_nodes;
 }
 __device__ __forceinline__ bool seq_shape_ok(const AttnParams& p, int b, int n, int L) {
-    if (!seq_tree_shape_ok(p, b, n) || L < 0) return false;
+    if (!seq_tree_shape_ok(p, seq_node_base(p, b), n) || L < 0) return false;
     long long keys = (long long)L + n;
     return keys <= (long long)p.max_pages_per_seq * p.page_size;
 }
@@ -174,52 +178,44 @@ __device__ __forceinline__ bool seq_shape_ok(const AttnParams& p, int b, int n, 
 // Schedule of a batch of at most 32 sequences, derived by one warp on its own: lane b holds sequence b, prefix sums
 // by shuffle, no shared memory.  The split-KV pass (its producer warp) and the merge that follows it (every warp) call the
 // same function on the same inputs, so the merge needs nothing from the pass but its partials.
+// The line is so short that everything fits 32 bits, a sequence's keys (2^24 tiles) included.
 constexpr int kSchedTileKeys = 128;      // key tile of the split-KV pass
+inline bool small_schedule(int batch, int num_kv_heads, int max_pages_per_seq, int page_size) {
+    const long long tiles = ((long long)max_pages_per_seq * page_size + kSchedTileKeys - 1) / kSchedTileKeys;
+    return batch <= 32 && (tiles + kBoundaryPenaltyTiles) * batch * num_kv_heads < (1ll << 24);
+}
 struct WarpSchedule {
     int n, L, node_base, tiles;          // this lane's sequence (tiles = 0 if it is not schedulable)
-    bool ok;
-    long long my_tiles, excl_t, total;   // tiles of this sequence (all KV heads), of the ones before it, of all
-    int my_units, excl_u, units;
-    int uniform_tiles;                   // tiles per unit if every schedulable sequence has the same count, else 0
+    unsigned ok;                         // the schedulable sequences
+    int begin, end;                      // this lane's sequence on the line
+    Partition<int> part;
 };
 __device__ __forceinline__ WarpSchedule warp_schedule(const AttnParams& p) {
+    constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     WarpSchedule ws;
-    ws.n = 0; ws.L = 0; ws.node_base = 0; ws.tiles = 0; ws.ok = false;
+    ws.n = 0; ws.L = 0; ws.node_base = 0;
+    bool ok = false;
     if (lane < p.batch) {
-        ws.n = seq_nodes(p, lane);
         ws.L = p.ctx_lens[lane];
         ws.node_base = seq_node_base(p, lane);
-        ws.ok = seq_shape_ok(p, lane, ws.n, ws.L);
-        ws.tiles = ws.ok ? (ws.L + ws.n + kSchedTileKeys - 1) / kSchedTileKeys : 0;
+        ws.n = seq_nodes(p, lane);
+        ok = seq_tree_shape_ok(p, ws.node_base, ws.n) && ws.L >= 0 &&
+             (unsigned)ws.L + (unsigned)ws.n <= (unsigned)p.max_pages_per_seq * (unsigned)p.page_size;
     }
-    ws.my_tiles = (long long)ws.tiles * p.num_kv_heads;
-    ws.my_units = ws.ok ? p.num_kv_heads : 0;
-    long long inc_t = ws.my_tiles;
-    int inc_u = ws.my_units, tmin = ws.ok ? ws.tiles : 0x7fffffff, tmax = ws.ok ? ws.tiles : 0;
-    // as many rounds as the batch needs (one sequence: none): this runs once per launch on every CTA's critical
-    // path, where an instruction costs tens of nanoseconds.  Lanes >= batch hold zeros / neutral elements.
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        if (o >= p.batch) break;
-        const long long vt = __shfl_up_sync(0xffffffffu, inc_t, o);
-        const int vu = __shfl_up_sync(0xffffffffu, inc_u, o);
-        if (lane >= o) { inc_t += vt; inc_u += vu; }
+    ws.tiles = ok ? (ws.L + ws.n + kSchedTileKeys - 1) / kSchedTileKeys : 0;
+    ws.ok = __ballot_sync(kAll, ok);
+    const int first_tiles = __shfl_sync(kAll, ws.tiles, ws.ok ? __ffs(ws.ok) - 1 : 0);
+    const bool uniform = __all_sync(kAll, !ok || ws.tiles == first_tiles);
+    // tiles of one KV head's units; as many rounds as the batch needs
+    int inc = ws.tiles;
+    for (int o = 1; o < p.batch; o <<= 1) {
+        const int v = __shfl_up_sync(kAll, inc, o);
+        if (lane >= o) inc += v;
     }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {               // after the rounds with o < batch, lane 0 covers [0, batch)
-        if (o >= p.batch) break;
-        tmin = min(tmin, __shfl_down_sync(0xffffffffu, tmin, o));
-        tmax = max(tmax, __shfl_down_sync(0xffffffffu, tmax, o));
-    }
-    tmin = __shfl_sync(0xffffffffu, tmin, 0);
-    tmax = __shfl_sync(0xffffffffu, tmax, 0);
-    const int last = p.batch < 32 ? p.batch - 1 : 31;
-    ws.total = __shfl_sync(0xffffffffu, inc_t, last);
-    ws.units = __shfl_sync(0xffffffffu, inc_u, last);
-    ws.uniform_tiles = (ws.units > 0 && tmin == tmax) ? tmin : 0;
-    ws.excl_t = inc_t - ws.my_tiles;
-    ws.excl_u = inc_u - ws.my_units;
+    ws.part.init(__shfl_sync(kAll, inc, p.batch - 1) * p.num_kv_heads, p.num_ctas, __popc(ws.ok) * p.num_kv_heads, uniform ? first_tiles : 0);
+    ws.end = (inc + ws.part.pen * __popc(ws.ok & (kAll >> (31 - lane)))) * p.num_kv_heads;
+    ws.begin = ws.end - (ok ? (ws.tiles + ws.part.pen) * p.num_kv_heads : 0);
     return ws;
 }
 

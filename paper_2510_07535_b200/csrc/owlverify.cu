@@ -361,6 +361,8 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     p.num_q_heads = d->num_q_heads;
     p.num_kv_heads = d->num_kv_heads;
     p.group = G;
+    p.group_magic = 65536u / (unsigned)G + 1u;
+    p.small = small_schedule(d->batch, d->num_kv_heads, d->max_pages_per_seq, d->page_size) ? 1 : 0;
     p.page_size = d->page_size;
     p.page_shift = log2_exact(d->page_size);
     p.max_pages_per_seq = d->max_pages_per_seq;
@@ -411,9 +413,9 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        // the instance that holds only this call's case: block-wide schedule above 32 sequences, the two-row-block
+        // the instance that holds only this call's case: block-wide schedule above 32 sequences (small_schedule), the two-row-block
         // mode only if a unit (G * max_nodes rows at most) can exceed 128 rows, the logits scan only in a step
-        const bool many = d->batch > 32, wide = G * d->max_nodes > 128;
+        const bool many = !p.small, wide = G * d->max_nodes > 128;
         cudaLaunchKernelEx(&cfg, umma_kernel(many, wide, ap && !own_scan, fp16), p, maps->kmap, maps->vmap, ap ? *ap : AcceptParams{});
     }
     ++ctx->launches;

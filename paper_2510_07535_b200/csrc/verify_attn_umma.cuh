@@ -115,9 +115,11 @@ static_assert(sizeof(Aux) <= kAuxBytes, "aux area too small");
 // Walks the CTA's piece [t, t_end) of the line unit by unit.  The producer warp does, one segment after the other, and
 // announces each to the other roles in shared memory: with a walker and the schedule's arithmetic in every role the
 // text was a third longer and a CTA barrier stood between the schedule and the first copy.
+template <bool kManySeqs>
 struct Walker {
+    using Place = typename std::conditional<kManySeqs, long long, int>::type;
     int b, pen;
-    long long seq_begin, t, t_end;      // places on the line of Partition
+    Place seq_begin, t, t_end;          // places on the line of Partition
     // the sequence `b` as last loaded (most segments of a piece lie in the same sequence)
     int cur_b = -1, cur_n = 0, cur_L = 0, cur_tiles = 0, cur_node_base = 0;
     bool cur_ok = false;
@@ -136,7 +138,7 @@ struct Walker {
         if (t >= t_end) return false;
         while (b < p.batch) {
             if (cur_b != b) load_seq(p);
-            const long long flat = cur_ok ? (long long)(cur_tiles + pen) * p.num_kv_heads : 0;
+            const Place flat = cur_ok ? (Place)(cur_tiles + pen) * p.num_kv_heads : 0;
             if (t < seq_begin + flat) break;
             seq_begin += flat;
             ++b;
@@ -147,7 +149,7 @@ struct Walker {
         g.b = b; g.n = cur_n; g.L = cur_L; g.tiles = cur_tiles;
         g.h = (int)(local / (unsigned)len);
         const int at = (int)(local - (unsigned)g.h * (unsigned)len);
-        const long long left = t_end - t;
+        const Place left = t_end - t;
         const int end = (int)(at + left < len ? at + left : len);
         t += end - at;
         g.tile0 = max(at - pen, 0);
@@ -162,7 +164,7 @@ struct Walker {
 
 // Block-wide: totals of tiles and units, the choice of partition and the first sequence of this
 // CTA's piece.  CTA 0 also leaves the per-sequence prefix and the header for the combine kernel.
-__device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker& w) {
+__device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker<true>& w) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int per = (p.batch + kThreads - 1) / kThreads;
     const int b_lo = tid * per, b_hi = min(p.batch, b_lo + per);
@@ -176,7 +178,7 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
             my_units += p.num_kv_heads;
             tmin = min(tmin, tiles); tmax = max(tmax, tiles);
         } else {
-            report(p.status, seq_tree_shape_ok(p, b, n) ? kErrBadPage : kErrBadTree);
+            report(p.status, seq_tree_shape_ok(p, seq_node_base(p, b), n) ? kErrBadPage : kErrBadTree);
         }
     }
     long long inc_t = my_tiles;
@@ -203,7 +205,7 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
         tmin = min(tmin, aux->scan_tmin[w2]); tmax = max(tmax, aux->scan_tmax[w2]);
     }
     const int uniform_tiles = (units > 0 && tmin == tmax) ? tmin : 0;
-    Partition part;
+    Partition<long long> part;
     part.init(total, gridDim.x, units, uniform_tiles);
     // this thread's sequences on the line
     const long long excl = off_t + inc_t - my_tiles + (long long)part.pen * (off_u + inc_u - my_units);
@@ -238,40 +240,26 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
 
 // Batches of at most 32 sequences: the producer warp derives the schedule on its own (lane b holds sequence
 // b, prefix sums by shuffle), with no shared memory and no CTA-wide barrier.
-__device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker& w) {
+__device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker<false>& w) {
     static_assert(kTileKeys == kSchedTileKeys, "the merge kernel derives the same schedule");
     const int lane = threadIdx.x & 31;
     const WarpSchedule ws = warp_schedule(p);
-    const int n = ws.n, L = ws.L, node_base = ws.node_base, tiles = ws.tiles;
-    if (lane < p.batch && !ws.ok) {
-        report(p.status, seq_tree_shape_ok(p, lane, n) ? kErrBadPage : kErrBadTree);
-    }
-    Partition part;
-    part.init(ws.total, gridDim.x, ws.units, ws.uniform_tiles);
-    const long long excl = ws.excl_t + (long long)part.pen * ws.excl_u, my_len = ws.my_tiles + (long long)part.pen * ws.my_units;
-    long long t_begin, t_end;
-    part.range(blockIdx.x, t_begin, t_end);
-    const unsigned owner = __ballot_sync(0xffffffffu, my_len > 0 && t_begin >= excl && t_begin < excl + my_len);
-    if (blockIdx.x == 0) {
-        if (lane < p.batch) p.sched_seq_begin[lane] = excl;
-        if (lane == 0) {
-            p.sched_seq_begin[p.batch] = part.total;
-            p.sched_header->total_tiles = ws.total;
-            p.sched_header->uniform_tiles = ws.uniform_tiles;
-            p.sched_header->units = ws.units;
-        }
-    }
-    w.pen = part.pen;
+    if (lane < p.batch && !(ws.ok >> lane & 1u))
+        report(p.status, seq_tree_shape_ok(p, ws.node_base, ws.n) ? kErrBadPage : kErrBadTree);
+    int t_begin, t_end;
+    ws.part.range(blockIdx.x, t_begin, t_end);
+    const unsigned owner = __ballot_sync(0xffffffffu, t_begin >= ws.begin && t_begin < ws.end);
+    w.pen = ws.part.pen;
     w.t = t_begin;
-    w.t_end = (t_begin < t_end && owner) ? t_end : t_begin;
+    w.t_end = owner ? t_end : t_begin;
     const int b0 = owner ? __ffs(owner) - 1 : 0;
     w.b = b0;
-    w.seq_begin = __shfl_sync(0xffffffffu, excl, b0);
+    w.seq_begin = __shfl_sync(0xffffffffu, ws.begin, b0);
     w.cur_b = b0;
-    w.cur_n = __shfl_sync(0xffffffffu, n, b0);
-    w.cur_L = __shfl_sync(0xffffffffu, L, b0);
-    w.cur_node_base = __shfl_sync(0xffffffffu, node_base, b0);
-    w.cur_tiles = __shfl_sync(0xffffffffu, tiles, b0);
+    w.cur_n = __shfl_sync(0xffffffffu, ws.n, b0);
+    w.cur_L = __shfl_sync(0xffffffffu, ws.L, b0);
+    w.cur_node_base = __shfl_sync(0xffffffffu, ws.node_base, b0);
+    w.cur_tiles = __shfl_sync(0xffffffffu, ws.tiles, b0);
     w.cur_ok = true;
 }
 
@@ -310,9 +298,9 @@ __device__ __forceinline__ bool readers_reached(Aux* aux, int seg_no) {
     return __all_sync(0xffffffffu, ok);
 }
 
-template <bool kWide>
+template <bool kWide, bool kManySeqs>
 __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtensorMap* kmap, const CUtensorMap* vmap,
-                                              Aux* aux, uint32_t ring, Walker w) {
+                                              Aux* aux, uint32_t ring, Walker<kManySeqs> w) {
     const int lane = threadIdx.x & 31;
     volatile int* abort_flag = &aux->abort_flag;
     const int ppt = kTileKeys >> p.page_shift;               // pages (= TMA boxes) per tile
@@ -323,7 +311,17 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
     const uint64_t stream_policy = l2_policy_evict_first();
     for (uint32_t seg_no = 0;; ++seg_no) {
         Segment g;
+        g.b = g.n = g.L = 0;
         const bool more = w.template next<kWide>(p, g);
+        // The page of the segment's first tile that this lane copies is asked for before the segment is announced.
+        const int keys = g.L + g.n;
+        const int pages_valid = (keys + p.page_size - 1) >> p.page_shift;
+        const int32_t* table = p.block_table + (long long)g.b * p.max_pages_per_seq;
+        auto page_of = [&](int t) {
+            const int lp = t * ppt + lane;
+            return lane < ppt && lp < pages_valid ? table[lp] : -1;
+        };
+        int page_next = more ? page_of(g.tile0) : -1;
         // a place is free again once the readers have come to the segment after the one that it held (not abortable:
         // their waits are bounded; should it give up all the same, nothing is announced any more and they do likewise)
         if (seg_no >= (uint32_t)kSegs && !readers_reached(aux, (int)seg_no - kSegs + 1)) break;
@@ -336,26 +334,17 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
         }
         __syncwarp();
         if (!more) break;
-        const int keys = g.L + g.n;
-        const int pages_valid = (keys + p.page_size - 1) >> p.page_shift;
-        const int32_t* table = p.block_table + (long long)g.b * p.max_pages_per_seq;
-        auto coord_of = [&](int t) {
-            int c = oob;
-            const int lp = t * ppt + lane;
-            if (lane < ppt && lp < pages_valid) {
-                const int pg = table[lp];
-                if ((unsigned)pg < (unsigned)p.num_pages) c = pg * p.num_kv_heads + g.h;
-                else {
-                    report(p.status, kErrBadPage);
-                    const_cast<volatile int&>(announced.bad_page) = 1;
-                }
+        auto coord_of = [&](int t, int pg) {
+            if ((unsigned)pg < (unsigned)p.num_pages) return pg * p.num_kv_heads + g.h;
+            if (lane < ppt && t * ppt + lane < pages_valid) {
+                report(p.status, kErrBadPage);
+                const_cast<volatile int&>(announced.bad_page) = 1;
             }
-            return c;
+            return oob;
         };
-        int c_next = coord_of(g.tile0);
         for (int t = g.tile0; t < g.tile1; ++t) {
-            const int c_cur = c_next;
-            if (t + 1 < g.tile1) c_next = coord_of(t + 1);
+            const int c_cur = coord_of(t, page_next);
+            if (t + 1 < g.tile1) page_next = page_of(t + 1);
 #pragma unroll
             for (int kv = 0; kv < 2; ++kv) {
                 const uint32_t slot = item % kSlots, ph = (item / kSlots) & 1u;
@@ -595,17 +584,22 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             const int r_first = (g.shared ? 0 : 64 * s) + (wtid >> 4);
             const int r_count = g.shared ? 16 : 8;                 // rows per thread, 8 apart
             const int c = wtid & 15;                               // 16-byte chunk of the row
-            const uint32_t qs = smem_u32(smem) + blk * kQBytes + (c >> 3) * 16384;
-#pragma unroll 2
+            uint32_t dst = smem_u32(smem) + blk * kQBytes + (c >> 3) * 16384 + r_first * 128 + (((c & 7) ^ (r_first & 7)) << 4);
+            // Eight rows on are dn nodes and dh heads on, and after a node's last head comes the next node's first: no division
+            // per row (the 240 rows of a unit at 47K context took 2.3 us to ask for with two).
+            const unsigned dn = row_node(p, 8), dh = 8u - dn * (unsigned)G;
+            unsigned rr = (unsigned)(blk * 128 + r_first);
+            const unsigned node = row_node(p, rr);
+            unsigned hg = rr - node * (unsigned)G;
+            const __nv_bfloat16* src = p.q + ((long long)(g.node_base + node) * p.num_q_heads + g.h * G + hg) * kHeadDim + c * 8;
+            const long long step = ((long long)dn * p.num_q_heads + dh) * kHeadDim, wrap = (long long)(p.num_q_heads - G) * kHeadDim;
+#pragma unroll 4
             for (int j = 0; j < r_count; ++j) {
-                const int r = r_first + 8 * j;
-                const unsigned rr = (unsigned)(blk * 128 + r);
                 const bool valid = rr < (unsigned)g.M;
-                const unsigned node = rr / (unsigned)G, hg = rr - node * (unsigned)G;
-                const __nv_bfloat16* src =
-                    valid ? p.q + ((long long)(g.node_base + node) * p.num_q_heads + g.h * G + hg) * kHeadDim + c * 8 : p.q;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(qs + r * 128 + (((c & 7) ^ (r & 7)) << 4)),
-                             "l"(src), "r"(valid ? 16 : 0) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(valid ? src : p.q), "r"(valid ? 16 : 0)
+                             : "memory");
+                dst += 1024; rr += 8; src += step; hg += dh;
+                if (hg >= (unsigned)G) { hg -= (unsigned)G; src += wrap; }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
@@ -634,7 +628,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         mbar_arrive(smem_u32(&aux->q_full));
 
         const int rr = (g.shared ? s * 128 : 0) + row_local;       // packed row of this thread
-        const unsigned long long anc_row = rr < g.M ? aux->anc[rr / G] : 0ull;
+        const unsigned long long anc_row = rr < g.M ? aux->anc[row_node(p, rr)] : 0ull;
         const bool bad_tree = aux->seg_bad_tree != 0;
         const int n_it = g.iters(s);
         const int live = g.template live_warps<kWide>();
@@ -865,7 +859,8 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         const bool write_ok = !bad && !*abort_flag;
         // only the first and the last unit of a CTA's piece can be cut: two partial slots per CTA
         const long long part_row = (2ll * blockIdx.x + (seg_no > 0 ? 1 : 0)) * kRows + rr;
-        const long long out_row = rr < g.M ? (long long)(g.node_base + rr / G) * p.num_q_heads + g.h * G + rr % G : 0;
+        const int node = (int)row_node(p, rr);
+        const long long out_row = rr < g.M ? (long long)(g.node_base + node) * p.num_q_heads + g.h * G + (rr - node * G) : 0;
         const bool row_ok = write_ok && rr < g.M;
         const bool whole = g.whole();
         // staging for coalesced stores: the Q blocks are idle now (every MMA of the segment is done); stream 1's
@@ -932,7 +927,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
 }
 
 // ------------------------------------------------------------------------------------------ kernel
-// kManySeqs: more than 32 sequences (the block-wide schedule); kWide: some unit may have more than 128 rows.
+// kManySeqs: the block-wide schedule (more than 32 sequences, or a line too long for 32 bits); kWide: some unit may have more than 128 rows.
 // Separate instances, so that a launch carries only the code of its own case: the text of the paths a launch never takes
 // still costs it time (3 us of 39 on a 32K-context, 32-node step when the block-wide schedule was compiled in).
 // kFused: the verify step's logits scan rides along.  Warps 2 and 3 have no part in the attention; they take the
@@ -974,6 +969,17 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = aux->tmem_base;
+    // What the schedule reads first is brought to L2 while the kernel before this one runs out (a prefetch reads nothing: it
+    // may come before the wait): lengths and offsets, and of the block table each CTA its own 32 lines.
+    if (warp == 2) {
+        const long long line = 32ll * blockIdx.x + lane;
+        if (line * 128 < (long long)p.batch * p.max_pages_per_seq * 4) l2_prefetch(reinterpret_cast<const char*>(p.block_table) + line * 128);
+        if (lane * 32 < p.batch) {
+            l2_prefetch(p.ctx_lens + lane * 32);
+            if (p.node_offsets) l2_prefetch(p.node_offsets + lane * 32);
+        }
+        if (lane * 32 < p.total_nodes) l2_prefetch(p.tree_parent + lane * 32);
+    }
     // Launched as a programmatic dependent itself: everything so far touched no input.  Each role waits for the kernel
     // before this one in the stream itself, after the jump into its code (a no-op in an ordinary launch).
     // The combine kernel is launched as a programmatic dependent and may queue up behind this grid's CTAs from then
@@ -983,8 +989,8 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     };
-    Walker w;
-    if (kManySeqs) {                    // the block-wide schedule
+    Walker<kManySeqs> w;
+    if constexpr (kManySeqs) {          // the block-wide schedule
         wait_for_inputs();
         build_walk(p, aux, w);
     }
@@ -999,8 +1005,8 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         if (!kManySeqs) wait_for_inputs();
         if (warp == 0) {
-            if (!kManySeqs) build_walk_small(p, w);
-            producer_loop<kWide>(p, &kmap, &vmap, aux, smem_base + kRingOff, w);
+            if constexpr (!kManySeqs) build_walk_small(p, w);
+            producer_loop<kWide, kManySeqs>(p, &kmap, &vmap, aux, smem_base + kRingOff, w);
         } else if (warp == 1) {
             mma_loop<kWide, kF16>(aux, smem_base, tmem);
         } else if (kFused) {

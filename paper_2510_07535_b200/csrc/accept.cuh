@@ -85,28 +85,55 @@ __device__ __forceinline__ unsigned long long argmax_key(float x, uint32_t idx) 
     return ((unsigned long long)u << 32) | (uint32_t)(~idx);
 }
 
-// Called by every thread of a CTA of kArgmaxThreads: a node's chunk keys are read by several neighbouring threads, all
-// in one memory round trip; after that thread i is node i and the others only keep the barriers company.
-__device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int b) {
-    const int i = threadIdx.x;
+// The kernel before this one in the stream has completed and its writes are visible; the next one may queue up.
+__device__ __forceinline__ void wait_and_let_dependents_start() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// One sequence's walk; called by the first kArgmaxThreads threads of a CTA.  A node's chunk keys are read by several
+// neighbouring threads, all in one memory round trip; the rest is the first warp's, two nodes per lane.
+// `keys()` waits for the kernel that leaves the arg-max keys and returns them.  The tree is read before: the kernels that
+// call this are dependents of one that lets them start only when everything before it has completed, and that writes no
+// tree.  With the ancestors as bits by then, what is left when the keys are there is one round of loads, one CTA barrier
+// and a handful of votes.
+template <typename Keys>
+__device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int b, Keys keys) {
+    constexpr unsigned kAll = 0xffffffffu;
+    static_assert(kMaxNodes == 64, "two nodes per lane of a warp");
+    static_assert(kArgmaxThreads >= 4 * kMaxNodes, "at least four threads per node");
+    __shared__ int s_parent[kMaxNodes], s_am[kMaxNodes];
+    const int i = threadIdx.x, lane = i & 31;
     const int base = p.node_offsets ? p.node_offsets[b] : b * p.nodes_uniform;
     const int n = p.node_offsets ? p.node_offsets[b + 1] - base : p.nodes_uniform;
-    __shared__ int s_parent[kMaxNodes], s_am[kMaxNodes], s_tok[kMaxNodes];
-    __shared__ int s_bad, s_win, s_leaf;
-    if (i == 0) {
-        s_bad = (n < 1 || n > p.max_nodes || n > p.path_stride || base < 0 || base + n > p.total_nodes) ? 1 : 0;
-        s_win = 0;
-        s_leaf = kMaxNodes;
+    const bool shape_ok = n >= 1 && n <= p.max_nodes && n <= p.path_stride && base >= 0 && base + n <= p.total_nodes;
+    int parent[2] = {-1, -1}, tok[2] = {-1, -1};
+    unsigned long long anc[2] = {0ull, 0ull};          // the node and its ancestors
+    bool bad = false;
+    if (i < 32 && shape_ok) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int node = lane + 32 * h;
+            if (node >= n) continue;
+            parent[h] = p.tree_parent[base + node];
+            tok[h] = p.draft_tokens[base + node];
+            bad = bad || (node == 0 ? parent[h] != -1 : parent[h] < 0 || parent[h] >= node);
+            s_parent[node] = parent[h];
+        }
+        bad = __any_sync(kAll, bad);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (!bad && lane + 32 * h < n)
+                for (int c = lane + 32 * h; c >= 0; c = s_parent[c]) anc[h] |= 1ull << c;      // parents come first: it ends
     }
-    __syncthreads();
-    if (s_bad) { if (i == 0) report(p.status, kErrBadTree); return; }
+    const unsigned long long* part_keys = keys();
+    if (!shape_ok) { if (i == 0) report(p.status, kErrBadTree); return; }
     {
-        static_assert(kArgmaxThreads >= 4 * kMaxNodes, "at least four threads per node");
         const int lg = n > 32 ? 2 : n > 16 ? 3 : n > 8 ? 4 : 5;       // 4 to 32 threads per node
         const int node = i >> lg, sub = i & ((1 << lg) - 1);
         unsigned long long k = 0;
         if (node < n) {
-            const unsigned long long* pk = p.part_keys + (long long)(base + node) * p.chunks;
+            const unsigned long long* pk = part_keys + (long long)(base + node) * p.chunks;
             for (int c0 = sub; c0 < p.chunks; c0 += 8 << lg) {
                 unsigned long long v[8];
 #pragma unroll
@@ -116,7 +143,7 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
             }
         }
         for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
+            const unsigned long long other = __shfl_xor_sync(kAll, k, o);
             k = other > k ? other : k;
         }
         if (node < n && sub == 0) {
@@ -125,45 +152,35 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
             if (p.node_argmax) p.node_argmax[base + node] = am;
         }
     }
-    if (i < n) {
-        const int pi = p.tree_parent[base + i];
-        s_parent[i] = pi;
-        s_tok[i] = p.draft_tokens[base + i];
-        if ((i == 0 && pi != -1) || (i > 0 && (pi < 0 || pi >= i))) atomicExch(&s_bad, 1);
-    }
-    __syncthreads();
-    if (s_bad) { if (i == 0) report(p.status, kErrBadTree); return; }
+    asm volatile("bar.sync 0, %0;" ::"n"(kArgmaxThreads) : "memory");
+    if (i >= 32) return;
+    if (bad) { if (i == 0) report(p.status, kErrBadTree); return; }
 
-    // ok(i): every edge on the root path of i matches; depth(i): number of edges
-    int key = 0;
-    if (i < n) {
-        bool ok = true;
-        int depth = 0;
-        for (int c = i; s_parent[c] >= 0 && depth < kMaxNodes; c = s_parent[c], ++depth)
-            ok = ok && s_tok[c] >= 0 && s_tok[c] == s_am[s_parent[c]];
-        if (ok) key = ((depth + 1) << 8) | (kMaxNodes - 1 - i);   // deeper first, then lower index
-    }
-    atomicMax(&s_win, key);
-    __syncthreads();
-    if (p.spec_node) {
-        // Section 3.2.2 "Decode Stage": the hidden state handed to the drafter is that of the [SPEC] which follows
-        // the accepted path, i.e. the [SPEC] child of its last node (lowest index if several, -1 if none)
-        const int win = kMaxNodes - 1 - (s_win & 0xff);
-        if (i < n && s_parent[i] == win && s_tok[i] < 0) atomicMin(&s_leaf, i);
-        __syncthreads();
-        if (i == 0) p.spec_node[b] = s_leaf < kMaxNodes ? s_leaf : -1;
-    }
-    {
-        const int win = kMaxNodes - 1 - (s_win & 0xff);
-        const int len = s_win >> 8;
-        int32_t* path = p.accept_path + (long long)b * p.path_stride;
-        for (int k = len + i; k < p.path_stride; k += blockDim.x) path[k] = -1;     // the padding, all threads
-        if (i == 0) {
-            p.accept_len[b] = len;
-            p.bonus_token[b] = s_am[win];
-            int k = len - 1;
-            for (int c = win; c >= 0 && k >= 0; c = s_parent[c]) path[k--] = c;
-        }
+    // a node is accepted if it and all its ancestors but the root are what the verifier chose at their parents
+    unsigned long long match = 1ull;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        match |= (unsigned long long)__ballot_sync(kAll, parent[h] >= 0 && tok[h] >= 0 && tok[h] == s_am[max(parent[h], 0)]) << (32 * h);
+    unsigned best = 0;                                  // deepest, then lowest index
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (anc[h] && !(anc[h] & ~match)) best = max(best, (unsigned)__popcll(anc[h]) << 8 | (unsigned)(kMaxNodes - 1 - lane - 32 * h));
+    best = __reduce_max_sync(kAll, best);
+    const int win = kMaxNodes - 1 - (int)(best & 0xffu), len = (int)(best >> 8);
+    const unsigned long long anc_win = __shfl_sync(kAll, win >= 32 ? anc[1] : anc[0], win & 31);
+    int32_t* path = p.accept_path + (long long)b * p.path_stride;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)                         // parents come first: a path is its nodes in ascending order
+        if (anc_win >> (lane + 32 * h) & 1ull) path[__popcll(anc_win & ((1ull << (lane + 32 * h)) - 1ull))] = lane + 32 * h;
+    for (int k = len + lane; k < p.path_stride; k += 32) path[k] = -1;
+    // Section 3.2.2 "Decode Stage": the hidden state handed to the drafter is that of the [SPEC] which follows
+    // the accepted path, i.e. the [SPEC] child of its last node (lowest index if several, -1 if none)
+    const unsigned leaf0 = __ballot_sync(kAll, lane < n && parent[0] == win && tok[0] < 0);
+    const unsigned leaf1 = __ballot_sync(kAll, lane + 32 < n && parent[1] == win && tok[1] < 0);
+    if (lane == 0) {
+        p.accept_len[b] = len;
+        p.bonus_token[b] = s_am[win];
+        if (p.spec_node) p.spec_node[b] = leaf0 ? __ffs(leaf0) - 1 : leaf1 ? __ffs(leaf1) + 31 : -1;
     }
 }
 
@@ -293,21 +310,22 @@ __global__ void __launch_bounds__(kArgmaxThreads, kArgmaxCtasPerSm) argmax_parti
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// One sequence's acceptance walk per CTA over the keys the scan left.  Launched as a programmatic dependent: it reads
-// nothing before the kernel before it has completed.
+// One sequence's acceptance walk per CTA over the keys the scan left.  Launched as a programmatic dependent of the scan.
 __global__ void __launch_bounds__(kArgmaxThreads) accept_walk_kernel(const AcceptParams p) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    accept_walk_seq(p, (int)blockIdx.x);
+    accept_walk_seq(p, (int)blockIdx.x, [&] {
+        wait_and_let_dependents_start();
+        return (const unsigned long long*)p.part_keys;
+    });
 }
 // The same over the keys of the LM-head product (a kernel of its own, so that the short acceptances do not carry the choice
 // of the set).
-__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_sets_kernel(AcceptParams p, const KeySets sets) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const uint32_t call = __ldcg(sets.call + 1);
-    p.part_keys = sets.keys + (size_t)(call & 1u) * sets.stride;
-    accept_walk_seq(p, (int)blockIdx.x);
+__global__ void __launch_bounds__(kArgmaxThreads) accept_walk_sets_kernel(const AcceptParams p, const KeySets sets) {
+    uint32_t call = 0;
+    accept_walk_seq(p, (int)blockIdx.x, [&] {
+        wait_and_let_dependents_start();
+        call = __ldcg(sets.call + 1);
+        return (const unsigned long long*)(sets.keys + (size_t)(call & 1u) * sets.stride);
+    });
     unsigned long long* idle = sets.keys + (size_t)((call + 1u) & 1u) * sets.stride;
     for (int i = blockIdx.x * kArgmaxThreads + threadIdx.x; i < sets.stride; i += gridDim.x * kArgmaxThreads) idle[i] = 0ull;
     if (blockIdx.x == 0 && threadIdx.x == 0) sets.call[0] = call + 1u;

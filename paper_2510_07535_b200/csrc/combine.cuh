@@ -10,6 +10,8 @@
 namespace owl {
 
 constexpr int kCombineWarps = 8;
+constexpr int kCombineThreads = (kCombineWarps + 1) * 32;     // and one that rehearses
+constexpr int kRehearsedPartials = 5;                         // the unrolled loops and what they leave over
 constexpr int kCombineCtasPerSm = 4;
 constexpr int kCombineRows = 8;            // a unit's rows that a CTA merges at a time
 
@@ -21,17 +23,28 @@ inline int combine_group(long long units, int ctas) {
     const long long g = (ctas + units - 1) / units + 2;
     return (int)(g < 4 ? 4 : g < 32 ? g : 32);
 }
-inline size_t combine_stage_bytes(int group) { return (size_t)kCombineWarps * group * 34 * sizeof(float4); }
+__host__ __device__ inline int rehearsed_partials(int group) { return group < kRehearsedPartials ? group : kRehearsedPartials; }
+inline size_t combine_stage_bytes(int group, int lg_parts) {
+    return (size_t)((kCombineWarps >> lg_parts) * group + rehearsed_partials(group)) * 34 * sizeof(float4);
+}
 inline int combine_ctas_per_sm(int group) {
-    const int fit = (int)((227u << 10) / (combine_stage_bytes(group) + 1024));
+    const int fit = (int)((227u << 10) / (combine_stage_bytes(group, 0) + 1024));
     return fit < kCombineCtasPerSm ? fit : kCombineCtasPerSm;
+}
+// CTAs that share a block's channels: 1, 2 or 4, as long as every one still has an SM to itself.  What a merge waits for is
+// the partials that one SM takes in and folds, 70 KB for the eight rows of a block at 2K context (chain of 8 nodes: 32 blocks on 128 SMs
+// instead of 32, and the schedule's shorter divisions, 12.1 -> 11.5 us per step).
+inline int combine_lg_parts(long long blocks, int other_ctas, int sms) {
+    int lg = 0;
+    while (lg < 2 && (blocks << (lg + 1)) + other_ctas <= sms) ++lg;
+    return lg;
 }
 // What a launch of `ctas` CTAs asks for: its stage, and enough that no SM takes more than its share of them.  The
 // SMs whose attention CTA ends first would otherwise collect several merge CTAs each (2K context, 33 CTAs: 15.5 -> 16.1 us
 // per step).
-inline size_t combine_smem_bytes(int group, unsigned ctas, int sms) {
+inline size_t combine_smem_bytes(int group, int lg_parts, unsigned ctas, int sms) {
     const unsigned share = (ctas + (unsigned)sms - 1) / (unsigned)sms;
-    const size_t spread = (227u << 10) / (share + 1) + 16, stage = combine_stage_bytes(group);
+    const size_t spread = (227u << 10) / (share + 1) + 16, stage = combine_stage_bytes(group, lg_parts);
     return stage > spread ? stage : spread;
 }
 
@@ -60,47 +73,62 @@ inline size_t combine_smem_bytes(int group, unsigned ctas, int sms) {
 // the fold were two loops unrolled 32 times, some 450 instructions that a warp with one row executes exactly once,
 // at the pace of instruction fetches from L2.
 template <bool kFused>
-__global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine_sched_kernel(const AttnParams p, const AcceptParams ap) {
+__global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sched_kernel(const AttnParams p, const AcceptParams ap) {
     const unsigned row_ctas = (unsigned)p.combine_row_ctas;
     if (kFused) {
         if (blockIdx.x >= row_ctas) {
-            static_assert(kCombineWarps * 32 == kArgmaxThreads, "the walk's block");
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            accept_walk_seq(ap, (int)(blockIdx.x - row_ctas));
+            static_assert(kCombineThreads >= kArgmaxThreads, "the walk's block");
+            if (threadIdx.x < kArgmaxThreads)
+                accept_walk_seq(ap, (int)(blockIdx.x - row_ctas), [&] {
+                    wait_and_let_dependents_start();
+                    return (const unsigned long long*)ap.part_keys;
+                });
             return;
         }
     }
-    // The row CTAs are persistent: a warp derives the schedule once and then takes blocks first, first + row_ctas, ...
+    // The row CTAs are persistent: a warp derives the schedule once and then takes blocks first, first + stride, ...
     // (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived 8192 times).  Blocks are
     // numbered unit by unit for the first eight rows of all units, then for the second eight and so on, up to the rows of
     // the most nodes a sequence may have: what shorter sequences lack lies at the end.
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = lane & 7, chunk = warp * 4 + (lane >> 3);      // row of the block; group of four channels
+    // The ninth warp rehearses: it runs the code that follows the wait on whatever the first slots hold (M stays 0, so
+    // nothing is written), while the others derive the schedule and wait.  That code runs once or twice per launch, and its lines
+    // used to be fetched when the partials were there already (2.9 -> 2.5 us after the wait; 2K step 12.4 -> 12.1 with the walk's
+    // reads before its wait).
+    const bool rehearsal = warp == kCombineWarps;
+    // A block is shared out to combine_parts CTAs, each with a part of the channels and of the eight warps.
+    const int warps = kCombineWarps >> p.combine_lg_parts, part_no = (int)blockIdx.x & ((1 << p.combine_lg_parts) - 1);
+    if (!rehearsal && warp >= warps) return;
+    const int r = lane & 7, chunk = rehearsal ? lane >> 3 : (part_no * warps + warp) * 4 + (lane >> 3);   // row of the block; four channels
+    const unsigned first_id = blockIdx.x >> p.combine_lg_parts, stride = row_ctas >> p.combine_lg_parts;
     extern __shared__ float4 combine_stage[];          // per warp: [group][32] pieces of the partials, [group][8] LSEs
-    const int group = p.combine_group;
-    float4* stage = combine_stage + warp * group * 34;
+    const int group = rehearsal ? rehearsed_partials(p.combine_group) : p.combine_group;
+    float4* stage = combine_stage + (rehearsal ? warps : warp) * p.combine_group * 34;
     float* lse_stage = reinterpret_cast<float*>(stage + group * 32);
     const uint32_t stage_u32 = (uint32_t)__cvta_generic_to_shared(stage + lane);
-    const unsigned units = (unsigned)(p.batch * p.num_kv_heads);
-    const unsigned blocks = units * (unsigned)((p.group * p.max_nodes + kCombineRows - 1) / kCombineRows);
     WarpSchedule ws{};
     // per block: its unit's row count, the first partial's slot and the number of partials (0: nothing to merge)
     int M = 0, h = 0, row = 0, node_base = 0, slot = 0, count = 0;
-    auto plan = [&](unsigned k, int n, int tiles, auto t0, const auto& part) {
-        row = (int)k * kCombineRows + r;
+    auto plan = [&](int k, int n, int tiles, auto t0, const auto& part) {
+        row = k * kCombineRows + r;
         M = n * p.group;
         count = 0;
-        if (tiles == 0 || (int)k * kCombineRows >= M) return;      // not scheduled, or no such rows
-        const int c0 = part.owner(t0 + part.pen), c1 = part.owner(t0 + part.pen + tiles - 1);
+        if (tiles == 0 || k * kCombineRows >= M) return;      // not scheduled, or no such rows
+        // the CTAs that hold its first tile, its last one and, if it is not the line's first, the place before its gap: three
+        // lanes find one each
+        auto place = t0 + part.pen;
+        if (lane == 1) place += tiles - 1;
+        if (lane == 2) place = t0 > 0 ? t0 - 1 : 0;
+        const int mine = part.owner(place);
+        const int c0 = __shfl_sync(0xffffffffu, mine, 0), c1 = __shfl_sync(0xffffffffu, mine, 1), before = __shfl_sync(0xffffffffu, mine, 2);
         if (c0 == c1) return;              // a single CTA saw every key of this unit and wrote the result itself
-        // the unit's first CTA may have come from another unit; the others' pieces start in this one
-        slot = 2 * c0 + (part.begin(c0) < t0 ? 1 : 0);
+        // the unit's first CTA may have come from another unit or from the gap before that; the others' pieces start in this one
+        slot = 2 * c0 + (t0 > 0 && before == c0 ? 1 : 0);
         count = c1 - c0 + 1;
     };
     auto locate = [&](unsigned id) {       // every lane of the warp, same block
-        const unsigned k = id / units, u = id - k * units, b = u / (unsigned)p.num_kv_heads;
-        h = (int)(u - b * (unsigned)p.num_kv_heads);
+        const int units = p.batch * p.num_kv_heads, k = div_small((int)id, units), u = (int)id - k * units, b = div_small(u, p.num_kv_heads);
+        h = u - b * p.num_kv_heads;
         if (p.small) {
             const int n = __shfl_sync(0xffffffffu, ws.n, b), tiles = __shfl_sync(0xffffffffu, ws.tiles, b);
             node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
@@ -110,22 +138,24 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             const SchedHeader hdr = *p.sched_header;      // larger batches read the schedule the pass left
             part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
             const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
-            node_base = seq_node_base(p, (int)b);
+            node_base = seq_node_base(p, b);
             const int tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
-            plan(k, seq_nodes(p, (int)b), tiles, sb + (long long)h * (tiles + part.pen), part);
+            plan(k, seq_nodes(p, b), tiles, sb + (long long)h * (tiles + part.pen), part);
         }
     };
     // latency after the pass has ended is what this kernel costs: whatever needs no output of the pass comes before
     // the wait - for batches of at most 32 sequences the whole plan of the first block
-    if (p.small) {
+    if (rehearsal) {
+        row = r;
+        count = min(kRehearsedPartials, p.num_ctas);
+    } else if (p.small) {
         ws = warp_schedule(p);
-        locate(blockIdx.x);
+        locate(first_id);
     }
     // from here on the split-KV pass has completed and its writes are visible (a no-op in an ordinary launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel in the stream may queue up
-    for (unsigned id = blockIdx.x; id < blocks; id += row_ctas) {
-        if (!p.small || id != blockIdx.x) locate(id);
+    if (!rehearsal) wait_and_let_dependents_start();
+    for (unsigned id = first_id; id < (unsigned)p.combine_blocks; id += stride) {
+        if (!rehearsal && (!p.small || id != first_id)) locate(id);
         if (count == 0) continue;
         // Partials are taken `group` at a time, their LSEs with them: one memory round trip per group.  Groups are folded
         // online (running maximum, each lane its own row's).
@@ -134,7 +164,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
         bool bad = false;
         // slots of neighbouring CTAs lie two apart; only the first CTA's partial may be its second
         const float4* src = reinterpret_cast<const float4*>(p.part_o) + (slot * 32ll + chunk) * kMaxRows + row;
-        const float4* next = src + (slot & 1 ? 32 : 64) * kMaxRows;
+        int step = slot & 1 ? 32 * kMaxRows : 64 * kMaxRows;
         for (int base = 0; base < count; base += group) {
             const int cnt = count - base < group ? count - base : group;
             if (base > 0) __syncwarp();                  // the stage's weights of the round before have been read
@@ -147,8 +177,8 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
 #pragma unroll 4
             for (int j = 0; j < cnt; ++j) {
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_u32 + (uint32_t)j * 512u), "l"(src) : "memory");
-                src = next;
-                next += 64 * kMaxRows;
+                src += step;
+                step = 64 * kMaxRows;
             }
             asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
             __syncwarp();
@@ -182,8 +212,6 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
                 acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
             }
         }
-        // a bad tree or page in the unit's sequence: no output (the same for all of its rows; rows past the last hold nothing)
-        if (__any_sync(0xffffffffu, bad) || row >= M) continue;
         const float inv = sum > 0.f ? 1.f / sum : 0.f;
         uint2 pk;
         if (p.f16) {
@@ -195,10 +223,16 @@ __global__ void __launch_bounds__(kCombineWarps * 32, kCombineCtasPerSm) combine
             pk.x = *reinterpret_cast<uint32_t*>(&lo2);
             pk.y = *reinterpret_cast<uint32_t*>(&hi2);
         }
+        const float lse = sum > 0.f ? mx + logf(sum) : -INFINITY;
         const int node = (int)row_node(p, row);
         const long long out_row = (long long)(node_base + node) * p.num_q_heads + h * p.group + (row - node * p.group);
-        *reinterpret_cast<uint2*>(p.out + out_row * kHeadDim + chunk * 4) = pk;
-        if (p.lse && chunk == 0) p.lse[out_row] = sum > 0.f ? mx + logf(sum) : -INFINITY;
+        // rows past the unit's last hold nothing; a bad tree or page in the unit's sequence (the same for all of its rows): no
+        // output
+        if (!__any_sync(0xffffffffu, bad) && row < M) {
+            *reinterpret_cast<uint2*>(p.out + out_row * kHeadDim + chunk * 4) = pk;
+            if (p.lse && chunk == 0) p.lse[out_row] = lse;
+        }
+        if (rehearsal) break;
     }
 }
 

@@ -48,7 +48,9 @@ struct AttnParams {
     int32_t small;                // the schedule is derived by single warps in 32-bit arithmetic (small_schedule)
     int32_t num_ctas;             // CTAs of the split-KV pass (the flat tile range is cut into this many pieces)
     int32_t combine_group;        // partials per round of the merge kernel, 4..32
-    int32_t combine_row_ctas;     // CTAs of the merge kernel that take output rows (persistent, eight warps each)
+    int32_t combine_blocks;       // blocks of eight packed rows that the merge kernel goes through
+    int32_t combine_lg_parts;     // log2 of the CTAs that share a block's channels
+    int32_t combine_row_ctas;     // the merge kernel's CTAs that take rows (persistent)
     int32_t f16;                  // q / caches / out are fp16 instead of bf16 (same size; typed as bf16 pointers here)
     float sm_scale;
 };
@@ -87,6 +89,17 @@ constexpr int kBoundaryPenaltyTiles = 5;
 // T: places on the line.  int where the host has made sure that the line is short (small_schedule).  Every CTA derives its
 // piece once, on its critical path, where the code is not in the instruction caches and one instruction waits for the one
 // before: instructions are time there.
+
+// x / d for 0 <= x < 2^24, 0 < d and a quotient below 2^21: both are exact in fp32, the quotient of __fdividef (2 ulp) is off by
+// less than one, and the remainder says which way.  Half the instructions of an integer division.
+__device__ __forceinline__ int div_small(int x, int d) {
+    int q = (int)__fdividef((float)x, (float)d);
+    const int r = x - q * d;
+    if (r < 0) --q;
+    if (r >= d) ++q;
+    return q;
+}
+
 template <typename T>
 struct Partition {
     static constexpr bool kShort = sizeof(T) == 4;
@@ -94,60 +107,52 @@ struct Partition {
     int rem, ctas;
     int unit_tiles, base, urem;   // aligned mode iff unit_tiles > 0
     int pen;                      // gap in front of a unit's tiles
-    __device__ __host__ void init(T tiles, int ctas_, int units, int uniform_tiles) {
+    static __device__ __forceinline__ T div(T x, T d) {
+        if constexpr (kShort) return div_small(x, d);
+        else if (x >= 0 && x <= 0x7fffffffll && d <= 0x7fffffffll) return (T)((unsigned)x / (unsigned)d);
+        else return x / d;
+    }
+    __device__ __forceinline__ void init(T tiles, int ctas_, int units, int uniform_tiles) {
         ctas = ctas_;
         pen = kBoundaryPenaltyTiles;
         total = tiles + (T)pen * units;
-        if (kShort || (total >= 0 && total <= 0x7fffffffll)) {
-            const unsigned qq = (unsigned)total / (unsigned)ctas_;
-            q = (T)qq; rem = (int)((unsigned)total - qq * (unsigned)ctas_);
-        } else {
-            q = total / ctas_; rem = (int)(total % ctas_);
-        }
+        q = div(total, ctas);
+        rem = (int)(total - q * ctas);
         unit_tiles = 0; base = 0; urem = 0;
-        if (uniform_tiles > 0 && units > 1 && units <= ctas_) {
-            const unsigned b = (unsigned)ctas_ / (unsigned)units;
-            if ((T)(((unsigned)uniform_tiles + b - 1u) / b) < q + (rem ? 1 : 0)) {
-                unit_tiles = uniform_tiles; base = (int)b; urem = ctas_ - (int)b * units;
+        if (uniform_tiles > 0 && units > 1 && units <= ctas) {
+            const int b = (int)div(ctas, units);
+            if (div((T)uniform_tiles + b - 1, b) < q + (rem ? 1 : 0)) {
+                unit_tiles = uniform_tiles; base = b; urem = ctas - b * units;
                 total = tiles; pen = 0;
             }
         }
     }
-    // [begin(c), begin(c + 1)) with one set of divisions (the pieces of a unit tile it exactly, so a piece's end is
-    // its begin plus its length in either mode)
-    __device__ __host__ void range(int c, T& t_begin, T& t_end) const {
+    // piece c, [t_begin, t_end)
+    __device__ __forceinline__ void range(int c, T& t_begin, T& t_end) const {
         if (unit_tiles == 0) {
-            t_begin = (T)c * q + (c < rem ? c : rem);
+            t_begin = (T)c * q + min(c, rem);
             t_end = t_begin + q + (c < rem ? 1 : 0);
             return;
         }
-        const int big = urem * (base + 1);
-        int u, k, cu;
-        if (c < big) { u = (int)((unsigned)c / (unsigned)(base + 1)); k = c - u * (base + 1); cu = base + 1; }
-        else { u = urem + (int)((unsigned)(c - big) / (unsigned)base); k = (c - big) - (u - urem) * base; cu = base; }
-        const int qq = (int)((unsigned)unit_tiles / (unsigned)cu), rr = unit_tiles - qq * cu;
-        t_begin = (T)u * unit_tiles + (T)k * qq + (k < rr ? k : rr);
+        // the first urem units have one piece more
+        const int big = urem * (base + 1), cu = c < big ? base + 1 : base;
+        const int x = c < big ? c : c - big, u = (int)div(x, cu), k = x - u * cu;
+        const int qq = (int)div(unit_tiles, cu), rr = unit_tiles - qq * cu;
+        t_begin = (T)(c < big ? u : urem + u) * unit_tiles + (T)k * qq + min(k, rr);
         t_end = t_begin + qq + (k < rr ? 1 : 0);
     }
-    __device__ __host__ T begin(int c) const {
-        T t_begin, t_end;
-        range(c, t_begin, t_end);
-        return t_begin;
-    }
-    __device__ __host__ int owner(T t) const {        // of a place on the line
-        if (unit_tiles == 0) {
-            const T big = (T)rem * (q + 1);
-            if (kShort || total <= 0x7fffffffll) {
-                const unsigned tt = (unsigned)t, qq = (unsigned)q, bb = (unsigned)big;
-                return tt < bb ? (int)(tt / (qq + 1u)) : rem + (int)((tt - bb) / qq);
-            }
-            return t < big ? (int)(t / (q + 1)) : rem + (int)((t - big) / q);
+    __device__ __forceinline__ int owner(T t) const {        // of a place on the line
+        T x = t, head = (T)rem * (q + 1), d = q;             // pieces, the first rem of them of d + 1 places
+        int first = 0, longer = rem;
+        if (unit_tiles > 0) {
+            const int u = (int)div(t, unit_tiles), cu = base + (u < urem ? 1 : 0);
+            x = t - (T)u * unit_tiles;
+            first = u * base + min(u, urem);
+            d = div(unit_tiles, cu);
+            longer = unit_tiles - (int)d * cu;
+            head = (T)longer * (d + 1);
         }
-        const int u = kShort || total <= 0x7fffffffll ? (int)((unsigned)t / (unsigned)unit_tiles) : (int)(t / unit_tiles);
-        const unsigned local = (unsigned)(t - (T)u * unit_tiles), cu = (unsigned)(base + (u < urem ? 1 : 0));
-        const int c0 = u * base + (u < urem ? u : urem);
-        const unsigned qq = (unsigned)unit_tiles / cu, rr = (unsigned)unit_tiles - qq * cu, bigl = rr * (qq + 1u);
-        return c0 + (int)(local < bigl ? local / (qq + 1u) : rr + (local - bigl) / qq);
+        return first + (x < head ? (int)div(x, d + 1) : longer + (int)div(x - head, d));
     }
 };
 

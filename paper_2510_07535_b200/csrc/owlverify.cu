@@ -275,7 +275,7 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
         ok = set_umma_smem_attr();
     }
     if (ok) {
-        const int most = (int)combine_stage_bytes(32);
+        const int most = (int)combine_stage_bytes(32, 0);
         ok = cudaFuncSetAttribute(combine_sched_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
              cudaFuncSetAttribute(combine_sched_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
     }
@@ -400,7 +400,9 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     p.combine_group = combine_group((long long)d->batch * d->num_kv_heads, ctx->num_ctas);
     const long long want_ctas = (long long)d->batch * d->num_kv_heads * ((G * d->max_nodes + kCombineRows - 1) / kCombineRows);
     const long long most_ctas = (long long)ctx->sm_count * combine_ctas_per_sm(p.combine_group);
-    const unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas : most_ctas);
+    p.combine_blocks = (int32_t)want_ctas;
+    p.combine_lg_parts = combine_lg_parts(want_ctas, ap ? d->batch : 0, ctx->sm_count);
+    const unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas << p.combine_lg_parts : most_ctas);
     p.combine_row_ctas = (int32_t)grid;
     {
         cudaLaunchConfig_t cfg = {};
@@ -422,12 +424,12 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     if (ctx->profiling) cudaEventRecord(ctx->ev[1], stream);
     if (own_scan && !ctx->profiling) launch_scan(ctx, *ap, stream, true);
     const bool walk_here = ap && !(own_scan && ctx->profiling);
-    const size_t stage_bytes = combine_smem_bytes(p.combine_group, grid + (walk_here ? (unsigned)d->batch : 0u), ctx->sm_count);
+    const size_t stage_bytes = combine_smem_bytes(p.combine_group, p.combine_lg_parts, grid + (walk_here ? (unsigned)d->batch : 0u), ctx->sm_count);
     if (walk_here)
-        launch_dependent_smem(combine_sched_kernel<true>, dim3(grid + (unsigned)d->batch), dim3(kCombineWarps * 32), stage_bytes, stream,
+        launch_dependent_smem(combine_sched_kernel<true>, dim3(grid + (unsigned)d->batch), dim3(kCombineThreads), stage_bytes, stream,
                               p, *ap);
     else
-        launch_dependent_smem(combine_sched_kernel<false>, dim3(grid), dim3(kCombineWarps * 32), stage_bytes, stream, p, AcceptParams{});
+        launch_dependent_smem(combine_sched_kernel<false>, dim3(grid), dim3(kCombineThreads), stage_bytes, stream, p, AcceptParams{});
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[2], stream); ctx->ev_attn_valid = true; }
     if (ap && !walk_here) launch_accept(ctx, *ap, stream);      // profiling: the halves timed apart

@@ -145,10 +145,10 @@ struct Walker {
         }
         if (b >= p.batch) { t = t_end; return false; }
         const int len = cur_tiles + pen;
-        const unsigned local = (unsigned)(t - seq_begin);   // < len * Hkv <= 2^24 * 2^7
+        const int local = (int)(t - seq_begin);             // < len * Hkv, a short line or at most 2^24 * 2^7
         g.b = b; g.n = cur_n; g.L = cur_L; g.tiles = cur_tiles;
-        g.h = (int)(local / (unsigned)len);
-        const int at = (int)(local - (unsigned)g.h * (unsigned)len);
+        g.h = kManySeqs ? (int)((unsigned)local / (unsigned)len) : div_small(local, len);
+        const int at = (int)((unsigned)local - (unsigned)g.h * (unsigned)len);
         const Place left = t_end - t;
         const int end = (int)(at + left < len ? at + left : len);
         t += end - at;
@@ -306,7 +306,7 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
     const int ppt = kTileKeys >> p.page_shift;               // pages (= TMA boxes) per tile
     const uint32_t box_bytes = (uint32_t)p.page_size * 256u;
     const int oob = p.num_pages * p.num_kv_heads;            // a coordinate past the end: the box reads zeros
-    uint32_t item = 0;
+    uint32_t slot = 0, free_parity = 1, tile_bar = 0;        // the ring goes round by tiles, K and V by turns
     // K/V are read once: let them leave L2 first, so that Q, the partials, the tables and the code stay
     const uint64_t stream_policy = l2_policy_evict_first();
     for (uint32_t seg_no = 0;; ++seg_no) {
@@ -347,20 +347,20 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
             if (t + 1 < g.tile1) page_next = page_of(t + 1);
 #pragma unroll
             for (int kv = 0; kv < 2; ++kv) {
-                const uint32_t slot = item % kSlots, ph = (item / kSlots) & 1u;
-                const uint32_t full = smem_u32(&aux->full[(item >> 1) % kTilesInFlight]);
-                // A slot whose wait gave up is left out, but `item` goes by the tiles all the same: K and V keep their slots, and
-                // the lanes, which may disagree about a wait that gives up, keep step.
-                const bool ok = mbar_wait(smem_u32(&aux->empty[slot]), ph ^ 1u, abort_flag);
+                const uint32_t full = smem_u32(&aux->full[tile_bar]);
+                // A slot whose wait gave up is left out, but the ring goes on by the tiles all the same: K and V keep their
+                // slots, and the lanes, which may disagree about a wait that gives up, keep step.
+                const bool ok = mbar_wait(smem_u32(&aux->empty[slot]), free_parity, abort_flag);
                 // the tile's barrier expects K and V together (announced with K; V follows as its slot frees up)
                 if (ok && lane == 0 && kv == 0) mbar_arrive_expect_tx(full, 2u * (uint32_t)kSlotBytes);
                 __syncwarp();
                 if (ok && lane < ppt)
                     tma_load_5d_hint(ring + slot * kSlotBytes + lane * box_bytes, kv ? vmap : kmap, full, 0, 0, 0, 0, c_cur,
                                      stream_policy);
-                ++item;
+                if (++slot == (uint32_t)kSlots) { slot = 0; free_parity ^= 1u; }
                 __syncwarp();
             }
+            if (++tile_bar == (uint32_t)kTilesInFlight) tile_bar = 0;
         }
     }
 }

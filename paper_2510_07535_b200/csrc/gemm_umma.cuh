@@ -493,119 +493,129 @@ struct CellParams {
     float alpha, eps;
 };
 
-// Sum of v over the CTA's threads; s_warp is free again after the second barrier.
-__device__ __forceinline__ float cell_block_sum(float v, float* s_warp) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+constexpr int kCellWarps = kCellThreads / 32;
+struct CellStats { float2 warp[kCellCluster][kCellWarps]; };      // (mean, sum of squared deviations) of a warp's columns
+
+__device__ __forceinline__ float cell_warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) s_warp[warp] = v;
-    __syncthreads();
-    float t = lane < kCellThreads / 32 ? s_warp[lane] : 0.f;
+    return v;
+}
+// Columns of a CTA with `count` of them that warp w holds.
+__device__ __forceinline__ int cell_warp_columns(int count, int w) {
+    int n = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    __syncthreads();
-    return t;
+    for (int k = 0; k < kCellPerThread; ++k) n += min(max(count - k * kCellThreads - w * 32, 0), 32);
+    return n;
 }
 
 // Mean and 1 / sqrt(variance + eps) over a whole row from the values x[] this thread holds (on[] says which exist).
-// Each CTA takes the mean and the sum of squared deviations of its own `count` columns (two block reductions), pushes
-// the pair into slot `which` of every CTA of the cluster, and after one cluster barrier all of them combine the eight
-// pairs in rank order by the pairwise-variance identity  M2 = sum_i M2_i + sum_i n_i (mean_i - mean)^2 : the same
-// numbers everywhere, no cancellation, and nobody reads a peer's shared memory after the barrier.
+// Each warp takes the mean and the sum of squared deviations of its own columns, pushes the pair into every CTA of the
+// cluster, and after one cluster barrier every warp combines all 128 pairs by the pairwise-variance identity
+// M2 = sum_i M2_i + sum_i n_i (mean_i - mean)^2 : the same numbers everywhere, no cancellation, and nobody reads a peer's
+// shared memory after the barrier.  (With a pair per CTA two block reductions, four barriers, stood before the exchange.)
 __device__ __forceinline__ void cluster_mean_rstd(const float (&x)[kCellPerThread], const bool (&on)[kCellPerThread], int count,
-                                                  int slice, int d, float eps, float* s_warp, float (*s_stat)[kCellCluster][2],
-                                                  int which, float& mean, float& rstd) {
+                                                  int slice, int d, float eps, CellStats& stats, float& mean, float& rstd) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float sum = 0.f;
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k) sum += on[k] ? x[k] : 0.f;
-    const float mean_cta = count > 0 ? cell_block_sum(sum, s_warp) / count : (cell_block_sum(sum, s_warp), 0.f);
+    const int n_warp = cell_warp_columns(count, warp);
+    const float mean_warp = cell_warp_sum(sum) / (float)max(n_warp, 1);
     float sq = 0.f;
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k)
-        if (on[k]) { const float t = x[k] - mean_cta; sq += t * t; }
-    const float m2_cta = cell_block_sum(sq, s_warp);
-    const int rank = (int)cluster.block_rank();
-    if (threadIdx.x < kCellCluster) {
-        float* dst = &cluster.map_shared_rank(s_stat, threadIdx.x)[which][rank][0];
-        dst[0] = mean_cta;
-        dst[1] = m2_cta;
-    }
+        if (on[k]) { const float t = x[k] - mean_warp; sq += t * t; }
+    const float m2_warp = cell_warp_sum(sq);
+    if (lane < kCellCluster) cluster.map_shared_rank(&stats, lane)->warp[cluster.block_rank()][warp] = make_float2(mean_warp, m2_warp);
     cluster.sync();
-    float total = 0.f;
+    constexpr int kPerLane = kCellCluster * kCellWarps / 32;
+    float2 pair[kPerLane];
+    float n[kPerLane], total = 0.f;
 #pragma unroll
-    for (int r = 0; r < kCellCluster; ++r) {
-        const int n_r = min(slice, max(d - r * slice, 0));
-        total += (float)n_r * s_stat[which][r][0];
+    for (int q = 0; q < kPerLane; ++q) {
+        const int at = q * 32 + lane, r = at / kCellWarps, w = at % kCellWarps;
+        pair[q] = stats.warp[r][w];
+        n[q] = (float)cell_warp_columns(min(slice, max(d - r * slice, 0)), w);
+        total += n[q] * pair[q].x;
     }
-    mean = total / d;
+    mean = cell_warp_sum(total) / d;
     float m2 = 0.f;
 #pragma unroll
-    for (int r = 0; r < kCellCluster; ++r) {
-        const int n_r = min(slice, max(d - r * slice, 0));
-        const float dm = s_stat[which][r][0] - mean;
-        m2 += s_stat[which][r][1] + (float)n_r * dm * dm;
+    for (int q = 0; q < kPerLane; ++q) {
+        const float dm = pair[q].x - mean;
+        m2 += pair[q].y + n[q] * dm * dm;
     }
-    rstd = rsqrtf(m2 / d + eps);
+    rstd = rsqrtf(cell_warp_sum(m2) / d + eps);
 }
 
 __device__ __forceinline__ float gelu_exact(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float sigmoid_f(float x) { return 1.f / (1.f + __expf(-x)); }
 
-__global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThreads) lstm_cell_kernel(const CellParams p) {
+__global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThreads, 2) lstm_cell_kernel(const CellParams p) {
     namespace cg = cooperative_groups;
-    __shared__ float s_warp[kCellThreads / 32];
-    __shared__ float s_stat[2][kCellCluster][2];     // [which normalisation][CTA of the cluster][mean, M2]
+    __shared__ CellStats s_stats[2];                 // of the two normalisations
     cg::cluster_group cluster = cg::this_cluster();
-    // may be launched as a programmatic dependent of the product that writes S; the kernel after this one may queue up
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long row = blockIdx.x / kCellCluster;
     const int d = p.d;
     const int slice = (d + kCellCluster - 1) / kCellCluster;
     const int j0 = (int)cluster.block_rank() * slice;             // this CTA's columns: [j0, min(j0 + slice, d))
     const int count = min(slice, max(d - j0, 0));
     const float* s = p.s + row * 4ll * d;
-    // everything a column needs is asked for at once: the four pre-activations, E(t) and z
+    // A programmatic dependent of the product that writes S and nothing else, and that lets its dependents start only when
+    // everything before it has completed: E(t), z and the affine parameters are read, and the cluster's CTAs meet (before anyone
+    // writes into a peer's shared memory), under the product's tail.
     float xc[kCellPerThread], sf[kCellPerThread], si[kCellPerThread], so[kCellPerThread], zo[kCellPerThread], zn[kCellPerThread];
+    float ae[kCellPerThread], gc[kCellPerThread], bc[kCellPerThread], gz[kCellPerThread], bz[kCellPerThread];
     bool on[kCellPerThread];
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k) {
         const int i = k * kCellThreads + threadIdx.x, j = j0 + i;
-        on[k] = i < slice && j < d;
-        xc[k] = sf[k] = si[k] = so[k] = zo[k] = zn[k] = 0.f;
+        on[k] = i < count;
+        xc[k] = sf[k] = si[k] = so[k] = zo[k] = zn[k] = ae[k] = bc[k] = bz[k] = 0.f;
+        gc[k] = gz[k] = 1.f;
         if (on[k]) {
-            const float ae = p.alpha * __bfloat162float(p.emb[row * d + j]);     // s^m = W^m h + alpha e  (Eq. 2)
-            sf[k] = s[j] + ae; si[k] = s[1ll * d + j] + ae; so[k] = s[2ll * d + j] + ae; xc[k] = s[3ll * d + j] + ae;
+            ae[k] = p.alpha * __bfloat162float(p.emb[row * d + j]);
             zo[k] = p.z[row * d + j];
+            if (p.gamma_c) gc[k] = p.gamma_c[j];
+            if (p.beta_c) bc[k] = p.beta_c[j];
+            if (p.gamma_z) gz[k] = p.gamma_z[j];
+            if (p.beta_z) bz[k] = p.beta_z[j];
         }
     }
-    cluster.sync();      // every CTA of the cluster is running before anyone writes into its shared memory (the loads fly)
+    cluster.sync();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the kernel after this one may queue up
+#pragma unroll
+    for (int k = 0; k < kCellPerThread; ++k) {
+        const int j = j0 + k * kCellThreads + threadIdx.x;
+        if (on[k]) {     // s^m = W^m h + alpha e  (Eq. 2)
+            xc[k] = __ldcg(s + 3ll * d + j) + ae[k]; sf[k] = __ldcg(s + j) + ae[k];
+            si[k] = __ldcg(s + 1ll * d + j) + ae[k]; so[k] = __ldcg(s + 2ll * d + j) + ae[k];
+        }
+    }
     float mean_c, rstd_c;
-    cluster_mean_rstd(xc, on, count, slice, d, p.eps, s_warp, s_stat, 0, mean_c, rstd_c);
+    cluster_mean_rstd(xc, on, count, slice, d, p.eps, s_stats[0], mean_c, rstd_c);
     // z' = z g^f + f(s^c) g^i  (Eq. 5-7)
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k) {
         const int j = j0 + k * kCellThreads + threadIdx.x;
         if (on[k]) {
-            float y = (xc[k] - mean_c) * rstd_c;
-            if (p.gamma_c) y *= p.gamma_c[j];
-            if (p.beta_c) y += p.beta_c[j];
+            const float y = (xc[k] - mean_c) * rstd_c * gc[k] + bc[k];
             zn[k] = zo[k] * sigmoid_f(sf[k]) + gelu_exact(y) * sigmoid_f(si[k]);
             p.z[row * d + j] = zn[k];
         }
     }
     float mean_z, rstd_z;
-    cluster_mean_rstd(zn, on, count, slice, d, p.eps, s_warp, s_stat, 1, mean_z, rstd_z);
+    cluster_mean_rstd(zn, on, count, slice, d, p.eps, s_stats[1], mean_z, rstd_z);
     // h' = f(z') g^o  (Eq. 8)
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k) {
         const int j = j0 + k * kCellThreads + threadIdx.x;
         if (on[k]) {
-            float y = (zn[k] - mean_z) * rstd_z;
-            if (p.gamma_z) y *= p.gamma_z[j];
-            if (p.beta_z) y += p.beta_z[j];
+            const float y = (zn[k] - mean_z) * rstd_z * gz[k] + bz[k];
             const float h = gelu_exact(y) * sigmoid_f(so[k]);
             if (p.h_f32) p.h_f32[row * d + j] = h;
             if (p.h_bf16) p.h_bf16[row * d + j] = __float2bfloat16_rn(h);

@@ -183,8 +183,10 @@ __device__ __forceinline__ void lane_row_argmax(const uint32_t (&v)[32], int cou
 }
 
 // gridDim.x is even: CTAs 2j and 2j + 1 are pair j.
+// (kEpiStore: at most 128 registers, so that a CTA of the cell kernel fits beside one: its reads before the wait then lie under
+// the product.  With 221, 10 states 71.1 us instead of 70.7.)
 template <int kEpi, int kGroups, bool kRowsOnLanes>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, kEpi == kEpiStore ? 2 : 1)
 gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap_hi,
                  const __grid_constant__ CUtensorMap bmap_lo) {
     extern __shared__ __align__(1024) unsigned char smem[];

@@ -51,11 +51,17 @@ constexpr int kTileKeys = 128;
 constexpr int kRows = kMaxRows;                 // packed rows per unit (two streams of 128)
 constexpr int kThreads = 384;
 constexpr int kSlots = 5;                  // ring of K / V tiles
+constexpr int kSlotsNarrow = 6;            // in the instances for units of up to 128 rows, which have one block of Q rows
 constexpr int kSlotBytes = kTileKeys * kHeadDim * 2;     // 32 KB
-constexpr int kTilesInFlight = 3;          // five slots never hold parts of more than three tiles
+// Arrival barriers: a tile's is that of the tile three before it, whose K has been read when the tile's K finds a slot.
+constexpr int kTilesInFlight = 3;
 constexpr int kQBytes = 128 * kHeadDim * 2;              // 32 KB per 128-row block
-constexpr int kRingOff = 2 * kQBytes;
-constexpr int kAuxOff = kRingOff + kSlots * kSlotBytes;  // 224 KB
+constexpr int kAuxOff = 2 * kQBytes + kSlots * kSlotBytes;  // 224 KB
+// Shared memory up to there: two blocks of Q and five slots, or one block and six (192 instead of 160 KB of K/V on their way to an
+// SM: 48 short sequences 132.0 -> 127.5 us per step, 16 mixed 737 -> 719, 32K 37.9 -> 37.2).
+template <bool kWide> constexpr int kRingSlots = kWide ? kSlots : kSlotsNarrow;
+template <bool kWide> constexpr int kRingOff = kWide ? 2 * kQBytes : kQBytes;
+static_assert(kRingOff<false> + kRingSlots<false> * kSlotBytes == kAuxOff && kRingOff<true> + kRingSlots<true> * kSlotBytes == kAuxOff, "layout");
 constexpr int kAuxBytes = 3072;
 constexpr int kSmemBytes = kAuxOff + kAuxBytes;          // 232448 = 227 KB
 constexpr uint32_t kTmemCols = 512;
@@ -78,7 +84,6 @@ struct Segment {
         return shared ? T : (s == 0 ? (T + 1) >> 1 : T >> 1);
     }
     __device__ __forceinline__ int tile(int s, int i) const { return tile0 + (shared ? i : 2 * i + s); }
-    __device__ __forceinline__ bool whole() const { return tile0 == 0 && tile1 == tiles; }
     // Warps of a stream's warpgroup that hold a row of a unit of up to 128 rows (both streams hold the same ones).  The
     // others take no part in the key loop.  A chain of 8 nodes x 4 heads fills one warp of four: its three idle warps used
     // to weigh 96 zero rows a tile, and their weights of 1 kept the multipliers of P V busy; left alone, those rows of P
@@ -92,7 +97,7 @@ struct Segment {
 struct Aux {
     uint64_t seg_full[kSegs];
     uint64_t full[kTilesInFlight];   // one per tile: its K and its V slot complete the same barrier
-    uint64_t empty[kSlots];
+    uint64_t empty[kSlotsNarrow];
     uint64_t s_full[2], o_done[2];
     uint64_t q_full;
     uint32_t tmem_base;
@@ -357,7 +362,7 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
                 if (ok && lane < ppt)
                     tma_load_5d_hint(ring + slot * kSlotBytes + lane * box_bytes, kv ? vmap : kmap, full, 0, 0, 0, 0, c_cur,
                                      stream_policy);
-                if (++slot == (uint32_t)kSlots) { slot = 0; free_parity ^= 1u; }
+                if (++slot == (uint32_t)kRingSlots<kWide>) { slot = 0; free_parity ^= 1u; }
                 __syncwarp();
             }
             if (++tile_bar == (uint32_t)kTilesInFlight) tile_bar = 0;
@@ -384,7 +389,7 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
     volatile int* abort_flag = &aux->abort_flag;
     constexpr uint32_t idesc_qk = umma_idesc_16bit(128, kTileKeys, 0, 0, kF16);
     constexpr uint32_t idesc_pv = umma_idesc_16bit(128, kHeadDim, 0, 1, kF16);
-    const uint32_t ring = smem_base + kRingOff;
+    const uint32_t ring = smem_base + kRingOff<kWide>;
     const uint32_t elected = elect_one() ? 1u : 0u;
     // descriptors of Q block 0 and of ring slot 0; those of the other blocks and slots differ in the start-address
     // field only (units of 16 bytes; shared memory ends below 2^18, so the field never carries)
@@ -405,7 +410,7 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
         const int n_it[2] = {shared ? T : (T + 1) >> 1, shared ? T : T >> 1};
 
         // ring slots of the V tile and of the K tile that the next turn needs
-        uint32_t k_slot = item_base % kSlots, v_slot = (item_base + 1u) % kSlots;
+        uint32_t k_slot = item_base % kRingSlots<kWide>, v_slot = (item_base + 1u) % kRingSlots<kWide>;
         // A turn: O_s += P_s V of the stream's tile i, then S_s = Q K^T of its tile i + 1 (which overwrites the P just
         // consumed; the tensor pipe runs them in order), each where the stream has such a tile; i = -1 issues the first S
         // of both streams.  The text of one turn serves both streams and all tiles: with the two streams unrolled (and the
@@ -443,8 +448,8 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
                     umma_commit_if(s ? issue : 0u, k_empty);
                     tS += 128; q_lo += kQBytes >> 4; s_bar += 8;
                 }
-                k_slot += 2u; if (k_slot >= (uint32_t)kSlots) k_slot -= kSlots;
-                v_slot += 2u; if (v_slot >= (uint32_t)kSlots) v_slot -= kSlots;
+                k_slot += 2u; if (k_slot >= (uint32_t)kRingSlots<kWide>) k_slot -= kRingSlots<kWide>;
+                v_slot += 2u; if (v_slot >= (uint32_t)kRingSlots<kWide>) v_slot -= kRingSlots<kWide>;
                 continue;
             }
 #pragma unroll 1
@@ -504,8 +509,8 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
                 // the tiles lie in the ring in the order of the turns that consume them, K and V by turns
                 if (last_reader) {
                     k_slot += 2u;
-                    if (k_slot >= (uint32_t)kSlots) k_slot -= kSlots;
-                    if (i >= 0) { v_slot += 2u; if (v_slot >= (uint32_t)kSlots) v_slot -= kSlots; }
+                    if (k_slot >= (uint32_t)kRingSlots<kWide>) k_slot -= kRingSlots<kWide>;
+                    if (i >= 0) { v_slot += 2u; if (v_slot >= (uint32_t)kRingSlots<kWide>) v_slot -= kRingSlots<kWide>; }
                 }
             }
         }
@@ -520,8 +525,9 @@ __device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(
 // Writes a warp's 32 rows x 32 columns (lane = row, v = its 32 fp32 values) to `out` as 16-bit values, through a per-warp
 // staging area in shared memory, so that every store instruction covers whole 64-byte row segments instead of 32 scattered
 // pieces.  `out_row` / `row_ok` are the lane's own row; the other rows' values come by shuffle.
-constexpr int kStageStride = 36;                     // floats per staged row: 16-byte aligned, conflict-free
-constexpr int kStageBytesPerWarp = 32 * kStageStride * 4;
+// Sixteen-byte piece c of row r lies at place c ^ (r & 7) of the row: no bank conflicts, and eight warps' areas fit a block of Q.
+constexpr int kStageBytesPerWarp = 32 * 32 * 4;
+static_assert(8 * kStageBytesPerWarp <= kQBytes, "the staging areas of both warpgroups");
 // Two floats to two 16-bit values of the cache's element type (x in the low half), round to nearest even.
 template <bool kF16>
 __device__ __forceinline__ uint32_t pack2_16bit(float x, float y) {
@@ -537,7 +543,7 @@ __device__ __forceinline__ void store_rows32(const AttnParams& p, float* stage, 
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<float4*>(stage + lane * kStageStride + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        *reinterpret_cast<float4*>(stage + lane * 32 + 4 * (j ^ (lane & 7))) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
     __syncwarp();
     // (rolled: this code runs a few times per launch, with cold instruction caches, where its length counts)
 #pragma unroll 1
@@ -545,8 +551,8 @@ __device__ __forceinline__ void store_rows32(const AttnParams& p, float* stage, 
         const int row = 8 * k + (lane >> 2), piece = lane & 3;
         const long long orow = __shfl_sync(0xffffffffu, out_row, row);
         const bool ok = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, row) != 0;
-        const float4 a = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 8);
-        const float4 b2 = *reinterpret_cast<const float4*>(stage + row * kStageStride + piece * 8 + 4);
+        const float4 a = *reinterpret_cast<const float4*>(stage + row * 32 + 4 * ((2 * piece) ^ (row & 7)));
+        const float4 b2 = *reinterpret_cast<const float4*>(stage + row * 32 + 4 * ((2 * piece + 1) ^ (row & 7)));
         uint4 u;
         u.x = pack2_16bit<kF16>(a.x, a.y); u.y = pack2_16bit<kF16>(a.z, a.w);
         u.z = pack2_16bit<kF16>(b2.x, b2.y); u.w = pack2_16bit<kF16>(b2.z, b2.w);
@@ -576,7 +582,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         // ancestor masks; every global read of the segment start is in flight at the same time
         int parent_i = -1;
         if (s == 0 && wtid < g.n) parent_i = p.tree_parent[g.node_base + wtid];
-        if (seg_no > 0) named_barrier(1, 256);   // the other warpgroup may still be reading its staging area in the Q blocks
+        if (seg_no > 0) named_barrier(1, 256);   // the other warpgroup may still be reading its staging area in the Q block
         if (leader) const_cast<volatile int&>(aux->seg_reached) = (int)seg_no;
         {
             // shared: this warpgroup loads its own 128-row block; split: rows [64 s, 64 s + 64) of block 0
@@ -629,7 +635,6 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
 
         const int rr = (g.shared ? s * 128 : 0) + row_local;       // packed row of this thread
         const unsigned long long anc_row = rr < g.M ? aux->anc[row_node(p, rr)] : 0ull;
-        const bool bad_tree = aux->seg_bad_tree != 0;
         const int n_it = g.iters(s);
         const int live = g.template live_warps<kWide>();
         const bool idle = (wtid >> 5) >= live;       // no row of the unit in this warp: straight to the segment's end
@@ -675,7 +680,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
                 if (kv_valid < kTileKeys) {
                     const int kv_end = min(kTileKeys, ((kv_valid + p.page_size - 1) >> p.page_shift) << p.page_shift);
                     const uint32_t seq = tile_base + (uint32_t)(g.shared ? i : 2 * i + s);
-                    unsigned char* vslot = smem + kRingOff + ((2u * seq + 1u) % kSlots) * kSlotBytes;
+                    unsigned char* vslot = smem + kRingOff<kWide> + ((2u * seq + 1u) % kRingSlots<kWide>) * kSlotBytes;
 #pragma unroll 1
                     for (int k = kv_valid + (wtid >> 4); k < kv_end; k += 2 * live)   // 16 threads x 16 bytes per 256-byte row
                         *reinterpret_cast<uint4*>(vslot + (k >> 3) * 2048 + ((wtid >> 3) & 1) * 1024 + (k & 7) * 128 +
@@ -851,21 +856,27 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             ++od_phase;
         }
         tc_fence_after();
-        // split mode: the streams exchange (m, l, lx) through the second Q block, which only the shared mode uses
-        float (*ml)[128][3] = reinterpret_cast<float (*)[128][3]>(smem + kQBytes);
-        if (!g.shared) { ml[s][row_local][0] = m; ml[s][row_local][1] = l; ml[s][row_local][2] = lx; }
+        // split mode: the streams exchange (m, l, lx) through the first columns of their S, which nobody needs any more (the
+        // warps of both warpgroups that hold the same rows reach the same lanes of tensor memory)
+        if (!g.shared) {
+            const uint32_t mine[4] = {__float_as_uint(m), __float_as_uint(l), __float_as_uint(lx), 0u};
+            tmem_st4(tS, mine);
+            tmem_wait_st();
+            tc_fence_before();
+        }
         meet_before_segment(aux, seg_no + 1, leader);    // both streams done: all MMAs of the segment have completed
-        const bool bad = bad_tree || const_cast<volatile int&>(aux->seg[seg_no % kSegs].bad_page);
+        // (what only the segment's ends need is read again here rather than held in registers through the key loop)
+        const volatile Segment& again = aux->seg[seg_no % kSegs];
+        const bool bad = const_cast<volatile int&>(aux->seg_bad_tree) || again.bad_page;
         const bool write_ok = !bad && !*abort_flag;
         // only the first and the last unit of a CTA's piece can be cut: two partial slots per CTA
         const long long part_row = (2ll * blockIdx.x + (seg_no > 0 ? 1 : 0)) * kRows + rr;
         const int node = (int)row_node(p, rr);
-        const long long out_row = rr < g.M ? (long long)(g.node_base + node) * p.num_q_heads + g.h * G + (rr - node * G) : 0;
+        const long long out_row = rr < g.M ? (long long)(again.node_base + node) * p.num_q_heads + again.h * G + (rr - node * G) : 0;
         const bool row_ok = write_ok && rr < g.M;
-        const bool whole = g.whole();
-        // staging for coalesced stores: the Q blocks are idle now (every MMA of the segment is done); stream 1's
-        // area starts after the (m, l, lx) exchange
-        float* stage = reinterpret_cast<float*>(smem + s * (kQBytes + 4096) + ((threadIdx.x >> 5) & 3) * kStageBytesPerWarp);
+        const bool whole = again.tile0 == 0 && again.tile1 == again.tiles;
+        // staging for coalesced stores: the first Q block is idle now (every MMA of the segment is done)
+        float* stage = reinterpret_cast<float*>(smem + (s * 4 + ((threadIdx.x >> 5) & 3)) * kStageBytesPerWarp);
         // a partial: [32 groups of four channels][kRows rows][4], so that a warp, one row per lane, stores whole lines
         float4* part = reinterpret_cast<float4*>(p.part_o) + (part_row - rr) * 32 + rr;
         // One loop writes both modes.  shared: this warpgroup's own rows, all 128 columns of its O, weight 1 / l.
@@ -879,10 +890,24 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             wa = l > 0.f ? 1.f / l : 0.f;
             lse = lx > 0.f ? (m + __log2f(lx)) * 0.6931471805599453f : -INFINITY;
         } else {
-            const float m0 = ml[0][row_local][0], l0 = ml[0][row_local][1], x0 = ml[0][row_local][2];
+            // (a stream without a tile has m = -inf and nothing in its sums)
             use_b = g.iters(1) > 0;
-            const float m1 = use_b ? ml[1][row_local][0] : -INFINITY, l1 = use_b ? ml[1][row_local][1] : 0.f;
-            const float x1 = use_b ? ml[1][row_local][2] : 0.f;
+            float m0 = m, l0 = l, x0 = lx, m1 = m, l1 = l, x1 = lx;
+            uint32_t st[4];
+            tc_fence_after();
+            // The instances for 256-row units read both streams' numbers: what is read again need not be kept.
+            if (kWide || s == 1) {
+                tmem_ld4(tmem + lane_sel, st);
+                tmem_wait_ld();
+                tmem_loaded(st);
+                m0 = __uint_as_float(st[0]); l0 = __uint_as_float(st[1]); x0 = __uint_as_float(st[2]);
+            }
+            if (kWide || s == 0) {
+                tmem_ld4(tmem + lane_sel + 128, st);
+                tmem_wait_ld();
+                tmem_loaded(st);
+                m1 = __uint_as_float(st[0]); l1 = __uint_as_float(st[1]); x1 = __uint_as_float(st[2]);
+            }
             const float mm = fmaxf(m0, m1);
             const float a0 = (m0 == -INFINITY) ? 0.f : fast_exp2(m0 - mm);
             const float a1 = (m1 == -INFINITY) ? 0.f : fast_exp2(m1 - mm);
@@ -947,7 +972,7 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         return;
     }
     if (tid == 0) {
-        for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&aux->empty[i]), 1);
+        for (int i = 0; i < kRingSlots<kWide>; ++i) mbar_init(smem_u32(&aux->empty[i]), 1);
         for (int i = 0; i < kTilesInFlight; ++i) mbar_init(smem_u32(&aux->full[i]), 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&aux->s_full[s]), 1);
@@ -1006,7 +1031,7 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
         if (!kManySeqs) wait_for_inputs();
         if (warp == 0) {
             if constexpr (!kManySeqs) build_walk_small(p, w);
-            producer_loop<kWide, kManySeqs>(p, &kmap, &vmap, aux, smem_base + kRingOff, w);
+            producer_loop<kWide, kManySeqs>(p, &kmap, &vmap, aux, smem_base + kRingOff<kWide>, w);
         } else if (warp == 1) {
             mma_loop<kWide, kF16>(aux, smem_base, tmem);
         } else if (kFused) {

@@ -371,9 +371,11 @@ __device__ __forceinline__ void producer_loop(const AttnParams& p, const CUtenso
 }
 
 // ------------------------------------------------------------------------------------------ MMA issuer
-// One thread's time is what bounds a 256-row unit: each tcgen05.mma costs the issuing thread about 60 clocks, and
-// whatever it executes between two batches (waits, slot arithmetic, commits) is added to that, not hidden behind it.
-// So the loop is kept lean:
+// A 256-row tile takes about 3480 clocks for 2048 of products: by clock stamps this warp waits 1411 of them for P, issues for
+// 590 and sits in commits, which push back while the pipe works, for 1260.  (Fed without a gap - one S buffer for both
+// streams, Q K^T of the next tile before P V of this one - the products took 71 and 77 clocks each instead of 64 plus the
+// commits, 3200 per tile, the ring ran dry, and 4 x 128K took 734 us instead of 639: shared memory is what they wait for.)
+// What this warp executes between two batches is added to the chain P -> P V -> Q K^T -> S, so the loop is kept lean:
 //  * the warp stays converged from top to bottom; all 32 lanes run the loop and the tensor-core instructions carry
 //    the guard (`elected` lane, waits succeeded, work to do) themselves.  What steers the loop (the segment's tile
 //    range and mode, the verdicts of the waits) goes through a warp reduction or a vote first, so that trip counts,
@@ -419,7 +421,7 @@ __device__ __forceinline__ void mma_loop(Aux* aux, uint32_t smem_base, uint32_t 
 #pragma unroll 1
         for (int i = -1; i < n_it[0]; ++i) {
             if (kWide && shared && ok && i >= 0 && i + 1 < T) {
-                // The middle of a 256-row unit, where this warp's time is what counts: both streams have both products, and
+                // The middle of a 256-row unit: both streams have both products, and
                 // a turn has no conditions but the stream's commits.  With the general turn here as well the 70B step took
                 // 693 us instead of 660.  Unrolled over the two streams 70B takes the same, 4 x 128K 633 us instead of
                 // 627, fp16 with 60 nodes 71.2 instead of 73.1.

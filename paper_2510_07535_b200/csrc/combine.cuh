@@ -134,13 +134,17 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
             node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
             plan(k, n, tiles, __shfl_sync(0xffffffffu, ws.begin, b) + h * (tiles + ws.part.pen), ws.part);
         } else {
+            // (with one tree of 64 nodes among chains of a few most blocks hold no rows: they cost two loads, not a schedule)
+            const int n = seq_nodes(p, b);
+            count = 0;
+            if (k * kCombineRows >= n * p.group) return;
             Partition<long long> part;
             const SchedHeader hdr = *p.sched_header;      // larger batches read the schedule the pass left
             part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
             const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
             node_base = seq_node_base(p, b);
             const int tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
-            plan(k, seq_nodes(p, b), tiles, sb + (long long)h * (tiles + part.pen), part);
+            plan(k, n, tiles, sb + (long long)h * (tiles + part.pen), part);
         }
     };
     // latency after the pass has ended is what this kernel costs: whatever needs no output of the pass comes before

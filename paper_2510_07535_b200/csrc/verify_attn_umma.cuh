@@ -852,15 +852,16 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
         it += (uint32_t)n_it;
 
         // ---- segment end: every product of this stream has completed
-        // (an idle warp sleeps on the hardware barrier below instead; it reads nothing)
+        // (an idle warp sleeps on the hardware barrier below instead; it touches no tensor memory)
         if (n_it > 0) {
             if (!idle) mbar_wait_certain(smem_u32(&aux->o_done[s]), od_phase & 1u, abort_flag);
             ++od_phase;
         }
         tc_fence_after();
         // split mode: the streams exchange (m, l, lx) through the first columns of their S, which nobody needs any more (the
-        // warps of both warpgroups that hold the same rows reach the same lanes of tensor memory)
-        if (!g.shared) {
+        // warps of both warpgroups that hold the same rows reach the same lanes of tensor memory).  Live warps only: an
+        // idle one has not waited for the products, which may still be writing and reading these columns of its lanes.
+        if (!g.shared && !idle) {
             const uint32_t mine[4] = {__float_as_uint(m), __float_as_uint(l), __float_as_uint(lx), 0u};
             tmem_st4(tS, mine);
             tmem_wait_st();
@@ -898,13 +899,13 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, Aux* aux, unsi
             uint32_t st[4];
             tc_fence_after();
             // The instances for 256-row units read both streams' numbers: what is read again need not be kept.
-            if (kWide || s == 1) {
+            if (!idle && (kWide || s == 1)) {
                 tmem_ld4(tmem + lane_sel, st);
                 tmem_wait_ld();
                 tmem_loaded(st);
                 m0 = __uint_as_float(st[0]); l0 = __uint_as_float(st[1]); x0 = __uint_as_float(st[2]);
             }
-            if (kWide || s == 0) {
+            if (!idle && (kWide || s == 0)) {
                 tmem_ld4(tmem + lane_sel + 128, st);
                 tmem_wait_ld();
                 tmem_loaded(st);

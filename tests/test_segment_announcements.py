@@ -1,7 +1,8 @@
 """A model of how the attention kernel's roles agree on the segments of a CTA's piece and hand over P tile by tile, run under
 random interleavings on the CPU.  A wait on a tile or on a free slot may give up at any point; from then on all of those
 return at once.  What is never abortable must still end: the hardware barriers, the wait for a score tile and the producer's
-look at `seg_reached`; every reader must have taken every segment; and a copy goes to the ring slot of its own tile and kind."""
+look at `seg_reached`; every reader must have taken every segment; a copy goes to the ring slot of its own tile and kind; and
+nobody writes over the scores of a segment whose products are under way."""
 import random
 import re
 from pathlib import Path
@@ -11,10 +12,14 @@ import pytest
 SOURCE = (Path(__file__).parent.parent / "paper_2510_07535_b200" / "csrc" / "verify_attn_umma.cuh").read_text()
 PLACES = int(re.search(r"constexpr int kSegs = (\d+);", SOURCE).group(1))
 SLOTS = int(re.search(r"constexpr int kSlots = (\d+);", SOURCE).group(1))
+SLOTS_NARROW = int(re.search(r"constexpr int kSlotsNarrow = (\d+);", SOURCE).group(1))
+# the condition under which a warp writes its maximum and sums over its scores at a segment's end
+EXCHANGE = re.search(r"if \((.*)\) \{\s*const uint32_t mine\[4\]", SOURCE).group(1)
 
 
 class Cta:
-    def __init__(self, rng, segments, paced, certain, by_tile):
+    def __init__(self, rng, segments, paced, certain, by_tile, idle_aside="!idle" in EXCHANGE, slots=SLOTS):
+        self.idle_aside, self.slots = idle_aside, slots
         self.rng, self.paced, self.certain, self.by_tile, self.abort = rng, paced, certain, by_tile, False
         self.tiles = [rng.randint(1, 3) for _ in range(segments)] + [0]       # 0: no more segments
         self.place, self.announced = [None] * PLACES, [0] * PLACES            # contents; completed phases
@@ -54,7 +59,7 @@ class Cta:
             yield None
             self.announced[k % PLACES] += 1
             for _ in range(2 * tiles):
-                free = lambda: item - 2 * self.freed < SLOTS
+                free = lambda: item - 2 * self.freed < self.slots
                 yield self.bounded(free)
                 if free():
                     assert item % 2 == wanted % 2, "K in a slot of V"
@@ -67,7 +72,7 @@ class Cta:
         if self.paced:
             if leader:
                 yield self.complete(k)
-            yield self.sync(3, 3)
+            yield self.sync(3, 4)
         else:
             yield self.complete(k)               # every reader for itself
         yield None
@@ -93,10 +98,10 @@ class Cta:
             taken.append(seg)
             if self.tiles[seg] == 0:
                 return
-            yield self.sync(1, 2)                # the Q blocks are free
+            yield self.sync(1, 3)                # the Q blocks are free
             if leader:
                 self.reached = k
-            yield self.sync(1, 2)                # the tree's masks
+            yield self.sync(1, 3)                # the tree's masks
             if leader:
                 self.q_full += 1
                 base = sum(self.tiles[:seg])
@@ -109,9 +114,23 @@ class Cta:
             yield from self.meet(k + 1, leader)
             assert not self.paced or self.place[k % PLACES] == seg        # bad_page is read here
 
+    def idle(self):
+        """The softmax warps without a row of the unit, if there are any: from the masks straight to the segment's end."""
+        yield from self.meet(0, False)
+        for k in range(len(self.tiles)):
+            seg = self.place[k % PLACES]
+            if self.tiles[seg] == 0:
+                return
+            yield self.sync(1, 3)
+            yield self.sync(1, 3)
+            if self.live[seg] < 4 and not self.idle_aside:
+                assert self.abort or self.products >= sum(self.tiles[:seg + 1]), "scores overwritten under the products"
+            yield from self.meet(k + 1, False)
+
     def run(self, abort_at):
         taken = [[], [], []]
-        roles = {r: next(r) for r in (self.producer(), self.mma(taken[0]), self.softmax(taken[1], True), self.softmax(taken[2], False))}
+        roles = {r: next(r) for r in (self.producer(), self.mma(taken[0]), self.softmax(taken[1], True), self.softmax(taken[2], False),
+                                      self.idle())}
         step = 0
         while roles:
             self.abort = self.abort or step >= abort_at
@@ -129,9 +148,9 @@ class Cta:
         return taken
 
 
-def segments_of(seed, segments, paced=True, certain=True, by_tile=True):
+def segments_of(seed, segments, paced=True, certain=True, by_tile=True, **more):
     rng = random.Random(seed)
-    return Cta(rng, segments, paced, certain, by_tile).run(abort_at=rng.choice([0, 10 ** 9, rng.randint(0, 12 * segments)]))
+    return Cta(rng, segments, paced, certain, by_tile, **more).run(abort_at=rng.choice([0, 10 ** 9, rng.randint(0, 12 * segments)]))
 
 
 @pytest.mark.parametrize("segments", [1, PLACES - 1, PLACES, PLACES + 1, 16, 40])
@@ -140,10 +159,16 @@ def test_all_roles_take_the_same_segments_whatever_gives_up(segments):
         assert segments_of(seed, segments) == [list(range(segments + 1))] * 3, seed
 
 
-@pytest.mark.parametrize("segments,without", [(40, "paced"), (4, "certain"), (4, "by_tile")])
+@pytest.mark.parametrize("segments", [1, PLACES + 1, 40])
+def test_the_same_with_the_longer_ring_of_narrow_units(segments):
+    for seed in range(300):
+        assert segments_of(seed, segments, slots=SLOTS_NARROW) == [list(range(segments + 1))] * 3, seed
+
+
+@pytest.mark.parametrize("segments,without", [(40, "paced"), (4, "certain"), (4, "by_tile"), (4, "idle_aside")])
 def test_the_model_shows_what_each_rule_is_for(segments, without):
     """A producer that nothing paces, softmax warps that hand over P of a tile whose S was not announced, a producer that
-    counts only what it has copied."""
+    counts only what it has copied, idle warps that take part in the exchange at a segment's end."""
     def broken(seed):
         try:
             return segments_of(seed, segments, **{without: False}) != [list(range(segments + 1))] * 3

@@ -121,6 +121,7 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
             s_parent[node] = parent[h];
         }
         bad = __any_sync(kAll, bad);
+        __syncwarp();                                  // a vote orders no memory: the lanes' parents are there, and checked
 #pragma unroll
         for (int h = 0; h < 2; ++h)
             if (!bad && lane + 32 * h < n)

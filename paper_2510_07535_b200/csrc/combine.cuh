@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
         int step = slot & 1 ? 32 * kMaxRows : 64 * kMaxRows;
         for (int base = 0; base < count; base += group) {
             const int cnt = count - base < group ? count - base : group;
-            if (base > 0) __syncwarp();                  // the stage's weights of the round before have been read
+            __syncwarp();                                // the stage's weights of the round or the block before have been read
             for (int j = lane; j < 2 * cnt; j += 32) {   // eight rows' LSEs: two pieces of 16 bytes
                 const int at = base + (j >> 1), sl = at == 0 ? slot : (slot & ~1) + 2 * at;
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(lse_stage + j * 4)),

@@ -93,9 +93,8 @@ __device__ __forceinline__ void wait_and_let_dependents_start() {
 
 // One sequence's walk; called by the first kArgmaxThreads threads of a CTA.  A node's chunk keys are read by several
 // neighbouring threads, all in one memory round trip; the rest is the first warp's, two nodes per lane.
-// `keys()` waits for the kernel that leaves the arg-max keys and returns them.  The tree is read before: the kernels that
-// call this are dependents of one that lets them start only when everything before it has completed, and that writes no
-// tree.  With the ancestors as bits by then, what is left when the keys are there is one round of loads, one CTA barrier
+// `keys()` waits for the kernel that leaves the arg-max keys and returns them.  The tree and the tokens are read before
+// (ld_early).  With the ancestors as bits by then, what is left when the keys are there is one round of loads, one CTA barrier
 // and a handful of votes.
 template <typename Keys>
 __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int b, Keys keys) {
@@ -104,8 +103,8 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
     static_assert(kArgmaxThreads >= 4 * kMaxNodes, "at least four threads per node");
     __shared__ int s_parent[kMaxNodes], s_am[kMaxNodes];
     const int i = threadIdx.x, lane = i & 31;
-    const int base = p.node_offsets ? p.node_offsets[b] : b * p.nodes_uniform;
-    const int n = p.node_offsets ? p.node_offsets[b + 1] - base : p.nodes_uniform;
+    const int base = p.node_offsets ? ld_early(p.node_offsets + b) : b * p.nodes_uniform;
+    const int n = p.node_offsets ? ld_early(p.node_offsets + b + 1) - base : p.nodes_uniform;
     const bool shape_ok = n >= 1 && n <= p.max_nodes && n <= p.path_stride && base >= 0 && base + n <= p.total_nodes;
     int parent[2] = {-1, -1}, tok[2] = {-1, -1};
     unsigned long long anc[2] = {0ull, 0ull};          // the node and its ancestors
@@ -115,8 +114,8 @@ __device__ __forceinline__ void accept_walk_seq(const AcceptParams& p, const int
         for (int h = 0; h < 2; ++h) {
             const int node = lane + 32 * h;
             if (node >= n) continue;
-            parent[h] = p.tree_parent[base + node];
-            tok[h] = p.draft_tokens[base + node];
+            parent[h] = ld_early(p.tree_parent + base + node);
+            tok[h] = ld_early(p.draft_tokens + base + node);
             bad = bad || (node == 0 ? parent[h] != -1 : parent[h] < 0 || parent[h] >= node);
             s_parent[node] = parent[h];
         }
@@ -288,7 +287,7 @@ __global__ void __launch_bounds__(kArgmaxThreads, kArgmaxCtasPerSm) argmax_parti
         }
     }
     if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may queue up; it waits likewise
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may queue up (what it reads early: ld_early)
     const int warp = threadIdx.x >> 5;
     if (blockIdx.x == 0) {
         // Do the packed offsets describe this call's rows: start at 0, end at total_nodes, 1..max_nodes nodes per sequence?

@@ -232,7 +232,7 @@ gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, c
     }
     // may be launched as a programmatic dependent of the kernel before it in the stream: the set-up above touched no
     // input and ran beside that kernel's tail; from here on it has completed (a no-op in an ordinary launch).  The
-    // kernel after this one may queue up in turn; it waits likewise before it reads anything.
+    // kernel after this one may queue up in turn; before its own wait it reads inputs of the call only (ld_early).
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tc_fence_before();
@@ -566,9 +566,8 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
     const int j0 = (int)cluster.block_rank() * slice;             // this CTA's columns: [j0, min(j0 + slice, d))
     const int count = min(slice, max(d - j0, 0));
     const float* s = p.s + row * 4ll * d;
-    // A programmatic dependent of the product that writes S and nothing else, and that lets its dependents start only when
-    // everything before it has completed: E(t), z and the affine parameters are read, and the cluster's CTAs meet (before anyone
-    // writes into a peer's shared memory), under the product's tail.
+    // A programmatic dependent of the product, which writes S and nothing else: E(t), z and the affine parameters are read
+    // (ld_early), and the cluster's CTAs meet (before anyone writes into a peer's shared memory), under the product's tail.
     float xc[kCellPerThread], sf[kCellPerThread], si[kCellPerThread], so[kCellPerThread], zo[kCellPerThread], zn[kCellPerThread];
     float ae[kCellPerThread], gc[kCellPerThread], bc[kCellPerThread], gz[kCellPerThread], bz[kCellPerThread];
     bool on[kCellPerThread];
@@ -579,12 +578,12 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
         xc[k] = sf[k] = si[k] = so[k] = zo[k] = zn[k] = ae[k] = bc[k] = bz[k] = 0.f;
         gc[k] = gz[k] = 1.f;
         if (on[k]) {
-            ae[k] = p.alpha * __bfloat162float(p.emb[row * d + j]);
-            zo[k] = p.z[row * d + j];
-            if (p.gamma_c) gc[k] = p.gamma_c[j];
-            if (p.beta_c) bc[k] = p.beta_c[j];
-            if (p.gamma_z) gz[k] = p.gamma_z[j];
-            if (p.beta_z) bz[k] = p.beta_z[j];
+            ae[k] = p.alpha * __bfloat162float(ld_early(p.emb + row * d + j));
+            zo[k] = ld_early(p.z + row * d + j);
+            if (p.gamma_c) gc[k] = ld_early(p.gamma_c + j);
+            if (p.beta_c) bc[k] = ld_early(p.beta_c + j);
+            if (p.gamma_z) gz[k] = ld_early(p.gamma_z + j);
+            if (p.beta_z) bz[k] = ld_early(p.beta_z + j);
         }
     }
     cluster.sync();

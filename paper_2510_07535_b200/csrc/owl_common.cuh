@@ -170,6 +170,13 @@ __device__ __forceinline__ int seq_node_base(const AttnParams& p, int b) {
     return p.node_offsets ? p.node_offsets[b] : b * p.nodes_uniform;
 }
 
+// Loads of a call's inputs before the kernel's own dependency wait (the merge's schedule, the walk's tree, the cell's states).
+// They may stand there because the kernel before it in the call lets its dependents start only after its own wait, when
+// everything before the call has completed, and because that kernel writes none of them.  They take what L2 holds: an input
+// that an earlier kernel wrote in place (lengths, z) may lie in the L1 of this SM as it was.
+template <typename T>
+__device__ __forceinline__ T ld_early(const T* p) { return __ldcg(p); }
+
 // A sequence is schedulable when its node count and lengths are inside the interface's limits.
 __device__ __forceinline__ bool seq_tree_shape_ok(const AttnParams& p, int base, int n) {
     return n >= 1 && n <= p.max_nodes && base >= 0 && base + n <= p.total_nodes;
@@ -202,9 +209,9 @@ __device__ __forceinline__ WarpSchedule warp_schedule(const AttnParams& p) {
     ws.n = 0; ws.L = 0; ws.node_base = 0;
     bool ok = false;
     if (lane < p.batch) {
-        ws.L = p.ctx_lens[lane];
-        ws.node_base = seq_node_base(p, lane);
-        ws.n = seq_nodes(p, lane);
+        ws.L = ld_early(p.ctx_lens + lane);
+        ws.node_base = p.node_offsets ? ld_early(p.node_offsets + lane) : lane * p.nodes_uniform;
+        ws.n = p.node_offsets ? ld_early(p.node_offsets + lane + 1) - ws.node_base : p.nodes_uniform;
         ok = seq_tree_shape_ok(p, ws.node_base, ws.n) && ws.L >= 0 &&
              (unsigned)ws.L + (unsigned)ws.n <= (unsigned)p.max_pages_per_seq * (unsigned)p.page_size;
     }

@@ -74,7 +74,8 @@ int cuda_fail(owl_ctx* ctx, cudaError_t e, const char* what) {
 }
 
 // Launch `kernel(arg)` so that it may be scheduled while the kernel before it in the stream is still running
-// (programmatic dependent launch); the kernel itself waits (griddepcontrol.wait) before it reads anything.
+// (programmatic dependent launch); the kernel itself waits (griddepcontrol.wait) before it reads anything that kernel writes.
+// What it may read before is stated at ld_early.
 template <typename... Args>
 cudaError_t launch_dependent_smem(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const Args&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -1011,8 +1011,8 @@ verify_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap 
     // Launched as a programmatic dependent itself: everything so far touched no input.  Each role waits for the kernel
     // before this one in the stream itself, after the jump into its code (a no-op in an ordinary launch).
     // The combine kernel is launched as a programmatic dependent and may queue up behind this grid's CTAs from then
-    // on.  It reads the call's inputs (lengths, offsets) before its own wait: triggering only after this grid's wait
-    // keeps those reads ordered after whatever kernel wrote them earlier in the stream.
+    // on.  It reads the call's inputs (lengths, offsets, trees, tokens) before its own wait (ld_early): triggering only
+    // after this grid's wait keeps those reads ordered after whatever kernel wrote them earlier in the stream.
     auto wait_for_inputs = [] {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -48,6 +48,36 @@ inline size_t combine_smem_bytes(int group, int lg_parts, unsigned ctas, int sms
     return stage > spread ? stage : spread;
 }
 
+// Blocks of eight rows that hold any, of all units of a sequence with n nodes.
+__host__ __device__ inline int seq_blocks(int n, int group, int num_kv_heads) {
+    return num_kv_heads * ((n * group + kCombineRows - 1) / kCombineRows);
+}
+// At most so many in a call: the host knows the nodes of the batch and the most that a sequence has.
+inline long long combine_most_blocks(long long batch, long long total_nodes, int max_nodes, int group, int num_kv_heads) {
+    const long long by_max = batch * seq_blocks(max_nodes, group, 1), by_total = (total_nodes * group + (kCombineRows - 1) * batch) / kCombineRows;
+    return num_kv_heads * (by_max < by_total ? by_max : by_total);
+}
+
+// Places where the line of a pass of `ctas` CTAs is cut (one CTA: none, but a grid is never empty).
+__host__ __device__ inline int combine_cuts(int ctas) { return ctas > 1 ? ctas - 1 : 1; }
+
+// Short lines: which block is whose.  Lane b holds sequence b, everything is derived from the inputs; a sequence that the pass
+// refuses has no blocks.  (Numbered for every sequence up to the largest tree's rows, the blocks of one tree of 64 nodes among
+// chains lay mostly empty and the full ones far apart, two and more to a CTA.  One such tree among 16 sequences of 100-1500
+// tokens: 31.2 us per step, now 27.6; among 8 of 200-6000: 46.8, now 44.8.)
+struct BlockNumbers {
+    int blocks, end;                 // of the call; where this lane's sequence ends
+    __device__ __forceinline__ void derive(const AttnParams& p, const WarpSchedule& ws) {
+        const int lane = threadIdx.x & 31;
+        end = ws.tiles > 0 ? seq_blocks(ws.n, p.group, p.num_kv_heads) : 0;
+        for (int o = 1; o < p.batch; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += v;
+        }
+        blocks = __shfl_sync(0xffffffffu, end, p.batch - 1);
+    }
+};
+
 // A block of eight of a unit's packed rows per CTA and turn, 16 of the 128 channels per warp: lane = (row, four
 // channels).  The warp finds the CTAs whose pieces cut the unit and merges their partials in CTA order.  A CTA stores at
 // most two partials: slot 2c if its piece starts inside the unit, else 2c + 1.
@@ -58,10 +88,10 @@ inline size_t combine_smem_bytes(int group, int lg_parts, unsigned ctas, int sms
 // epilogue took 1.9 us instead of 1.0 at 2K context, 3.5 instead of 3.0 for 240 rows at 47K.)
 //
 // The kernel is launched as a programmatic dependent of that pass and its time after the pass has ended is pure
-// latency, so everything that needs no output of the pass comes before the wait: for batches of at most 32
-// sequences the warp derives the schedule from the inputs exactly as the pass did (warp_schedule) and knows its
-// block's partial slots when the wait returns; what is left is one round of loads.  Larger batches read the
-// schedule the pass left in global memory (first flat tile of every sequence, totals, choice of partition).
+// latency, so everything that needs no output of the pass comes before the wait: on short lines (small_schedule) the
+// warp derives the schedule from the inputs exactly as the pass did (warp_schedule) and knows its
+// block's partial slots when the wait returns; what is left is one round of loads.  Otherwise (kManySeqs) it reads the
+// schedule the pass left in global memory (first place of every sequence, totals, choice of partition).
 //
 // kFused (verify step): the grid has one more CTA per sequence after the row CTAs; each of those runs one
 // sequence's acceptance walk over the arg-max keys that the pass's spare warps left (`ap`).
@@ -69,10 +99,10 @@ inline size_t combine_smem_bytes(int group, int lg_parts, unsigned ctas, int sms
 // p.combine_group: partials fetched per round, at most 32 (combine_group above).  A round's rows go through a
 // warp-private stage in shared memory of that many pieces, which is what limits the CTAs per SM.
 //
-// The stage is there for the sake of the code's length, not of the data: with the rows in registers the fetch and
-// the fold were two loops unrolled 32 times, some 450 instructions that a warp with one row executes exactly once,
-// at the pace of instruction fetches from L2.
-template <bool kFused>
+// The stage is there for the sake of the code's length, not of the data: with the pieces in registers the fetch and
+// the fold were two loops unrolled 32 times, some 450 instructions that a warp executes once per block, mostly once in
+// all, at the pace of instruction fetches from L2.
+template <bool kFused, bool kManySeqs>
 __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sched_kernel(const AttnParams p, const AcceptParams ap) {
     const unsigned row_ctas = (unsigned)p.combine_row_ctas;
     if (kFused) {
@@ -86,80 +116,112 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
             return;
         }
     }
-    // The row CTAs are persistent: a warp derives the schedule once and then takes blocks first, first + stride, ...
-    // (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived 8192 times).  Blocks are
-    // numbered unit by unit for the first eight rows of all units, then for the second eight and so on, up to the rows of
-    // the most nodes a sequence may have: what shorter sequences lack lies at the end.
+    // The row CTAs are persistent (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived
+    // 8192 times).  Short lines: a warp derives the schedule once and then takes blocks first, first + stride, ..., numbered
+    // sequence by sequence, unit by unit, and only those that hold rows (BlockNumbers).  Otherwise there are mostly more units
+    // than pieces, and only those that a piece's end cuts have anything to merge: a CTA goes by one cut and takes its share of
+    // that unit's blocks.  (Every block of every unit looked up in turn, us per step: 64 sequences of 100-1500 tokens with one
+    // tree of 64 nodes 91.6, now 79.4; 300 of 50-300 tokens 124.6, now 120.7; 1000 with one such tree 539, now 355.)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // The ninth warp rehearses: it runs the code that follows the wait on whatever the first slots hold (M stays 0, so
+    // The ninth warp rehearses: it runs the code that follows the wait on whatever the first slots hold (out_row stays -1, so
     // nothing is written), while the others derive the schedule and wait.  That code runs once or twice per launch, and its lines
     // used to be fetched when the partials were there already (2.9 -> 2.5 us after the wait; 2K step 12.4 -> 12.1 with the walk's
     // reads before its wait).
     const bool rehearsal = warp == kCombineWarps;
-    // A block is shared out to combine_parts CTAs, each with a part of the channels and of the eight warps.
+    // A block is shared out to 1 << combine_lg_parts CTAs, each with a part of the channels and of the eight warps.
     const int warps = kCombineWarps >> p.combine_lg_parts, part_no = (int)blockIdx.x & ((1 << p.combine_lg_parts) - 1);
     if (!rehearsal && warp >= warps) return;
     const int r = lane & 7, chunk = rehearsal ? lane >> 3 : (part_no * warps + warp) * 4 + (lane >> 3);   // row of the block; four channels
-    const unsigned first_id = blockIdx.x >> p.combine_lg_parts, stride = row_ctas >> p.combine_lg_parts;
     extern __shared__ float4 combine_stage[];          // per warp: [group][32] pieces of the partials, [group][8] LSEs
     const int group = rehearsal ? rehearsed_partials(p.combine_group) : p.combine_group;
     float4* stage = combine_stage + (rehearsal ? warps : warp) * p.combine_group * 34;
     float* lse_stage = reinterpret_cast<float*>(stage + group * 32);
     const uint32_t stage_u32 = (uint32_t)__cvta_generic_to_shared(stage + lane);
-    WarpSchedule ws{};
-    // per block: its unit's row count, the first partial's slot and the number of partials (0: nothing to merge)
-    int M = 0, h = 0, row = 0, node_base = 0, slot = 0, count = 0;
-    auto plan = [&](int k, int n, int tiles, auto t0, const auto& part) {
-        row = k * kCombineRows + r;
-        M = n * p.group;
+    // The unit: its sequence's nodes and their offset, its KV head; the first partial's slot and the number of partials (0:
+    // nothing to merge).  The block: its first row, this lane's row of the output (-1: past the unit's last).
+    int n = 0, node_base = 0, h = 0, slot = 0, count = 0, row0 = 0;
+    long long out_row = -1;
+    int c0 = 0;
+    auto plan = [&](auto t0, int tiles, const auto& part) {       // the unit's place on the line and its tiles
         count = 0;
-        if (tiles == 0 || k * kCombineRows >= M) return;      // not scheduled, or no such rows
         // the CTAs that hold its first tile, its last one and, if it is not the line's first, the place before its gap: three
         // lanes find one each
         auto place = t0 + part.pen;
         if (lane == 1) place += tiles - 1;
         if (lane == 2) place = t0 > 0 ? t0 - 1 : 0;
         const int mine = part.owner(place);
-        const int c0 = __shfl_sync(0xffffffffu, mine, 0), c1 = __shfl_sync(0xffffffffu, mine, 1), before = __shfl_sync(0xffffffffu, mine, 2);
+        c0 = __shfl_sync(0xffffffffu, mine, 0);
+        const int c1 = __shfl_sync(0xffffffffu, mine, 1), before = __shfl_sync(0xffffffffu, mine, 2);
         if (c0 == c1) return;              // a single CTA saw every key of this unit and wrote the result itself
         // the unit's first CTA may have come from another unit or from the gap before that; the others' pieces start in this one
         slot = 2 * c0 + (t0 > 0 && before == c0 ? 1 : 0);
         count = c1 - c0 + 1;
     };
-    auto locate = [&](unsigned id) {       // every lane of the warp, same block
-        const int units = p.batch * p.num_kv_heads, k = div_small((int)id, units), u = (int)id - k * units, b = div_small(u, p.num_kv_heads);
-        h = u - b * p.num_kv_heads;
-        if (p.small) {
-            const int n = __shfl_sync(0xffffffffu, ws.n, b), tiles = __shfl_sync(0xffffffffu, ws.tiles, b);
-            node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
-            plan(k, n, tiles, __shfl_sync(0xffffffffu, ws.begin, b) + h * (tiles + ws.part.pen), ws.part);
-        } else {
-            // (with one tree of 64 nodes among chains of a few most blocks hold no rows: they cost two loads, not a schedule)
-            const int n = seq_nodes(p, b);
-            count = 0;
-            if (k * kCombineRows >= n * p.group) return;
-            Partition<long long> part;
-            const SchedHeader hdr = *p.sched_header;      // larger batches read the schedule the pass left
-            part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
-            const long long sb = p.sched_seq_begin[b], se = p.sched_seq_begin[b + 1];
-            node_base = seq_node_base(p, b);
-            const int tiles = se > sb ? (int)((se - sb) / p.num_kv_heads) - part.pen : 0;
-            plan(k, n, tiles, sb + (long long)h * (tiles + part.pen), part);
-        }
+    auto take_rows = [&](int block) {      // of the unit
+        row0 = block * kCombineRows;
+        const int row = row0 + r, node = (int)row_node(p, row);
+        out_row = row < n * p.group ? (long long)(node_base + node) * p.num_q_heads + h * p.group + (row - node * p.group) : -1;
     };
+    WarpSchedule ws;
+    BlockNumbers num;
+    auto locate = [&](int id) {            // every lane of the warp, same block
+        const int b = __ffs(__ballot_sync(0xffffffffu, id < num.end)) - 1;
+        n = __shfl_sync(0xffffffffu, ws.n, b);
+        node_base = __shfl_sync(0xffffffffu, ws.node_base, b);
+        const int tiles = __shfl_sync(0xffffffffu, ws.tiles, b), unit_blocks = seq_blocks(n, p.group, 1);
+        const int local = id - __shfl_sync(0xffffffffu, num.end, b) + p.num_kv_heads * unit_blocks;
+        h = div_small(local, unit_blocks);
+        take_rows(local - h * unit_blocks);
+        plan(__shfl_sync(0xffffffffu, ws.begin, b) + h * (tiles + ws.part.pen), tiles, ws.part);
+    };
+    // Block numbers are the call's for short lines, the unit's otherwise.
+    int id = (int)blockIdx.x >> p.combine_lg_parts, stride = (int)row_ctas >> p.combine_lg_parts, end = 1;
     // latency after the pass has ended is what this kernel costs: whatever needs no output of the pass comes before
-    // the wait - for batches of at most 32 sequences the whole plan of the first block
+    // the wait - for short lines the whole plan of the first block
     if (rehearsal) {
-        row = r;
         count = min(kRehearsedPartials, p.num_ctas);
-    } else if (p.small) {
-        ws = warp_schedule(p);
-        locate(first_id);
+        id = 0;
+    } else {
+        if (!kManySeqs) {
+            ws = warp_schedule(p);
+            num.derive(p, ws);
+            end = num.blocks;
+            if (id < end) locate(id);
+        }
+        // from here on the split-KV pass has completed and its writes are visible (a no-op in an ordinary launch)
+        wait_and_let_dependents_start();
+        if (kManySeqs) {
+            // a cut per CTA: the first place of piece `cut`; which sequence it lies in, 32 of them at a look
+            const int cuts = combine_cuts(p.num_ctas), turn = div_small(id, cuts), cut = id - turn * cuts + 1;
+            const SchedHeader hdr = *p.sched_header;
+            Partition<long long> part;
+            part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
+            long long t, t_end;
+            part.range(cut, t, t_end);
+            if (t >= part.total) return;
+            int b = 0;
+            for (int per = p.batch > 32 ? 32 : 1; per > 0; per >>= 5) {
+                const int at = b + lane * per;
+                const unsigned from = __ballot_sync(0xffffffffu, at < p.batch && p.sched_seq_begin[at] <= t);
+                b += (31 - __clz((int)from)) * per;
+            }
+            const long long begin = p.sched_seq_begin[b];
+            n = seq_nodes(p, b);
+            node_base = seq_node_base(p, b);
+            const int len = (int)((unsigned)(p.sched_seq_begin[b + 1] - begin) / (unsigned)p.num_kv_heads), local = (int)(t - begin);
+            h = (int)((unsigned)local / (unsigned)len);
+            if (local - h * len <= part.pen) return;       // the piece begins with a unit, not inside one
+            plan(begin + (long long)h * len, len - part.pen, part);
+            // a unit's cuts share its blocks
+            const int turns = div_small((int)row_ctas, cuts);
+            id = (cut - c0 - 1) * turns + turn;
+            stride = (count - 1) * turns;
+            end = seq_blocks(n, p.group, 1);
+        }
     }
-    // from here on the split-KV pass has completed and its writes are visible (a no-op in an ordinary launch)
-    if (!rehearsal) wait_and_let_dependents_start();
-    for (unsigned id = first_id; id < (unsigned)p.combine_blocks; id += stride) {
-        if (!rehearsal && (!p.small || id != first_id)) locate(id);
+    for (bool first = true; id < end; id += stride, first = false) {
+        if (kManySeqs) { if (!rehearsal) take_rows(id); }
+        else if (!first) locate(id);
         if (count == 0) continue;
         // Partials are taken `group` at a time, their LSEs with them: one memory round trip per group.  Groups are folded
         // online (running maximum, each lane its own row's).
@@ -167,7 +229,7 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
         float sum = 0.f, mx = -INFINITY;
         bool bad = false;
         // slots of neighbouring CTAs lie two apart; only the first CTA's partial may be its second
-        const float4* src = reinterpret_cast<const float4*>(p.part_o) + (slot * 32ll + chunk) * kMaxRows + row;
+        const float4* src = reinterpret_cast<const float4*>(p.part_o) + (slot * 32ll + chunk) * kMaxRows + row0 + r;
         int step = slot & 1 ? 32 * kMaxRows : 64 * kMaxRows;
         for (int base = 0; base < count; base += group) {
             const int cnt = count - base < group ? count - base : group;
@@ -175,7 +237,7 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
             for (int j = lane; j < 2 * cnt; j += 32) {   // eight rows' LSEs: two pieces of 16 bytes
                 const int at = base + (j >> 1), sl = at == 0 ? slot : (slot & ~1) + 2 * at;
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(lse_stage + j * 4)),
-                             "l"(p.part_lse + (long long)sl * kMaxRows + (row - r) + (j & 1) * 4) : "memory");
+                             "l"(p.part_lse + (long long)sl * kMaxRows + row0 + (j & 1) * 4) : "memory");
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll 4
@@ -190,7 +252,7 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
             float mx_new = mx;
             for (int j = lane >> 3; j < cnt; j += 4) {
                 const float l = lse_stage[j * 8 + r];
-                bad = bad || (row < M && __float_as_uint(l) == kBadPartial);
+                bad = bad || (out_row >= 0 && __float_as_uint(l) == kBadPartial);
                 mx_new = fmaxf(mx_new, l);
             }
             mx_new = fmaxf(mx_new, __shfl_xor_sync(0xffffffffu, mx_new, 8));
@@ -228,15 +290,12 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
             pk.y = *reinterpret_cast<uint32_t*>(&hi2);
         }
         const float lse = sum > 0.f ? mx + logf(sum) : -INFINITY;
-        const int node = (int)row_node(p, row);
-        const long long out_row = (long long)(node_base + node) * p.num_q_heads + h * p.group + (row - node * p.group);
         // rows past the unit's last hold nothing; a bad tree or page in the unit's sequence (the same for all of its rows): no
         // output
-        if (!__any_sync(0xffffffffu, bad) && row < M) {
+        if (!__any_sync(0xffffffffu, bad) && out_row >= 0) {
             *reinterpret_cast<uint2*>(p.out + out_row * kHeadDim + chunk * 4) = pk;
             if (p.lse && chunk == 0) p.lse[out_row] = lse;
         }
-        if (rehearsal) break;
     }
 }
 

@@ -48,7 +48,6 @@ struct AttnParams {
     int32_t small;                // the schedule is derived by single warps in 32-bit arithmetic (small_schedule)
     int32_t num_ctas;             // CTAs of the split-KV pass (the flat tile range is cut into this many pieces)
     int32_t combine_group;        // partials per round of the merge kernel, 4..32
-    int32_t combine_blocks;       // blocks of eight packed rows that the merge kernel goes through
     int32_t combine_lg_parts;     // log2 of the CTAs that share a block's channels
     int32_t combine_row_ctas;     // the merge kernel's CTAs that take rows (persistent)
     int32_t f16;                  // q / caches / out are fp16 instead of bf16 (same size; typed as bf16 pointers here)

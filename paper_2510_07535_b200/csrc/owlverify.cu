@@ -95,8 +95,8 @@ cudaError_t launch_dependent(void (*kernel)(Args...), dim3 grid, dim3 block, cud
     return launch_dependent_smem(kernel, grid, block, 0, stream, args...);
 }
 
-// The attention kernel's instances: [more than 32 sequences][units above 128 rows][logits scan fused in], bf16;
-// and the fp16 ones (attention only): [more than 32 sequences][units above 128 rows]
+// The attention kernel's instances: [block-wide schedule][units above 128 rows][logits scan fused in], bf16;
+// and the fp16 ones (attention only): [block-wide schedule][units above 128 rows]
 using UmmaKernel = void (*)(AttnParams, CUtensorMap, CUtensorMap, AcceptParams);
 UmmaKernel umma_kernel(bool many, bool wide, bool fused, bool fp16) {
     using namespace umma_path;
@@ -109,6 +109,12 @@ UmmaKernel umma_kernel(bool many, bool wide, bool fused, bool fp16) {
         {verify_attn_umma_kernel<false, false, false, true>, verify_attn_umma_kernel<false, true, false, true>},
         {verify_attn_umma_kernel<true, false, false, true>, verify_attn_umma_kernel<true, true, false, true>}};
     return fp16 ? table16[many][wide] : table[many][wide][fused];
+}
+// The merge kernel's: [acceptance walk in extra CTAs][the pass's schedule read from global memory]
+using CombineKernel = void (*)(AttnParams, AcceptParams);
+CombineKernel combine_kernel(bool fused, bool many) {
+    return fused ? (many ? combine_sched_kernel<true, true> : combine_sched_kernel<true, false>)
+                 : (many ? combine_sched_kernel<false, true> : combine_sched_kernel<false, false>);
 }
 bool set_umma_smem_attr() {
     bool ok = true;
@@ -277,8 +283,8 @@ int owl_create(owl_ctx** out, int device, const owl_dims* max_dims) {
     }
     if (ok) {
         const int most = (int)combine_stage_bytes(32, 0);
-        ok = cudaFuncSetAttribute(combine_sched_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
-             cudaFuncSetAttribute(combine_sched_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
+        for (int i = 0; ok && i < 4; ++i)
+            ok = cudaFuncSetAttribute(combine_kernel(i & 2, i & 1), cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
     }
     if (ok) {
         using namespace gemm_path;
@@ -397,13 +403,18 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     }
 
     if (ctx->profiling) cudaEventRecord(ctx->ev[0], stream);
-    // one CTA per block of rows while all are resident at once; beyond that the merge kernel's CTAs stride over the blocks
+    // one CTA per block of rows while all are resident at once, beyond that the merge kernel's CTAs stride over the blocks; on a
+    // line that is not short the same for each cut, whose CTAs come in whole turns over the cuts
     p.combine_group = combine_group((long long)d->batch * d->num_kv_heads, ctx->num_ctas);
-    const long long want_ctas = (long long)d->batch * d->num_kv_heads * ((G * d->max_nodes + kCombineRows - 1) / kCombineRows);
+    const long long want_ctas = combine_most_blocks(d->batch, d->total_nodes, d->max_nodes, G, d->num_kv_heads);
     const long long most_ctas = (long long)ctx->sm_count * combine_ctas_per_sm(p.combine_group);
-    p.combine_blocks = (int32_t)want_ctas;
-    p.combine_lg_parts = combine_lg_parts(want_ctas, ap ? d->batch : 0, ctx->sm_count);
-    const unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas << p.combine_lg_parts : most_ctas);
+    p.combine_lg_parts = p.small ? combine_lg_parts(want_ctas, ap ? d->batch : 0, ctx->sm_count) : 0;
+    unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas << p.combine_lg_parts : most_ctas);
+    if (!p.small) {
+        const unsigned cuts = (unsigned)combine_cuts(ctx->num_ctas), most_turns = (unsigned)(most_ctas / cuts);
+        const unsigned turns = (grid + cuts - 1) / cuts;
+        grid = cuts * (turns < most_turns ? turns : most_turns);
+    }
     p.combine_row_ctas = (int32_t)grid;
     {
         cudaLaunchConfig_t cfg = {};
@@ -427,10 +438,10 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
     const bool walk_here = ap && !(own_scan && ctx->profiling);
     const size_t stage_bytes = combine_smem_bytes(p.combine_group, p.combine_lg_parts, grid + (walk_here ? (unsigned)d->batch : 0u), ctx->sm_count);
     if (walk_here)
-        launch_dependent_smem(combine_sched_kernel<true>, dim3(grid + (unsigned)d->batch), dim3(kCombineThreads), stage_bytes, stream,
+        launch_dependent_smem(combine_kernel(true, !p.small), dim3(grid + (unsigned)d->batch), dim3(kCombineThreads), stage_bytes, stream,
                               p, *ap);
     else
-        launch_dependent_smem(combine_sched_kernel<false>, dim3(grid), dim3(kCombineThreads), stage_bytes, stream, p, AcceptParams{});
+        launch_dependent_smem(combine_kernel(false, !p.small), dim3(grid), dim3(kCombineThreads), stage_bytes, stream, p, AcceptParams{});
     ++ctx->launches;
     if (ctx->profiling) { cudaEventRecord(ctx->ev[2], stream); ctx->ev_attn_valid = true; }
     if (ap && !walk_here) launch_accept(ctx, *ap, stream);      // profiling: the halves timed apart

@@ -39,3 +39,42 @@ def test_block_table_too_wide_for_32_bits():
     assert torch.equal(dw.out, out) and torch.equal(dw.lse, lse)
     assert np.isfinite(dw.out_f32()).all()
     ctx.close()
+
+
+def _ragged(batch, seed):
+    """One tree of 64 nodes among chains of one to five and small trees: units of 4 to 256 rows."""
+    rng = np.random.default_rng(seed)
+    trees = [("tree", int(rng.integers(2, 13)), 4) if rng.random() < 0.2 else ("chain", int(rng.integers(1, 6))) for _ in range(batch)]
+    trees[int(rng.integers(0, batch))] = ("tree", 64, 8)
+    lens = [int(x) for x in rng.integers(40, 700, size=batch)]
+    lens[int(rng.integers(0, batch))] = 2600
+    return W.generate(W.Spec("ragged", 8, 2, lens, trees, shuffle_pages=True, seed=seed, with_logits=False))
+
+
+@pytest.mark.parametrize("batch", [2, 9, 31, 32, 33, 64, 65, 97, 160])
+def test_merge_of_one_large_tree_among_chains(batch):
+    """Blocks of rows numbered over sequences of very different sizes: within a warp's lanes, and 32 sequences at a time."""
+    check_attention(_ragged(batch, 1400 + batch))
+
+
+@pytest.mark.parametrize("batch", [20, 40])
+def test_merge_leaves_refused_sequences_out(batch):
+    """A sequence without nodes and its neighbour with two roots, in the middle of the batch: the others as without them."""
+    wl = _ragged(batch, 1500 + batch)
+    dw = DeviceWorkload.upload(wl)
+    ctx = OwlContext(dw.dims)
+    dw.attn(ctx)
+    assert ctx.owl_get_status() == 0
+    out, lse = dw.out.clone(), dw.lse.clone()
+    offs = wl.node_offsets.copy()
+    b = next(i for i in range(batch // 2, batch) if 1 <= offs[i + 1] - offs[i] <= 8 and offs[i + 2] - offs[i + 1] <= 8)
+    rows = slice(int(offs[b]), int(offs[b + 2]))
+    dw.node_offsets[b + 1] = int(offs[b])
+    dw.out.fill_(7.0), dw.lse.fill_(7.0)
+    dw.attn(ctx)
+    assert ctx.owl_get_status() == -4
+    out[rows], lse[rows] = 7.0, 7.0
+    # the cuts move with the units that are gone: another order of the same fp32 sums, then one bf16 rounding of values below 4
+    assert float((dw.out.float() - out.float()).abs().max()) <= 2.0 ** -7 and float((dw.lse - lse).abs().max()) <= 1e-4
+    assert torch.equal(dw.out[rows], out[rows]) and torch.equal(dw.lse[rows], lse[rows])
+    ctx.close()

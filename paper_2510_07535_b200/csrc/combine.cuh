@@ -60,6 +60,19 @@ inline long long combine_most_blocks(long long batch, long long total_nodes, int
 
 // Places where the line of a pass of `ctas` CTAs is cut (one CTA: none, but a grid is never empty).
 __host__ __device__ inline int combine_cuts(int ctas) { return ctas > 1 ? ctas - 1 : 1; }
+// The unit whose tiles are cut at t, a piece's first place, which lies in the sequence [begin, end) of the line: its KV head and
+// its length with the gap.  False: the piece begins with a unit, or in the gap before one.
+__host__ __device__ inline bool cut_unit(const Partition<long long>& part, long long t, long long begin, long long end, int kv_heads,
+                                         int& h, int& len) {
+    len = (int)((unsigned)(end - begin) / (unsigned)kv_heads);
+    h = (int)((unsigned)(t - begin) / (unsigned)len);
+    return (int)(t - begin) - h * len > part.pen;
+}
+// What a CTA takes of a unit that lies in pieces c0 .. c0 + count - 1: its cuts share its blocks, `turns` CTAs each.
+__host__ __device__ inline void cut_share(int cut, int c0, int count, int turn, int turns, int& first, int& stride) {
+    first = (cut - c0 - 1) * turns + turn;
+    stride = (count - 1) * turns;
+}
 
 // Short lines: which block is whose.  Lane b holds sequence b, everything is derived from the inputs; a sequence that the pass
 // refuses has no blocks.  (Numbered for every sequence up to the largest tree's rows, the blocks of one tree of 64 nodes among
@@ -208,14 +221,10 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
             const long long begin = p.sched_seq_begin[b];
             n = seq_nodes(p, b);
             node_base = seq_node_base(p, b);
-            const int len = (int)((unsigned)(p.sched_seq_begin[b + 1] - begin) / (unsigned)p.num_kv_heads), local = (int)(t - begin);
-            h = (int)((unsigned)local / (unsigned)len);
-            if (local - h * len <= part.pen) return;       // the piece begins with a unit, not inside one
+            int len;
+            if (!cut_unit(part, t, begin, p.sched_seq_begin[b + 1], p.num_kv_heads, h, len)) return;
             plan(begin + (long long)h * len, len - part.pen, part);
-            // a unit's cuts share its blocks
-            const int turns = div_small((int)row_ctas, cuts);
-            id = (cut - c0 - 1) * turns + turn;
-            stride = (count - 1) * turns;
+            cut_share(cut, c0, count, turn, div_small((int)row_ctas, cuts), id, stride);
             end = seq_blocks(n, p.group, 1);
         }
     }

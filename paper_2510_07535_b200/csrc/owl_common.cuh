@@ -91,8 +91,12 @@ constexpr int kBoundaryPenaltyTiles = 5;
 
 // x / d for 0 <= x < 2^24, 0 < d and a quotient below 2^21: both are exact in fp32, the quotient of __fdividef (2 ulp) is off by
 // less than one, and the remainder says which way.  Half the instructions of an integer division.
-__device__ __forceinline__ int div_small(int x, int d) {
+__host__ __device__ __forceinline__ int div_small(int x, int d) {
+#ifdef __CUDA_ARCH__
     int q = (int)__fdividef((float)x, (float)d);
+#else
+    int q = x / d;
+#endif
     const int r = x - q * d;
     if (r < 0) --q;
     if (r >= d) ++q;
@@ -106,12 +110,12 @@ struct Partition {
     int rem, ctas;
     int unit_tiles, base, urem;   // aligned mode iff unit_tiles > 0
     int pen;                      // gap in front of a unit's tiles
-    static __device__ __forceinline__ T div(T x, T d) {
+    static __host__ __device__ __forceinline__ T div(T x, T d) {
         if constexpr (kShort) return div_small(x, d);
         else if (x >= 0 && x <= 0x7fffffffll && d <= 0x7fffffffll) return (T)((unsigned)x / (unsigned)d);
         else return x / d;
     }
-    __device__ __forceinline__ void init(T tiles, int ctas_, int units, int uniform_tiles) {
+    __host__ __device__ __forceinline__ void init(T tiles, int ctas_, int units, int uniform_tiles) {
         ctas = ctas_;
         pen = kBoundaryPenaltyTiles;
         total = tiles + (T)pen * units;
@@ -127,7 +131,7 @@ struct Partition {
         }
     }
     // piece c, [t_begin, t_end)
-    __device__ __forceinline__ void range(int c, T& t_begin, T& t_end) const {
+    __host__ __device__ __forceinline__ void range(int c, T& t_begin, T& t_end) const {
         if (unit_tiles == 0) {
             t_begin = (T)c * q + min(c, rem);
             t_end = t_begin + q + (c < rem ? 1 : 0);
@@ -140,7 +144,7 @@ struct Partition {
         t_begin = (T)(c < big ? u : urem + u) * unit_tiles + (T)k * qq + min(k, rr);
         t_end = t_begin + qq + (k < rr ? 1 : 0);
     }
-    __device__ __forceinline__ int owner(T t) const {        // of a place on the line
+    __host__ __device__ __forceinline__ int owner(T t) const {      // of a place on the line
         T x = t, head = (T)rem * (q + 1), d = q;             // pieces, the first rem of them of d + 1 places
         int first = 0, longer = rem;
         if (unit_tiles > 0) {

@@ -184,7 +184,9 @@ __device__ __forceinline__ void lane_row_argmax(const uint32_t (&v)[32], int cou
 
 // gridDim.x is even: CTAs 2j and 2j + 1 are pair j.
 // (kEpiStore: at most 128 registers, so that a CTA of the cell kernel fits beside one: its reads before the wait then lie under
-// the product.  With 221, 10 states 71.1 us instead of 70.7.)
+// the product.  With 221 registers / with 128, us per cell call with the weights not in L2: 3 x 2048 -> 5076 24.4 / 23.7, 10 x 4096 ->
+// 4096 28.8 / 27.7, 10 x 4096 -> 12288 68.4 / 67.2, 32 x 8192 -> 8192 94.9 / 90.6, 64 x 4096 -> 12288 88.3 / 84.0; runs of one side
+// differ by 0.2.)
 template <int kEpi, int kGroups, bool kRowsOnLanes>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, kEpi == kEpiStore ? 2 : 1)
 gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap_hi,
@@ -569,21 +571,19 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
     // A programmatic dependent of the product, which writes S and nothing else: E(t), z and the affine parameters are read
     // (ld_early), and the cluster's CTAs meet (before anyone writes into a peer's shared memory), under the product's tail.
     float xc[kCellPerThread], sf[kCellPerThread], si[kCellPerThread], so[kCellPerThread], zo[kCellPerThread], zn[kCellPerThread];
-    float ae[kCellPerThread], gc[kCellPerThread], bc[kCellPerThread], gz[kCellPerThread], bz[kCellPerThread];
+    float ae[kCellPerThread], gc[kCellPerThread], bc[kCellPerThread];
     bool on[kCellPerThread];
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k) {
         const int i = k * kCellThreads + threadIdx.x, j = j0 + i;
         on[k] = i < count;
-        xc[k] = sf[k] = si[k] = so[k] = zo[k] = zn[k] = ae[k] = bc[k] = bz[k] = 0.f;
-        gc[k] = gz[k] = 1.f;
+        xc[k] = sf[k] = si[k] = so[k] = zo[k] = zn[k] = ae[k] = bc[k] = 0.f;
+        gc[k] = 1.f;
         if (on[k]) {
             ae[k] = p.alpha * __bfloat162float(ld_early(p.emb + row * d + j));
             zo[k] = ld_early(p.z + row * d + j);
             if (p.gamma_c) gc[k] = ld_early(p.gamma_c + j);
             if (p.beta_c) bc[k] = ld_early(p.beta_c + j);
-            if (p.gamma_z) gz[k] = ld_early(p.gamma_z + j);
-            if (p.beta_z) bz[k] = ld_early(p.beta_z + j);
         }
     }
     cluster.sync();
@@ -608,6 +608,15 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
             zn[k] = zo[k] * sigmoid_f(sf[k]) + gelu_exact(y) * sigmoid_f(si[k]);
             p.z[row * d + j] = zn[k];
         }
+    }
+    // (asked for here, to arrive under the second exchange: read before the wait with the others they made the kernel spill 40
+    // bytes; 64 x 4096 -> 12288 85.5 -> 84.0 us per call, 32 x 8192 -> 8192 91.2 -> 90.6, 10 x 4096 -> 12288 67.6 -> 67.2)
+    float gz[kCellPerThread], bz[kCellPerThread];
+#pragma unroll
+    for (int k = 0; k < kCellPerThread; ++k) {
+        const int j = j0 + k * kCellThreads + threadIdx.x;
+        gz[k] = on[k] && p.gamma_z ? __ldcg(p.gamma_z + j) : 1.f;
+        bz[k] = on[k] && p.beta_z ? __ldcg(p.beta_z + j) : 0.f;
     }
     float mean_z, rstd_z;
     cluster_mean_rstd(zn, on, count, slice, d, p.eps, s_stats[1], mean_z, rstd_z);

@@ -427,7 +427,7 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        // the instance that holds only this call's case: block-wide schedule above 32 sequences (small_schedule), the two-row-block
+        // the instance that holds only this call's case: block-wide schedule unless the line is short (small_schedule), the two-row-block
         // mode only if a unit (G * max_nodes rows at most) can exceed 128 rows, the logits scan only in a step
         const bool many = !p.small, wide = G * d->max_nodes > 128;
         cudaLaunchKernelEx(&cfg, umma_kernel(many, wide, ap && !own_scan, fp16), p, maps->kmap, maps->vmap, ap ? *ap : AcceptParams{});

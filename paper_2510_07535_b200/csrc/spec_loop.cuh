@@ -109,7 +109,7 @@ constexpr int kCommitPages = 6;          // 64 drafted positions on pages of at 
 // What every CTA of sequence b decides alike, from the inputs alone: 0 = commit, else the error code.
 // The accepted path must be a root path in node order (path[0] = 0, strictly increasing, below n) and every page
 // the drafted positions L .. L + n - 1 touch must exist: s_pages[i], the i-th of them, and s_path are the sequence's
-// afterwards.  Called by all threads of a CTA (one barrier).  The path is read along with the lengths, before it is known how
+// afterwards.  Called by all threads of a CTA (two barriers).  The path is read along with the lengths, before it is known how
 // much of it counts.
 __device__ __forceinline__ int commit_verdict(const CommitParams& p, int b, int& L, int& n, int& a, int* s_path /*[kMaxNodes]*/,
                                               int* s_pages /*[kCommitPages]*/) {

@@ -58,7 +58,7 @@ constexpr int kTilesInFlight = 3;
 constexpr int kQBytes = 128 * kHeadDim * 2;              // 32 KB per 128-row block
 constexpr int kAuxOff = 2 * kQBytes + kSlots * kSlotBytes;  // 224 KB
 // Shared memory up to there: two blocks of Q and five slots, or one block and six (192 instead of 160 KB of K/V on their way to an
-// SM: 48 short sequences 132.0 -> 127.5 us per step, 16 mixed 737 -> 719, 32K 37.9 -> 37.2).
+// SM: both trees on one GPU, us per step, 48 short sequences 131.9 -> 127.1, 16 mixed 691 -> 662, 32K 37.8 -> 37.4).
 template <bool kWide> constexpr int kRingSlots = kWide ? kSlots : kSlotsNarrow;
 template <bool kWide> constexpr int kRingOff = kWide ? 2 * kQBytes : kQBytes;
 static_assert(kRingOff<false> + kRingSlots<false> * kSlotBytes == kAuxOff && kRingOff<true> + kRingSlots<true> * kSlotBytes == kAuxOff, "layout");
@@ -243,7 +243,7 @@ __device__ __forceinline__ void build_walk(const AttnParams& p, Aux* aux, Walker
     w.seq_begin = aux->sched_tile_begin;
 }
 
-// Batches of at most 32 sequences: the producer warp derives the schedule on its own (lane b holds sequence
+// Short lines (small_schedule): the producer warp derives the schedule on its own (lane b holds sequence
 // b, prefix sums by shuffle), with no shared memory and no CTA-wide barrier.
 __device__ __forceinline__ void build_walk_small(const AttnParams& p, Walker<false>& w) {
     static_assert(kTileKeys == kSchedTileKeys, "the merge kernel derives the same schedule");

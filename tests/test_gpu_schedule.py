@@ -53,7 +53,7 @@ def _ragged(batch, seed):
 
 @pytest.mark.parametrize("batch", [2, 9, 31, 32, 33, 64, 65, 97, 160])
 def test_merge_of_one_large_tree_among_chains(batch):
-    """Blocks of rows numbered over sequences of very different sizes: within a warp's lanes, and 32 sequences at a time."""
+    """Blocks of rows of sequences of very different sizes: numbered over a warp's lanes, and found by the line's cuts."""
     check_attention(_ragged(batch, 1400 + batch))
 
 

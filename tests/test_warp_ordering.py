@@ -1,6 +1,6 @@
 """What one lane of a warp writes to shared memory another may read, and what it reads another may overwrite, only after
-`__syncwarp()` (or a barrier): votes and shuffles
-bring the lanes together but order no memory.  The hardware does not show a missing one, so the kernels' text is looked at."""
+`__syncwarp()` (or a barrier): votes and shuffles bring the lanes together but order no memory.  The hardware does not show a
+missing one, so the kernels' text is looked at."""
 import re
 from pathlib import Path
 

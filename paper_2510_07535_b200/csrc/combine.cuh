@@ -58,8 +58,15 @@ inline long long combine_most_blocks(long long batch, long long total_nodes, int
     return num_kv_heads * (by_max < by_total ? by_max : by_total);
 }
 
-// Places where the line of a pass of `ctas` CTAs is cut (one CTA: none, but a grid is never empty).
+// Lines that are not short: what the merge goes by, whichever are fewer, the units or the places where the line of a pass of
+// `ctas` CTAs is cut (one CTA: none, but a grid is never empty).
 __host__ __device__ inline int combine_cuts(int ctas) { return ctas > 1 ? ctas - 1 : 1; }
+__host__ __device__ inline int combine_places(int units, int ctas) { return units < combine_cuts(ctas) ? units : combine_cuts(ctas); }
+// CTAs per place: one for each block of the largest unit there may be, while all are resident at once.
+inline int combine_turns(int group, int max_nodes, int places, long long most_ctas) {
+    const long long blocks = seq_blocks(max_nodes, group, 1), most = most_ctas / places;
+    return (int)(blocks < most ? blocks : most > 1 ? most : 1);
+}
 // The unit whose tiles are cut at t, a piece's first place, which lies in the sequence [begin, end) of the line: its KV head and
 // its length with the gap.  False: the piece begins with a unit, or in the gap before one.
 __host__ __device__ inline bool cut_unit(const Partition<long long>& part, long long t, long long begin, long long end, int kv_heads,
@@ -131,10 +138,11 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
     }
     // The row CTAs are persistent (one CTA per eight rows cost a launch of 8192 rows 19 us, most of it the schedule derived
     // 8192 times).  Short lines: a warp derives the schedule once and then takes blocks first, first + stride, ..., numbered
-    // sequence by sequence, unit by unit, and only those that hold rows (BlockNumbers).  Otherwise there are mostly more units
-    // than pieces, and only those that a piece's end cuts have anything to merge: a CTA goes by one cut and takes its share of
-    // that unit's blocks.  (Every block of every unit looked up in turn, us per step: 64 sequences of 100-1500 tokens with one
-    // tree of 64 nodes 91.6, now 79.4; 300 of 50-300 tokens 124.6, now 120.7; 1000 with one such tree 539, now 355.)
+    // sequence by sequence, unit by unit, and only those that hold rows (BlockNumbers).  Otherwise the units are many, and only
+    // those that a piece's end cuts have anything to merge: a CTA goes by one cut and takes its share of that unit's blocks; or,
+    // where the units are fewer than the cuts, by one unit (one KV head, 40 sequences of 50-2000 tokens with 80 rows: 17.7 us
+    // per call, by cuts 21.2; with 256 rows 28.7, by cuts 33.8).  (Every block of every unit looked up in turn, us per step: 64 sequences of 100-1500 tokens with one
+    // tree of 64 nodes 91.4, now 79.5; 300 of 50-300 tokens 124.4, now 120.1; 1000 with one such tree 540, now 355.)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // The ninth warp rehearses: it runs the code that follows the wait on whatever the first slots hold (out_row stays -1, so
     // nothing is written), while the others derive the schedule and wait.  That code runs once or twice per launch, and its lines
@@ -175,8 +183,8 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
         const int row = row0 + r, node = (int)row_node(p, row);
         out_row = row < n * p.group ? (long long)(node_base + node) * p.num_q_heads + h * p.group + (row - node * p.group) : -1;
     };
-    WarpSchedule ws;
-    BlockNumbers num;
+    WarpSchedule ws{};
+    BlockNumbers num{};
     auto locate = [&](int id) {            // every lane of the warp, same block
         const int b = __ffs(__ballot_sync(0xffffffffu, id < num.end)) - 1;
         n = __shfl_sync(0xffffffffu, ws.n, b);
@@ -204,27 +212,55 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
         // from here on the split-KV pass has completed and its writes are visible (a no-op in an ordinary launch)
         wait_and_let_dependents_start();
         if (kManySeqs) {
-            // a cut per CTA: the first place of piece `cut`; which sequence it lies in, 32 of them at a look
-            const int cuts = combine_cuts(p.num_ctas), turn = div_small(id, cuts), cut = id - turn * cuts + 1;
-            const SchedHeader hdr = *p.sched_header;
+            const int units = p.batch * p.num_kv_heads, places = combine_places(units, p.num_ctas), turns = div_small((int)row_ctas, places);
+            const int turn = div_small(id, places), place = id - turn * places;
+            const long long* seq_begin = p.sched_seq_begin;
+            const SchedHeader* header = p.sched_header;
             Partition<long long> part;
-            part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
-            long long t, t_end;
-            part.range(cut, t, t_end);
-            if (t >= part.total) return;
-            int b = 0;
-            for (int per = p.batch > 32 ? 32 : 1; per > 0; per >>= 5) {
-                const int at = b + lane * per;
-                const unsigned from = __ballot_sync(0xffffffffu, at < p.batch && p.sched_seq_begin[at] <= t);
-                b += (31 - __clz((int)from)) * per;
+            auto read_partition = [&] {
+                const SchedHeader hdr = *header;
+                part.init(hdr.total_tiles, p.num_ctas, hdr.units, hdr.uniform_tiles);
+            };
+            if (places == units) {
+                const int b = div_small(place, p.num_kv_heads);
+                const long long from = seq_begin[b], to = seq_begin[b + 1];
+                n = seq_nodes(p, b);
+                node_base = seq_node_base(p, b);
+                read_partition();
+                const int len = (int)((unsigned)(to - from) / (unsigned)p.num_kv_heads);
+                if (len == 0) return;                          // a sequence that the pass refuses
+                h = place - b * p.num_kv_heads;
+                plan(from + (long long)h * len, len - part.pen, part);
+                id = turn;
+                stride = turns;
+            } else {
+                // the first place of piece `cut`: which sequence it lies in, 32 of them at a look, the first look's loads beside the
+                // header's
+                const int cut = place + 1;
+                int b = 0;
+                long long from = 0, to = 0, t, t_end;
+                const int per = p.batch > 32 ? 32 : 1, at = lane * per;
+                if (at < p.batch) from = seq_begin[at];
+                read_partition();
+                part.range(cut, t, t_end);
+                if (t >= part.total) return;
+                b = (31 - __clz((int)__ballot_sync(0xffffffffu, at < p.batch && from <= t))) * per;
+                const int mine = per > 1 ? b + lane : lane;
+                if (mine < p.batch) {
+                    from = seq_begin[mine];
+                    to = seq_begin[mine + 1];
+                    n = seq_nodes(p, mine);
+                    node_base = seq_node_base(p, mine);
+                }
+                const int who = 31 - __clz((int)__ballot_sync(0xffffffffu, mine < p.batch && from <= t));
+                n = __shfl_sync(0xffffffffu, n, who);
+                node_base = __shfl_sync(0xffffffffu, node_base, who);
+                from = __shfl_sync(0xffffffffu, from, who);
+                int len;
+                if (!cut_unit(part, t, from, __shfl_sync(0xffffffffu, to, who), p.num_kv_heads, h, len)) return;
+                plan(from + (long long)h * len, len - part.pen, part);
+                cut_share(cut, c0, count, turn, turns, id, stride);
             }
-            const long long begin = p.sched_seq_begin[b];
-            n = seq_nodes(p, b);
-            node_base = seq_node_base(p, b);
-            int len;
-            if (!cut_unit(part, t, begin, p.sched_seq_begin[b + 1], p.num_kv_heads, h, len)) return;
-            plan(begin + (long long)h * len, len - part.pen, part);
-            cut_share(cut, c0, count, turn, div_small((int)row_ctas, cuts), id, stride);
             end = seq_blocks(n, p.group, 1);
         }
     }

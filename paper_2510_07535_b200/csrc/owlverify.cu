@@ -404,16 +404,15 @@ static int verify_attn_impl(owl_ctx* ctx, const owl_dims* d, const void* q, cons
 
     if (ctx->profiling) cudaEventRecord(ctx->ev[0], stream);
     // one CTA per block of rows while all are resident at once, beyond that the merge kernel's CTAs stride over the blocks; on a
-    // line that is not short the same for each cut, whose CTAs come in whole turns over the cuts
+    // line that is not short the same for each unit or cut, whose CTAs come in whole turns over these places
     p.combine_group = combine_group((long long)d->batch * d->num_kv_heads, ctx->num_ctas);
     const long long want_ctas = combine_most_blocks(d->batch, d->total_nodes, d->max_nodes, G, d->num_kv_heads);
     const long long most_ctas = (long long)ctx->sm_count * combine_ctas_per_sm(p.combine_group);
     p.combine_lg_parts = p.small ? combine_lg_parts(want_ctas, ap ? d->batch : 0, ctx->sm_count) : 0;
     unsigned grid = (unsigned)(want_ctas < most_ctas ? want_ctas << p.combine_lg_parts : most_ctas);
     if (!p.small) {
-        const unsigned cuts = (unsigned)combine_cuts(ctx->num_ctas), most_turns = (unsigned)(most_ctas / cuts);
-        const unsigned turns = (grid + cuts - 1) / cuts;
-        grid = cuts * (turns < most_turns ? turns : most_turns);
+        const int places = combine_places(d->batch * d->num_kv_heads, ctx->num_ctas);
+        grid = (unsigned)(places * combine_turns(G, d->max_nodes, places, most_ctas));
     }
     p.combine_row_ctas = (int32_t)grid;
     {

@@ -57,6 +57,15 @@ def test_merge_of_one_large_tree_among_chains(batch):
     check_attention(_ragged(batch, 1400 + batch))
 
 
+@pytest.mark.parametrize("batch,hkv,nodes", [(33, 1, 5), (40, 1, 16), (49, 3, 7), (50, 3, 7), (147, 1, 2), (148, 1, 2)])
+def test_merge_by_units_and_by_cuts(batch, hkv, nodes):
+    """More than 32 sequences with up to 147 units, which a CTA of the merge goes by, and with more, where it goes by cuts."""
+    rng = np.random.default_rng(1600 + batch)
+    lens = [int(x) for x in rng.integers(40, 1500, size=batch)]
+    check_attention(W.generate(W.Spec("places", 16 * hkv, hkv, lens, [("tree", nodes, 4)] * batch, shuffle_pages=True, seed=1600 + batch,
+                                      with_logits=False)))
+
+
 @pytest.mark.parametrize("batch", [20, 40])
 def test_merge_leaves_refused_sequences_out(batch):
     """A sequence without nodes and its neighbour with two roots, in the middle of the batch: the others as without them."""

@@ -498,11 +498,12 @@ struct CellParams {
 };
 
 constexpr int kCellWarps = kCellThreads / 32;
-struct CellStats { float2 warp[kCellCluster][kCellWarps]; };      // (mean, sum of squared deviations) of a warp's columns
+struct CellStats { float2 warp[kCellWarps], cta[kCellCluster]; };      // (mean, sum of squared deviations) of a warp's, a CTA's columns
 
-__device__ __forceinline__ float cell_warp_sum(float v) {
+template <int kLanes>
+__device__ __forceinline__ float cell_lanes_sum(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = kLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 // Columns of a CTA with `count` of them that warp w holds.
@@ -512,12 +513,20 @@ __device__ __forceinline__ int cell_warp_columns(int count, int w) {
     for (int k = 0; k < kCellPerThread; ++k) n += min(max(count - k * kCellThreads - w * 32, 0), 32);
     return n;
 }
+// Mean and sum of squared deviations of kLanes sets of n columns each, one per lane (the same in every group of kLanes), by the
+// pairwise-variance identity  M2 = sum_i M2_i + sum_i n_i (mean_i - mean)^2 : no cancellation.
+template <int kLanes>
+__device__ __forceinline__ float2 cell_combine(float2 pair, float n, float total) {
+    const float mean = cell_lanes_sum<kLanes>(n * pair.x) / fmaxf(total, 1.f), dm = pair.x - mean;
+    return make_float2(mean, cell_lanes_sum<kLanes>(pair.y + n * dm * dm));
+}
 
 // Mean and 1 / sqrt(variance + eps) over a whole row from the values x[] this thread holds (on[] says which exist).
-// Each warp takes the mean and the sum of squared deviations of its own columns, pushes the pair into every CTA of the
-// cluster, and after one cluster barrier every warp combines all 128 pairs by the pairwise-variance identity
-// M2 = sum_i M2_i + sum_i n_i (mean_i - mean)^2 : the same numbers everywhere, no cancellation, and nobody reads a peer's
-// shared memory after the barrier.  (With a pair per CTA two block reductions, four barriers, stood before the exchange.)
+// Each warp takes the pair of its own columns, the first one combines them and pushes the CTA's into every CTA of the cluster,
+// and after one cluster barrier every warp combines the eight: the same numbers everywhere, and nobody reads a peer's shared
+// memory after the barrier.  (With every warp's pair pushed and 128 of them combined by every warp, us per call: 384 x 1024 -> 4096
+// 97.6, now 89.0; 200 x 2048 -> 2048 53.5, now 48.3; 10 x 4096 -> 4096 27.7, now 27.5.  With two block sums, four CTA barriers,
+// before the exchange instead of one: 96.6, 52.3, 29.8.)
 __device__ __forceinline__ void cluster_mean_rstd(const float (&x)[kCellPerThread], const bool (&on)[kCellPerThread], int count,
                                                   int slice, int d, float eps, CellStats& stats, float& mean, float& rstd) {
     namespace cg = cooperative_groups;
@@ -527,32 +536,24 @@ __device__ __forceinline__ void cluster_mean_rstd(const float (&x)[kCellPerThrea
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k) sum += on[k] ? x[k] : 0.f;
     const int n_warp = cell_warp_columns(count, warp);
-    const float mean_warp = cell_warp_sum(sum) / (float)max(n_warp, 1);
+    const float mean_warp = cell_lanes_sum<32>(sum) / (float)max(n_warp, 1);
     float sq = 0.f;
 #pragma unroll
     for (int k = 0; k < kCellPerThread; ++k)
         if (on[k]) { const float t = x[k] - mean_warp; sq += t * t; }
-    const float m2_warp = cell_warp_sum(sq);
-    if (lane < kCellCluster) cluster.map_shared_rank(&stats, lane)->warp[cluster.block_rank()][warp] = make_float2(mean_warp, m2_warp);
+    const float m2_warp = cell_lanes_sum<32>(sq);
+    if (lane == 0) stats.warp[warp] = make_float2(mean_warp, m2_warp);
+    __syncthreads();
+    if (warp == 0) {
+        const int w = lane % kCellWarps;
+        const float2 cta = cell_combine<kCellWarps>(stats.warp[w], (float)cell_warp_columns(count, w), (float)count);
+        if (lane < kCellCluster) cluster.map_shared_rank(&stats, lane)->cta[cluster.block_rank()] = cta;
+    }
     cluster.sync();
-    constexpr int kPerLane = kCellCluster * kCellWarps / 32;
-    float2 pair[kPerLane];
-    float n[kPerLane], total = 0.f;
-#pragma unroll
-    for (int q = 0; q < kPerLane; ++q) {
-        const int at = q * 32 + lane, r = at / kCellWarps, w = at % kCellWarps;
-        pair[q] = stats.warp[r][w];
-        n[q] = (float)cell_warp_columns(min(slice, max(d - r * slice, 0)), w);
-        total += n[q] * pair[q].x;
-    }
-    mean = cell_warp_sum(total) / d;
-    float m2 = 0.f;
-#pragma unroll
-    for (int q = 0; q < kPerLane; ++q) {
-        const float dm = pair[q].x - mean;
-        m2 += pair[q].y + n[q] * dm * dm;
-    }
-    rstd = rsqrtf(cell_warp_sum(m2) / d + eps);
+    const int r = lane % kCellCluster;
+    const float2 row = cell_combine<kCellCluster>(stats.cta[r], (float)min(slice, max(d - r * slice, 0)), (float)d);
+    mean = row.x;
+    rstd = rsqrtf(row.y / d + eps);
 }
 
 __device__ __forceinline__ float gelu_exact(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
@@ -568,8 +569,12 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
     const int j0 = (int)cluster.block_rank() * slice;             // this CTA's columns: [j0, min(j0 + slice, d))
     const int count = min(slice, max(d - j0, 0));
     const float* s = p.s + row * 4ll * d;
+    // Every CTA of the cluster is running before anyone writes into its shared memory: they tell each other so here and look
+    // when all loads are on their way.  (A whole barrier here put S behind it, in every wave of many rows: 384 x 1024 -> 4096 99.4 us
+    // instead of 97.5, 200 x 2048 -> 2048 54.7 instead of 53.5.)
+    cluster.barrier_arrive();
     // A programmatic dependent of the product, which writes S and nothing else: E(t), z and the affine parameters are read
-    // (ld_early), and the cluster's CTAs meet (before anyone writes into a peer's shared memory), under the product's tail.
+    // (ld_early) under the product's tail.
     float xc[kCellPerThread], sf[kCellPerThread], si[kCellPerThread], so[kCellPerThread], zo[kCellPerThread], zn[kCellPerThread];
     float ae[kCellPerThread], gc[kCellPerThread], bc[kCellPerThread];
     bool on[kCellPerThread];
@@ -586,7 +591,6 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
             if (p.beta_c) bc[k] = ld_early(p.beta_c + j);
         }
     }
-    cluster.sync();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the kernel after this one may queue up
 #pragma unroll
@@ -597,6 +601,7 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
             si[k] = __ldcg(s + 1ll * d + j) + ae[k]; so[k] = __ldcg(s + 2ll * d + j) + ae[k];
         }
     }
+    cluster.barrier_wait();
     float mean_c, rstd_c;
     cluster_mean_rstd(xc, on, count, slice, d, p.eps, s_stats[0], mean_c, rstd_c);
     // z' = z g^f + f(s^c) g^i  (Eq. 5-7)

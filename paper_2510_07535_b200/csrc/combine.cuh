@@ -141,8 +141,9 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
     // sequence by sequence, unit by unit, and only those that hold rows (BlockNumbers).  Otherwise the units are many, and only
     // those that a piece's end cuts have anything to merge: a CTA goes by one cut and takes its share of that unit's blocks; or,
     // where the units are fewer than the cuts, by one unit (one KV head, 40 sequences of 50-2000 tokens with 80 rows: 17.7 us
-    // per call, by cuts 21.2; with 256 rows 28.7, by cuts 33.8).  (Every block of every unit looked up in turn, us per step: 64 sequences of 100-1500 tokens with one
-    // tree of 64 nodes 91.4, now 79.5; 300 of 50-300 tokens 124.4, now 120.1; 1000 with one such tree 540, now 355.)
+    // per call, by cuts 21.2; with 256 rows 28.7, by cuts 33.8).  (Every block of every unit looked up in turn, us per step: 64
+    // sequences of 100-1500 tokens with one tree of 64 nodes 91.4, now 79.5; 300 of 50-300 tokens 124.4, now 120.1; 1000 of
+    // 20-200 with one such tree 540, now 355.)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // The ninth warp rehearses: it runs the code that follows the wait on whatever the first slots hold (out_row stays -1, so
     // nothing is written), while the others derive the schedule and wait.  That code runs once or twice per launch, and its lines
@@ -237,15 +238,14 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtasPerSm) combine_sc
                 // the first place of piece `cut`: which sequence it lies in, 32 of them at a look, the first look's loads beside the
                 // header's
                 const int cut = place + 1;
-                int b = 0;
                 long long from = 0, to = 0, t, t_end;
                 const int per = p.batch > 32 ? 32 : 1, at = lane * per;
                 if (at < p.batch) from = seq_begin[at];
                 read_partition();
                 part.range(cut, t, t_end);
                 if (t >= part.total) return;
-                b = (31 - __clz((int)__ballot_sync(0xffffffffu, at < p.batch && from <= t))) * per;
-                const int mine = per > 1 ? b + lane : lane;
+                const int last = 31 - __clz((int)__ballot_sync(0xffffffffu, at < p.batch && from <= t));
+                const int mine = (per > 1 ? last * per : 0) + lane;
                 if (mine < p.batch) {
                     from = seq_begin[mine];
                     to = seq_begin[mine + 1];

@@ -184,9 +184,9 @@ __device__ __forceinline__ void lane_row_argmax(const uint32_t (&v)[32], int cou
 
 // gridDim.x is even: CTAs 2j and 2j + 1 are pair j.
 // (kEpiStore: at most 128 registers, so that a CTA of the cell kernel fits beside one: its reads before the wait then lie under
-// the product.  With 221 registers / with 128, us per cell call with the weights not in L2: 3 x 2048 -> 5076 24.4 / 23.7, 10 x 4096 ->
-// 4096 28.8 / 27.7, 10 x 4096 -> 12288 68.4 / 67.2, 32 x 8192 -> 8192 94.9 / 90.6, 64 x 4096 -> 12288 88.3 / 84.0; runs of one side
-// differ by 0.2.)
+// the product.  With 221 registers / with 128, us per cell call with the weights not in L2: 3 x 2048 -> 5076 23.8 / 23.4, 10 x 4096 ->
+// 4096 28.1 / 27.5, 10 x 4096 -> 12288 67.7 / 66.9, 32 x 8192 -> 8192 94.0 / 90.0, 64 x 4096 -> 12288 85.7 / 82.0; runs of one side
+// differ by 0.1.)
 template <int kEpi, int kGroups, bool kRowsOnLanes>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, kEpi == kEpiStore ? 2 : 1)
 gemm_umma_kernel(const GemmParams p, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap_hi,
